@@ -42,6 +42,7 @@
 
 #include "devutil.cuh"
 #include "internal.h"
+#include "lookback.cuh"
 #include "runtime.h"
 
 namespace lx {
@@ -76,11 +77,10 @@ struct Geo {
 };
 constexpr uint32_t SPARSE_LIMIT = Geo<0>::LIMIT;
 constexpr uint32_t SPILL_CAP = Geo<DENSE>::LIMIT;   // spill slot entries per warp: a tile's kept tokens, at most
-constexpr uint32_t GS = 64;                   // tiles per look-back group
 constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t BIG = 0x7FFFFFFFu;
 constexpr int MAX_WARPS = 20;                 // warps per CTA at most (as many as shared memory allows)
-constexpr unsigned ERR_TIMEOUT = 1u;
+constexpr unsigned ERR_TIMEOUT = ERR_TIMEOUT_BIT;
 constexpr unsigned ERR_SMEM = 2u;
 constexpr unsigned ERR_SPARSE = 4u;   // a chunk ran past the sparse limit: certified bytes too far apart
 constexpr unsigned ERR_LOOKAHEAD = 8u;   // backtracking past its step budget (failed lookahead)
@@ -131,8 +131,8 @@ struct WParams {
     uint64_t cap;
     uint32_t *spill;               // SPILL_CAP stage entries per warp of the grid
     unsigned long long *status;    // per tile: ST_AGG | kept count
-    unsigned long long *gstatus;   // per group of GS tiles: ST_AGG | group count, or ST_INCL | inclusive prefix
-    unsigned int *gdone;           // per group: tiles that have published
+    unsigned long long *gagg;      // per group of GS tiles: its tiles' counts (lookback.cuh)
+    unsigned long long *ginc;      // per group: ST_INCL | inclusive prefix
     unsigned int *tile_counter;
     WResult *res;
     uint32_t n_tiles;
@@ -145,6 +145,10 @@ struct WParams {
     WDocRes *dres;
     uint32_t sets_off;          // WSet array in the table blob
     uint32_t n_ctx;             // split-window context classes of the table (0: none)
+    // look-back (lookback.cuh)
+    static constexpr unsigned long long COUNT = (1ull << GW_SHIFT) - 1;
+    static constexpr bool SMALL = false;
+    __device__ unsigned int *error() const { return &res->error; }
 };
 
 // Shared addresses of the tables and of this warp's buffers, and the tile.
@@ -548,137 +552,11 @@ __device__ __forceinline__ uint32_t event_mask(uint32_t w)  // bit 7 of every no
     return (((w | 0x80808080u) - 0x01010101u) | w) & 0x80808080u;
 }
 
-// ---- two-level decoupled look-back ----
-// Tiles form groups of GS.  A tile publishes its kept count (ST_AGG) and
-// counts itself into its group; the warp that completes a group sums the
-// group's counts and publishes the group aggregate (group 0: its inclusive
-// prefix).  A tile's output offset is the exclusive prefix of its group
-// (a look-back over group words, a few dozen deep) plus the counts of the
-// tiles before it in the group.  Every wait is bounded by the time budget
-// and ends early once another warp has given up.
-// Polls back off exponentially (64 ns doubling to 4 us): while one slow tile
-// (say, a chunk walked byte by byte) holds up its group, thousands of waiting
-// warps must not flood L2 with status reads and starve that tile's own loads.
-struct Waiter {
-    uint64_t t0;
-    uint32_t spins;
-    // false (and the error flag raised) once the budget is spent
-    __device__ bool again(const WParams &P)
-    {
-        if ((++spins & 3) == 0 &&
-            (globaltimer() - t0 > P.timeout_ns || *(volatile const unsigned int *)&P.res->error != 0)) {
-            if ((threadIdx.x & 31) == 0) atomicOr(&P.res->error, ERR_TIMEOUT);
-            return false;
-        }
-        __nanosleep(64u << min(spins, 6u));
-        return true;
-    }
-};
-
+// The tile's kept count for the look-back (lookback.cuh).
 __device__ void publish_tile(const WParams &P, uint32_t tile, uint64_t agg)
 {
-    const int lane = threadIdx.x & 31;
-    const uint32_t g = tile / GS, f = g * GS;
-    const uint32_t gsize = min(GS, P.n_tiles - f);
-    uint32_t last = 0;
-    if (lane == 0 && agg) atomicAdd(&P.res->total, agg);
-    if (lane == 0 && tile != P.withhold) {
-        st_status(&P.status[tile], ST_AGG | agg);
-        // release: the status store before the count; acquire: the group's
-        // other status stores visible to the warp that completes it
-        uint32_t old;
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&P.gdone[g]) : "memory");
-        last = old + 1 == gsize ? 1u : 0u;
-    }
-    if (!__shfl_sync(0xffffffffu, last, 0)) return;
-    __threadfence();   // every lane reads the statuses lane 0's acquire made visible
-    // every tile of the group has published: its aggregate
-    unsigned long long x = 0;
-    for (uint32_t j = lane; j < gsize; j += 32) x += ld_status(&P.status[f + j]) & ST_VAL;
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) st_status(&P.gstatus[g], (g == 0 ? ST_INCL : ST_AGG) | x);
-}
-
-// Lane 0 waits until status word *p is published; the warp learns whether
-// the wait ended in time.  Only one word is polled: thousands of waiting warps
-// re-reading whole rounds of status words would crowd the L2 lines that
-// every warp reads and slow the very tile they wait for.
-__device__ bool wait_word(const WParams &P, Waiter &W, const unsigned long long *p)
-{
-    uint32_t ok = 1;
-    if ((threadIdx.x & 31) == 0)
-        while (ld_status(p) == 0)
-            if (!W.again(P)) {
-                ok = 0;
-                break;
-            }
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
-
-// The output offset of `tile`; false when a wait ran out of time.
-__device__ bool resolve_tile(const WParams &P, uint32_t tile, uint64_t &G)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t g = tile / GS, f = g * GS;
-    Waiter W{globaltimer(), 0};
-    // the tiles before this one in its group (at most GS - 1 < 64 words)
-    unsigned long long w = 0;
-    for (;;) {
-        uint32_t miss = NONE;
-        w = 0;
-        for (uint32_t j = f + lane; j < tile; j += 32) {
-            const unsigned long long v = ld_status(&P.status[j]);
-            if (v == 0) miss = min(miss, j);
-            w += v & ST_VAL;
-        }
-        miss = __reduce_min_sync(0xffffffffu, miss);
-        if (miss == NONE) break;
-        if (!wait_word(P, W, &P.status[miss])) return false;
-    }
-    for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    // the groups before: sum aggregates back to the nearest inclusive prefix
-    uint64_t GE = 0;
-    int64_t base = (int64_t)g - 1;
-    while (base >= 0) {
-        unsigned long long v[LB_PER_LANE];
-#pragma unroll
-        for (int j = 0; j < LB_PER_LANE; j++) {
-            const int64_t k = base - (int64_t)LB_PER_LANE * lane - j;
-            v[j] = k >= 0 ? ld_status(&P.gstatus[k]) : ST_INCL;
-        }
-        int jstar = LB_PER_LANE;
-        uint32_t zk = NONE;   // an unpublished group word of this lane before its first inclusive one
-        unsigned long long lsum = 0;
-#pragma unroll
-        for (int j = 0; j < LB_PER_LANE; j++) {
-            if (jstar == LB_PER_LANE) {
-                const unsigned long long fl = v[j] & ~ST_VAL;
-                if (fl == 0 && zk == NONE) zk = (uint32_t)(base - (int64_t)LB_PER_LANE * lane - j);
-                lsum += v[j] & ST_VAL;
-                if (fl == ST_INCL) jstar = j;
-            }
-        }
-        const unsigned incl = __ballot_sync(0xffffffffu, jstar < LB_PER_LANE);
-        const unsigned upto = incl ? (incl & (0u - incl)) : 0u;
-        const unsigned lanes = incl ? ((upto - 1u) | upto) : 0xffffffffu;
-        const uint32_t wait_k = __reduce_min_sync(0xffffffffu, ((lanes >> lane) & 1u) ? zk : NONE);
-        if (wait_k != NONE) {
-            if (!wait_word(P, W, &P.gstatus[wait_k])) return false;
-            continue;
-        }
-        unsigned long long x = ((lanes >> lane) & 1u) ? lsum : 0ull;
-        for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        GE += x;
-        if (incl) break;
-        base -= 32 * LB_PER_LANE;
-    }
-    // once the group is complete, its inclusive prefix shortens later look-backs
-    if (lane == 0 && g > 0) {
-        const unsigned long long gv = ld_status(&P.gstatus[g]);
-        if ((gv & ~ST_VAL) == ST_AGG) st_status(&P.gstatus[g], ST_INCL | (GE + (gv & ST_VAL)));
-    }
-    G = GE + w;
-    return true;
+    if ((threadIdx.x & 31) == 0 && agg) atomicAdd(&P.res->total, agg);
+    publish_word(P, tile, agg);
 }
 
 // A tile whose tokens wait in the warp's stage for their output offset.
@@ -886,6 +764,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_warps(WParams P)
     const uint32_t ahead = gridDim.x * (blockDim.x / 32);   // tiles the other warps take meanwhile
 
     Pending pend{NONE, 0, NONE64, 0, 0, 0, 0};
+    unsigned long long before;   // (the status word before a resolved tile: not used here)
     for (;;) {
         uint32_t tile = 0;
         if (lane == 0) {
@@ -1069,7 +948,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_warps(WParams P)
         // the previous tile's output: its predecessors have had a whole tile to publish
         if (pend.tile != NONE) {
             uint64_t G = 0;
-            if (!resolve_tile(P, pend.tile, G)) break;
+            if (!resolve_tile(P, pend.tile, G, before)) break;
             report_failure<BATCH>(P, pend.tile, pend.fail, G, pend.agg, pend.doc, pend.dtile);
             copy_stage<dense ? 4 : 2>(P, pend.kmap_s, stage, spill, dense ? pend.staged >> 16 : STAGE_CAP,
                        dense ? pend.staged & 0xFFFFu : pend.staged, G);
@@ -1083,7 +962,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_warps(WParams P)
         uint64_t G = 0;
         uint32_t split = STAGE_CAP;   // dense: how many kept tokens are in the stage (the rest: spill slot)
         if (!defer) {   // rare: a chunk past the halo is written at once
-            if (!resolve_tile(P, tile, G)) break;
+            if (!resolve_tile(P, tile, G, before)) break;
             report_failure<BATCH>(P, tile, fpos, G, agg, doc, dtile);
         }
         if (c0 != NONE) {
@@ -1172,7 +1051,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_warps(WParams P)
     }
     if (pend.tile != NONE) {
         uint64_t G = 0;
-        if (resolve_tile(P, pend.tile, G)) {
+        if (resolve_tile(P, pend.tile, G, before)) {
             report_failure<BATCH>(P, pend.tile, pend.fail, G, pend.agg, pend.doc, pend.dtile);
             copy_stage<dense ? 4 : 2>(P, pend.kmap_s, stage, spill, dense ? pend.staged >> 16 : STAGE_CAP,
                        dense ? pend.staged & 0xFFFFu : pend.staged, G);
@@ -1342,8 +1221,8 @@ int warp_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     L.grid = (uint32_t)std::min<uint64_t>((uint64_t)occ * c->num_sms, (n_tiles + L.nwarps - 1) / L.nwarps);
 
     const uint32_t n_groups = (n_tiles + GS - 1) / GS;
-    const size_t o_gstatus = 64 + 8 * (size_t)n_tiles, o_gdone = o_gstatus + 8 * (size_t)n_groups;
-    L.need = o_gdone + 4 * (size_t)n_groups;   // zeroed per call
+    const size_t o_gagg = 64 + 8 * (size_t)n_tiles, o_ginc = o_gagg + 8 * (size_t)n_groups;
+    L.need = o_ginc + 8 * (size_t)n_groups;   // zeroed per call
     rc = grow(&c->scratch, &c->scratch_bytes, L.need);
     if (rc != LX_OK) return rc;
     uint8_t *scr = static_cast<uint8_t *>(c->scratch);
@@ -1371,8 +1250,8 @@ int warp_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     P.res = reinterpret_cast<WResult *>(scr);
     P.tile_counter = reinterpret_cast<unsigned int *>(scr + sizeof(WResult));
     P.status = reinterpret_cast<unsigned long long *>(scr + 64);
-    P.gstatus = reinterpret_cast<unsigned long long *>(scr + o_gstatus);
-    P.gdone = reinterpret_cast<unsigned int *>(scr + o_gdone);
+    P.gagg = reinterpret_cast<unsigned long long *>(scr + o_gagg);
+    P.ginc = reinterpret_cast<unsigned long long *>(scr + o_ginc);
     P.n_tiles = n_tiles;
     P.timeout_ns = c->timeout_ns;
     P.withhold = c->withhold;
@@ -1698,8 +1577,8 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
 
     // device scratch: [zeroed: record, counter, statuses, group words, document records][documents][tile map]
     auto al = [](size_t x, size_t a) { return (x + a - 1) / a * a; };
-    const size_t o_status = 64, o_gstatus = al(o_status + 8 * (size_t)n_tiles, 64);
-    const size_t o_gdone = al(o_gstatus + 8 * (size_t)n_groups, 64), o_dres = al(o_gdone + 4 * (size_t)n_groups, 64);
+    const size_t o_status = 64, o_gagg = al(o_status + 8 * (size_t)n_tiles, 64);
+    const size_t o_ginc = al(o_gagg + 8 * (size_t)n_groups, 64), o_dres = al(o_ginc + 8 * (size_t)n_groups, 64);
     const size_t zero_end = o_dres + sizeof(WDocRes) * D;
     const size_t o_docs = al(zero_end, 256), o_tdoc = al(o_docs + sizeof(WDoc) * D, 256);
     const size_t dev_total = o_tdoc + 4 * (size_t)n_tiles;
@@ -1747,8 +1626,8 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
         P.res = reinterpret_cast<WResult *>(dv);
         P.tile_counter = reinterpret_cast<unsigned int *>(dv + sizeof(WResult));
         P.status = reinterpret_cast<unsigned long long *>(dv + o_status);
-        P.gstatus = reinterpret_cast<unsigned long long *>(dv + o_gstatus);
-        P.gdone = reinterpret_cast<unsigned int *>(dv + o_gdone);
+        P.gagg = reinterpret_cast<unsigned long long *>(dv + o_gagg);
+        P.ginc = reinterpret_cast<unsigned long long *>(dv + o_ginc);
         P.n_tiles = n_tiles;
         P.timeout_ns = c->timeout_ns;
         P.withhold = NONE;
