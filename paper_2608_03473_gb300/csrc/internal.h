@@ -115,6 +115,11 @@ struct WalkTable {
     // at byte b when the byte before has context k; row 0: single bytes)
     uint32_t n_ctx = 0, ctx_off = 0;
     std::vector<uint8_t> blob;
+    // synchronizing bytes (rows.cu): for every byte (byte form) or class
+    // (class form), the row every run over Q+ is in right after it, as a
+    // relative row address; p_pre where the runs end in different rows
+    std::vector<uint16_t> sync;
+    uint32_t n_sync = 0;                  // byte values that synchronize
 };
 
 // ---------------------------------------------------------------------------

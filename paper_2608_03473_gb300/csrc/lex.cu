@@ -1032,7 +1032,12 @@ int lx::ensure_device_tables(const lx_tokenset *cts, int device, DeviceTables *o
     }
     if (rc == LX_OK && ts->scan.status == LX_OK) rc = upload(ts->scan.blob, &dt.d_scan);
     for (int m = 0; m < 3 && rc == LX_OK; m++)
-        if (ts->walk[m].status == LX_OK) rc = upload(ts->walk[m].blob, &dt.d_walk[m]);
+        if (ts->walk[m].status == LX_OK) {   // the synchronizing rows right behind the table
+            std::vector<uint8_t> w = ts->walk[m].blob;
+            const uint8_t *y = reinterpret_cast<const uint8_t *>(ts->walk[m].sync.data());
+            w.insert(w.end(), y, y + 2 * ts->walk[m].sync.size());
+            rc = upload(w, &dt.d_walk[m]);
+        }
     if (rc == LX_OK && ts->liveness.status == LX_OK) rc = upload(ts->liveness.blob, &dt.d_live);
     if (rc != LX_OK) {
         for (int m = 0; m < 3; m++) {
@@ -1343,6 +1348,10 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     const bool can_enumerate = !force && c->kernel == LX_KERNEL_AUTO && ts->scan.status == LX_OK;
     const lx_tuned *tu = tuned_for(c, ts, mode);
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;
+    if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
+        const int rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        if (rc != LX_ROWS) return rc;
+    }
     const bool warp_ok = !force && c->kernel != LX_KERNEL_TILE && warp_path_ok(ts, mode, d_in);
     // the tile kernel cuts at single certified bytes only; the warp kernel also at windows
     const bool warp_windows = warp_ok && !mode_has_cuts(ts, mode) && warp_has_cuts(ts, mode);

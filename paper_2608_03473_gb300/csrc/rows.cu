@@ -1,0 +1,977 @@
+// rows.cu -- GB300 (sm_103a) lexing from known entry rows: the kernels that
+// lx_lex takes first (lexwarp.cu and lex.cu hold the paths for what these
+// refuse).
+//
+// The longest-match scanner of Section 3, as the event-code walk table of
+// internal.h runs it, is in one row after every input byte.  If the row at
+// the start of every slice of the input is known, all slices walk at once
+// from there, each over its own bytes and no others.  Two kernels:
+//
+//   row_guess   the entry row of every slice.  After a synchronizing byte
+//               every run over Q+ is in the same row (WalkTable::sync; the
+//               certified bytes of the mode are among them), so a lane that
+//               starts a few bytes before the slice in the PRE row, which
+//               absorbs bytes up to the first synchronizing one, reaches the
+//               slice in the scanner's row.
+//   lex_rows    every warp claims tiles of 32 slices; lane i walks slice i
+//               from its entry row, stores the event codes in its part of
+//               the warp's event buffer, counts them, and turns them into
+//               (kind, length) pairs in a shared stage; the warp resolves
+//               the tile's output offset (lookback.cuh) after its next
+//               tile's walk and copies the stage out, coalesced.
+//
+// The entry rows need not be right: each lane checks that it leaves its slice
+// in the next one's entry row (across tiles, when the offset is resolved).
+// Where every slice agrees from START at offset 0 on, the rows are the serial
+// scan's by induction.  A disagreement, an entry row that was not found or a
+// backtrack to before a slice stops the call (ERR_ROWS) and the caller
+// lexes the input another way; what was written is overwritten.
+//
+// Backtracking inside a slice (SLOW) is replayed by its lane (relex), and the
+// first lexing failure ends the stream (Corollary 1).
+//
+// Against the chunks of lexwarp.cu, which start at a certified byte and run
+// on past their lane's bytes to the next one: no lane walks another's bytes
+// (that tail was 16-26 % of the time), no halo, 16-byte event stores, and
+// token-driven instead of byte-driven emission (instructions per input byte
+// 1.02 -> 0.68).  A call: 512 MiB of JSON 1 003 -> 642 us, 192 MiB of C-like
+// text 630 -> 397 us, 1 MiB of arith tokens 84 -> 41 us, 40 MiB not 16-byte
+// aligned (formerly the tile kernel) 333 -> 114 us.  What bounds it: the
+// dependent table lookups of the walk (40 % of a warp's cycles) and the
+// emission (27 %), at 17-20 warps per SM, which shared memory limits.
+
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "devutil.cuh"
+#include "internal.h"
+#include "lookback.cuh"
+#include "runtime.h"
+
+namespace lx {
+namespace {
+
+constexpr uint32_t NONE = 0xFFFFFFFFu;
+constexpr uint32_t BIG = 0x7FFFFFFFu;
+constexpr uint32_t ROW_UNKNOWN = 0xFFFFu;   // entry row: none found (rows are at even addresses)
+constexpr int MAX_WARPS = 20;               // warps per CTA at most
+constexpr uint32_t LEN_MAX = 511;           // a stage entry's length field; this value: kept aside
+constexpr uint32_t GUESS_MAX = 8192;        // bytes before a slice searched for a synchronizing byte
+constexpr int GUESS_NT = 512;
+constexpr unsigned ERR_TIMEOUT = ERR_TIMEOUT_BIT;
+constexpr unsigned ERR_SMEM = 2u;
+constexpr unsigned ERR_ROWS = 4u;           // entry rows do not fit together: lex the input another way
+
+// A warp's shared memory: the event buffer, SLICE + 16 bytes per lane (the
+// 16-byte stores and loads of eight lanes then fall in different banks), and
+// the stage of STAGE tokens, 2 bytes each (event code << 8 | length).
+template <int NW>   // event mask words per lane
+struct Geo {
+    static constexpr uint32_t SLICE = 32 * NW;
+    static constexpr uint32_t TILE = 32 * SLICE;
+    static constexpr uint32_t STRIDE = SLICE + 16;
+    static constexpr uint32_t STAGE = NW < 3 ? TILE : 512 + 256 * NW;
+    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE;
+    static_assert(WAREA % 16 == 0, "geometry");
+};
+
+struct RResult {
+    unsigned long long total;          // kept tokens over all tiles
+    unsigned long long inv_fail_pos;   // ~min failure position, 0 = none
+    unsigned long long inv_fail_tok;   // ~output index at that failure
+    unsigned int error;
+    unsigned int pad;
+};
+
+struct RParams {
+    const uint8_t *in;             // 16-byte aligned; the input is [lo, n) of it
+    uint64_t n;
+    uint32_t lo;                   // 0..15
+    uint32_t slice;                // bytes per slice
+    const uint8_t *blob;           // walk table, then WalkTable::sync
+    uint32_t blob_bytes, rows_bytes, row_shift, sync_bytes;   // multiples of 16 but the shift
+    uint32_t p_start, p_pre, acc_off, kmap_off, cmap_off;
+    uint32_t guess;                // bytes walked before a slice at first
+    uint16_t *rows;                // entry row of every slice (relative address)
+    uint64_t n_slices;
+    uint16_t *out_kinds;
+    uint32_t *out_lens;
+    uint64_t cap;
+    uint16_t *spill;               // per warp of the grid: a tile's stage entries beyond the shared stage
+    unsigned long long *status;    // per tile: ST_AGG | exit row << 32 | last event position + 1 << 16 | kept count
+    unsigned long long *gagg, *ginc;   // per group of tiles (lookback.cuh)
+    unsigned int *tile_counter;
+    RResult *res;
+    uint64_t zero_bytes;           // of the scratch from res on, zeroed by row_guess
+    uint32_t n_tiles;
+    uint64_t timeout_ns;
+    uint32_t withhold;
+    uint32_t n_pat;                // synchronizing byte values where they are few (0: more than four)
+    uint32_t pat[4];               // each four times
+    static constexpr unsigned long long COUNT = 0xFFFFull;
+    static constexpr bool SMALL = true;
+    __device__ unsigned int *error() const { return &res->error; }
+};
+
+// Shared addresses of the tables.
+struct REnv {
+    uint32_t tb, start, pre, slow, acc, kmap, cmap, shift;
+};
+
+__device__ __forceinline__ uint4 ldg16(const uint8_t *p)
+{
+    return __ldg(reinterpret_cast<const uint4 *>(p));
+}
+__device__ __forceinline__ void sts16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint4 lds16(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+
+template <int FORM>
+__device__ __forceinline__ uint32_t wstep(const REnv &E, uint32_t e, uint32_t b)
+{
+    const uint32_t a = FORM == FORM_BYTE ? ((e & ~0x1FEu) | (b << 1)) : ((e & ~0xFFu) | lds_u8(E.cmap + b));
+    return lds_u16(a);
+}
+__device__ __forceinline__ uint32_t acc_code(const REnv &E, uint32_t e)
+{
+    return lds_u8(E.acc + ((e - E.tb) >> E.shift));
+}
+
+// Four byte steps over the little-endian word w (per byte one LOP3 and the
+// dependent table load; the class form adds a PRMT and the class map's load,
+// which depend on the input alone); returns the four event codes.
+#define LXR_B(XOP, VIN, VOUT)                                                  \
+    XOP "lop3.b32 a, " VIN ", t, %4, 0xD8;\n\t"                                \
+        "ld.shared.u16 " VOUT ", [a];\n\t"
+#define LXR_C(SEL, VIN, VOUT)                                                  \
+    "prmt.b32 t, %2, %3, " SEL ";\n\t"                                         \
+    "ld.shared.u8 c, [t];\n\t"                                                 \
+    "lop3.b32 a, " VIN ", c, %4, 0xD8;\n\t"                                    \
+    "ld.shared.u16 " VOUT ", [a];\n\t"
+#define LXR_HEAD "{\n\t.reg .b32 t, a, c, v0, v1, v2, t0, t1;\n\t"
+#define LXR_PACK                                                               \
+    "prmt.b32 t0, v0, v1, 0x0040;\n\t"                                         \
+    "prmt.b32 t1, v2, %0, 0x0040;\n\t"                                         \
+    "prmt.b32 %1, t0, t1, 0x5410;\n\t}"
+
+template <int FORM>
+__device__ __forceinline__ uint32_t wword(uint32_t &e, uint32_t w, uint32_t cm)
+{
+    uint32_t pk;
+    if (FORM == FORM_BYTE)
+        asm volatile(LXR_HEAD LXR_B("shl.b32 t, %2, 1;\n\t", "%0", "v0") LXR_B("shr.b32 t, %2, 7;\n\t", "v0", "v1")
+                         LXR_B("shr.b32 t, %2, 15;\n\t", "v1", "v2") LXR_B("shr.b32 t, %2, 23;\n\t", "v2", "%0")
+                             LXR_PACK
+                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0x1FEu) : "memory");
+    else
+        asm volatile(LXR_HEAD LXR_C("0x7650", "%0", "v0") LXR_C("0x7651", "v0", "v1") LXR_C("0x7652", "v1", "v2")
+                         LXR_C("0x7653", "v2", "%0") LXR_PACK
+                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0xFFu) : "memory");
+    return pk;
+}
+
+__device__ __forceinline__ uint32_t top_bit(uint32_t x)   // index of the highest one, NONE for 0
+{
+    uint32_t b;
+    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(x));
+    return b;
+}
+
+// A kept token (code >= 4) of length d into the stage at sa, which advances.
+__device__ __forceinline__ void put_token(uint32_t &sa, uint32_t code, uint32_t d)
+{
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 v;\n\t"
+                 "setp.gt.u32 p, %1, 3;\n\t"
+                 "mad.lo.u32 v, %1, 256, %2;\n\t"
+                 "@p st.shared.u16 [%0], v;\n\t"
+                 "@p add.u32 %0, %0, 2;\n\t}"
+                 : "+r"(sa) : "r"(code), "r"(d) : "memory");
+}
+
+__device__ __forceinline__ uint32_t kept_mask(uint32_t w)   // bit 7 of every byte >= 4 (a kept code)
+{
+    return (((w | 0x80808080u) - 0x04040404u) | w) & 0x80808080u;
+}
+__device__ __forceinline__ uint32_t event_mask(uint32_t w)  // bit 7 of every nonzero byte
+{
+    return (((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u;
+}
+
+// Stage the walk table (row offsets become shared addresses) with the PRE
+// row replaced by the synchronizing one; false where the 16-bit row
+// addresses would not reach every row.
+template <int FORM>
+__device__ bool stage_table(const RParams &P, uint8_t *smem, REnv &E)
+{
+    const uint32_t sbase = smem_u32(smem), tb = (sbase + 511u) & ~511u;
+    if (tb + P.rows_bytes > 65536u) {
+        if (threadIdx.x == 0) atomicOr(P.error(), ERR_SMEM);
+        return false;
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(smem + (tb - sbase));
+    const uint4 *src = reinterpret_cast<const uint4 *>(P.blob);
+    const uint32_t n = P.blob_bytes / 16, r = P.rows_bytes / 16, pre = P.p_pre / 16, tb2 = tb * 0x10001u;
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        uint4 v = __ldg(src + (i - pre < P.sync_bytes / 16 ? n + (i - pre) : i));
+        if (i < r) v = make_uint4(__vadd2(v.x, tb2), __vadd2(v.y, tb2), __vadd2(v.z, tb2), __vadd2(v.w, tb2));
+        dst[i] = v;
+    }
+    E.tb = E.slow = tb;
+    E.start = tb + P.p_start;
+    E.pre = tb + P.p_pre;
+    E.acc = tb + P.acc_off;
+    E.kmap = tb + P.kmap_off;
+    E.cmap = tb + P.cmap_off;
+    E.shift = P.row_shift;
+    return true;
+}
+
+// Whether one of the few synchronizing byte values is among a block's bytes.
+__device__ __forceinline__ bool has_sync(const RParams &P, const uint4 &c)
+{
+    uint32_t z = 0;
+    for (uint32_t i = 0; i < P.n_pat; i++) {
+        const uint32_t x = c.x ^ P.pat[i], y = c.y ^ P.pat[i], u = c.z ^ P.pat[i], v = c.w ^ P.pat[i];
+        z |= ((x - 0x01010101u) & ~x) | ((y - 0x01010101u) & ~y) | ((u - 0x01010101u) & ~u) | ((v - 0x01010101u) & ~v);
+    }
+    return (z & 0x80808080u) != 0;
+}
+
+// The row at position p (a multiple of 16, 0 < p < n) by walking to it from
+// the PRE row: from the block of the nearest synchronizing byte before it
+// where few byte values synchronize (compared a word at a time, which takes
+// no table lookups), else from `guess` bytes before, four times as many where
+// none of them synchronizes; at most GUESS_MAX bytes back, and from START where
+// the input begins there.  SLOW looks for the next synchronizing byte (the
+// row need not be right).  All lanes of a warp call it together.
+template <int FORM>
+__device__ uint32_t guess_row(const RParams &P, const REnv &E, uint64_t p, bool has)
+{
+    uint32_t e = E.pre, w = P.guess;
+    if (P.n_pat && has) {
+        w = 0;
+        bool hit = false;
+        while (!hit && w < GUESS_MAX && w < p) {   // 64 bytes at a time
+            uint4 c[4];
+#pragma unroll
+            for (uint32_t k = 0; k < 4; k++)
+                c[k] = w + 16 * (k + 1) <= p ? ldg16(P.in + (p - w - 16 * (k + 1))) : make_uint4(0, 0, 0, 0);
+            uint32_t back = 64;
+#pragma unroll
+            for (int k = 3; k >= 0; k--)
+                if (w + 16 * (k + 1) <= p && has_sync(P, c[k])) {
+                    back = 16 * (k + 1);
+                    hit = true;
+                }
+            w += back;
+        }
+    }
+    bool todo = has;
+    while (__any_sync(0xffffffffu, todo)) {
+        if (todo) {
+            uint64_t a = p > w ? p - w : 0;
+            e = E.pre;
+            if (a == 0) {
+                e = E.start;
+                if (P.lo) {
+                    for (uint32_t k = P.lo; k < 16; k++) e = wstep<FORM>(E, e, __ldg(P.in + k));
+                    a = 16;
+                }
+            }
+            for (; a < p; a += 16) {
+                const uint4 c = ldg16(P.in + a);
+                wword<FORM>(e, c.x, E.cmap);
+                wword<FORM>(e, c.y, E.cmap);
+                wword<FORM>(e, c.z, E.cmap);
+                wword<FORM>(e, c.w, E.cmap);
+                if (e == E.slow) e = E.pre;
+            }
+            todo = e >= E.pre && w < GUESS_MAX && w < p;
+        }
+        w *= 4;
+    }
+    return e >= E.pre || e == E.slow ? ROW_UNKNOWN : (e & ~0xFFu) - E.tb;
+}
+
+template <int FORM>
+__global__ void __launch_bounds__(GUESS_NT) row_guess(RParams P)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    // the scratch of lex_rows, which runs next on the stream
+    uint4 *z = reinterpret_cast<uint4 *>(P.res);
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < P.zero_bytes / 16;
+         i += (uint64_t)gridDim.x * blockDim.x)
+        z[i] = make_uint4(0, 0, 0, 0);
+    REnv E;
+    if (!stage_table<FORM>(P, smem, E)) return;
+    __syncthreads();
+    for (uint64_t s0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ull; s0 < P.n_slices;
+         s0 += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t s = s0 + (threadIdx.x & 31);
+        const bool has = s > 0 && s < P.n_slices;
+        uint32_t r = guess_row<FORM>(P, E, s * P.slice, has);
+        if (s == 0) r = P.p_start;
+        if (s < P.n_slices) P.rows[s] = (uint16_t)r;
+    }
+}
+
+// The slice [ps, pe) of a lane token by token, from the last event that its
+// walk stored (or from the entry row): the walk ran into SLOW, or the input
+// ends at pe in a row that does not accept.  Codes go to ev + position - p0.
+// Sets the exit row, the code that ends at pe == end of input (tail), a
+// failure offset, or `back` where the token in progress at ps does not
+// accept in the slice (it has to be replayed from before it).
+template <int FORM>
+__device__ __noinline__ void relex(const REnv &E, const uint8_t *in, uint32_t ev, uint32_t p0, uint32_t ps, uint32_t pe,
+                                   uint32_t e_in, bool at_end, uint32_t *exit, uint32_t *tail, uint32_t *fail,
+                                   bool *back)
+{
+    uint32_t tok = ps, q = e_in, r = NONE, rc = 0, k;
+    bool own = false;   // a token start lies in the slice
+    for (uint32_t j = pe; j-- > ps;)
+        if (lds_u8(ev + j - p0)) {
+            tok = j;
+            own = true;
+            break;
+        }
+    if (own || q == E.start) {
+        q = E.start;
+        own = true;
+    } else if ((rc = acc_code(E, q)) != 0) {
+        r = ps;
+    }
+    k = tok;
+    for (;;) {
+        uint32_t v = E.slow;
+        if (k < pe) {
+            v = wstep<FORM>(E, q, __ldg(in + k));
+        } else if (!at_end) {
+            *exit = q & ~0xFFu;
+            return;
+        } else if (q != E.start) {
+            const uint32_t ac = acc_code(E, q);
+            if (ac) {
+                *tail = ac;
+                return;
+            }
+        } else {
+            return;
+        }
+        if (v != E.slow) {
+            const uint32_t code = v & 0xFEu;
+            if (code) {   // the token ends before this byte
+                sts_u8(ev + k - p0, code);
+                tok = k;
+                own = true;
+                r = NONE;
+            }
+            q = v;
+            k++;
+            const uint32_t ac = acc_code(E, q);
+            if (ac) {
+                r = k;
+                rc = ac;
+            }
+            continue;
+        }
+        if (r == NONE) {
+            if (own) *fail = tok;
+            else *back = true;
+            return;
+        }
+        sts_u8(ev + r - p0, rc);
+        tok = k = r;
+        own = true;
+        q = E.start;
+        r = NONE;
+    }
+}
+
+// A tile whose tokens wait in the warp's stage for their output offset.
+struct Pending {
+    uint32_t tile;      // NONE: nothing pending
+    uint32_t staged;    // kept tokens
+    uint32_t split;     // of them in the shared stage (the rest: spill slot)
+    uint32_t entry;     // entry row of its first lane
+    uint32_t open;      // its first event ended a kept token that began in an earlier tile
+    uint32_t fail;      // failure position in the tile, or NONE
+    uint32_t lidx, llen;   // per lane: a token whose length the stage does not hold
+};
+
+// The staged tokens of a tile to the output from index G: each lane two
+// consecutive tokens at a time from the first index where G + i is even, when
+// the arrays are aligned for it and the capacity does not cut the tile.
+__device__ __forceinline__ void copy_stage(const RParams &P, uint32_t kmap, uint32_t stage, const uint16_t *spill,
+                                           uint32_t split, uint32_t staged, uint64_t G)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    auto val = [&](uint32_t i) { return i < split ? lds_u16(stage + 2 * i) : (uint32_t)spill[i - split]; };
+    auto kind = [&](uint32_t v) { return lds_u16(kmap + ((v >> 8) & 0xFEu)); };
+    auto one = [&](uint32_t i) {
+        const uint64_t o = G + i;
+        if (o < P.cap) {
+            const uint32_t v = val(i);
+            P.out_kinds[o] = (uint16_t)kind(v);
+            P.out_lens[o] = v & 0x1FFu;
+        }
+    };
+    const bool aligned = ((reinterpret_cast<uintptr_t>(P.out_kinds) & 3u) |
+                          (reinterpret_cast<uintptr_t>(P.out_lens) & 7u)) == 0;
+    if (!aligned || G + staged > P.cap) {
+        for (uint32_t i = lane; i < staged; i += 32) one(i);
+        return;
+    }
+    const uint32_t h = min((uint32_t)(G & 1u), staged);
+    if (lane < h) one(lane);
+    const uint32_t ng = (staged - h) / 2;
+    uint16_t *const ok = P.out_kinds + G + h;
+    uint32_t *const ol = P.out_lens + G + h;
+    auto put = [&](uint32_t q, uint32_t v0, uint32_t v1, uint32_t k0, uint32_t k1) {
+        *reinterpret_cast<uint32_t *>(ok + 2 * q) = k0 | (k1 << 16);
+        *reinterpret_cast<uint2 *>(ol + 2 * q) = make_uint2(v0 & 0x1FFu, v1 & 0x1FFu);
+    };
+    uint32_t q = lane;
+    if (split == staged)   // two pairs at a time: their stage and kind lookups overlap
+        for (; q + 32 < ng; q += 64) {
+            const uint32_t s0 = stage + 2 * h + 4 * q;
+            const uint32_t v0 = lds_u16(s0), v1 = lds_u16(s0 + 2), v2 = lds_u16(s0 + 128), v3 = lds_u16(s0 + 130);
+            const uint32_t k0 = kind(v0), k1 = kind(v1), k2 = kind(v2), k3 = kind(v3);
+            put(q, v0, v1, k0, k1);
+            put(q + 32, v2, v3, k2, k3);
+        }
+    for (; q < ng; q += 32) {
+        const uint32_t i = h + 2 * q, v0 = val(i), v1 = val(i + 1);
+        put(q, v0, v1, kind(v0), kind(v1));
+    }
+    const uint32_t t = h + 2 * ng;
+    if (lane < staged - t) one(t + lane);
+}
+
+// Resolve the pending tile's output offset, check its entry row against the
+// previous tile's exit row, and copy its tokens out.  False: stop (an error
+// is flagged).
+template <int NW>
+__device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, uint32_t stage, const uint16_t *spill)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    constexpr uint32_t TILE = Geo<NW>::TILE;
+    uint64_t G = 0, carry = 0;
+    unsigned long long w;   // the previous tile's status word
+    if (!resolve_tile(P, D.tile, G, w)) return false;
+    if (D.tile) {
+        const uint32_t x = (uint32_t)(w >> 32) & 0xFFFFu;
+        if (x && x != D.entry) {
+            if (lane == 0) atomicOr(P.error(), ERR_ROWS);
+            return false;
+        }
+        if (D.open) {   // where the open token began: the last event before the tile (every earlier tile has published)
+            bool good = true;
+            if (lane == 0) {
+                Waiter W;
+                uint32_t t = D.tile - 1;
+                while (good && !((w >> 16) & 0xFFFFu) && t > 0) {
+                    t--;
+                    while ((w = ld_status(&P.status[t])) == 0 && (good = W.again(P))) {}
+                }
+                const uint32_t lp = (uint32_t)(w >> 16) & 0xFFFFu;
+                carry = (uint64_t)(D.tile - t) * TILE - (lp ? lp - 1 : P.lo);
+            }
+            if (!__shfl_sync(0xffffffffu, good ? 1u : 0u, 0)) return false;
+            carry = __shfl_sync(0xffffffffu, carry, 0);
+        }
+    }
+    if (lane == 0) {
+        if (D.fail != NONE) {
+            atomicMax(&P.res->inv_fail_pos, ~(unsigned long long)((uint64_t)D.tile * TILE + D.fail));
+            atomicMax(&P.res->inv_fail_tok, ~(unsigned long long)(G + D.staged));
+        }
+        if (D.tile == P.n_tiles - 1) P.res->total = G + D.staged;
+    }
+    copy_stage(P, E.kmap, stage, spill, D.split, D.staged, G);
+    __syncwarp();
+    if (D.lidx != NONE && G + D.lidx < P.cap)
+        P.out_lens[G + D.lidx] = (uint32_t)(D.llen + (D.open && D.lidx == 0 ? carry : 0));
+    return true;
+}
+
+template <int FORM, int NW, bool FUSED>
+__global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    constexpr uint32_t SLICE = Geo<NW>::SLICE, TILE = Geo<NW>::TILE, STRIDE = Geo<NW>::STRIDE;
+    constexpr uint32_t STAGE = Geo<NW>::STAGE, WAREA = Geo<NW>::WAREA;
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    REnv E;
+    if (!stage_table<FORM>(P, smem, E)) return;
+    __syncthreads();
+    const uint32_t area = ((E.tb + P.blob_bytes + 15u) & ~15u) + wid * WAREA;
+    const uint32_t stage = area + 32 * STRIDE, evl = area + lane * STRIDE;
+    uint16_t *const spill = P.spill + ((size_t)blockIdx.x * (blockDim.x >> 5) + wid) * (TILE + 1);
+    const uint32_t ahead = gridDim.x * (blockDim.x / 32);
+    const uint32_t lt = (1u << lane) - 1u;
+
+    Pending pend;
+    pend.tile = NONE;
+    for (;;) {
+        uint32_t tile = 0;
+        if (lane == 0) {
+            tile = atomicAdd(P.tile_counter, 1u);
+            if (*(volatile unsigned int *)P.error() != 0) tile = P.n_tiles;
+        }
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+        if (tile >= P.n_tiles) break;
+        const uint8_t *in = P.in + (uint64_t)tile * TILE;
+        const uint64_t left = P.n - (uint64_t)tile * TILE;
+        const uint32_t nrel = left < BIG ? (uint32_t)left : BIG;   // bytes from the tile's start on
+        const uint32_t lo = tile == 0 ? P.lo : 0u;
+        if (lane == 0 && tile + ahead < P.n_tiles) {   // a tile some warp takes about one tile from now, into L2
+            const uint64_t fb = (uint64_t)(tile + ahead) * TILE, fl = P.n - fb;
+            const uint32_t bytes = (uint32_t)(fl < TILE ? fl : TILE) & ~15u;
+            if (bytes)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.in + fb), "r"(bytes) : "memory");
+        }
+        const uint32_t p0 = lane * SLICE;
+        const bool has = p0 < nrel, whole = nrel >= TILE && lo == 0;
+        uint4 A, B;
+        if (whole) {   // in flight while the entry row is read or found
+            A = ldg16(in + p0);
+            B = ldg16(in + p0 + 16);
+        }
+        uint32_t er;
+        if (FUSED) {
+            const uint64_t p = (uint64_t)tile * TILE + p0;
+            er = guess_row<FORM>(P, E, p, has && p > 0);
+            if (p == 0) er = P.p_start;
+        } else {
+            er = has ? P.rows[(uint64_t)tile * 32 + lane] : 0u;
+        }
+        const bool act = has && er != ROW_UNKNOWN;
+        const uint32_t e_in = er + E.tb, ps = max(p0, lo), pe = min(p0 + SLICE, nrel);
+        uint32_t e = e_in;
+
+        // walk the slice
+        if (whole) {
+            if (act) {
+#pragma unroll 1
+                for (uint32_t b = 0; b < SLICE; b += 32) {
+                    const uint32_t a0 = wword<FORM>(e, A.x, E.cmap), a1 = wword<FORM>(e, A.y, E.cmap);
+                    const uint32_t a2 = wword<FORM>(e, A.z, E.cmap), a3 = wword<FORM>(e, A.w, E.cmap);
+                    sts16(evl + b, a0, a1, a2, a3);
+                    if (b + 32 < SLICE) A = ldg16(in + p0 + b + 32);
+                    const uint32_t b0 = wword<FORM>(e, B.x, E.cmap), b1 = wword<FORM>(e, B.y, E.cmap);
+                    const uint32_t b2 = wword<FORM>(e, B.z, E.cmap), b3 = wword<FORM>(e, B.w, E.cmap);
+                    sts16(evl + b + 16, b0, b1, b2, b3);
+                    if (b + 32 < SLICE) B = ldg16(in + p0 + b + 48);
+                }
+            }
+        } else if (act) {   // the input's first or last tile: partial blocks byte by byte
+            for (uint32_t b = p0; b < pe; b += 16) {
+                if (b >= lo && b + 16 <= nrel) {
+                    A = ldg16(in + b);
+                    const uint32_t a0 = wword<FORM>(e, A.x, E.cmap), a1 = wword<FORM>(e, A.y, E.cmap);
+                    const uint32_t a2 = wword<FORM>(e, A.z, E.cmap), a3 = wword<FORM>(e, A.w, E.cmap);
+                    sts16(evl + b - p0, a0, a1, a2, a3);
+                } else {
+                    sts16(evl + b - p0, 0, 0, 0, 0);
+                    for (uint32_t k = max(b, lo); k < min(b + 16, nrel); k++) {
+                        e = wstep<FORM>(E, e, __ldg(in + k));
+                        sts_u8(evl + k - p0, e & 0xFEu);
+                    }
+                }
+            }
+        }
+
+        // the lane's end: backtracking, the end of the input, the exit row
+        const bool at_end = act && pe == nrel;
+        uint32_t tail = 0, fail = NONE, exit = e & ~0xFFu;   // without the event code
+        bool back = has && !act;
+        if (at_end && e != E.slow && e < E.pre) tail = acc_code(E, e);
+        if (act && (e == E.slow || (at_end && !tail)))
+            relex<FORM>(E, in, evl, p0, ps, pe, e_in, at_end, &exit, &tail, &fail, &back);
+        const uint32_t fmin = __reduce_min_sync(0xffffffffu, fail);
+        {
+            const uint32_t ner = __shfl_down_sync(0xffffffffu, er, 1);
+            bool bad = back;
+            if (lane < 31 && act && !back && fail == NONE && !at_end && exit - E.tb != ner) bad = true;
+            if (__any_sync(0xffffffffu, bad && p0 <= fmin)) {
+                if (lane == 0) atomicOr(P.error(), ERR_ROWS);
+                break;
+            }
+        }
+
+        // (d) event masks (bit j: position 32 w + j of the slice) and the kept count
+        uint32_t m[NW], cnt = 0;
+        const uint32_t used = act && ps <= fmin ? pe - p0 : 0u;
+#pragma unroll
+        for (uint32_t w = 0; w < NW; w++) {
+            m[w] = 0;
+            if (32 * w < used) {
+                const uint4 x = lds16(evl + 32 * w);
+                uint4 y = make_uint4(0, 0, 0, 0);
+                if (32 * w + 16 < used) y = lds16(evl + 32 * w + 16);
+                const uint32_t s0 = __dp4a(event_mask(x.y), 0x80402010u, __dp4a(event_mask(x.x), 0x08040201u, 0u));
+                const uint32_t s1 = __dp4a(event_mask(x.w), 0x80402010u, __dp4a(event_mask(x.z), 0x08040201u, 0u));
+                const uint32_t s2 = __dp4a(event_mask(y.y), 0x80402010u, __dp4a(event_mask(y.x), 0x08040201u, 0u));
+                const uint32_t s3 = __dp4a(event_mask(y.w), 0x80402010u, __dp4a(event_mask(y.z), 0x08040201u, 0u));
+                m[w] = (s0 >> 7) | (s1 << 1) | (s2 << 9) | (s3 << 17);
+                uint32_t c = __dp4a(kept_mask(x.x), 0x01010101u, __dp4a(kept_mask(x.y), 0x01010101u, 0u));
+                c = __dp4a(kept_mask(x.z), 0x01010101u, __dp4a(kept_mask(x.w), 0x01010101u, c));
+                c = __dp4a(kept_mask(y.x), 0x01010101u, __dp4a(kept_mask(y.y), 0x01010101u, c));
+                c = __dp4a(kept_mask(y.z), 0x01010101u, __dp4a(kept_mask(y.w), 0x01010101u, c));
+                cnt += c;
+            }
+        }
+        cnt >>= 7;
+        if (fmin != NONE) {   // nothing after the failure counts
+            cnt = 0;
+#pragma unroll
+            for (uint32_t w = 0; w < NW; w++) {
+                const uint32_t at = p0 + 32 * w;
+                if (at > fmin) m[w] = 0;
+                else if (fmin - at < 31) m[w] &= (2u << (fmin - at)) - 1u;
+                for (uint32_t x = m[w]; x; x &= x - 1) cnt += lds_u8(evl + 32 * w + __ffs(x) - 1) >= 4 ? 1u : 0u;
+            }
+            if (pe > fmin) tail = 0;
+        }
+        cnt += tail >= 4 ? 1u : 0u;
+        // the last event position of the lane (+ 1), and of the lanes before it
+        uint32_t lp = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < NW; w++)
+            if (m[w]) lp = p0 + 32 * w + 32 - __clz(m[w]);
+        if (tail) lp = pe + 1;
+        const uint32_t evb = __ballot_sync(0xffffffffu, lp != 0);
+        const uint32_t below = evb & lt;
+        const uint32_t prev1 = __shfl_sync(0xffffffffu, lp, below ? 31 - __clz(below) : 0);
+        const uint32_t last1 = __shfl_sync(0xffffffffu, lp, evb ? 31 - __clz(evb) : 0);
+        uint32_t excl = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, excl, o);
+            if (lane >= (uint32_t)o) excl += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, excl, 31);
+        excl -= cnt;
+        const uint32_t xr = __shfl_sync(0xffffffffu, exit, 31);   // 0 where the input ended or failed
+        const uint32_t x31 = __shfl_sync(0xffffffffu, (act && !at_end && fmin == NONE) ? 1u : 0u, 31) ? xr - E.tb : 0u;
+        publish_word(P, tile, ((unsigned long long)x31 << 32) | ((unsigned long long)last1 << 16) | total);
+
+        // the previous tile's output: its predecessors have had a whole tile to publish
+        if (pend.tile != NONE) {
+            if (!finish_tile<NW>(P, E, pend, stage, spill)) {
+                pend.tile = NONE;
+                break;
+            }
+            __syncwarp();
+        }
+
+        // (e) the kept events into the stage, in order
+        pend.tile = tile;
+        pend.staged = total;
+        pend.fail = fmin;
+        pend.entry = __shfl_sync(0xffffffffu, er, 0);
+        pend.lidx = NONE;
+        pend.llen = 0;
+        bool open = false;
+        uint32_t split = total;
+        uint16_t *gp = nullptr;
+        if (total > STAGE) {   // excl + cnt ascends with the lane: those that fit are a prefix
+            const uint32_t fit = __popc(__ballot_sync(0xffffffffu, excl + cnt <= STAGE));
+            split = fit == 32 ? total : __shfl_sync(0xffffffffu, excl, fit & 31u);
+            if (lane >= fit) gp = spill + (excl - split);
+        }
+        pend.split = split;
+        // the first event's token may begin in another lane or tile
+        int prev = 0;   // the last event's position, relative to the slice
+        if (lp) {
+            uint32_t f = NONE;
+#pragma unroll
+            for (int w = NW - 1; w >= 0; w--)
+                if (m[w]) f = 32 * w + __ffs(m[w]) - 1;
+            const uint32_t fp = f == NONE ? pe - p0 : f;             // its position in the slice
+            const uint32_t fc = f == NONE ? tail : lds_u8(evl + f);  // its code
+            if (below) prev = (int)prev1 - 1 - (int)p0;
+            else if (tile == 0) prev = (int)lo - (int)p0;
+            else prev = -(int)p0, open = true;
+            const uint32_t d = (uint32_t)((int)fp - prev);
+            if (open || d >= LEN_MAX) {
+                if (fc >= 4) {
+                    pend.lidx = excl;
+                    pend.llen = d;
+                } else {
+                    open = false;
+                }
+                prev = (int)fp - (int)LEN_MAX;
+            }
+        }
+        uint32_t sa = stage + 2 * excl;
+        if (total <= STAGE) {
+            // every lane its events in order, the warp as many steps per mask
+            // word as its fullest lane has events, four at a time so that their
+            // code lookups overlap
+            uint32_t nmax[NW];
+#pragma unroll
+            for (uint32_t w = 0; w < NW; w++) nmax[w] = __reduce_max_sync(0xffffffffu, __popc(m[w]));
+#pragma unroll
+            for (uint32_t w = 0; w < NW; w++) {
+                uint32_t x = m[w];
+                for (int n = (int)nmax[w]; n > 0; n -= 4) {
+                    uint32_t b[4], code[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        b[i] = top_bit(x & (0u - x));   // NONE once the events have run out
+                        x &= x - 1;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; i++) code[i] = b[i] != NONE ? lds_u8(evl + 32 * w + b[i]) : 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const int pos = (int)(32 * w + b[i]);
+                        put_token(sa, code[i], (uint32_t)(pos - prev));
+                        prev = code[i] ? pos : prev;
+                    }
+                }
+            }
+            if (tail >= 4) sts_u16(sa, (tail << 8) + (uint32_t)((int)(pe - p0) - prev));
+        } else {
+#pragma unroll
+            for (uint32_t w = 0; w < NW; w++)
+                for (uint32_t x = m[w]; x; x &= x - 1) {
+                    const int pos = (int)(32 * w) + __ffs(x) - 1;
+                    const uint32_t code = lds_u8(evl + pos), v = (code << 8) + (uint32_t)(pos - prev);
+                    if (code >= 4) {
+                        if (gp) *gp++ = (uint16_t)v;
+                        else sts_u16(sa, v), sa += 2;
+                    }
+                    prev = pos;
+                }
+            if (tail >= 4) {
+                const uint32_t v = (tail << 8) + (uint32_t)((int)(pe - p0) - prev);
+                if (gp) *gp = (uint16_t)v;
+                else sts_u16(sa, v);
+            }
+        }
+        pend.open = __any_sync(0xffffffffu, open) ? 1u : 0u;
+        __syncwarp();
+    }
+    if (pend.tile != NONE) finish_tile<NW>(P, E, pend, stage, spill);
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+constexpr uint32_t SMEM_BUDGET = 227 * 1024;
+
+struct RLaunch {
+    RParams P;
+    uint32_t grid = 0, nwarps = 0, smem = 0;
+    uint32_t ggrid = 0, gsmem = 0;
+    bool fused = false;
+    int form = FORM_BYTE, nw = 1;
+};
+
+// Up to this many bytes lex_rows finds the entry rows itself: one launch less.
+constexpr uint64_t FUSED_MAX = 4ull << 20;
+// A warp's time for a tile of 32 slices of 32 k bytes, in units of its fixed
+// part (measured, JSON: 25.7, 29.9, 34.4, 35.8 and 39.1 thousand cycles for
+// k = 4 to 8); a launch takes its rounds of tiles and half a round more, the
+// last one's share.
+constexpr double TILE_FIXED = 1.0, TILE_STEP = 0.265;
+
+using RowsKernel = void (*)(RParams);
+
+// The kernel of a table form and geometry, and its per-warp shared bytes.
+template <int FORM>
+RowsKernel rows_kernel(int nw, bool fused)
+{
+    switch (nw) {
+    case 1: return fused ? lex_rows<FORM, 1, true> : lex_rows<FORM, 1, false>;
+    case 2: return fused ? lex_rows<FORM, 2, true> : lex_rows<FORM, 2, false>;
+    case 3: return lex_rows<FORM, 3, false>;
+    case 4: return lex_rows<FORM, 4, false>;
+    case 5: return lex_rows<FORM, 5, false>;
+    case 6: return lex_rows<FORM, 6, false>;
+    case 7: return lex_rows<FORM, 7, false>;
+    default: return lex_rows<FORM, 8, false>;
+    }
+}
+constexpr uint32_t AREA[9] = {0, Geo<1>::WAREA, Geo<2>::WAREA, Geo<3>::WAREA, Geo<4>::WAREA,
+                              Geo<5>::WAREA, Geo<6>::WAREA, Geo<7>::WAREA, Geo<8>::WAREA};
+
+RowsKernel rows_kernel(int form, int nw, bool fused)
+{
+    return form == FORM_BYTE ? rows_kernel<FORM_BYTE>(nw, fused) : rows_kernel<FORM_CLASS>(nw, fused);
+}
+
+// Whether the kernels may use the shared memory they are launched with (once per context and kernel).
+int allow_smem(lx_ctx *c, int form, int nw, bool fused)
+{
+    const uint64_t key = (2ull << 62) | ((uint64_t)form << 8) | ((uint64_t)fused << 7) | (uint64_t)nw;
+    for (auto &kv : c->occupancy)
+        if (kv.first == key) return LX_OK;
+    cudaError_t e = cudaFuncSetAttribute(rows_kernel(form, nw, fused), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         SMEM_BUDGET);
+    if (e == cudaSuccess)
+        e = form == FORM_BYTE
+                ? cudaFuncSetAttribute(row_guess<FORM_BYTE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 66 * 1024)
+                : cudaFuncSetAttribute(row_guess<FORM_CLASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 66 * 1024);
+    if (e != cudaSuccess) return LX_E_CUDA;
+    c->occupancy.emplace_back(key, 1);
+    return LX_OK;
+}
+
+// Geometry of a launch over L.P.n bytes: the slice length (32 nw bytes), the
+// warps per CTA and the grid (one CTA per SM).
+int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L)
+{
+    const WalkTable &w = ts->walk[mode];
+    const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16, want = warps_setting(c, ts, mode);
+    const uint64_t n = L.P.n;
+    L.fused = n <= FUSED_MAX;
+    double best = 0;
+    int nw = 0;
+    for (int k = 1; k <= (L.fused ? 2 : 8); k++) {
+        if (fixed + AREA[k] > SMEM_BUDGET) break;
+        uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[k]);
+        if (want) warps = std::min(warps, want);
+        const uint64_t tiles = (n + 1024 * k - 1) / (1024 * k), all = (uint64_t)warps * c->num_sms;
+        const double cost = ((double)tiles / (double)all + 0.5) * (TILE_FIXED + TILE_STEP * k);
+        if (!nw || cost < best) {
+            best = cost;
+            nw = k;
+        }
+    }
+    if (!nw) return LX_E_TOOBIG;
+    L.nw = nw;
+    L.P.slice = 32 * nw;
+    L.P.n_slices = (n + L.P.slice - 1) / L.P.slice;
+    const uint64_t tiles = (n + 1024 * nw - 1) / (1024 * nw);
+    if (tiles > 0xFFFFFFF0ull) return LX_E_INVAL;
+    L.P.n_tiles = (uint32_t)tiles;
+    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[nw]);
+    if (want) warps = std::min(warps, want);
+    // few tiles: one CTA on every SM, no more warps than its share (eight stage the table)
+    L.nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(8, (tiles + c->num_sms - 1) / c->num_sms));
+    L.smem = fixed + L.nwarps * AREA[nw];
+    L.grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, tiles);
+    L.gsmem = fixed;
+    return allow_smem(c, w.form, nw, L.fused);
+}
+
+void launch(const RLaunch &L, cudaStream_t st)
+{
+    if (!L.fused) {
+        if (L.form == FORM_BYTE) row_guess<FORM_BYTE><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
+        else row_guess<FORM_CLASS><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
+    }
+    rows_kernel(L.form, L.nw, L.fused)<<<L.grid, 32 * L.nwarps, L.smem, st>>>(L.P);
+}
+
+}  // namespace
+
+bool rows_path_ok(const lx_tokenset *ts, int mode)
+{
+    return ts->walk[mode].status == LX_OK && ts->walk[mode].n_sync > 0;
+}
+
+int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st)
+{
+    if (n == 0) {
+        *n_tokens = 0;
+        *consumed = 0;
+        return LX_OK;
+    }
+    const WalkTable &w = ts->walk[mode];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev != c->device) return LX_E_INVAL;
+    DeviceTables dt;
+    int rc = ensure_device_tables(ts, dev, &dt);
+    if (rc != LX_OK) return rc;
+    RLaunch L;
+    RParams &P = L.P;
+    P = RParams{};
+    P.lo = (uint32_t)(reinterpret_cast<uintptr_t>(d_in) & 15u);
+    P.in = d_in - P.lo;
+    P.n = n + P.lo;
+    L.form = w.form;
+    rc = shape(c, ts, mode, L);
+    if (rc == LX_E_TOOBIG) return LX_ROWS;
+    if (rc != LX_OK) return rc;
+    P.blob = static_cast<const uint8_t *>(dt.d_walk[mode]);
+    P.blob_bytes = (uint32_t)w.blob.size();
+    P.rows_bytes = w.rows_bytes;
+    P.row_shift = w.row_shift;
+    P.sync_bytes = 2 * (uint32_t)w.sync.size();
+    P.p_start = w.p_start;
+    P.p_pre = w.p_pre;
+    P.acc_off = w.acc_off;
+    P.kmap_off = w.kmap_off;
+    P.cmap_off = w.cmap_off;
+    P.guess = 32;
+    if (w.n_sync <= 4)   // few byte values synchronize: they are searched for
+        for (uint32_t b = 0; b < 256; b++)
+            if (w.sync[w.form == FORM_BYTE ? b : ts->byte_class[b]] != w.p_pre) P.pat[P.n_pat++] = b * 0x01010101u;
+    P.out_kinds = d_kinds;
+    P.out_lens = d_lens;
+    P.cap = capacity;
+    P.timeout_ns = c->timeout_ns;
+    P.withhold = c->withhold;
+    // scratch: record and tile counter, status words, group words and counters
+    // (zeroed), entry rows, spill slots
+    auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
+    const uint64_t groups = (P.n_tiles + GS - 1) / GS;
+    const uint64_t o_g = 64 + 8ull * P.n_tiles, o_i = o_g + 8 * groups, zero = (o_i + 8 * groups + 15) & ~15ull;
+    const uint64_t o_rows = al(zero), o_spill = al(o_rows + (L.fused ? 0 : 2 * P.n_slices));
+    const uint64_t need = o_spill + 2ull * (32 * P.slice + 1) * L.grid * L.nwarps;
+    rc = grow(&c->scratch, &c->scratch_bytes, need);
+    if (rc != LX_OK) return rc;
+    uint8_t *scr = static_cast<uint8_t *>(c->scratch);
+    static_assert(sizeof(RResult) == 32 && sizeof(RResult) <= LAUNCH_RECORD_BYTES, "record layout");
+    P.res = reinterpret_cast<RResult *>(scr);
+    P.tile_counter = reinterpret_cast<unsigned int *>(scr + sizeof(RResult));
+    P.status = reinterpret_cast<unsigned long long *>(scr + 64);
+    P.gagg = reinterpret_cast<unsigned long long *>(scr + o_g);
+    P.ginc = reinterpret_cast<unsigned long long *>(scr + o_i);
+    P.zero_bytes = zero;
+    P.rows = reinterpret_cast<uint16_t *>(scr + o_rows);
+    P.spill = reinterpret_cast<uint16_t *>(scr + o_spill);
+    L.ggrid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (P.n_slices + GUESS_NT - 1) / GUESS_NT);
+    if (L.fused) {
+        rc = cuda_err(cudaMemsetAsync(scr, 0, zero, st));
+        if (rc != LX_OK) return rc;
+    }
+    if (c->timing) cudaEventRecord(c->ev[0], st);
+    launch(L, st);
+    rc = cuda_err(cudaGetLastError());
+    if (c->timing) cudaEventRecord(c->ev[1], st);
+    if (rc != LX_OK) return rc;
+    rc = cuda_err(cudaMemcpyAsync(c->h_res, P.res, sizeof(RResult), cudaMemcpyDeviceToHost, st));
+    if (rc == LX_OK) rc = cuda_err(cudaStreamSynchronize(st));
+    if (rc != LX_OK) return rc;
+    const RResult r = *static_cast<const RResult *>(c->h_res);
+    if (r.error & ERR_TIMEOUT) return r.error == ERR_TIMEOUT ? LX_E_TIMEOUT : LX_ROWS;
+    if (r.error) return LX_ROWS;
+    uint64_t tokens = r.total, con = n;
+    if (r.inv_fail_pos) {
+        con = ~r.inv_fail_pos - P.lo;
+        tokens = ~r.inv_fail_tok;
+    }
+    *n_tokens = tokens;
+    *consumed = con;
+    return tokens > capacity ? LX_E_CAPACITY : LX_OK;
+}
+
+}  // namespace lx

@@ -115,6 +115,14 @@ int ensure_device_tables(const lx_tokenset *ts, int device, DeviceTables *out);
 // LX_LOOKAHEAD, leaving the input to the enumerative path (guarded).
 constexpr int LX_SPARSE = -100;   // internal status, never returned by the C ABI
 bool warp_path_ok(const lx_tokenset *ts, int mode, const uint8_t *d_in);
+// Lexing from the entry rows of fixed slices (rows.cu; same contract as
+// lx_lex, any input alignment), for token sets with a synchronizing byte.
+// LX_ROWS: the entry rows were not found or do not fit together; the caller
+// lexes the input another way.
+constexpr int LX_ROWS = -102;   // internal status, never returned by the C ABI
+bool rows_path_ok(const lx_tokenset *ts, int mode);
+int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st);
 // Warps per CTA for the warp-tile kernel on (ts, mode): the context's
 // setting, else lx_autotune's choice, else 0 (as many as fit).
 uint32_t warps_setting(const lx_ctx *c, const lx_tokenset *ts, int mode);

@@ -418,6 +418,30 @@ void build_walk_table(const lx_tokenset &t, int mode, lx::WalkTable &wt, bool fo
         for (uint32_t k = 0; k <= K; k++) wt.blob[wt.cut_off + 256 * k + b] = (cut_c[c] || foll[k][c]) ? 1 : 0;
         wt.blob[wt.ctx_off + b] = (uint8_t)ctx_of[c];
     }
+    // Synchronizing classes: a token that reads a byte of class c moves some
+    // q in Q+ (q0 at its first byte) to delta(q, c), in Q+ as well, or, where
+    // the byte is a cut, starts on it; one such row for the class means that
+    // the scan is in that row after the byte, wherever the byte stands.
+    wt.sync.assign(wt.form == lx::FORM_BYTE ? 256 : 128, (uint16_t)wt.p_pre);
+    for (uint32_t c = 0; c < C; c++) {
+        uint32_t to = 0, distinct = 0;
+        auto add = [&](uint32_t d) {
+            if (d == LX_NONE || !t.live[d] || (distinct && to == Rq(d))) return;
+            to = Rq(d);
+            distinct++;
+        };
+        if (cut_c[c]) add(nx(c, q0));
+        else
+            for (uint32_t q = 0; q < S; q++)
+                if (t.live[q]) add(nx(c, q));
+        if (distinct != 1) continue;
+        if (wt.form == lx::FORM_CLASS) wt.sync[c] = (uint16_t)(to << wt.row_shift);
+        for (uint32_t b = 0; b < 256; b++)
+            if (t.byte_class[b] == c) {
+                wt.n_sync++;
+                if (wt.form == lx::FORM_BYTE) wt.sync[b] = (uint16_t)(to << wt.row_shift);
+            }
+    }
     wt.status = LX_OK;
 }
 
