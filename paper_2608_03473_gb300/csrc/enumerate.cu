@@ -969,20 +969,27 @@ struct EnRun {
     uint16_t *guess_buf = nullptr;   // [M] scratch for predicted contexts
 };
 
-// Validate, upload tables, size the scratch and fill the parameters.
-int en_setup(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
-             uint32_t *d_lens, uint64_t capacity, void *stream, EnRun &R, bool stage = false)
+int en_args(const lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, const uint16_t *d_kinds,
+            const uint32_t *d_lens, uint64_t capacity)
 {
     if (!c || !ts) return LX_E_INVAL;
     if (mode < LX_FULL_EXACT || mode > LX_FILTERED_MODULO) return LX_E_MODE;
     if (n && !d_in) return LX_E_INVAL;
     if (capacity && (!d_kinds || !d_lens)) return LX_E_INVAL;
+    return ts->scan.status;
+}
+
+// Validate, upload tables, size the scratch and fill the parameters.
+int en_setup(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+             uint32_t *d_lens, uint64_t capacity, void *stream, EnRun &R, bool stage = false)
+{
+    int rc = en_args(c, ts, d_in, n, mode, d_kinds, d_lens, capacity);
+    if (rc != LX_OK) return rc;
     const ScanTable &st = ts->scan;
-    if (st.status != LX_OK) return st.status;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != c->device) return LX_E_INVAL;
     DeviceTables dt;
-    int rc = ensure_device_tables(ts, dev, &dt);
+    rc = ensure_device_tables(ts, dev, &dt);
     if (rc != LX_OK) return rc;
     void *scan = dt.d_scan;
     const uint64_t M64 = (n + CHUNK - 1) / CHUNK;
@@ -1194,7 +1201,13 @@ int lx::lex_enumerative_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *
     *n_tokens = 0;
     *consumed = 0;
     EnRun R;
-    int rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R);
+    int rc;
+    if (!guard && n && en_args(c, ts, d_in, n, mode, d_kinds, d_lens, capacity) == LX_OK && contexts_path_ok(ts, mode)) {
+        rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, stream, nullptr,
+                                 nullptr);
+        if (rc != LX_ROWS) return rc;
+    }
+    rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R);
     if (rc != LX_OK || n == 0) return rc;
     if (c->timing) cudaEventRecord(c->ev[0], R.s);
     if (guard && (rc = en_guard(c, ts, R)) != LX_OK) return rc;
@@ -1250,7 +1263,18 @@ extern "C" int lx_lex_speculative(lx_ctx *c, const lx_tokenset *ts, lx_model *mo
     *consumed = 0;
     if (stats) *stats = lx_spec_stats{0, 0, 0, 0};
     EnRun R;
-    int rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R, true);
+    int rc = en_args(c, ts, d_in, n, mode, d_kinds, d_lens, capacity);
+    if (rc == LX_OK && n && (!model || model_contexts(model) == ts->scan.S + 1) && contexts_path_ok(ts, mode) &&
+        (reinterpret_cast<uintptr_t>(d_in) & 15u) == 0) {   // chunk targets count from the input's start
+        lx_spec_stats sp{0, 0, 0, 0};
+        rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed,
+                                 static_cast<cudaStream_t>(stream), model, &sp);
+        if (rc != LX_ROWS) {
+            if (stats) *stats = sp;
+            return rc;
+        }
+    }
+    rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R, true);
     if (rc != LX_OK || n == 0) return rc;
     if (model && model_contexts(model) != ts->scan.S + 1) return LX_E_INVAL;
     if (c->timing) cudaEventRecord(c->ev[0], R.s);

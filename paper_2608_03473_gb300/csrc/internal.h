@@ -120,6 +120,7 @@ struct WalkTable {
     // relative row address; p_pre where the runs end in different rows
     std::vector<uint16_t> sync;
     uint32_t n_sync = 0;                  // byte values that synchronize
+    std::vector<uint8_t> noacc;           // per row: no run from q0 to it passes or ends in an accepting state
 };
 
 // ---------------------------------------------------------------------------

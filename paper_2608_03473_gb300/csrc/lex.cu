@@ -1032,10 +1032,11 @@ int lx::ensure_device_tables(const lx_tokenset *cts, int device, DeviceTables *o
     }
     if (rc == LX_OK && ts->scan.status == LX_OK) rc = upload(ts->scan.blob, &dt.d_scan);
     for (int m = 0; m < 3 && rc == LX_OK; m++)
-        if (ts->walk[m].status == LX_OK) {   // the synchronizing rows right behind the table
+        if (ts->walk[m].status == LX_OK) {   // the synchronizing rows and the noacc bytes right behind the table
             std::vector<uint8_t> w = ts->walk[m].blob;
             const uint8_t *y = reinterpret_cast<const uint8_t *>(ts->walk[m].sync.data());
             w.insert(w.end(), y, y + 2 * ts->walk[m].sync.size());
+            w.insert(w.end(), ts->walk[m].noacc.begin(), ts->walk[m].noacc.end());
             rc = upload(w, &dt.d_walk[m]);
         }
     if (rc == LX_OK && ts->liveness.status == LX_OK) rc = upload(ts->liveness.blob, &dt.d_live);
@@ -1350,6 +1351,8 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;
     if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
         const int rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        if (rc == LX_FAR)   // contexts are enumerated instead
+            return lx_lex_enumerative(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
         if (rc != LX_ROWS) return rc;
     }
     const bool warp_ok = !force && c->kernel != LX_KERNEL_TILE && warp_path_ok(ts, mode, d_in);

@@ -45,199 +45,11 @@
 #include <algorithm>
 #include <cstdint>
 
-#include "devutil.cuh"
-#include "internal.h"
-#include "lookback.cuh"
+#include "rows.cuh"
 #include "runtime.h"
 
 namespace lx {
 namespace {
-
-constexpr uint32_t NONE = 0xFFFFFFFFu;
-constexpr uint32_t BIG = 0x7FFFFFFFu;
-constexpr uint32_t ROW_UNKNOWN = 0xFFFFu;   // entry row: none found (rows are at even addresses)
-constexpr int MAX_WARPS = 20;               // warps per CTA at most
-constexpr uint32_t LEN_MAX = 511;           // a stage entry's length field; this value: kept aside
-constexpr uint32_t GUESS_MAX = 8192;        // bytes before a slice searched for a synchronizing byte
-constexpr int GUESS_NT = 512;
-constexpr unsigned ERR_TIMEOUT = ERR_TIMEOUT_BIT;
-constexpr unsigned ERR_SMEM = 2u;
-constexpr unsigned ERR_ROWS = 4u;           // entry rows do not fit together: lex the input another way
-
-// A warp's shared memory: the event buffer, SLICE + 16 bytes per lane (the
-// 16-byte stores and loads of eight lanes then fall in different banks), and
-// the stage of STAGE tokens, 2 bytes each (event code << 8 | length).
-template <int NW>   // event mask words per lane
-struct Geo {
-    static constexpr uint32_t SLICE = 32 * NW;
-    static constexpr uint32_t TILE = 32 * SLICE;
-    static constexpr uint32_t STRIDE = SLICE + 16;
-    static constexpr uint32_t STAGE = NW < 3 ? TILE : 512 + 256 * NW;
-    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE;
-    static_assert(WAREA % 16 == 0, "geometry");
-};
-
-struct RResult {
-    unsigned long long total;          // kept tokens over all tiles
-    unsigned long long inv_fail_pos;   // ~min failure position, 0 = none
-    unsigned long long inv_fail_tok;   // ~output index at that failure
-    unsigned int error;
-    unsigned int pad;
-};
-
-struct RParams {
-    const uint8_t *in;             // 16-byte aligned; the input is [lo, n) of it
-    uint64_t n;
-    uint32_t lo;                   // 0..15
-    uint32_t slice;                // bytes per slice
-    const uint8_t *blob;           // walk table, then WalkTable::sync
-    uint32_t blob_bytes, rows_bytes, row_shift, sync_bytes;   // multiples of 16 but the shift
-    uint32_t p_start, p_pre, acc_off, kmap_off, cmap_off;
-    uint32_t guess;                // bytes walked before a slice at first
-    uint16_t *rows;                // entry row of every slice (relative address)
-    uint64_t n_slices;
-    uint16_t *out_kinds;
-    uint32_t *out_lens;
-    uint64_t cap;
-    uint16_t *spill;               // per warp of the grid: a tile's stage entries beyond the shared stage
-    unsigned long long *status;    // per tile: ST_AGG | exit row << 32 | last event position + 1 << 16 | kept count
-    unsigned long long *gagg, *ginc;   // per group of tiles (lookback.cuh)
-    unsigned int *tile_counter;
-    RResult *res;
-    uint64_t zero_bytes;           // of the scratch from res on, zeroed by row_guess
-    uint32_t n_tiles;
-    uint64_t timeout_ns;
-    uint32_t withhold;
-    uint32_t n_pat;                // synchronizing byte values where they are few (0: more than four)
-    uint32_t pat[4];               // each four times
-    static constexpr unsigned long long COUNT = 0xFFFFull;
-    static constexpr bool SMALL = true;
-    __device__ unsigned int *error() const { return &res->error; }
-};
-
-// Shared addresses of the tables.
-struct REnv {
-    uint32_t tb, start, pre, slow, acc, kmap, cmap, shift;
-};
-
-__device__ __forceinline__ uint4 ldg16(const uint8_t *p)
-{
-    return __ldg(reinterpret_cast<const uint4 *>(p));
-}
-__device__ __forceinline__ void sts16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
-}
-__device__ __forceinline__ uint4 lds16(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
-}
-
-template <int FORM>
-__device__ __forceinline__ uint32_t wstep(const REnv &E, uint32_t e, uint32_t b)
-{
-    const uint32_t a = FORM == FORM_BYTE ? ((e & ~0x1FEu) | (b << 1)) : ((e & ~0xFFu) | lds_u8(E.cmap + b));
-    return lds_u16(a);
-}
-__device__ __forceinline__ uint32_t acc_code(const REnv &E, uint32_t e)
-{
-    return lds_u8(E.acc + ((e - E.tb) >> E.shift));
-}
-
-// Four byte steps over the little-endian word w (per byte one LOP3 and the
-// dependent table load; the class form adds a PRMT and the class map's load,
-// which depend on the input alone); returns the four event codes.
-#define LXR_B(XOP, VIN, VOUT)                                                  \
-    XOP "lop3.b32 a, " VIN ", t, %4, 0xD8;\n\t"                                \
-        "ld.shared.u16 " VOUT ", [a];\n\t"
-#define LXR_C(SEL, VIN, VOUT)                                                  \
-    "prmt.b32 t, %2, %3, " SEL ";\n\t"                                         \
-    "ld.shared.u8 c, [t];\n\t"                                                 \
-    "lop3.b32 a, " VIN ", c, %4, 0xD8;\n\t"                                    \
-    "ld.shared.u16 " VOUT ", [a];\n\t"
-#define LXR_HEAD "{\n\t.reg .b32 t, a, c, v0, v1, v2, t0, t1;\n\t"
-#define LXR_PACK                                                               \
-    "prmt.b32 t0, v0, v1, 0x0040;\n\t"                                         \
-    "prmt.b32 t1, v2, %0, 0x0040;\n\t"                                         \
-    "prmt.b32 %1, t0, t1, 0x5410;\n\t}"
-
-template <int FORM>
-__device__ __forceinline__ uint32_t wword(uint32_t &e, uint32_t w, uint32_t cm)
-{
-    uint32_t pk;
-    if (FORM == FORM_BYTE)
-        asm volatile(LXR_HEAD LXR_B("shl.b32 t, %2, 1;\n\t", "%0", "v0") LXR_B("shr.b32 t, %2, 7;\n\t", "v0", "v1")
-                         LXR_B("shr.b32 t, %2, 15;\n\t", "v1", "v2") LXR_B("shr.b32 t, %2, 23;\n\t", "v2", "%0")
-                             LXR_PACK
-                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0x1FEu) : "memory");
-    else
-        asm volatile(LXR_HEAD LXR_C("0x7650", "%0", "v0") LXR_C("0x7651", "v0", "v1") LXR_C("0x7652", "v1", "v2")
-                         LXR_C("0x7653", "v2", "%0") LXR_PACK
-                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0xFFu) : "memory");
-    return pk;
-}
-
-__device__ __forceinline__ uint32_t top_bit(uint32_t x)   // index of the highest one, NONE for 0
-{
-    uint32_t b;
-    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(x));
-    return b;
-}
-
-// A kept token (code >= 4) of length d into the stage at sa, which advances.
-__device__ __forceinline__ void put_token(uint32_t &sa, uint32_t code, uint32_t d)
-{
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 v;\n\t"
-                 "setp.gt.u32 p, %1, 3;\n\t"
-                 "mad.lo.u32 v, %1, 256, %2;\n\t"
-                 "@p st.shared.u16 [%0], v;\n\t"
-                 "@p add.u32 %0, %0, 2;\n\t}"
-                 : "+r"(sa) : "r"(code), "r"(d) : "memory");
-}
-
-__device__ __forceinline__ uint32_t kept_mask(uint32_t w)   // bit 7 of every byte >= 4 (a kept code)
-{
-    return (((w | 0x80808080u) - 0x04040404u) | w) & 0x80808080u;
-}
-__device__ __forceinline__ uint32_t event_mask(uint32_t w)  // bit 7 of every nonzero byte
-{
-    return (((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u;
-}
-
-// Stage the walk table (row offsets become shared addresses) with the PRE
-// row replaced by the synchronizing one; false where the 16-bit row
-// addresses would not reach every row.
-template <int FORM>
-__device__ bool stage_table(const RParams &P, uint8_t *smem, REnv &E)
-{
-    const uint32_t sbase = smem_u32(smem), tb = (sbase + 511u) & ~511u;
-    if (tb + P.rows_bytes > 65536u) {
-        if (threadIdx.x == 0) atomicOr(P.error(), ERR_SMEM);
-        return false;
-    }
-    uint4 *dst = reinterpret_cast<uint4 *>(smem + (tb - sbase));
-    const uint4 *src = reinterpret_cast<const uint4 *>(P.blob);
-    const uint32_t n = P.blob_bytes / 16, r = P.rows_bytes / 16, pre = P.p_pre / 16, tb2 = tb * 0x10001u;
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        uint4 v = __ldg(src + (i - pre < P.sync_bytes / 16 ? n + (i - pre) : i));
-        if (i < r) v = make_uint4(__vadd2(v.x, tb2), __vadd2(v.y, tb2), __vadd2(v.z, tb2), __vadd2(v.w, tb2));
-        dst[i] = v;
-    }
-    E.tb = E.slow = tb;
-    E.start = tb + P.p_start;
-    E.pre = tb + P.p_pre;
-    E.acc = tb + P.acc_off;
-    E.kmap = tb + P.kmap_off;
-    E.cmap = tb + P.cmap_off;
-    E.shift = P.row_shift;
-    return true;
-}
 
 // Whether one of the few synchronizing byte values is among a block's bytes.
 __device__ __forceinline__ bool has_sync(const RParams &P, const uint4 &c)
@@ -522,6 +334,10 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
     uint16_t *const spill = P.spill + ((size_t)blockIdx.x * (blockDim.x >> 5) + wid) * (TILE + 1);
     const uint32_t ahead = gridDim.x * (blockDim.x / 32);
     const uint32_t lt = (1u << lane) - 1u;
+    if (P.before && *P.before != 0) {   // no rows to start from
+        if (threadIdx.x == 0) atomicOr(P.error(), ERR_ROWS);
+        return;
+    }
 
     Pending pend;
     pend.tile = NONE;
@@ -556,9 +372,9 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
             er = guess_row<FORM>(P, E, p, has && p > 0);
             if (p == 0) er = P.p_start;
         } else {
-            er = has ? P.rows[(uint64_t)tile * 32 + lane] : 0u;
+            er = has ? P.rows[((uint64_t)tile * 32 + lane) * P.row_step] : 0u;
         }
-        const bool act = has && er != ROW_UNKNOWN;
+        const bool act = has && er < ROW_DEAD;
         const uint32_t e_in = er + E.tb, ps = max(p0, lo), pe = min(p0 + SLICE, nrel);
         uint32_t e = e_in;
 
@@ -597,7 +413,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         // the lane's end: backtracking, the end of the input, the exit row
         const bool at_end = act && pe == nrel;
         uint32_t tail = 0, fail = NONE, exit = e & ~0xFFu;   // without the event code
-        bool back = has && !act;
+        bool back = has && er == ROW_UNKNOWN;
         if (at_end && e != E.slow && e < E.pre) tail = acc_code(E, e);
         if (act && (e == E.slow || (at_end && !tail)))
             relex<FORM>(E, in, evl, p0, ps, pe, e_in, at_end, &exit, &tail, &fail, &back);
@@ -605,9 +421,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         {
             const uint32_t ner = __shfl_down_sync(0xffffffffu, er, 1);
             bool bad = back;
-            if (lane < 31 && act && !back && fail == NONE && !at_end && exit - E.tb != ner) bad = true;
+            const bool far = has && er == ROW_UNKNOWN;
+            if (lane < 31 && act && fail == NONE && !at_end && exit - E.tb != ner) bad = true;
             if (__any_sync(0xffffffffu, bad && p0 <= fmin)) {
-                if (lane == 0) atomicOr(P.error(), ERR_ROWS);
+                const unsigned err = __any_sync(0xffffffffu, far && p0 <= fmin) ? ERR_FAR : ERR_ROWS;
+                if (lane == 0) atomicOr(P.error(), err);
                 break;
             }
         }
@@ -834,16 +652,17 @@ int allow_smem(lx_ctx *c, int form, int nw, bool fused)
 
 // Geometry of a launch over L.P.n bytes: the slice length (32 nw bytes), the
 // warps per CTA and the grid (one CTA per SM).
-int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L)
+int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGiven *given)
 {
     const WalkTable &w = ts->walk[mode];
     const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16, want = warps_setting(c, ts, mode);
     const uint64_t n = L.P.n;
-    L.fused = n <= FUSED_MAX;
+    L.fused = !given && n <= FUSED_MAX;
     double best = 0;
     int nw = 0;
     for (int k = 1; k <= (L.fused ? 2 : 8); k++) {
         if (fixed + AREA[k] > SMEM_BUDGET) break;
+        if (given && 32 * k % given->step != 0) continue;
         uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[k]);
         if (want) warps = std::min(warps, want);
         const uint64_t tiles = (n + 1024 * k - 1) / (1024 * k), all = (uint64_t)warps * c->num_sms;
@@ -870,9 +689,9 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L)
     return allow_smem(c, w.form, nw, L.fused);
 }
 
-void launch(const RLaunch &L, cudaStream_t st)
+void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
 {
-    if (!L.fused) {
+    if (!L.fused && !given) {
         if (L.form == FORM_BYTE) row_guess<FORM_BYTE><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
         else row_guess<FORM_CLASS><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
     }
@@ -886,8 +705,24 @@ bool rows_path_ok(const lx_tokenset *ts, int mode)
     return ts->walk[mode].status == LX_OK && ts->walk[mode].n_sync > 0;
 }
 
+void rows_table(const lx_tokenset *ts, int mode, const DeviceTables &dt, RParams &P)
+{
+    const WalkTable &w = ts->walk[mode];
+    P.blob = static_cast<const uint8_t *>(dt.d_walk[mode]);
+    P.blob_bytes = (uint32_t)w.blob.size();
+    P.rows_bytes = w.rows_bytes;
+    P.row_shift = w.row_shift;
+    P.sync_bytes = 2 * (uint32_t)w.sync.size();
+    P.p_start = w.p_start;
+    P.p_pre = w.p_pre;
+    P.acc_off = w.acc_off;
+    P.kmap_off = w.kmap_off;
+    P.cmap_off = w.cmap_off;
+}
+
 int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
-                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st)
+                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
+                    const RowsGiven *given)
 {
     if (n == 0) {
         *n_tokens = 0;
@@ -907,19 +742,10 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     P.in = d_in - P.lo;
     P.n = n + P.lo;
     L.form = w.form;
-    rc = shape(c, ts, mode, L);
+    rc = shape(c, ts, mode, L, given);
     if (rc == LX_E_TOOBIG) return LX_ROWS;
     if (rc != LX_OK) return rc;
-    P.blob = static_cast<const uint8_t *>(dt.d_walk[mode]);
-    P.blob_bytes = (uint32_t)w.blob.size();
-    P.rows_bytes = w.rows_bytes;
-    P.row_shift = w.row_shift;
-    P.sync_bytes = 2 * (uint32_t)w.sync.size();
-    P.p_start = w.p_start;
-    P.p_pre = w.p_pre;
-    P.acc_off = w.acc_off;
-    P.kmap_off = w.kmap_off;
-    P.cmap_off = w.cmap_off;
+    rows_table(ts, mode, dt, P);
     P.guess = 32;
     if (w.n_sync <= 4)   // few byte values synchronize: they are searched for
         for (uint32_t b = 0; b < 256; b++)
@@ -929,12 +755,12 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     P.cap = capacity;
     P.timeout_ns = c->timeout_ns;
     P.withhold = c->withhold;
-    // scratch: record and tile counter, status words, group words and counters
-    // (zeroed), entry rows, spill slots
+    // scratch: record and tile counter, status words, group words (zeroed),
+    // entry rows, spill slots
     auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
     const uint64_t groups = (P.n_tiles + GS - 1) / GS;
     const uint64_t o_g = 64 + 8ull * P.n_tiles, o_i = o_g + 8 * groups, zero = (o_i + 8 * groups + 15) & ~15ull;
-    const uint64_t o_rows = al(zero), o_spill = al(o_rows + (L.fused ? 0 : 2 * P.n_slices));
+    const uint64_t o_rows = al(zero), o_spill = al(o_rows + (L.fused || given ? 0 : 2 * P.n_slices));
     const uint64_t need = o_spill + 2ull * (32 * P.slice + 1) * L.grid * L.nwarps;
     rc = grow(&c->scratch, &c->scratch_bytes, need);
     if (rc != LX_OK) return rc;
@@ -946,15 +772,17 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     P.gagg = reinterpret_cast<unsigned long long *>(scr + o_g);
     P.ginc = reinterpret_cast<unsigned long long *>(scr + o_i);
     P.zero_bytes = zero;
-    P.rows = reinterpret_cast<uint16_t *>(scr + o_rows);
+    P.rows = given ? given->rows : reinterpret_cast<uint16_t *>(scr + o_rows);
+    P.row_step = given ? P.slice / given->step : 1;
+    P.before = given ? given->error : nullptr;
     P.spill = reinterpret_cast<uint16_t *>(scr + o_spill);
     L.ggrid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (P.n_slices + GUESS_NT - 1) / GUESS_NT);
-    if (L.fused) {
+    if (L.fused || given) {
         rc = cuda_err(cudaMemsetAsync(scr, 0, zero, st));
         if (rc != LX_OK) return rc;
     }
-    if (c->timing) cudaEventRecord(c->ev[0], st);
-    launch(L, st);
+    if (c->timing && !given) cudaEventRecord(c->ev[0], st);
+    launch(L, given, st);
     rc = cuda_err(cudaGetLastError());
     if (c->timing) cudaEventRecord(c->ev[1], st);
     if (rc != LX_OK) return rc;
@@ -962,7 +790,8 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     if (rc == LX_OK) rc = cuda_err(cudaStreamSynchronize(st));
     if (rc != LX_OK) return rc;
     const RResult r = *static_cast<const RResult *>(c->h_res);
-    if (r.error & ERR_TIMEOUT) return r.error == ERR_TIMEOUT ? LX_E_TIMEOUT : LX_ROWS;
+    if (r.error == ERR_TIMEOUT) return LX_E_TIMEOUT;
+    if ((r.error & ~ERR_TIMEOUT) == ERR_FAR) return LX_FAR;   // (waits end early once an error is flagged)
     if (r.error) return LX_ROWS;
     uint64_t tokens = r.total, con = n;
     if (r.inv_fail_pos) {

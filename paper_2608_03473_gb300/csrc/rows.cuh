@@ -1,0 +1,210 @@
+// rows.cuh -- device parts shared by the kernels that walk the event-code
+// tables from known rows (rows.cu, ctxmap.cu): launch parameters, table
+// staging, the byte and word steps.  Not part of the C ABI.
+#pragma once
+
+#include <cstdint>
+
+#include "devutil.cuh"
+#include "internal.h"
+#include "lookback.cuh"
+
+namespace lx {
+
+struct RResult {
+    unsigned long long total;          // kept tokens over all tiles
+    unsigned long long inv_fail_pos;   // ~min failure position, 0 = none
+    unsigned long long inv_fail_tok;   // ~output index at that failure
+    unsigned int error;
+    unsigned int pad;
+};
+
+struct RParams {
+    const uint8_t *in;             // 16-byte aligned; the input is [lo, n) of it
+    uint64_t n;
+    uint32_t lo;                   // 0..15
+    uint32_t slice;                // bytes per slice
+    const uint8_t *blob;           // walk table, then WalkTable::sync
+    uint32_t blob_bytes, rows_bytes, row_shift, sync_bytes;   // multiples of 16 but the shift
+    uint32_t p_start, p_pre, acc_off, kmap_off, cmap_off;
+    uint32_t guess;                // bytes walked before a slice at first
+    uint16_t *rows;                // entry row of every slice (relative address)
+    uint32_t row_step;             // rows per slice of lex_rows
+    const unsigned int *before;    // an error word that the kernels before lex_rows may have set, or nullptr
+    uint64_t n_slices;
+    uint16_t *out_kinds;
+    uint32_t *out_lens;
+    uint64_t cap;
+    uint16_t *spill;               // per warp of the grid: a tile's stage entries beyond the shared stage
+    unsigned long long *status;    // per tile: ST_AGG | exit row << 32 | last event position + 1 << 16 | kept count
+    unsigned long long *gagg, *ginc;   // per group of tiles (lookback.cuh)
+    unsigned int *tile_counter;
+    RResult *res;
+    uint64_t zero_bytes;           // of the scratch from res on, zeroed by row_guess
+    uint32_t n_tiles;
+    uint64_t timeout_ns;
+    uint32_t withhold;
+    uint32_t n_pat;                // synchronizing byte values where they are few (0: more than four)
+    uint32_t pat[4];               // each four times
+    static constexpr unsigned long long COUNT = 0xFFFFull;
+    static constexpr bool SMALL = true;
+    __device__ unsigned int *error() const { return &res->error; }
+};
+
+// The table parameters of a token set's walk table (rows.cu).
+void rows_table(const lx_tokenset *ts, int mode, const DeviceTables &dt, RParams &P);
+
+namespace {   // each translation unit its own copy
+
+constexpr uint32_t NONE = 0xFFFFFFFFu;
+constexpr uint32_t BIG = 0x7FFFFFFFu;
+constexpr uint32_t ROW_UNKNOWN = 0xFFFFu;   // entry row: none found (rows are at even addresses)
+constexpr uint32_t ROW_DEAD = 0xFFFEu;      // entry row: after the first failure
+constexpr int MAX_WARPS = 20;               // warps per CTA at most
+constexpr uint32_t LEN_MAX = 511;           // a stage entry's length field; this value: kept aside
+constexpr uint32_t GUESS_MAX = 8192;        // bytes before a slice searched for a synchronizing byte
+constexpr int GUESS_NT = 512;
+constexpr unsigned ERR_TIMEOUT = ERR_TIMEOUT_BIT;
+constexpr unsigned ERR_SMEM = 2u;
+constexpr unsigned ERR_ROWS = 4u;           // entry rows do not fit together: lex the input another way
+constexpr unsigned ERR_FAR = 8u;            // no synchronizing byte near a slice
+
+// A warp's shared memory: the event buffer, SLICE + 16 bytes per lane (the
+// 16-byte stores and loads of eight lanes then fall in different banks), and
+// the stage of STAGE tokens, 2 bytes each (event code << 8 | length).
+template <int NW>   // event mask words per lane
+struct Geo {
+    static constexpr uint32_t SLICE = 32 * NW;
+    static constexpr uint32_t TILE = 32 * SLICE;
+    static constexpr uint32_t STRIDE = SLICE + 16;
+    static constexpr uint32_t STAGE = NW < 3 ? TILE : 512 + 256 * NW;
+    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE;
+    static_assert(WAREA % 16 == 0, "geometry");
+};
+
+// Shared addresses of the tables.
+struct REnv {
+    uint32_t tb, start, pre, slow, acc, kmap, cmap, shift;
+};
+
+__device__ __forceinline__ uint4 ldg16(const uint8_t *p)
+{
+    return __ldg(reinterpret_cast<const uint4 *>(p));
+}
+__device__ __forceinline__ void sts16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint4 lds16(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+
+template <int FORM>
+__device__ __forceinline__ uint32_t wstep(const REnv &E, uint32_t e, uint32_t b)
+{
+    const uint32_t a = FORM == FORM_BYTE ? ((e & ~0x1FEu) | (b << 1)) : ((e & ~0xFFu) | lds_u8(E.cmap + b));
+    return lds_u16(a);
+}
+__device__ __forceinline__ uint32_t acc_code(const REnv &E, uint32_t e)
+{
+    return lds_u8(E.acc + ((e - E.tb) >> E.shift));
+}
+
+// Four byte steps over the little-endian word w (per byte one LOP3 and the
+// dependent table load; the class form adds a PRMT and the class map's load,
+// which depend on the input alone); returns the four event codes.
+#define LXR_B(XOP, VIN, VOUT)                                                  \
+    XOP "lop3.b32 a, " VIN ", t, %4, 0xD8;\n\t"                                \
+        "ld.shared.u16 " VOUT ", [a];\n\t"
+#define LXR_C(SEL, VIN, VOUT)                                                  \
+    "prmt.b32 t, %2, %3, " SEL ";\n\t"                                         \
+    "ld.shared.u8 c, [t];\n\t"                                                 \
+    "lop3.b32 a, " VIN ", c, %4, 0xD8;\n\t"                                    \
+    "ld.shared.u16 " VOUT ", [a];\n\t"
+#define LXR_HEAD "{\n\t.reg .b32 t, a, c, v0, v1, v2, t0, t1;\n\t"
+#define LXR_PACK                                                               \
+    "prmt.b32 t0, v0, v1, 0x0040;\n\t"                                         \
+    "prmt.b32 t1, v2, %0, 0x0040;\n\t"                                         \
+    "prmt.b32 %1, t0, t1, 0x5410;\n\t}"
+
+template <int FORM>
+__device__ __forceinline__ uint32_t wword(uint32_t &e, uint32_t w, uint32_t cm)
+{
+    uint32_t pk;
+    if (FORM == FORM_BYTE)
+        asm volatile(LXR_HEAD LXR_B("shl.b32 t, %2, 1;\n\t", "%0", "v0") LXR_B("shr.b32 t, %2, 7;\n\t", "v0", "v1")
+                         LXR_B("shr.b32 t, %2, 15;\n\t", "v1", "v2") LXR_B("shr.b32 t, %2, 23;\n\t", "v2", "%0")
+                             LXR_PACK
+                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0x1FEu) : "memory");
+    else
+        asm volatile(LXR_HEAD LXR_C("0x7650", "%0", "v0") LXR_C("0x7651", "v0", "v1") LXR_C("0x7652", "v1", "v2")
+                         LXR_C("0x7653", "v2", "%0") LXR_PACK
+                     : "+r"(e), "=r"(pk) : "r"(w), "r"(cm), "r"(0xFFu) : "memory");
+    return pk;
+}
+
+__device__ __forceinline__ uint32_t top_bit(uint32_t x)   // index of the highest one, NONE for 0
+{
+    uint32_t b;
+    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(x));
+    return b;
+}
+
+// A kept token (code >= 4) of length d into the stage at sa, which advances.
+__device__ __forceinline__ void put_token(uint32_t &sa, uint32_t code, uint32_t d)
+{
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 v;\n\t"
+                 "setp.gt.u32 p, %1, 3;\n\t"
+                 "mad.lo.u32 v, %1, 256, %2;\n\t"
+                 "@p st.shared.u16 [%0], v;\n\t"
+                 "@p add.u32 %0, %0, 2;\n\t}"
+                 : "+r"(sa) : "r"(code), "r"(d) : "memory");
+}
+
+__device__ __forceinline__ uint32_t kept_mask(uint32_t w)   // bit 7 of every byte >= 4 (a kept code)
+{
+    return (((w | 0x80808080u) - 0x04040404u) | w) & 0x80808080u;
+}
+__device__ __forceinline__ uint32_t event_mask(uint32_t w)  // bit 7 of every nonzero byte
+{
+    return (((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u;
+}
+
+// Stage the walk table (row offsets become shared addresses) with the PRE
+// row replaced by the synchronizing one; false where the 16-bit row
+// addresses would not reach every row.
+template <int FORM>
+__device__ bool stage_table(const RParams &P, uint8_t *smem, REnv &E)
+{
+    const uint32_t sbase = smem_u32(smem), tb = (sbase + 511u) & ~511u;
+    if (tb + P.rows_bytes > 65536u) {
+        if (threadIdx.x == 0) atomicOr(P.error(), ERR_SMEM);
+        return false;
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(smem + (tb - sbase));
+    const uint4 *src = reinterpret_cast<const uint4 *>(P.blob);
+    const uint32_t n = P.blob_bytes / 16, r = P.rows_bytes / 16, pre = P.p_pre / 16, tb2 = tb * 0x10001u;
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        uint4 v = __ldg(src + (i - pre < P.sync_bytes / 16 ? n + (i - pre) : i));
+        if (i < r) v = make_uint4(__vadd2(v.x, tb2), __vadd2(v.y, tb2), __vadd2(v.z, tb2), __vadd2(v.w, tb2));
+        dst[i] = v;
+    }
+    E.tb = E.slow = tb;
+    E.start = tb + P.p_start;
+    E.pre = tb + P.p_pre;
+    E.acc = tb + P.acc_off;
+    E.kmap = tb + P.kmap_off;
+    E.cmap = tb + P.cmap_off;
+    E.shift = P.row_shift;
+    return true;
+}
+
+}  // namespace
+}  // namespace lx

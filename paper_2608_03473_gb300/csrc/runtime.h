@@ -119,10 +119,27 @@ bool warp_path_ok(const lx_tokenset *ts, int mode, const uint8_t *d_in);
 // lx_lex, any input alignment), for token sets with a synchronizing byte.
 // LX_ROWS: the entry rows were not found or do not fit together; the caller
 // lexes the input another way.
-constexpr int LX_ROWS = -102;   // internal status, never returned by the C ABI
+// LX_FAR: only because synchronizing bytes lie too far apart.
+constexpr int LX_ROWS = -102;   // internal statuses, never returned by the C ABI
+constexpr int LX_FAR = -103;
 bool rows_path_ok(const lx_tokenset *ts, int mode);
+// Rows already found, one every `step` bytes from the input's first 16-byte
+// block on, and the error word of the kernels that find them.
+struct RowsGiven {
+    uint16_t *rows;
+    uint32_t step;
+    const unsigned int *error;
+};
 int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
-                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st);
+                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
+                    const RowsGiven *given = nullptr);
+// The same with the entry rows found by enumerating contexts (ctxmap.cu): any
+// token set with a walk and a scan table.  With `spec`, the speculative path's
+// predictions and rounds as well (model: nullptr for BOUNDARY everywhere).
+bool contexts_path_ok(const lx_tokenset *ts, int mode);
+int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+                        uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
+                        lx_model *model, lx_spec_stats *spec);
 // Warps per CTA for the warp-tile kernel on (ts, mode): the context's
 // setting, else lx_autotune's choice, else 0 (as many as fit).
 uint32_t warps_setting(const lx_ctx *c, const lx_tokenset *ts, int mode);

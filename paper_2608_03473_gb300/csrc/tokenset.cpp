@@ -442,6 +442,22 @@ void build_walk_table(const lx_tokenset &t, int mode, lx::WalkTable &wt, bool fo
                 if (wt.form == lx::FORM_BYTE) wt.sync[b] = (uint16_t)(to << wt.row_shift);
             }
     }
+    // States that a run can be in after it passed an accepting one: the others
+    // have nothing to backtrack to.
+    std::vector<uint8_t> past(S, 0);
+    std::vector<uint32_t> todo;
+    for (uint32_t q = 0; q < S; q++)
+        if (t.accept[q] != LX_NO_KIND) past[q] = 1, todo.push_back(q);
+    while (!todo.empty()) {
+        const uint32_t q = todo.back();
+        todo.pop_back();
+        for (uint32_t c = 0; c < C; c++) {
+            const uint32_t d = nx(c, q);
+            if (d != LX_NONE && !past[d]) past[d] = 1, todo.push_back(d);
+        }
+    }
+    wt.noacc.assign((R + 15) & ~15u, 0);
+    for (uint32_t q = 0; q < S; q++) wt.noacc[Rq(q)] = !past[q];
     wt.status = LX_OK;
 }
 
