@@ -377,7 +377,8 @@ def lx_ctx_last_kernel_ms(ctx: Ctx) -> float:
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the raw handle: building a Stream object takes 4.6 us, a fifth of a small call
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return int(getattr(stream, "cuda_stream", stream))
 
 

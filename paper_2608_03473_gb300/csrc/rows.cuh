@@ -19,6 +19,11 @@ struct RResult {
     unsigned int pad;
 };
 
+struct HostRecord {
+    RResult r;
+    uint32_t seq;                      // of the last launch that has finished
+};
+
 struct RParams {
     const uint8_t *in;             // 16-byte aligned; the input is [lo, n) of it
     uint64_t n;
@@ -44,6 +49,11 @@ struct RParams {
     uint32_t n_tiles;
     uint64_t timeout_ns;
     uint32_t withhold;
+    // the end of the launch: the last CTA writes the record and then `seq` to
+    // pinned host memory, and with `clean` zeroes the scratch for the next call
+    unsigned int *done;            // CTAs that have finished
+    HostRecord *host;
+    uint32_t seq, clean;
     uint32_t n_pat;                // synchronizing byte values where they are few (0: more than four)
     uint32_t pat[4];               // each four times
     static constexpr unsigned long long COUNT = 0xFFFFull;

@@ -78,6 +78,12 @@ struct lx_ctx {
     // the warp-tile kernel's per-warp spill slots (kept tokens of a tile beyond its shared stage)
     void *w_spill = nullptr;
     size_t w_spill_bytes = 0;
+    // rows.cu: the scratch of small launches (its first part is zero between
+    // them while small_clean), and the last launch's sequence number
+    void *small = nullptr;
+    size_t small_bytes = 0;
+    bool small_clean = false;
+    uint32_t seq = 0;
     // optional kernel timing
     bool timing = false;
     cudaEvent_t ev[2] = {nullptr, nullptr};
