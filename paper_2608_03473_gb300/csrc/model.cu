@@ -41,7 +41,7 @@ constexpr uint32_t MPOOL = 4;        // max-pool width (and stride)
 constexpr uint32_t MU = MW / MPOOL;  // pooled positions
 constexpr uint32_t MIN_ = MU * MF;   // MLP input width (512)
 constexpr int GT = 16;               // GEMM tile
-constexpr uint32_t PRED_BATCH = 16384;
+constexpr uint32_t PRED_BATCH = 24576;
 constexpr float WEIGHT_DECAY = 1e-2f;   // AdamW, on Wc, W1 and W2
 
 }  // namespace
@@ -61,6 +61,8 @@ struct lx_model {
     float *act = nullptr;
     size_t act_floats = 0;
     uint16_t *win = nullptr;
+    bool mg_ready = false;          // k_mlp_grad may use its shared memory
+    float *h_g = nullptr;           // pinned: the gradient and the loss on their way to the caller
     int device = -1;
 };
 
@@ -76,45 +78,406 @@ __device__ __forceinline__ uint32_t window_byte(const uint8_t *in, uint64_t n, u
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-// Convolution, ReLU and max pooling, one thread per (window, pooled
-// position u, filter f): the four convolution outputs t = 4u .. 4u+3 over
-// the eight embedded bytes they touch, the first maximum of their ReLU into
-// m[b, u * MF + f], and its index (with whether it was positive) for the
-// backward pass.
-template <class TW>
-__global__ void k_conv_pool(const uint16_t *win, uint32_t B, const TW *emb, const TW *wc, const TW *bc, float *mo,
-                            uint8_t *arg)
+// Convolution, ReLU and max pooling, one warp per window, lane = filter: the
+// filter's 40 weights stay in registers, the window's embedded bytes in shared
+// memory (two zero rows on either side), and each of them is read once per
+// four outputs: 65 us per 16 384 windows (1.6 times its multiply-adds).  The convolution outputs t = 4u .. 4u+3 give the first maximum
+// of their ReLU into m[b, u * MF + f], and its index (with whether it was
+// positive) for the backward pass.  One thread per (window, u, f), reading
+// embedding and weights from global memory for each, took 258 us per 16 384
+// windows and 11.6 us for 512.
+constexpr int CP_WARPS = 8;
+constexpr uint32_t MPAD = MK / 2, MHR = MW + 2 * MPAD;   // rows of a window in shared memory
+
+__device__ __forceinline__ void load_window(const uint16_t *w, const __nv_bfloat16 *emb, float (*h)[MD], uint32_t lane)
 {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * MIN_) return;
-    const uint32_t b = i / MIN_, r = i % MIN_, u = r / MF, f = r % MF;
-    float h[MPOOL + MK - 1][MD];
+    for (uint32_t t = lane; t < MHR; t += 32) {
+        float v[MD] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (t >= MPAD && t < MPAD + MW) {
+            const uint4 e = __ldg(reinterpret_cast<const uint4 *>(emb + (size_t)w[t - MPAD] * MD));   // MD bf16
+            const uint32_t p[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
-    for (uint32_t j = 0; j < MPOOL + MK - 1; j++) {
-        const int t = (int)(u * MPOOL + j) - (int)(MK / 2);
-        const bool in = t >= 0 && t < (int)MW;
-        const uint32_t x = in ? win[(size_t)b * MW + t] : 0u;
-#pragma unroll
-        for (uint32_t d = 0; d < MD; d++) h[j][d] = in ? to_f(emb[(size_t)x * MD + d]) : 0.0f;
+            for (uint32_t i = 0; i < 4; i++) {
+                v[2 * i] = __uint_as_float(p[i] << 16);
+                v[2 * i + 1] = __uint_as_float(p[i] & 0xFFFF0000u);
+            }
+        }
+        *reinterpret_cast<float4 *>(&h[t][0]) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4 *>(&h[t][4]) = make_float4(v[4], v[5], v[6], v[7]);
     }
-    float best = -1.0f;
-    uint32_t bj = 0, pos = 0;
+}
+
+__global__ void __launch_bounds__(32 * CP_WARPS) k_conv_pool(const uint16_t *win, uint32_t B, const __nv_bfloat16 *emb,
+                                                             const __nv_bfloat16 *wc, const __nv_bfloat16 *bc, float *mo,
+                                                             uint8_t *arg)
+{
+    __shared__ __align__(16) float hs[CP_WARPS][MHR][MD];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float w[MK][MD];
 #pragma unroll
-    for (uint32_t j = 0; j < MPOOL; j++) {
-        float a = to_f(bc[f]);
+    for (uint32_t k = 0; k < MK; k++)
+#pragma unroll
+        for (uint32_t d = 0; d < MD; d++) w[k][d] = to_f(wc[((size_t)lane * MK + k) * MD + d]);
+    const float bias = to_f(bc[lane]);
+    float(*h)[MD] = hs[wid];
+    for (uint32_t b = blockIdx.x * CP_WARPS + wid; b < B; b += gridDim.x * CP_WARPS) {
+        __syncwarp();
+        load_window(win + (size_t)b * MW, emb, h, lane);
+        __syncwarp();
+#pragma unroll 1
+        for (uint32_t u = 0; u < MU; u++) {
+            float a[MPOOL] = {bias, bias, bias, bias};
+#pragma unroll
+            for (uint32_t r = 0; r < MPOOL + MK - 1; r++) {   // row t = 4u + r - 2; every output sums k, d in order
+                const float4 x = *reinterpret_cast<const float4 *>(&h[MPOOL * u + r][0]);
+                const float4 y = *reinterpret_cast<const float4 *>(&h[MPOOL * u + r][4]);
+                const float v[MD] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (uint32_t j = 0; j < MPOOL; j++)
+                    if (r >= j && r - j < MK) {
+#pragma unroll
+                        for (uint32_t d = 0; d < MD; d++) a[j] = fmaf(w[r - j][d], v[d], a[j]);
+                    }
+            }
+            float best = -1.0f;
+            uint32_t bj = 0, pos = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < MPOOL; j++) {
+                const float rr = a[j] > 0.0f ? a[j] : 0.0f;
+                if (rr > best) {
+                    best = rr;
+                    bj = j;
+                    pos = a[j] > 0.0f ? 1u : 0u;
+                }
+            }
+            const size_t i = (size_t)b * MIN_ + u * MF + lane;
+            mo[i] = best;
+            if (arg) arg[i] = (uint8_t)(bj | (pos << 2));
+        }
+    }
+}
+
+// ---- one training batch: k_conv_pool, k_mlp_grad, k_outer ----
+// Everything of a window but the weight gradients is its own: k_mlp_grad takes
+// MG windows per CTA through both dense layers, the softmax and back through
+// the convolution, with the activations in shared memory.  It replaces ten
+// launches (products in 16 x 16 tiles that left most SMs idle, column sums by
+// one thread per column, a thread per convolution weight): a gradient of 512
+// windows 391 -> 88 us, 58 of them in the three kernels, which wait on
+// shared and L2 loads with 16 warps per SM.
+constexpr uint32_t MG = 4;            // windows per CTA
+constexpr uint32_t MG_NT = 512;       // (256 left the SM's schedulers two warps each: 46 us for 512 windows)
+constexpr uint32_t MG_KP = 8;         // parts of the first product's sum
+constexpr uint32_t MG_MAXH = 256, MG_MAXC = 1024;
+constexpr uint32_t DA_LD = MF + 1;    // row stride of the dense pooled gradient (bank spread)
+
+struct MgSmem {   // float offsets of k_mlp_grad's shared memory
+    uint32_t mo, a1, h1, z, dh, part, total;
+    __host__ __device__ MgSmem(uint32_t H, uint32_t C)
+    {
+        uint32_t o = 0;
+        auto take = [&](uint32_t n) { const uint32_t at = o; o += (n + 3) & ~3u; return at; };
+        mo = take(MIN_ * MG);      // [k][window]; later the gradient of m
+        a1 = take(H * MG);
+        h1 = take(H * MG);
+        dh = take(H * MG);
+        z = take(C * MG);          // logits, then their gradient, [c][window]
+        // partial sums of the first product, or the convolution's part: windows,
+        // dense pooled gradients, per-warp weight sums, weights, embedding sums
+        const uint32_t conv = MG * MHR * MD + MG * MHR * DA_LD + (MG_NT / 32) * MF * MK * MD + MF * MK * MD + MROWS * MD;
+        const uint32_t p1 = MG_KP * H * MG, p2 = 2 * C * MG, p = p1 > p2 ? p1 : p2;
+        part = take(conv > p ? conv : p);
+        total = o;
+    }
+};
+
+__global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const uint16_t *y, uint32_t B, uint32_t H,
+                                                    uint32_t C, const float *mo, const uint8_t *arg,
+                                                    const __nv_bfloat16 *emb, const __nv_bfloat16 *wc,
+                                                    const __nv_bfloat16 *w1, const __nv_bfloat16 *b1,
+                                                    const __nv_bfloat16 *w2, const __nv_bfloat16 *b2, float *h1o,
+                                                    float *dzo, float *dho, float *gemb, float *gwc, float *gbc,
+                                                    float *loss)
+{
+    extern __shared__ __align__(16) float sm[];
+    const MgSmem L(H, C);
+    const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, b0 = blockIdx.x * MG;
+    float4 *smo = reinterpret_cast<float4 *>(sm + L.mo), *sa1 = reinterpret_cast<float4 *>(sm + L.a1);
+    float4 *sh1 = reinterpret_cast<float4 *>(sm + L.h1), *sdh = reinterpret_cast<float4 *>(sm + L.dh);
+    float4 *sz = reinterpret_cast<float4 *>(sm + L.z), *sp = reinterpret_cast<float4 *>(sm + L.part);
+    const bool ok[MG] = {b0 < B, b0 + 1 < B, b0 + 2 < B, b0 + 3 < B};
+    static_assert(MG == 4, "one float4 per (feature, four windows)");
+    for (uint32_t i = tid; i < MIN_; i += MG_NT) {
+        float4 v = make_float4(0, 0, 0, 0);
+        if (ok[0]) v.x = mo[(size_t)(b0 + 0) * MIN_ + i];
+        if (ok[1]) v.y = mo[(size_t)(b0 + 1) * MIN_ + i];
+        if (ok[2]) v.z = mo[(size_t)(b0 + 2) * MIN_ + i];
+        if (ok[3]) v.w = mo[(size_t)(b0 + 3) * MIN_ + i];
+        smo[i] = v;
+    }
+    __syncthreads();
+    auto fma4 = [](float4 &a, float w, const float4 &v) {
+        a.x = fmaf(w, v.x, a.x);
+        a.y = fmaf(w, v.y, a.y);
+        a.z = fmaf(w, v.z, a.z);
+        a.w = fmaf(w, v.w, a.w);
+    };
+    auto add4 = [](float4 a, const float4 &v) { return make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w); };
+    // a1 = m W1 + b1, the sum over k in parts
+    for (uint32_t q = tid; q < MG_KP * H; q += MG_NT) {
+        const uint32_t j = q % H, part = q / H;
+        float4 a = make_float4(0, 0, 0, 0);
+#pragma unroll 32
+        for (uint32_t k = part * (MIN_ / MG_KP); k < (part + 1) * (MIN_ / MG_KP); k++) fma4(a, to_f(w1[(size_t)k * H + j]), smo[k]);
+        sp[q] = a;
+    }
+    __syncthreads();
+    for (uint32_t j = tid; j < H; j += MG_NT) {
+        float4 a = sp[j];
+#pragma unroll
+        for (uint32_t q = 1; q < MG_KP; q++) a = add4(a, sp[q * H + j]);
+        const float b = to_f(b1[j]);
+        a = make_float4(a.x + b, a.y + b, a.z + b, a.w + b);
+        sa1[j] = a;
+        a = make_float4(fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f), fmaxf(a.z, 0.0f), fmaxf(a.w, 0.0f));
+        sh1[j] = a;
+        if (ok[0]) h1o[(size_t)(b0 + 0) * H + j] = a.x;
+        if (ok[1]) h1o[(size_t)(b0 + 1) * H + j] = a.y;
+        if (ok[2]) h1o[(size_t)(b0 + 2) * H + j] = a.z;
+        if (ok[3]) h1o[(size_t)(b0 + 3) * H + j] = a.w;
+    }
+    __syncthreads();
+    // z = h1 W2 + b2, the sum over k in two halves
+    for (uint32_t q = tid; q < 2 * C; q += MG_NT) {
+        const uint32_t c = q % C, half = q / C;
+        float4 a = make_float4(0, 0, 0, 0);
+#pragma unroll 16
+        for (uint32_t k = half ? H / 2 : 0; k < (half ? H : H / 2); k++) fma4(a, to_f(w2[(size_t)k * C + c]), sh1[k]);
+        sp[q] = a;
+    }
+    __syncthreads();
+    for (uint32_t c = tid; c < C; c += MG_NT) {
+        const float b = to_f(b2[c]);
+        const float4 a = add4(sp[c], sp[C + c]);
+        sz[c] = make_float4(a.x + b, a.y + b, a.z + b, a.w + b);
+    }
+    __syncthreads();
+    // softmax cross-entropy, a warp per window: dz = (softmax(z) - onehot(y)) / B
+    if (wid < MG && b0 + wid < B) {
+        float *zr = sm + L.z + wid;
+        const uint32_t yb = y[b0 + wid];
+        float mx = -INFINITY;
+        for (uint32_t c = lane; c < C; c += 32) mx = fmaxf(mx, zr[MG * c]);
+        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float se = 0.0f;
+        for (uint32_t c = lane; c < C; c += 32) se += expf(zr[MG * c] - mx);
+        for (int o = 16; o; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+        const float lse = mx + logf(se);
+        if (lane == 0) atomicAdd(loss, (lse - (yb < C ? zr[MG * yb] : 0.0f)) / (float)B);
+        __syncwarp();
+        for (uint32_t c = lane; c < C; c += 32) {
+            const float g = (expf(zr[MG * c] - lse) - (c == yb ? 1.0f : 0.0f)) / (float)B;
+            zr[MG * c] = g;
+            dzo[(size_t)(b0 + wid) * C + c] = g;
+        }
+    } else if (wid < MG) {
+        for (uint32_t c = lane; c < C; c += 32) sm[L.z + MG * c + wid] = 0.0f;
+    }
+    __syncthreads();
+    // dh1 = dz W2^T where a1 > 0: a warp per row of W2
+    for (uint32_t j = wid; j < H; j += MG_NT / 32) {
+        float4 a = make_float4(0, 0, 0, 0);
+        for (uint32_t c = lane; c < C; c += 32) fma4(a, to_f(w2[(size_t)j * C + c]), sz[c]);
+        for (int o = 16; o; o >>= 1) {
+            a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+            a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+            a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
+            a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
+        }
+        if (lane == 0) {
+            const float4 s = sa1[j];
+            a = make_float4(s.x > 0.0f ? a.x : 0.0f, s.y > 0.0f ? a.y : 0.0f, s.z > 0.0f ? a.z : 0.0f,
+                            s.w > 0.0f ? a.w : 0.0f);
+            sdh[j] = a;
+            if (ok[0]) dho[(size_t)(b0 + 0) * H + j] = a.x;
+            if (ok[1]) dho[(size_t)(b0 + 1) * H + j] = a.y;
+            if (ok[2]) dho[(size_t)(b0 + 2) * H + j] = a.z;
+            if (ok[3]) dho[(size_t)(b0 + 3) * H + j] = a.w;
+        }
+    }
+    __syncthreads();
+    // dm = dh1 W1^T, into the place of m
+    for (uint32_t i = tid; i < MIN_; i += MG_NT) {
+        float4 a = make_float4(0, 0, 0, 0);
+        if (H % 8 == 0) {   // a row of W1 is a lane's own: 16 bytes at a time
+            const uint4 *row = reinterpret_cast<const uint4 *>(w1 + (size_t)i * H);
+#pragma unroll 4
+            for (uint32_t j = 0; j < H / 8; j++) {
+                const uint4 v = __ldg(row + j);
+                const uint32_t p[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (uint32_t q = 0; q < 4; q++) {
+                    fma4(a, __uint_as_float(p[q] << 16), sdh[8 * j + 2 * q]);
+                    fma4(a, __uint_as_float(p[q] & 0xFFFF0000u), sdh[8 * j + 2 * q + 1]);
+                }
+            }
+        } else {
+            for (uint32_t j = 0; j < H; j++) fma4(a, to_f(w1[(size_t)i * H + j]), sdh[j]);
+        }
+        smo[i] = a;
+    }
+    // the convolution's part of shared memory
+    float *hs = sm + L.part, *da = hs + MG * MHR * MD, *pw = da + MG * MHR * DA_LD;
+    float *swc = pw + (MG_NT / 32) * MF * MK * MD, *ge = swc + MF * MK * MD;
+    for (uint32_t i = tid; i < MG * MHR * DA_LD; i += MG_NT) da[i] = 0.0f;
+    for (uint32_t i = tid; i < MF * MK * MD; i += MG_NT) swc[i] = to_f(wc[i]);
+    for (uint32_t i = tid; i < MROWS * MD; i += MG_NT) ge[i] = 0.0f;
+    __syncthreads();
+    if (wid < MG && b0 + wid < B)
+        load_window(win + (size_t)(b0 + wid) * MW, emb, reinterpret_cast<float(*)[MD]>(hs + wid * MHR * MD), lane);
+    // the gradient of each pooled maximum at the position that gave it
+    {
+        uint32_t av[MG * MIN_ / MG_NT];   // all loads first
+#pragma unroll
+        for (uint32_t i = 0; i < MG * MIN_ / MG_NT; i++) {
+            const uint32_t q = tid + i * MG_NT;
+            av[i] = b0 + q / MIN_ < B ? arg[(size_t)b0 * MIN_ + q] : 0u;
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < MG * MIN_ / MG_NT; i++) {
+            const uint32_t q = tid + i * MG_NT, w = q / MIN_, r = q % MIN_, u = r / MF, f = r % MF;
+            if (av[i] & 4u) da[(w * MHR + MPAD + MPOOL * u + (av[i] & 3u)) * DA_LD + f] = sm[L.mo + MG * r + w];
+        }
+    }
+    __syncthreads();
+    {   // weights and bias: lane = filter, some warps per window, each its share of the pooled positions
+        constexpr uint32_t WPW = MG_NT / 32 / MG, UP = MU / WPW;
+        const uint32_t w = wid / WPW, u0 = (wid % WPW) * UP;
+        float acc[MK][MD], sb = 0.0f;
 #pragma unroll
         for (uint32_t k = 0; k < MK; k++)
 #pragma unroll
-            for (uint32_t d = 0; d < MD; d++) a = fmaf(to_f(wc[((size_t)f * MK + k) * MD + d]), h[j + k][d], a);
-        const float rr = a > 0.0f ? a : 0.0f;
-        if (rr > best) {
-            best = rr;
-            bj = j;
-            pos = a > 0.0f ? 1u : 0u;
+            for (uint32_t d = 0; d < MD; d++) acc[k][d] = 0.0f;
+        uint32_t av[UP];
+#pragma unroll
+        for (uint32_t i = 0; i < UP; i++) av[i] = b0 + w < B ? arg[(size_t)(b0 + w) * MIN_ + (u0 + i) * MF + lane] : 0u;
+        if (b0 + w < B)
+#pragma unroll
+            for (uint32_t i = 0; i < UP; i++) {
+                const uint32_t u = u0 + i, ar = av[i];
+                const float g = (ar & 4u) ? sm[L.mo + MG * (u * MF + lane) + w] : 0.0f;
+                sb += g;
+                const float *h = hs + (w * MHR + MPOOL * u + (ar & 3u)) * MD;   // row t - 2
+#pragma unroll
+                for (uint32_t k = 0; k < MK; k++) {
+                    const float4 p = *reinterpret_cast<const float4 *>(h + k * MD);
+                    const float4 q = *reinterpret_cast<const float4 *>(h + k * MD + 4);
+                    const float v[MD] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (uint32_t d = 0; d < MD; d++) acc[k][d] = fmaf(g, v[d], acc[k][d]);
+                }
+            }
+#pragma unroll
+        for (uint32_t k = 0; k < MK; k++)
+#pragma unroll
+            for (uint32_t d = 0; d < MD; d++) pw[(wid * MK * MD + k * MD + d) * MF + lane] = acc[k][d];
+        atomicAdd(&gbc[lane], sb);
+    }
+    float dx[MD] = {0, 0, 0, 0, 0, 0, 0, 0};
+    constexpr uint32_t FP = MG_NT / (MG * MW);   // parts of the filters
+    const uint32_t part = tid / (MG * MW), at = tid % (MG * MW);
+    static_assert(FP == 2, "two places for the parts below");
+    {   // dh0: a thread per position of a window and half of the filters
+        const uint32_t w = at / MW, t = at % MW;
+        for (uint32_t k = 0; k < MK; k++) {
+            const float *g = da + (w * MHR + MPAD + t + MPAD - k) * DA_LD;   // output position t + 2 - k
+#pragma unroll 4
+            for (uint32_t f = part * (MF / FP); f < (part + 1) * (MF / FP); f++) {
+                const float gv = g[f];
+                const float4 p = *reinterpret_cast<const float4 *>(swc + (f * MK + k) * MD);
+                const float4 q = *reinterpret_cast<const float4 *>(swc + (f * MK + k) * MD + 4);
+                const float v[MD] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (uint32_t d = 0; d < MD; d++) dx[d] = fmaf(gv, v[d], dx[d]);
+            }
         }
     }
-    mo[i] = best;
-    if (arg) arg[i] = (uint8_t)(bj | (pos << 2));
+    __syncthreads();
+    // into the embedding's rows, eight lanes per position: the lanes of a warp
+    // meet in a word at most four times, however often a byte repeats
+    float *const half0 = hs, *const half1 = sm + L.mo;   // (windows and dm are done with)
+    float *const mine = (part ? half1 : half0) + at * MD;
+    *reinterpret_cast<float4 *>(mine) = make_float4(dx[0], dx[1], dx[2], dx[3]);
+    *reinterpret_cast<float4 *>(mine + 4) = make_float4(dx[4], dx[5], dx[6], dx[7]);
+    __syncthreads();
+    for (uint32_t i = tid; i < MG * MW * MD; i += MG_NT) {
+        const uint32_t t = i / MD;   // window * 64 + position
+        const float v = half0[i] + half1[i];
+        if (v != 0.0f) atomicAdd(&ge[win[(size_t)b0 * MW + t] * MD + i % MD], v);   // 0 past the batch
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < MF * MK * MD; i += MG_NT) {   // i = (k, d) * MF + f
+        float s = 0.0f;
+#pragma unroll
+        for (uint32_t q = 0; q < MG_NT / 32; q++) s += pw[q * MF * MK * MD + i];
+        atomicAdd(&gwc[(i % MF) * MK * MD + i / MF], s);
+    }
+    for (uint32_t i = tid; i < MROWS * MD; i += MG_NT)
+        if (ge[i] != 0.0f) atomicAdd(&gemb[i], ge[i]);
+}
+
+// Weight gradients: G[M x N] += A^T D over a slice of the batch, A [B][M], D
+// [B][N], and the column sums of D (the bias) from the first row of tiles.  64
+// x 64 tiles, 4 x 4 per thread; blockIdx.z: which of the two layers.
+constexpr uint32_t OT = 64, OK = 16, OSLICE = 64;
+
+__global__ void __launch_bounds__(256) k_outer(uint32_t B, const float *A0, const float *D0, uint32_t M0, uint32_t N0,
+                                               float *G0, float *s0, const float *A1, const float *D1, uint32_t M1,
+                                               uint32_t N1, float *G1, float *s1)
+{
+    const bool one = blockIdx.z != 0;
+    const float *A = one ? A1 : A0, *D = one ? D1 : D0;
+    float *G = one ? G1 : G0, *cs = one ? s1 : s0;
+    const uint32_t M = one ? M1 : M0, N = one ? N1 : N0;
+    const uint32_t nt = (N + OT - 1) / OT, m0 = (blockIdx.x / nt) * OT, n0 = (blockIdx.x % nt) * OT;
+    if (m0 >= M) return;
+    __shared__ __align__(16) float As[OK][OT], Ds[OK][OT];
+    const uint32_t tid = threadIdx.x, tx = tid & 15u, ty = tid >> 4;
+    const uint32_t k0 = blockIdx.y * OSLICE, k1 = min(B, k0 + OSLICE);
+    float acc[4][4], sum = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] = 0.0f;
+    for (uint32_t k = k0; k < k1; k += OK) {
+#pragma unroll
+        for (uint32_t i = 0; i < OK * OT / 256; i++) {
+            const uint32_t q = tid + 256 * i, r = q / OT, c = q % OT;
+            As[r][c] = k + r < k1 && m0 + c < M ? A[(size_t)(k + r) * M + m0 + c] : 0.0f;
+            Ds[r][c] = k + r < k1 && n0 + c < N ? D[(size_t)(k + r) * N + n0 + c] : 0.0f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t r = 0; r < OK; r++) {
+            const float4 a = *reinterpret_cast<const float4 *>(&As[r][4 * ty]);
+            const float4 d = *reinterpret_cast<const float4 *>(&Ds[r][4 * tx]);
+            const float av[4] = {a.x, a.y, a.z, a.w}, dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) acc[i][j] = fmaf(av[i], dv[j], acc[i][j]);
+        }
+        if (m0 == 0 && tid < OT)
+            for (uint32_t r = 0; r < OK; r++) sum += Ds[r][tid];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if (m0 + 4 * ty + i < M && n0 + 4 * tx + j < N)
+                atomicAdd(&G[(size_t)(m0 + 4 * ty + i) * N + n0 + 4 * tx + j], acc[i][j]);
+    if (m0 == 0 && tid < OT && n0 + tid < N) atomicAdd(&cs[n0 + tid], sum);
 }
 
 // Backward through pooling and the convolution's weights: each thread one
@@ -190,58 +553,62 @@ __global__ void k_gemm(const float *A, const TW *Bm, float *Cm, const TW *bias, 
 }
 
 // Inference products: C[M x N] = A[M x K] B[K x N] + bias (ReLU optional),
-// each CTA a 64 x 64 tile of C, each thread a 4 x 4 block of it in
-// registers, K in steps of 16 through shared memory.
-constexpr int RB_T = 64, RB_K = 16;
+// each CTA a 128 x 64 tile of C, each thread 8 x 4 of it in registers, K in
+// steps of 16 through shared memory, the next step's loads under way during
+// this one's products.
+constexpr int RB_M = 128, RB_N = 64, RB_K = 16;
 
 template <class TW>
 __global__ void __launch_bounds__(256) k_gemm_rb(const float *A, const TW *Bm, float *Cm, const TW *bias, uint32_t M,
                                                  uint32_t N, uint32_t K, int relu_out)
 {
-    __shared__ __align__(16) float As[RB_K][RB_T + 4];   // A tile, k-major
-    __shared__ __align__(16) float Bs[RB_K][RB_T + 4];
+    __shared__ __align__(16) float As[RB_K][RB_M + 4];   // A tile, k-major
+    __shared__ __align__(16) float Bs[RB_K][RB_N];
     const uint32_t tid = threadIdx.x, tx = tid & 15u, ty = tid >> 4;
-    const uint32_t m0 = blockIdx.y * RB_T, n0 = blockIdx.x * RB_T;
-    float acc[4][4];
+    const uint32_t m0 = blockIdx.y * RB_M, n0 = blockIdx.x * RB_N;
+    const uint32_t ar = tid >> 1, ak = (tid & 1u) * 8u, br = tid >> 4, bc = (tid & 15u) * 4u;
+    float acc[8][4], pa[8], pb[4];
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < 8; i++)
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] = 0.0f;
+    auto fetch = [&](uint32_t k0) {
+        const uint32_t m = m0 + ar;
+        const float *row = A + (size_t)m * K + k0 + ak;
+        if (m < M && K % 4 == 0 && k0 + ak + 8 <= K) {   // rows on 16-byte boundaries
+            const float4 x = *reinterpret_cast<const float4 *>(row), y = *reinterpret_cast<const float4 *>(row + 4);
+            pa[0] = x.x, pa[1] = x.y, pa[2] = x.z, pa[3] = x.w, pa[4] = y.x, pa[5] = y.y, pa[6] = y.z, pa[7] = y.w;
+        } else {
+#pragma unroll
+            for (uint32_t i = 0; i < 8; i++) pa[i] = m < M && k0 + ak + i < K ? row[i] : 0.0f;
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < 4; i++)
+            pb[i] = k0 + br < K && n0 + bc + i < N ? to_f(Bm[(size_t)(k0 + br) * N + n0 + bc + i]) : 0.0f;
+    };
+    fetch(0);
     for (uint32_t k0 = 0; k0 < K; k0 += RB_K) {
-        {
-            const uint32_t r = tid >> 2, kk = (tid & 3u) * 4u, m = m0 + r;
 #pragma unroll
-            for (uint32_t i = 0; i < 4; i++) {
-                const uint32_t k = k0 + kk + i;
-                float v = 0.0f;
-                if (m < M && k < K) v = A[(size_t)m * K + k];
-                As[kk + i][r] = v;
-            }
-        }
-        {
-            const uint32_t kr = tid >> 4, c = (tid & 15u) * 4u, k = k0 + kr;
-#pragma unroll
-            for (uint32_t i = 0; i < 4; i++) {
-                const uint32_t nn = n0 + c + i;
-                Bs[kr][c + i] = (k < K && nn < N) ? to_f(Bm[(size_t)k * N + nn]) : 0.0f;
-            }
-        }
+        for (uint32_t i = 0; i < 8; i++) As[ak + i][ar] = pa[i];
+        *reinterpret_cast<float4 *>(&Bs[br][bc]) = make_float4(pb[0], pb[1], pb[2], pb[3]);
         __syncthreads();
+        if (k0 + RB_K < K) fetch(k0 + RB_K);
 #pragma unroll
         for (int k = 0; k < RB_K; k++) {
-            const float4 a = *reinterpret_cast<const float4 *>(&As[k][ty * 4]);
+            const float4 a = *reinterpret_cast<const float4 *>(&As[k][ty * 8]);
+            const float4 c = *reinterpret_cast<const float4 *>(&As[k][ty * 8 + 4]);
             const float4 b = *reinterpret_cast<const float4 *>(&Bs[k][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+            const float av[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-            for (int i = 0; i < 4; i++)
+            for (int i = 0; i < 8; i++)
 #pragma unroll
                 for (int j = 0; j < 4; j++) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const uint32_t m = m0 + ty * 4 + i;
+    for (int i = 0; i < 8; i++) {
+        const uint32_t m = m0 + ty * 8 + i;
         if (m >= M) continue;
 #pragma unroll
         for (int j = 0; j < 4; j++) {
@@ -389,9 +756,10 @@ using namespace lx;
 
 namespace {
 
-int ensure_act(lx_model *m, uint32_t B)
+int ensure_act(lx_model *m, uint32_t B, bool predict = false)
 {
-    const size_t need = (size_t)B * (MIN_ * 2 + MW * MD + m->H * 3 + m->C * 2) + 16;
+    const size_t need = predict ? (size_t)B * (MIN_ + m->H + m->C) + 16
+                                : (size_t)B * (MIN_ * 2 + MW * MD + m->H * 3 + m->C * 2) + 16;
     if (m->act_floats < need) {
         if (m->act) cudaFree(m->act);
         m->act = nullptr;
@@ -399,7 +767,7 @@ int ensure_act(lx_model *m, uint32_t B)
         if (cudaMalloc(&m->act, need * sizeof(float)) != cudaSuccess) return LX_E_NOMEM;
         m->act_floats = need;
     }
-    const size_t abytes = (size_t)B * MIN_;
+    const size_t abytes = predict ? 0 : (size_t)B * MIN_;
     if (m->arg_bytes < abytes) {
         if (m->arg) cudaFree(m->arg);
         m->arg = nullptr;
@@ -411,7 +779,8 @@ int ensure_act(lx_model *m, uint32_t B)
 }
 
 dim3 gemm_grid(uint32_t M, uint32_t N) { return dim3((N + GT - 1) / GT, (M + GT - 1) / GT); }
-dim3 rb_grid(uint32_t M, uint32_t N) { return dim3((N + RB_T - 1) / RB_T, (M + RB_T - 1) / RB_T); }
+uint32_t conv_grid(uint32_t B) { return std::min<uint32_t>((B + CP_WARPS - 1) / CP_WARPS, 8 * 152); }
+dim3 rb_grid(uint32_t M, uint32_t N) { return dim3((N + RB_N - 1) / RB_N, (M + RB_M - 1) / RB_M); }
 
 // Forward (and with labels, backward into m->g) for a batch of windows, on
 // the BF16 weights.  Activations: m | a1 | h1 | z | dz | dh1 | dm | dh0 | loss
@@ -427,8 +796,30 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
     const __nv_bfloat16 *w = m->w16;
     const dim3 t2(GT, GT);
     const uint32_t nm = B * MIN_;
-    k_conv_pool<__nv_bfloat16><<<(nm + 255) / 256, 256, 0, s>>>(d_win, B, w + m->o_emb, w + m->o_wc, w + m->o_bc, mo,
-                                                               m->arg);
+    k_conv_pool<<<conv_grid(B), 32 * CP_WARPS, 0, s>>>(d_win, B, w + m->o_emb, w + m->o_wc, w + m->o_bc, mo, m->arg);
+    if (d_y && !d_logits_out && H <= MG_MAXH && C <= MG_MAXC) {
+        const uint32_t smem = 4 * MgSmem(H, C).total;
+        if (!m->mg_ready) {   // once per model; the largest sizes', which all models share
+            rc = cuda_err(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               4 * MgSmem(MG_MAXH, MG_MAXC).total));
+            if (rc != LX_OK) return rc;
+            m->mg_ready = true;
+        }
+        float *g = m->g;   // the loss follows the gradient
+        cudaMemsetAsync(g, 0, sizeof(float) * (m->n_params + 1), s);
+        k_mlp_grad<<<(B + MG - 1) / MG, MG_NT, smem, s>>>(d_win, d_y, B, H, C, mo, m->arg, w + m->o_emb, w + m->o_wc,
+                                                         w + m->o_w1, w + m->o_b1, w + m->o_w2, w + m->o_b2, h1, dz, dh1,
+                                                         g + m->o_emb, g + m->o_wc, g + m->o_bc, g + m->n_params);
+        const uint32_t t1 = (MIN_ / OT) * ((H + OT - 1) / OT), t2n = ((H + OT - 1) / OT) * ((C + OT - 1) / OT);
+        k_outer<<<dim3(std::max(t1, t2n), (B + OSLICE - 1) / OSLICE, 2), 256, 0, s>>>(
+            B, mo, dh1, MIN_, H, g + m->o_w1, g + m->o_b1, h1, dz, H, C, g + m->o_w2, g + m->o_b2);
+        rc = cuda_err(cudaGetLastError());
+        if (rc == LX_OK && h_loss) {
+            rc = cuda_err(cudaMemcpyAsync(h_loss, g + m->n_params, sizeof(float), cudaMemcpyDeviceToHost, s));
+            if (rc == LX_OK) rc = cuda_err(cudaStreamSynchronize(s));
+        }
+        return rc;
+    }
     k_gemm<__nv_bfloat16><<<gemm_grid(B, H), t2, 0, s>>>(mo, w + m->o_w1, a1, w + m->o_b1, B, H, MIN_, 0, 0, 0);
     cudaMemcpyAsync(h1, a1, sizeof(float) * B * H, cudaMemcpyDeviceToDevice, s);
     k_relu_back<<<(B * H + 255) / 256, 256, 0, s>>>(h1, a1, (size_t)B * H);   // h1 = relu(a1)
@@ -453,6 +844,7 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
     k_conv_back_w<__nv_bfloat16><<<gw, 128, 0, s>>>(d_win, B, w + m->o_emb, dm, m->arg, g + m->o_wc, g + m->o_bc, per);
     k_conv_back_x<__nv_bfloat16><<<(nm + 255) / 256, 256, 0, s>>>(B, w + m->o_wc, dm, m->arg, dh0);
     k_emb_back<<<(B * MW * MD + 255) / 256, 256, 0, s>>>(d_win, B, dh0, g + m->o_emb);
+    cudaMemcpyAsync(g + m->n_params, loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
     rc = cuda_err(cudaGetLastError());
     if (rc == LX_OK && h_loss) {
         rc = cuda_err(cudaMemcpyAsync(h_loss, loss, sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -478,8 +870,8 @@ int lx::model_predict(lx_model *m, const uint8_t *in, uint64_t n, const uint64_t
                       const uint8_t *scan_blob, uint32_t cbeg_off, uint32_t cand_off, uint32_t M, uint16_t *guess,
                       cudaStream_t s)
 {
-    const uint32_t B = std::min<uint32_t>(M, PRED_BATCH);
-    int rc = ensure_act(m, B);
+    const uint32_t parts = (M + PRED_BATCH - 1) / PRED_BATCH, B = (M + parts - 1) / parts;   // batches of equal size
+    int rc = ensure_act(m, B, true);
     if (rc != LX_OK) return rc;
     if (!m->win && cudaMalloc(&m->win, sizeof(uint16_t) * PRED_BATCH * MW) != cudaSuccess) return LX_E_NOMEM;
     const uint32_t H = m->H, C = m->C;
@@ -488,8 +880,8 @@ int lx::model_predict(lx_model *m, const uint8_t *in, uint64_t n, const uint64_t
     for (uint32_t j0 = 0; j0 < M; j0 += B) {
         const uint32_t cnt = std::min<uint32_t>(B, M - j0);
         k_windows<<<(cnt * MW + 255) / 256, 256, 0, s>>>(in, n, start, j0, cnt, m->win);
-        k_conv_pool<__nv_bfloat16><<<(cnt * MIN_ + 255) / 256, 256, 0, s>>>(m->win, cnt, w + m->o_emb, w + m->o_wc,
-                                                                           w + m->o_bc, mo, nullptr);
+        k_conv_pool<<<conv_grid(cnt), 32 * CP_WARPS, 0, s>>>(m->win, cnt, w + m->o_emb, w + m->o_wc, w + m->o_bc, mo,
+                                                             nullptr);
         // h1 = relu(m W1 + b1), z = h1 W2 + b2
         k_gemm_rb<__nv_bfloat16><<<rb_grid(cnt, H), 256, 0, s>>>(mo, w + m->o_w1, h1, w + m->o_b1, cnt, H, MIN_, 1);
         k_gemm_rb<__nv_bfloat16><<<rb_grid(cnt, C), 256, 0, s>>>(h1, w + m->o_w2, z, w + m->o_b2, cnt, C, H, 0);
@@ -526,7 +918,8 @@ extern "C" int lx_model_create(uint32_t n_contexts, uint32_t hidden, uint64_t se
     for (size_t i = m->o_w2; i < m->o_b2; i++) h[i] = init_value(st, a2);
     const size_t bytes = sizeof(float) * m->n_params;
     bool ok = cudaMalloc(&m->w, bytes) == cudaSuccess && cudaMalloc(&m->m, bytes) == cudaSuccess &&
-              cudaMalloc(&m->v, bytes) == cudaSuccess && cudaMalloc(&m->g, bytes) == cudaSuccess &&
+              cudaMalloc(&m->v, bytes) == cudaSuccess &&
+              cudaMalloc(&m->g, bytes + sizeof(float)) == cudaSuccess &&
               cudaMalloc(&m->w16, sizeof(__nv_bfloat16) * m->n_params) == cudaSuccess;
     ok = ok && cudaMemcpy(m->w, h.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(m->m, 0, bytes) == cudaSuccess && cudaMemset(m->v, 0, bytes) == cudaSuccess;
@@ -553,6 +946,7 @@ extern "C" void lx_model_free(lx_model *m)
     cudaFree(m->act);
     cudaFree(m->arg);
     cudaFree(m->win);
+    cudaFreeHost(m->h_g);
     delete m;
 }
 
@@ -608,10 +1002,15 @@ extern "C" int lx_model_gradient(lx_model *m, const uint16_t *d_windows, const u
 {
     if (!m || !d_windows || !d_labels || batch == 0 || !host_grad || count != m->n_params) return LX_E_INVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    float l = 0.0f;
-    int rc = model_pass(m, d_windows, d_labels, batch, nullptr, s, &l);
-    if (rc == LX_OK) rc = cuda_err(cudaMemcpy(host_grad, m->g, sizeof(float) * count, cudaMemcpyDeviceToHost));
-    if (loss) *loss = l;
+    // the gradient and the loss behind it in one copy to pinned memory: a copy
+    // to pageable memory of this size takes longer than the kernels
+    if (!m->h_g && cudaMallocHost(&m->h_g, sizeof(float) * (count + 1)) != cudaSuccess) return LX_E_NOMEM;
+    int rc = model_pass(m, d_windows, d_labels, batch, nullptr, s, nullptr);
+    if (rc == LX_OK) rc = cuda_err(cudaMemcpyAsync(m->h_g, m->g, sizeof(float) * (count + 1), cudaMemcpyDeviceToHost, s));
+    if (rc == LX_OK) rc = cuda_err(cudaStreamSynchronize(s));
+    if (rc != LX_OK) return rc;
+    std::memcpy(host_grad, m->h_g, sizeof(float) * count);
+    if (loss) *loss = m->h_g[count];
     return rc;
 }
 

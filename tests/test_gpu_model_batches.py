@@ -1,0 +1,70 @@
+"""The context model's gradient and loss against the FP64 reference at the
+BF16-rounded weights: batches at the edges of the windows one CTA takes and of
+the batch slices of the weight gradients, layer sizes at the edges of their
+tiles, up to and past the sizes of the fused kernel, and windows of one
+repeated byte and of padding.  FP32 sums of at most a few thousand terms:
+tolerances as in test_gpu_speculative.py."""
+
+import numpy as np
+import pytest
+
+from lexinputs import corpus
+from oracle import model as OM
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lg(lexlib):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return lexlib
+
+
+@pytest.mark.parametrize("batch,hidden,contexts", [
+    (1, 64, 211), (3, 64, 211), (4, 64, 211), (5, 16, 2), (63, 64, 64), (64, 32, 65), (65, 64, 63), (130, 1, 33),
+    (257, 100, 300), (8, 256, 1024), (8, 257, 40), (8, 40, 1025)])
+def test_gradient_sizes(lg, batch, hidden, contexts):
+    import torch
+    rng = np.random.default_rng(batch * 7 + hidden)
+    m = lg.Model(contexts, hidden=hidden, seed=11)
+    w = corpus.generate("clike_block", 1 << 16, seed=501)
+    pos = np.sort(rng.integers(0, w.size, size=batch))
+    win = OM.windows(w, pos)
+    win[0] = 256                       # padding alone
+    if batch > 2:
+        win[1] = 32                    # one byte value: every position adds to the same embedding row
+    y = rng.integers(0, contexts, size=batch)
+    p = OM.to_bf16(m.get_params().astype(np.float64))
+    dw = torch.from_numpy(win.astype(np.int16)).cuda()
+    dy = torch.from_numpy(y.astype(np.uint16).view(np.int16)).cuda()
+    rl, rg = OM.loss_and_grad(p, win, y, hidden, contexts)
+    for _ in range(2):                 # and again on used buffers
+        g, loss = m.gradient(dw, dy)
+        assert abs(loss - rl) < 1e-4 * (1 + abs(rl))
+        blocks = np.cumsum([0] + OM.sizes(hidden, contexts))
+        for lo, hi in zip(blocks[:-1], blocks[1:]):
+            assert np.max(np.abs(g[lo:hi] - rg[lo:hi])) < 1e-5 + 1e-3 * np.max(np.abs(rg[lo:hi])), (lo, hi)
+    z = m.forward(dw).cpu().numpy()
+    rz, _ = OM.forward(p, win, hidden, contexts)
+    assert np.max(np.abs(z - rz)) < 1e-4 * (1 + np.max(np.abs(rz)))
+
+
+def test_step_equals_its_gradient(lg):
+    # the first AdamW step moves every weight by lr against its gradient's sign
+    import torch
+    rng = np.random.default_rng(5)
+    m = lg.Model(40, hidden=32, seed=12)
+    w = corpus.generate("clike_block", 1 << 14, seed=502)
+    win = OM.windows(w, np.sort(rng.integers(0, w.size, size=48)))
+    y = rng.integers(0, 40, size=48)
+    dw = torch.from_numpy(win.astype(np.int16)).cuda()
+    dy = torch.from_numpy(y.astype(np.int16)).cuda()
+    p0 = m.get_params()
+    g, loss = m.gradient(dw, dy)
+    assert abs(m.train_step(dw, dy, 1e-3) - loss) < 1e-5 * (1 + abs(loss))
+    big = np.abs(g) > 1e-4
+    step = (m.get_params() - p0)[big]
+    assert big.sum() > 1000 and np.all(np.sign(step) == -np.sign(g[big]))
+    assert np.max(np.abs(np.abs(step) - 1e-3)) < 1e-5
