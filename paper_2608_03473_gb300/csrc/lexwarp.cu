@@ -98,28 +98,6 @@ struct WResult {
     unsigned int pad2[3];
 };
 
-// Batches: a document's tiles are consecutive in the launch's tile sequence
-// from first_tile; `set` indexes the WSet array staged with the tables.
-struct WDoc {
-    const uint8_t *in;
-    uint64_t n;
-    uint32_t first_tile;
-    uint32_t set;
-};
-
-// One token set's rows and maps in a batch's combined table (offsets from
-// the table's start; the rows of all sets lie in one 16-bit address window).
-struct WSet {
-    uint32_t p_start, p_pre, p_slow, kmap_off, cmap_off, cut_off, ctx_off, pad;
-};
-
-struct WDocRes {
-    unsigned long long total;          // kept tokens of the document's tiles (any after a failure included)
-    unsigned long long inv_fail_pos;   // ~min failure offset within the document, 0 = none
-    unsigned long long inv_fail_tok;   // ~output index at that failure
-    unsigned long long out_off1;       // output index of its first token + 1 (0: not yet resolved)
-};
-
 struct WParams {
     const uint8_t *in;
     uint64_t n;
@@ -1468,6 +1446,7 @@ namespace {
 struct Combined {
     std::vector<uint8_t> blob;
     uint32_t rows_bytes = 0, acc_off = 0, sets_off = 0;
+    bool sync = true;   // every set has a synchronizing byte
 };
 
 const WalkTable *class_walk(const lx_tokenset *ts, int mode)
@@ -1518,9 +1497,21 @@ int combine(const lx_tokenset *const *sets, uint32_t n_sets, int mode, Combined 
         std::memcpy(out.blob.data() + maps[s] + 256, t.blob.data() + t.cmap_off, 256);
         std::memcpy(out.blob.data() + maps[s] + 512, t.blob.data() + t.cut_off, 256);
         ws[s] = WSet{base[s] + t.p_start, base[s] + t.p_pre, base[s], maps[s], maps[s] + 256, maps[s] + 512,
-                     maps[s] + 768, 0};
+                     maps[s] + 768, 0, {0, 0, 0, 0}};
+        out.sync = out.sync && t.n_sync > 0;
+        if (t.n_sync <= 4)   // few byte values synchronize: they are searched for
+            for (uint32_t b = 0; b < 256; b++)
+                if (t.sync[sets[s]->byte_class[b]] != t.p_pre) ws[s].pat[ws[s].n_pat++] = b * 0x01010101u;
     }
     std::memcpy(out.blob.data() + out.sets_off, ws.data(), sizeof(WSet) * n_sets);
+    // behind it the same table for rows.cu: the PRE rows synchronize
+    const size_t bytes = out.blob.size();
+    out.blob.resize(2 * bytes);
+    std::memcpy(out.blob.data() + bytes, out.blob.data(), bytes);
+    for (uint32_t s = 0; s < n_sets; s++) {
+        uint16_t *pre = reinterpret_cast<uint16_t *>(out.blob.data() + bytes + base[s] + w[s]->p_pre);
+        for (uint32_t k = 0; k < 128; k++) pre[k] = (uint16_t)(w[s]->sync[k] + base[s]);
+    }
     return LX_OK;
 }
 
@@ -1546,10 +1537,19 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
         r2 = cuda_err(cudaMemcpy(c->wb_dev, cb.blob.data(), cb.blob.size(), cudaMemcpyHostToDevice));
         if (r2 != LX_OK) return r2;
         c->wb_key = key;
-        c->wb_blob_bytes = (uint32_t)cb.blob.size();
+        c->wb_blob_bytes = (uint32_t)(cb.blob.size() / 2);
+        c->wb_sync = cb.sync;
         c->wb_rows = cb.rows_bytes;
         c->wb_acc_off = cb.acc_off;
         c->wb_sets_off = cb.sets_off;
+    }
+
+    // from entry rows (rows.cu) where every set synchronizes
+    if (c->kernel == LX_KERNEL_AUTO && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && c->wb_sync) {
+        const int rc = lex_batch_rows(c, key, docs, n_docs, mode, d_kinds, d_lens, capacity, results, n_total, st);
+        if (rc != LX_ROWS && rc != LX_FAR) return rc;
+        for (uint32_t i = 0; i < n_docs; i++) results[i] = lx_doc_result{0, 0, 0};
+        *n_total = 0;
     }
 
     // documents in their order; empty ones take no tile

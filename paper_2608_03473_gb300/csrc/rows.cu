@@ -46,18 +46,27 @@
 #include <atomic>
 #include <chrono>
 #include <cstdint>
+#include <cstring>
+#include <vector>
 
 #include "rows.cuh"
-#include "runtime.h"
 
 namespace lx {
 namespace {
 
+// One input (of a batch: a document) as guess_row sees it.
+struct GuessIn {
+    const uint8_t *in;
+    uint32_t lo, guess, n_pat, pat[4];
+};
+
 // Whether one of the few synchronizing byte values is among a block's bytes.
-__device__ __forceinline__ bool has_sync(const RParams &P, const uint4 &c)
+__device__ __forceinline__ bool has_sync(const GuessIn &P, const uint4 &c)
 {
     uint32_t z = 0;
-    for (uint32_t i = 0; i < P.n_pat; i++) {
+#pragma unroll
+    for (uint32_t i = 0; i < 4; i++) {
+        if (i >= P.n_pat) break;
         const uint32_t x = c.x ^ P.pat[i], y = c.y ^ P.pat[i], u = c.z ^ P.pat[i], v = c.w ^ P.pat[i];
         z |= ((x - 0x01010101u) & ~x) | ((y - 0x01010101u) & ~y) | ((u - 0x01010101u) & ~u) | ((v - 0x01010101u) & ~v);
     }
@@ -72,7 +81,7 @@ __device__ __forceinline__ bool has_sync(const RParams &P, const uint4 &c)
 // the input begins there.  SLOW looks for the next synchronizing byte (the
 // row need not be right).  All lanes of a warp call it together.
 template <int FORM>
-__device__ uint32_t guess_row(const RParams &P, const REnv &E, uint64_t p, bool has)
+__device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool has)
 {
     uint32_t e = E.pre, w = P.guess;
     if (P.n_pat && has) {
@@ -120,7 +129,24 @@ __device__ uint32_t guess_row(const RParams &P, const REnv &E, uint64_t p, bool 
     return e >= E.pre || e == E.slow ? ROW_UNKNOWN : (e & ~0xFFu) - E.tb;
 }
 
-template <int FORM>
+__device__ __forceinline__ GuessIn guess_in(const RParams &P)
+{
+    return GuessIn{P.in, P.lo, P.guess, P.n_pat, {P.pat[0], P.pat[1], P.pat[2], P.pat[3]}};
+}
+
+// The tables of a batch's set, and its documents' synchronizing bytes.
+__device__ __forceinline__ GuessIn use_set(const RParams &P, REnv &E, const WDoc &D)
+{
+    const uint32_t ws = E.tb + P.sets_off + D.set * (uint32_t)sizeof(WSet);
+    E.start = E.tb + lds_u32(ws);
+    E.pre = E.tb + lds_u32(ws + 4);
+    E.slow = E.tb + lds_u32(ws + 8);
+    E.kmap = E.tb + lds_u32(ws + 12);
+    E.cmap = E.tb + lds_u32(ws + 16);
+    return GuessIn{D.in, 0, P.guess, lds_u32(ws + 28), {lds_u32(ws + 32), lds_u32(ws + 36), lds_u32(ws + 40), lds_u32(ws + 44)}};
+}
+
+template <int FORM, bool BATCH>
 __global__ void __launch_bounds__(GUESS_NT) row_guess(RParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -132,13 +158,21 @@ __global__ void __launch_bounds__(GUESS_NT) row_guess(RParams P)
     REnv E;
     if (!stage_table<FORM>(P, smem, E)) return;
     __syncthreads();
+    GuessIn in = guess_in(P);
     for (uint64_t s0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ull; s0 < P.n_slices;
          s0 += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t s = s0 + (threadIdx.x & 31);
-        const bool has = s > 0 && s < P.n_slices;
-        uint32_t r = guess_row<FORM>(P, E, s * P.slice, has);
-        if (s == 0) r = P.p_start;
-        if (s < P.n_slices) P.rows[s] = (uint16_t)r;
+        uint64_t p = s * P.slice, n = P.n;   // the slice's position in its input
+        if (BATCH) {   // a warp's 32 slices are one tile
+            const uint32_t t = (uint32_t)(s0 / 32);
+            const WDoc D = P.docs[__ldg(P.tile_doc + t)];
+            in = use_set(P, E, D);
+            p = (uint64_t)(t - D.first_tile) * 32 * P.slice + (uint64_t)(threadIdx.x & 31) * P.slice;
+            n = D.n;
+        }
+        uint32_t r = guess_row<FORM>(in, E, p, p > 0 && p < n);
+        if (p == 0) r = E.start - E.tb;
+        if (p < n) P.rows[s] = (uint16_t)r;
     }
 }
 
@@ -223,6 +257,7 @@ struct Pending {
     uint32_t open;      // its first event ended a kept token that began in an earlier tile
     uint32_t fail;      // failure position in the tile, or NONE
     uint32_t lidx, llen;   // per lane: a token whose length the stage does not hold
+    uint32_t doc, dtile, kmap;   // batches: its document, its index there, its set's kind map
 };
 
 // The staged tokens of a tile to the output from index G: each lane two
@@ -277,7 +312,7 @@ __device__ __forceinline__ void copy_stage(const RParams &P, uint32_t kmap, uint
 // Resolve the pending tile's output offset, check its entry row against the
 // previous tile's exit row, and copy its tokens out.  False: stop (an error
 // is flagged).
-template <int NW>
+template <int NW, bool BATCH>
 __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, uint32_t stage, const uint16_t *spill)
 {
     const uint32_t lane = threadIdx.x & 31;
@@ -285,7 +320,8 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
     uint64_t G = 0, carry = 0;
     unsigned long long w;   // the previous tile's status word
     if (!resolve_tile(P, D.tile, G, w)) return false;
-    if (D.tile) {
+    const uint32_t dtile = BATCH ? D.dtile : D.tile;
+    if (dtile) {
         const uint32_t x = (uint32_t)(w >> 32) & 0xFFFFu;
         if (x && x != D.entry) {
             if (lane == 0) atomicOr(P.error(), ERR_ROWS);
@@ -296,7 +332,7 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
             if (lane == 0) {
                 Waiter W;
                 uint32_t t = D.tile - 1;
-                while (good && !((w >> 16) & 0xFFFFu) && t > 0) {
+                while (good && !((w >> 16) & 0xFFFFu) && t > D.tile - dtile) {
                     t--;
                     while ((w = ld_status(&P.status[t])) == 0 && (good = W.again(P))) {}
                 }
@@ -308,13 +344,19 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
         }
     }
     if (lane == 0) {
+        unsigned long long *fp = BATCH ? &P.dres[D.doc].inv_fail_pos : &P.res->inv_fail_pos;
+        unsigned long long *ft = BATCH ? &P.dres[D.doc].inv_fail_tok : &P.res->inv_fail_tok;
         if (D.fail != NONE) {
-            atomicMax(&P.res->inv_fail_pos, ~(unsigned long long)((uint64_t)D.tile * TILE + D.fail));
-            atomicMax(&P.res->inv_fail_tok, ~(unsigned long long)(G + D.staged));
+            atomicMax(fp, ~(unsigned long long)((uint64_t)dtile * TILE + D.fail));
+            atomicMax(ft, ~(unsigned long long)(G + D.staged));
+        }
+        if (BATCH) {
+            if (dtile == 0) P.dres[D.doc].out_off1 = G + 1;
+            if (D.staged) atomicAdd(&P.dres[D.doc].total, (unsigned long long)D.staged);
         }
         if (D.tile == P.n_tiles - 1) P.res->total = G + D.staged;
     }
-    copy_stage(P, E.kmap, stage, spill, D.split, D.staged, G);
+    copy_stage(P, BATCH ? D.kmap : E.kmap, stage, spill, D.split, D.staged, G);
     __syncwarp();
     if (D.lidx != NONE && G + D.lidx < P.cap)
         P.out_lens[G + D.lidx] = (uint32_t)(D.llen + (D.open && D.lidx == 0 ? carry : 0));
@@ -325,12 +367,26 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
 // less per call than reading it back), and leaves a small launch's scratch
 // zeroed (a memset less): 1 500 B of JSON 31.3 -> 24.7 us a call, 1 MiB of
 // arith tokens 41 -> 36 us.
+template <bool BATCH>
 __device__ void finish_launch(const RParams &P)
 {
     __threadfence();
     __syncthreads();   // (no static shared memory: the dynamic part takes all of it)
     if (!__syncthreads_or(threadIdx.x == 0 && atomicAdd(P.done, 1u) == gridDim.x - 1)) return;
     __threadfence();
+    if (BATCH) {   // the record and, 64 bytes from it, the documents' records
+        const uint32_t words = 8 + (uint32_t)(sizeof(WDocRes) / 8) * P.n_docs;
+        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(P.res);
+        for (uint32_t i = threadIdx.x; i < words; i += blockDim.x)
+            reinterpret_cast<volatile unsigned long long *>(P.down)[i] = __ldcg(src + i);
+        __threadfence_system();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence_system();
+            reinterpret_cast<volatile unsigned long long *>(P.down)[words] = P.seq;
+        }
+        return;
+    }
     if (threadIdx.x == 0) {
         RResult r;
         r.total = __ldcg(&P.res->total);
@@ -356,7 +412,7 @@ __device__ void finish_launch(const RParams &P)
     }
 }
 
-template <int FORM, int NW, bool FUSED>
+template <int FORM, int NW, bool FUSED, bool BATCH>
 __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -389,10 +445,19 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         tile = __shfl_sync(0xffffffffu, tile, 0);
         if (tile >= P.n_tiles) break;
         const uint8_t *in = P.in + (uint64_t)tile * TILE;
-        const uint64_t left = P.n - (uint64_t)tile * TILE;
+        uint64_t left = P.n - (uint64_t)tile * TILE;
+        uint32_t doc = 0, dtile = tile;
+        if (BATCH) {   // the tile's document and its set's tables
+            doc = __ldg(P.tile_doc + tile);
+            const WDoc D = P.docs[doc];
+            dtile = tile - D.first_tile;
+            in = D.in + (uint64_t)dtile * TILE;
+            left = D.n - (uint64_t)dtile * TILE;
+            use_set(P, E, D);
+        }
         const uint32_t nrel = left < BIG ? (uint32_t)left : BIG;   // bytes from the tile's start on
-        const uint32_t lo = tile == 0 ? P.lo : 0u;
-        if (lane == 0 && tile + ahead < P.n_tiles) {   // a tile some warp takes about one tile from now, into L2
+        const uint32_t lo = BATCH || tile ? 0u : P.lo;
+        if (!BATCH && lane == 0 && tile + ahead < P.n_tiles) {   // a tile some warp takes about one tile from now, into L2
             const uint64_t fb = (uint64_t)(tile + ahead) * TILE, fl = P.n - fb;
             const uint32_t bytes = (uint32_t)(fl < TILE ? fl : TILE) & ~15u;
             if (bytes)
@@ -408,7 +473,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         uint32_t er;
         if (FUSED) {
             const uint64_t p = (uint64_t)tile * TILE + p0;
-            er = guess_row<FORM>(P, E, p, has && p > 0);
+            er = guess_row<FORM>(guess_in(P), E, p, has && p > 0);
             if (p == 0) er = P.p_start;
         } else {
             er = has ? P.rows[((uint64_t)tile * 32 + lane) * P.row_step] : 0u;
@@ -527,7 +592,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
 
         // the previous tile's output: its predecessors have had a whole tile to publish
         if (pend.tile != NONE) {
-            if (!finish_tile<NW>(P, E, pend, stage, spill)) {
+            if (!finish_tile<NW, BATCH>(P, E, pend, stage, spill)) {
                 pend.tile = NONE;
                 break;
             }
@@ -541,6 +606,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         pend.entry = __shfl_sync(0xffffffffu, er, 0);
         pend.lidx = NONE;
         pend.llen = 0;
+        if (BATCH) {
+            pend.doc = doc;
+            pend.dtile = dtile;
+            pend.kmap = E.kmap;
+        }
         bool open = false;
         uint32_t split = total;
         uint16_t *gp = nullptr;
@@ -560,7 +630,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
             const uint32_t fp = f == NONE ? pe - p0 : f;             // its position in the slice
             const uint32_t fc = f == NONE ? tail : lds_u8(evl + f);  // its code
             if (below) prev = (int)prev1 - 1 - (int)p0;
-            else if (tile == 0) prev = (int)lo - (int)p0;
+            else if (dtile == 0) prev = (int)lo - (int)p0;
             else prev = -(int)p0, open = true;
             const uint32_t d = (uint32_t)((int)fp - prev);
             if (open || d >= LEN_MAX) {
@@ -623,8 +693,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         pend.open = __any_sync(0xffffffffu, open) ? 1u : 0u;
         __syncwarp();
     }
-    if (pend.tile != NONE) finish_tile<NW>(P, E, pend, stage, spill);
-    finish_launch(P);
+    if (pend.tile != NONE) finish_tile<NW, BATCH>(P, E, pend, stage, spill);
+    finish_launch<BATCH>(P);
 }
 
 // ---------------------------------------------------------------------------
@@ -655,67 +725,85 @@ constexpr double TILE_FIXED = 1.0, TILE_STEP = 0.265;
 using RowsKernel = void (*)(RParams);
 
 // The kernel of a table form and geometry, and its per-warp shared bytes.
-template <int FORM>
+template <int FORM, bool BATCH>
 RowsKernel rows_kernel(int nw, bool fused)
 {
+    if constexpr (!BATCH)
+        if (fused) return nw == 1 ? lex_rows<FORM, 1, true, false> : lex_rows<FORM, 2, true, false>;
     switch (nw) {
-    case 1: return fused ? lex_rows<FORM, 1, true> : lex_rows<FORM, 1, false>;
-    case 2: return fused ? lex_rows<FORM, 2, true> : lex_rows<FORM, 2, false>;
-    case 3: return lex_rows<FORM, 3, false>;
-    case 4: return lex_rows<FORM, 4, false>;
-    case 5: return lex_rows<FORM, 5, false>;
-    case 6: return lex_rows<FORM, 6, false>;
-    case 7: return lex_rows<FORM, 7, false>;
-    default: return lex_rows<FORM, 8, false>;
+    case 1: return lex_rows<FORM, 1, false, BATCH>;
+    case 2: return lex_rows<FORM, 2, false, BATCH>;
+    case 3: return lex_rows<FORM, 3, false, BATCH>;
+    case 4: return lex_rows<FORM, 4, false, BATCH>;
+    case 5: return lex_rows<FORM, 5, false, BATCH>;
+    case 6: return lex_rows<FORM, 6, false, BATCH>;
+    case 7: return lex_rows<FORM, 7, false, BATCH>;
+    default: return lex_rows<FORM, 8, false, BATCH>;
     }
 }
 constexpr uint32_t AREA[9] = {0, Geo<1>::WAREA, Geo<2>::WAREA, Geo<3>::WAREA, Geo<4>::WAREA,
                               Geo<5>::WAREA, Geo<6>::WAREA, Geo<7>::WAREA, Geo<8>::WAREA};
 
-RowsKernel rows_kernel(int form, int nw, bool fused)
+RowsKernel rows_kernel(int form, int nw, bool fused, bool batch = false)
 {
-    return form == FORM_BYTE ? rows_kernel<FORM_BYTE>(nw, fused) : rows_kernel<FORM_CLASS>(nw, fused);
+    if (batch) return rows_kernel<FORM_CLASS, true>(nw, false);
+    return form == FORM_BYTE ? rows_kernel<FORM_BYTE, false>(nw, fused) : rows_kernel<FORM_CLASS, false>(nw, fused);
+}
+
+RowsKernel guess_kernel(int form, bool batch)
+{
+    if (batch) return row_guess<FORM_CLASS, true>;
+    return form == FORM_BYTE ? row_guess<FORM_BYTE, false> : row_guess<FORM_CLASS, false>;
 }
 
 // Whether the kernels may use the shared memory they are launched with (once per context and kernel).
-int allow_smem(lx_ctx *c, int form, int nw, bool fused)
+int allow_smem(lx_ctx *c, int form, int nw, bool fused, bool batch = false)
 {
-    const uint64_t key = (2ull << 62) | ((uint64_t)form << 8) | ((uint64_t)fused << 7) | (uint64_t)nw;
+    const uint64_t key = (2ull << 62) | ((uint64_t)batch << 9) | ((uint64_t)form << 8) | ((uint64_t)fused << 7) | (uint64_t)nw;
     for (auto &kv : c->occupancy)
         if (kv.first == key) return LX_OK;
-    cudaError_t e = cudaFuncSetAttribute(rows_kernel(form, nw, fused), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_BUDGET);
+    cudaError_t e = cudaFuncSetAttribute(rows_kernel(form, nw, fused, batch),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
     if (e == cudaSuccess)
-        e = form == FORM_BYTE
-                ? cudaFuncSetAttribute(row_guess<FORM_BYTE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 66 * 1024)
-                : cudaFuncSetAttribute(row_guess<FORM_CLASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 66 * 1024);
+        e = cudaFuncSetAttribute(guess_kernel(form, batch), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 batch ? SMEM_BUDGET : 66 * 1024);
     if (e != cudaSuccess) return LX_E_CUDA;
     c->occupancy.emplace_back(key, 1);
     return LX_OK;
 }
 
-// Geometry of a launch over L.P.n bytes: the slice length (32 nw bytes), the
-// warps per CTA and the grid (one CTA per SM).
+// The slice length (32 nw bytes) for `tiles_of(nw)` tiles beside `fixed` bytes
+// of tables, among 1 .. most and multiples of `step` bytes; 0: none fits.
+template <class F>
+int choose_nw(const lx_ctx *c, uint32_t fixed, uint32_t want, int most, uint32_t step, F tiles_of)
+{
+    double best = 0;
+    int nw = 0;
+    for (int k = 1; k <= most; k++) {
+        if (fixed + AREA[k] > SMEM_BUDGET) break;
+        if (32 * k % step != 0) continue;
+        uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[k]);
+        if (want) warps = std::min(warps, want);
+        const uint64_t all = (uint64_t)warps * c->num_sms;
+        const double cost = ((double)tiles_of(k) / (double)all + 0.5) * (TILE_FIXED + TILE_STEP * k);
+        if (!nw || cost < best) {
+            best = cost;
+            nw = k;
+        }
+    }
+    return nw;
+}
+
+// Geometry of a launch over L.P.n bytes: the slice length, the warps per CTA
+// and the grid (one CTA per SM).
 int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGiven *given)
 {
     const WalkTable &w = ts->walk[mode];
     const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16, want = warps_setting(c, ts, mode);
     const uint64_t n = L.P.n;
     L.fused = !given && n <= FUSED_MAX;
-    double best = 0;
-    int nw = 0;
-    for (int k = 1; k <= (L.fused ? 2 : 8); k++) {
-        if (fixed + AREA[k] > SMEM_BUDGET) break;
-        if (given && 32 * k % given->step != 0) continue;
-        uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[k]);
-        if (want) warps = std::min(warps, want);
-        const uint64_t tiles = (n + 1024 * k - 1) / (1024 * k), all = (uint64_t)warps * c->num_sms;
-        const double cost = ((double)tiles / (double)all + 0.5) * (TILE_FIXED + TILE_STEP * k);
-        if (!nw || cost < best) {
-            best = cost;
-            nw = k;
-        }
-    }
+    const int nw = choose_nw(c, fixed, want, L.fused ? 2 : 8, given ? given->step : 1,
+                             [&](int k) { return (n + 1024 * k - 1) / (1024 * k); });
     if (!nw) return LX_E_TOOBIG;
     L.nw = nw;
     L.P.slice = 32 * nw;
@@ -736,8 +824,7 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGive
 void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
 {
     if (!L.fused && !given) {
-        if (L.form == FORM_BYTE) row_guess<FORM_BYTE><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
-        else row_guess<FORM_CLASS><<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
+        guess_kernel(L.form, false)<<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
     }
     if (L.fused || given) {
         rows_kernel(L.form, L.nw, L.fused)<<<L.grid, 32 * L.nwarps, L.smem, st>>>(L.P);
@@ -756,6 +843,24 @@ void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, rows_kernel(L.form, L.nw, L.fused), L.P);
+}
+
+// The last CTA of a launch has written its record to pinned memory: a launch
+// that takes long (or failed) is waited for by the runtime.
+template <class F>
+int wait_record(cudaStream_t st, F there)
+{
+    const auto t0 = std::chrono::steady_clock::now();
+    bool ok = there();
+    for (uint32_t i = 1; !ok; i++, ok = there())
+        if (i % 1024 == 0 && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(2)) break;
+    if (!ok) {
+        const int rc = cuda_err(cudaStreamSynchronize(st));
+        if (rc != LX_OK) return rc;
+        if (!there()) return LX_E_CUDA;
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return LX_OK;
 }
 
 }  // namespace
@@ -851,23 +956,15 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     }
     volatile HostRecord *hr = P.host;
     hr->seq = 0;
+    std::atomic_thread_fence(std::memory_order_seq_cst);
     if (L.fused) c->small_clean = false;   // until this launch has finished without an error
     if (c->timing && !given) cudaEventRecord(c->ev[0], st);
     launch(L, given, st);
     rc = cuda_err(cudaGetLastError());
     if (c->timing) cudaEventRecord(c->ev[1], st);
     if (rc != LX_OK) return rc;
-    // the record arrives with the launch's sequence number; a launch that takes
-    // long (or failed) is waited for by the runtime
-    const auto t0 = std::chrono::steady_clock::now();
-    for (uint32_t i = 1; hr->seq != P.seq; i++)
-        if (i % 1024 == 0 && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(2)) break;
-    if (hr->seq != P.seq) {
-        rc = cuda_err(cudaStreamSynchronize(st));
-        if (rc != LX_OK) return rc;
-        if (hr->seq != P.seq) return LX_E_CUDA;
-    }
-    std::atomic_thread_fence(std::memory_order_acquire);
+    rc = wait_record(st, [&] { return hr->seq == P.seq; });
+    if (rc != LX_OK) return rc;
     const RResult r = static_cast<const HostRecord *>(c->h_res)->r;
     if (L.fused && r.error == 0) c->small_clean = true;
     if (r.error == ERR_TIMEOUT) return LX_E_TIMEOUT;
@@ -881,6 +978,172 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     *n_tokens = tokens;
     *consumed = con;
     return tokens > capacity ? LX_E_CAPACITY : LX_OK;
+}
+
+// ---------------------------------------------------------------------------
+// batches: every document of every token set in one graph launch
+// ---------------------------------------------------------------------------
+namespace {
+
+// One warp per document takes its descriptor from pinned memory and writes the
+// document's index over its tiles.
+__global__ void br_tile_docs(const WDoc *docs, uint32_t n_docs, uint32_t tile, WDoc *dev, uint32_t *tile_doc)
+{
+    const uint32_t lane = threadIdx.x & 31u, nw = gridDim.x * (blockDim.x / 32u);
+    for (uint32_t d = (blockIdx.x * blockDim.x + threadIdx.x) / 32u; d < n_docs; d += nw) {
+        const WDoc D = docs[d];
+        if (lane == 0) dev[d] = D;
+        const uint32_t nt = (uint32_t)((D.n + tile - 1) / tile);
+        for (uint32_t k = lane; k < nt; k += 32) tile_doc[D.first_tile + k] = d;
+    }
+}
+
+}  // namespace
+
+int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_doc *docs, uint32_t n_docs, int mode,
+                   uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, lx_doc_result *results, uint64_t *n_total,
+                   cudaStream_t st)
+{
+    const uint32_t fixed = 512 + c->wb_blob_bytes + 16;
+    uint64_t bytes = 0;
+    uint32_t D = 0;
+    for (uint32_t i = 0; i < n_docs; i++)
+        if (docs[i].n) {
+            bytes += docs[i].n;
+            D++;
+        }
+    if (!D) return LX_OK;
+    // half a tile of every document is empty on average
+    const int nw = choose_nw(c, fixed, c->warps, 8, 1, [&](int k) { return bytes / (1024 * k) + (D + 1) / 2; });
+    if (!nw) return LX_ROWS;
+    const uint32_t tile = 1024 * nw;
+    std::vector<WDoc> hd;
+    std::vector<uint32_t> idx;
+    hd.reserve(D);
+    idx.reserve(D);
+    uint64_t TT = 0;
+    for (uint32_t i = 0; i < n_docs; i++) {
+        if (!docs[i].n) continue;
+        hd.push_back(WDoc{docs[i].data, docs[i].n, (uint32_t)TT, docs[i].set});
+        idx.push_back(i);
+        TT += (docs[i].n + tile - 1) / tile;
+        if (TT > 0xFFFFFFF0ull) return LX_E_INVAL;
+    }
+    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[nw]);
+    if (c->warps) warps = std::min(warps, c->warps);
+    const uint32_t n_tiles = (uint32_t)TT;
+    const uint32_t nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(16, (TT + c->num_sms - 1) / c->num_sms));
+    const uint32_t smem = fixed + nwarps * AREA[nw], grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, TT);
+    int rc = allow_smem(c, FORM_CLASS, nw, false, true);
+    if (rc != LX_OK) return rc;
+
+    // device scratch: [record, document records, statuses, group words: zeroed][documents][tile map][rows][spill]
+    auto al = [](size_t x, size_t a) { return (x + a - 1) / a * a; };
+    const size_t groups = (n_tiles + GS - 1) / GS;
+    const size_t o_dres = 64, down = o_dres + sizeof(WDocRes) * D, o_status = al(down, 64);
+    const size_t o_gagg = o_status + 8 * (size_t)n_tiles, o_ginc = o_gagg + 8 * groups, zero_end = al(o_ginc + 8 * groups, 16);
+    const size_t o_docs = al(zero_end, 256), o_tdoc = al(o_docs + sizeof(WDoc) * D, 256);
+    const size_t o_rows = al(o_tdoc + 4 * (size_t)n_tiles, 256), o_spill = al(o_rows + 64 * (size_t)n_tiles, 256);
+    const size_t dev_total = o_spill + 2 * (size_t)(tile + 1) * grid * nwarps;
+    const size_t h_down = al(sizeof(WDoc) * D, 64), host_total = h_down + down + 8;
+    void *od = c->b_dev, *oh = c->b_host;
+    rc = grow(&c->b_dev, &c->b_dev_bytes, dev_total);
+    if (rc == LX_OK) rc = grow_host(&c->b_host, &c->b_host_bytes, host_total);
+    if (rc != LX_OK) return rc;
+    const bool moved = od != c->b_dev || oh != c->b_host;
+    uint8_t *dv = static_cast<uint8_t *>(c->b_dev), *hs = static_cast<uint8_t *>(c->b_host);
+    std::memcpy(hs, hd.data(), sizeof(WDoc) * D);
+
+    std::vector<uint64_t> gkey = {0xB47C6ull, D, TT, (uint64_t)mode, (uint64_t)(uintptr_t)d_kinds,
+                                  (uint64_t)(uintptr_t)d_lens, capacity, (uint64_t)(uintptr_t)dv,
+                                  (uint64_t)(uintptr_t)hs, c->timeout_ns, grid, nwarps, (uint64_t)nw,
+                                  (uint64_t)(uintptr_t)c->wb_dev};
+    gkey.insert(gkey.end(), sets_key.begin(), sets_key.end());
+    if (moved || gkey != c->b_key || !c->b_exec) {
+        if (c->b_exec) cudaGraphExecDestroy(c->b_exec);
+        c->b_exec = nullptr;
+        c->b_key.clear();
+        if (!c->b_stream && cudaStreamCreateWithFlags(&c->b_stream, cudaStreamNonBlocking) != cudaSuccess)
+            return LX_E_CUDA;
+        cudaStream_t cs = c->b_stream;
+        RParams P{};
+        P.blob = static_cast<const uint8_t *>(c->wb_dev) + c->wb_blob_bytes;
+        P.blob_bytes = c->wb_blob_bytes;
+        P.rows_bytes = c->wb_rows;
+        P.row_shift = 8;
+        P.acc_off = c->wb_acc_off;
+        P.sets_off = c->wb_sets_off;
+        P.guess = 32;
+        P.slice = 32 * nw;
+        P.n_slices = 32ull * n_tiles;
+        P.row_step = 1;
+        P.out_kinds = d_kinds;
+        P.out_lens = d_lens;
+        P.cap = capacity;
+        P.res = reinterpret_cast<RResult *>(dv);
+        P.tile_counter = reinterpret_cast<unsigned int *>(dv + sizeof(RResult));
+        P.done = P.tile_counter + 1;
+        P.down = reinterpret_cast<unsigned long long *>(hs + h_down);
+        P.n_docs = D;
+        P.seq = 1;
+        P.dres = reinterpret_cast<WDocRes *>(dv + o_dres);
+        P.status = reinterpret_cast<unsigned long long *>(dv + o_status);
+        P.gagg = reinterpret_cast<unsigned long long *>(dv + o_gagg);
+        P.ginc = reinterpret_cast<unsigned long long *>(dv + o_ginc);
+        P.zero_bytes = zero_end;
+        P.docs = reinterpret_cast<const WDoc *>(dv + o_docs);
+        P.tile_doc = reinterpret_cast<const uint32_t *>(dv + o_tdoc);
+        P.rows = reinterpret_cast<uint16_t *>(dv + o_rows);
+        P.spill = reinterpret_cast<uint16_t *>(dv + o_spill);
+        P.n_tiles = n_tiles;
+        P.timeout_ns = c->timeout_ns;
+        P.withhold = NONE;
+        const uint32_t gmax = SMEM_BUDGET / (fixed + 1024) * c->num_sms;   // guess CTAs resident at once, at most four per SM
+        const uint32_t gg = std::min(std::min(gmax, 4u * (uint32_t)c->num_sms), (32u * n_tiles + GUESS_NT - 1) / GUESS_NT);
+        if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LX_E_CUDA;
+        br_tile_docs<<<(D + 7) / 8, 256, 0, cs>>>(reinterpret_cast<const WDoc *>(hs), D, tile,
+                                                 const_cast<WDoc *>(P.docs), const_cast<uint32_t *>(P.tile_doc));
+        guess_kernel(FORM_CLASS, true)<<<std::max(1u, gg), GUESS_NT, fixed, cs>>>(P);
+        rows_kernel(FORM_CLASS, nw, false, true)<<<grid, 32 * nwarps, smem, cs>>>(P);
+        cudaGraph_t graph = nullptr;
+        cudaError_t e = cudaStreamEndCapture(cs, &graph);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->b_exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess) {
+            c->b_exec = nullptr;
+            cudaGetLastError();
+            return LX_E_CUDA;
+        }
+        c->b_key = gkey;
+    }
+    volatile unsigned long long *seq = reinterpret_cast<volatile unsigned long long *>(hs + h_down + down);
+    *seq = 0;
+    std::atomic_thread_fence(std::memory_order_seq_cst);
+    if (c->timing) cudaEventRecord(c->ev[0], st);
+    rc = cuda_err(cudaGraphLaunch(c->b_exec, st));
+    if (c->timing) cudaEventRecord(c->ev[1], st);
+    if (rc == LX_OK) rc = wait_record(st, [&] { return *seq == 1; });
+    if (rc != LX_OK) return rc;
+
+    const RResult r = *reinterpret_cast<const RResult *>(hs + h_down);
+    if (r.error == ERR_TIMEOUT) return LX_E_TIMEOUT;
+    if (r.error) return LX_ROWS;
+    const WDocRes *dres = reinterpret_cast<const WDocRes *>(hs + h_down + o_dres);
+    for (uint32_t j = 0; j < D; j++) {
+        const WDocRes &x = dres[j];
+        lx_doc_result &o = results[idx[j]];
+        if (x.out_off1 == 0) return LX_E_CUDA;   // every document's first tile reports its offset
+        o.out_off = x.out_off1 - 1;
+        if (x.inv_fail_pos) {
+            o.consumed = ~x.inv_fail_pos;
+            o.n_tokens = ~x.inv_fail_tok - o.out_off;
+        } else {
+            o.consumed = hd[j].n;
+            o.n_tokens = x.total;
+        }
+    }
+    *n_total = r.total;
+    return r.total > capacity ? LX_E_CAPACITY : LX_OK;
 }
 
 }  // namespace lx

@@ -8,6 +8,7 @@
 #include "devutil.cuh"
 #include "internal.h"
 #include "lookback.cuh"
+#include "runtime.h"
 
 namespace lx {
 
@@ -56,6 +57,13 @@ struct RParams {
     uint32_t seq, clean;
     uint32_t n_pat;                // synchronizing byte values where they are few (0: more than four)
     uint32_t pat[4];               // each four times
+    // batches
+    const WDoc *docs;
+    const uint32_t *tile_doc;      // document of every tile
+    WDocRes *dres;
+    uint32_t sets_off;             // WSet array in the table
+    unsigned long long *down;      // pinned: the record and the document records (D), then the sequence number
+    uint32_t n_docs;
     static constexpr unsigned long long COUNT = 0xFFFFull;
     static constexpr bool SMALL = true;
     __device__ unsigned int *error() const { return &res->error; }

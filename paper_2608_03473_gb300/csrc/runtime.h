@@ -71,6 +71,7 @@ struct lx_ctx {
     size_t wb_dev_bytes = 0;
     std::vector<uint64_t> wb_key;
     uint32_t wb_blob_bytes = 0, wb_rows = 0, wb_acc_off = 0, wb_sets_off = 0;
+    bool wb_sync = false;   // every set has a synchronizing byte; rows.cu's table lies behind the other
     // the warp-tile kernel's geometry (lx_ctx_set_warp_geometry) and, in
     // LX_WARP_GEOMETRY_AUTO, the choice per (token set serial * 8 + mode)
     int warp_geometry = 0;
@@ -90,6 +91,29 @@ struct lx_ctx {
 };
 
 namespace lx {
+
+// Batches: a document's tiles are consecutive in the launch's tile sequence
+// from first_tile; `set` indexes the WSet array staged with the tables.
+struct WDoc {
+    const uint8_t *in;
+    uint64_t n;
+    uint32_t first_tile;
+    uint32_t set;
+};
+
+// One token set's rows and maps in a batch's combined table (offsets from
+// the table's start; the rows of all sets lie in one 16-bit address window).
+struct WSet {
+    uint32_t p_start, p_pre, p_slow, kmap_off, cmap_off, cut_off, ctx_off;
+    uint32_t n_pat, pat[4];   // synchronizing byte values where they are few (rows.cu)
+};
+
+struct WDocRes {
+    unsigned long long total;          // kept tokens of the document's tiles (any after a failure included)
+    unsigned long long inv_fail_pos;   // ~min failure offset within the document, 0 = none
+    unsigned long long inv_fail_tok;   // ~output index at that failure
+    unsigned long long out_off1;       // output index of its first token + 1 (0: not yet resolved)
+};
 
 // lx_lex_host on the warp-tile kernel (lexwarp.cu): the K pieces [b[i],
 // b[i+1]) of the host input (cut at certified bytes) each copied to a
@@ -139,7 +163,12 @@ struct RowsGiven {
 int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
                     uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
                     const RowsGiven *given = nullptr);
-// The same with the entry rows found by enumerating contexts (ctxmap.cu): any
+// lx_lex_batch in one launch from entry rows (rows.cu), with the context's
+// combined table (its key: part of the graph's); LX_ROWS, LX_FAR as above.
+int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_doc *docs, uint32_t n_docs, int mode,
+                   uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, lx_doc_result *results, uint64_t *n_total,
+                   cudaStream_t st);
+// lex_rows_device with the entry rows found by enumerating contexts (ctxmap.cu): any
 // token set with a walk and a scan table.  With `spec`, the speculative path's
 // predictions and rounds as well (model: nullptr for BOUNDARY everywhere).
 bool contexts_path_ok(const lx_tokenset *ts, int mode);
