@@ -429,6 +429,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
     uint16_t *const spill = P.spill + ((size_t)blockIdx.x * (blockDim.x >> 5) + wid) * (TILE + 1);
     const uint32_t ahead = gridDim.x * (blockDim.x / 32);
     const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t mbar = stage + 2 * STAGE;
+    uint32_t phase = 0;
+    if (lane == 0) mbar_init(mbar);
+    fence_proxy_async();
+    __syncwarp();
     if (P.before && *P.before != 0) {   // no rows to start from
         if (threadIdx.x == 0) atomicOr(P.error(), ERR_ROWS);
         go = false;
@@ -465,10 +470,12 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         }
         const uint32_t p0 = lane * SLICE;
         const bool has = p0 < nrel, whole = nrel >= TILE && lo == 0;
-        uint4 A, B;
-        if (whole) {   // in flight while the entry row is read or found
-            A = ldg16(in + p0);
-            B = ldg16(in + p0 + 16);
+        if (whole) {   // every lane's slice into its place, while the entry row is read or found
+            fence_proxy_async();   // (after the last tile's events were read there)
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(TILE) : "memory");
+            __syncwarp();
+            bulk_load(evl, in + p0, SLICE, mbar);
         }
         uint32_t er;
         if (FUSED) {
@@ -482,25 +489,32 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         const uint32_t e_in = er + E.tb, ps = max(p0, lo), pe = min(p0 + SLICE, nrel);
         uint32_t e = e_in;
 
-        // walk the slice
+        // walk the slice, its codes over its bytes.  (With 16-byte loads from
+        // global memory instead, 32 lines a load, the input alone took a quarter
+        // of the shared-memory and L1 pipe that bounds this kernel.)
         if (whole) {
+            const bool there = mbar_wait(mbar, phase, P.timeout_ns);
+            phase ^= 1u;
+            if (!__all_sync(0xffffffffu, there)) {
+                if (lane == 0) atomicOr(P.error(), ERR_TIMEOUT);
+                mbar_wait(mbar, phase ^ 1u, P.timeout_ns);   // the copies must not land in a finished CTA
+                break;
+            }
             if (act) {
-#pragma unroll 1
-                for (uint32_t b = 0; b < SLICE; b += 32) {
-                    const uint32_t a0 = wword<FORM>(e, A.x, E.cmap), a1 = wword<FORM>(e, A.y, E.cmap);
-                    const uint32_t a2 = wword<FORM>(e, A.z, E.cmap), a3 = wword<FORM>(e, A.w, E.cmap);
+                uint4 A = lds16(evl);
+#pragma unroll 2
+                for (uint32_t b = 0; b < SLICE; b += 16) {
+                    const uint4 c = A;
+                    if (b + 16 < SLICE) A = lds16(evl + b + 16);
+                    const uint32_t a0 = wword<FORM>(e, c.x, E.cmap), a1 = wword<FORM>(e, c.y, E.cmap);
+                    const uint32_t a2 = wword<FORM>(e, c.z, E.cmap), a3 = wword<FORM>(e, c.w, E.cmap);
                     sts16(evl + b, a0, a1, a2, a3);
-                    if (b + 32 < SLICE) A = ldg16(in + p0 + b + 32);
-                    const uint32_t b0 = wword<FORM>(e, B.x, E.cmap), b1 = wword<FORM>(e, B.y, E.cmap);
-                    const uint32_t b2 = wword<FORM>(e, B.z, E.cmap), b3 = wword<FORM>(e, B.w, E.cmap);
-                    sts16(evl + b + 16, b0, b1, b2, b3);
-                    if (b + 32 < SLICE) B = ldg16(in + p0 + b + 48);
                 }
             }
         } else if (act) {   // the input's first or last tile: partial blocks byte by byte
             for (uint32_t b = p0; b < pe; b += 16) {
                 if (b >= lo && b + 16 <= nrel) {
-                    A = ldg16(in + b);
+                    const uint4 A = ldg16(in + b);
                     const uint32_t a0 = wword<FORM>(e, A.x, E.cmap), a1 = wword<FORM>(e, A.y, E.cmap);
                     const uint32_t a2 = wword<FORM>(e, A.z, E.cmap), a3 = wword<FORM>(e, A.w, E.cmap);
                     sts16(evl + b - p0, a0, a1, a2, a3);

@@ -87,16 +87,17 @@ constexpr unsigned ERR_SMEM = 2u;
 constexpr unsigned ERR_ROWS = 4u;           // entry rows do not fit together: lex the input another way
 constexpr unsigned ERR_FAR = 8u;            // no synchronizing byte near a slice
 
-// A warp's shared memory: the event buffer, SLICE + 16 bytes per lane (the
-// 16-byte stores and loads of eight lanes then fall in different banks), and
-// the stage of STAGE tokens, 2 bytes each (event code << 8 | length).
+// A warp's shared memory: the slices' bytes and then, in their place, their
+// event codes, SLICE + 16 bytes per lane (the 16-byte stores and loads of eight
+// lanes then fall in different banks); the stage of STAGE tokens, 2 bytes each
+// (event code << 8 | length); the mbarrier of the copies.
 template <int NW>   // event mask words per lane
 struct Geo {
     static constexpr uint32_t SLICE = 32 * NW;
     static constexpr uint32_t TILE = 32 * SLICE;
     static constexpr uint32_t STRIDE = SLICE + 16;
     static constexpr uint32_t STAGE = NW < 3 ? TILE : 512 + 256 * NW;
-    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE;
+    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE + 16;
     static_assert(WAREA % 16 == 0, "geometry");
 };
 
@@ -122,6 +123,37 @@ __device__ __forceinline__ uint4 lds16(uint32_t a)
 __device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
 {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t mbar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+}
+__device__ __forceinline__ void fence_proxy_async()
+{
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+// `bytes` (a multiple of 16, both addresses 16-byte aligned) global -> shared.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const uint8_t *src, uint32_t bytes, uint32_t mbar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(mbar) : "memory");
+}
+// Bounded wait for a phase of the mbarrier; false when the time budget runs out.
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint64_t timeout_ns)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 0;; it++) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
+        if (done) return true;
+        if (it % 16 == 0) {
+            const uint64_t t = globaltimer();
+            if (!t0) t0 = t;
+            else if (t - t0 > timeout_ns) return false;
+        }
+    }
 }
 
 template <int FORM>
