@@ -165,7 +165,11 @@ __global__ void __launch_bounds__(CM_NT) cm_starts(CParams P)
 constexpr uint32_t CH = 6;
 #define LXM_ROW(E) "lop3.b32 a, " E ", t, %7, 0xD8;\n\tld.shared.u16 " E ", [a];\n\t"
 #define LXM_ROWS LXM_ROW("%0") LXM_ROW("%1") LXM_ROW("%2") LXM_ROW("%3") LXM_ROW("%4") LXM_ROW("%5")
-#define LXM_C(SEL) "prmt.b32 t, %6, %8, " SEL ";\n\tld.shared.u8 t, [t];\n\t" LXM_ROWS
+#define LXM_SROW(E)                                                            \
+    "shr.b32 a, " E ", 6;\n\tlop3.b32 a, a, 0x7C, t, 0x6A;\n\t"                \
+    "lop3.b32 a, " E ", a, %7, 0xD8;\n\tld.shared.u16 " E ", [a];\n\t"
+#define LXM_SROWS LXM_SROW("%0") LXM_SROW("%1") LXM_SROW("%2") LXM_SROW("%3") LXM_SROW("%4") LXM_SROW("%5")
+#define LXM_C(SEL) "prmt.b32 t, %6, %8, " SEL ";\n\tld.shared.u8 t, [t];\n\t" LXM_SROWS
 #define LXM_OPS(MASK)                                                          \
     : "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4]), "+r"(e[5])   \
     : "r"(w), "r"(MASK), "r"(cm) : "memory"
@@ -199,7 +203,7 @@ __device__ __noinline__ uint32_t hard_run(const CParams &P, const REnv &E, uint6
             atomicOr(P.R.error(), ERR_ROWS);
             return E.slow;
         }
-        const uint32_t v = wstep<FORM>(E, q, __ldg(P.R.in + p));
+        const uint32_t v = wstep<FORM, true>(E, q, __ldg(P.R.in + p));
         if (v != E.slow && v != E.pre) {
             if (v & 0xFEu) r = NOPOS64;
             q = v;
@@ -248,7 +252,7 @@ __device__ uint32_t block_fix(const REnv &E, const uint8_t *in, uint64_t p, bool
 {
     uint32_t q = row, r = acc_code(E, row) ? 0u : NONE;
     for (uint32_t j = 0; j < 16;) {
-        const uint32_t v = wstep<FORM>(E, q, __ldg(in + p + j));
+        const uint32_t v = wstep<FORM, true>(E, q, __ldg(in + p + j));
         if (v == E.slow) return v;
         if (v == E.pre) {
             if (r == NONE) return v;
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     REnv E;
-    if (!stage_table<FORM>(P.R, smem, E)) return;
+    if (!stage_table<FORM, true>(P.R, smem, E)) return;
     __syncthreads();
     hard_rows(P, smem, E);
     __syncthreads();
@@ -332,16 +336,18 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
                     e[i] = E.start;
                 } else if (k < nc) {
                     const uint32_t row = E.tb + ((1u + __ldg(P.cand + c0 + k - 1)) << E.shift);
-                    const uint32_t v = wstep<FORM>(E, row, b0);
+                    const uint32_t v = wstep<FORM, true>(E, row, b0);
                     if (v != E.slow && v != E.pre && !(v & 0xFEu)) e[i] = row;
                 }
             }
             auto scalar = [&](uint64_t to) {
                 for (; p < to; p++) {
                     const uint32_t b = __ldg(in + p);
-                    const uint32_t x = FORM == FORM_BYTE ? b << 1 : lds_u8(E.cmap + b), m = FORM == FORM_BYTE ? ~0x1FEu : ~0xFFu;
+                    const uint32_t x = FORM == FORM_BYTE ? b << 1 : lds_u8(E.cmap + b);
 #pragma unroll
-                    for (uint32_t i = 0; i < CH; i++) e[i] = lds_u16((e[i] & m) | x);
+                    for (uint32_t i = 0; i < CH; i++)
+                        e[i] = lds_u16(FORM == FORM_BYTE ? (e[i] & ~0x1FEu) | x
+                                                         : (e[i] & ~0xFFu) | (x ^ ((e[i] >> 6) & 0x7Cu)));
                 }
             };
             auto words = [&](uint64_t to) {   // p a multiple of 4
@@ -396,7 +402,7 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
                     if (k >= KMAX) break;
                     uint32_t x = DEAD;
                     if (e[i] != E.slow && e[i] < E.start) {
-                        const uint32_t v = wstep<FORM>(E, e[i], nb);
+                        const uint32_t v = wstep<FORM, true>(E, e[i], nb);
                         if (v == E.slow ? acc_code(E, e[i]) != 0 : (v & 0xFEu) != 0) {
                             x = 0;   // the token ends there
                         } else if (v != E.slow && v != E.pre) {

@@ -34,11 +34,12 @@
 // on past their lane's bytes to the next one: no lane walks another's bytes
 // (that tail was 16-26 % of the time), no halo, 16-byte event stores, and
 // token-driven instead of byte-driven emission (instructions per input byte
-// 1.02 -> 0.68).  A call: 512 MiB of JSON 1 003 -> 642 us, 192 MiB of C-like
-// text 630 -> 397 us, 1 MiB of arith tokens 84 -> 41 us, 40 MiB not 16-byte
-// aligned (formerly the tile kernel) 333 -> 114 us.  What bounds it: the
-// dependent table lookups of the walk (40 % of a warp's cycles) and the
-// emission (27 %), at 17-20 warps per SM, which shared memory limits.
+// 1.02 -> 0.7).  A call: 512 MiB of JSON 1 003 -> 545 us, 192 MiB of C-like
+// text 630 -> 334 us, 1 MiB of arith tokens 84 -> 30 us, 40 MiB not 16-byte
+// aligned (formerly the tile kernel) 333 -> 79 us.  What bounds it: the
+// load/store pipe, 66-80 % busy (1 460 wavefronts per 6 KiB tile of JSON: 614
+// for the table lookups, 420 for the emission's code lookups and stage
+// stores), with half the issue slots taken.
 
 #include <cuda_runtime.h>
 
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr uint32_t SLICE = Geo<NW>::SLICE, TILE = Geo<NW>::TILE, STRIDE = Geo<NW>::STRIDE;
-    constexpr uint32_t STAGE = Geo<NW>::STAGE, WAREA = Geo<NW>::WAREA;
+    const uint32_t STAGE = P.stage, WAREA = warp_area(NW, P.stage);
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     REnv E;
     bool go = stage_table<FORM>(P, smem, E);
@@ -669,20 +670,17 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
             for (uint32_t w = 0; w < NW; w++) {
                 uint32_t x = m[w];
                 for (int n = (int)nmax[w]; n > 0; n -= 4) {
-                    uint32_t b[4], code[4];
+                    uint32_t b[4], v[4], code[4];
 #pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        b[i] = top_bit(x & (0u - x));   // NONE once the events have run out
+                    for (int i = 0; i < 4; i++) {   // x's lowest one; 32 once the events have run out
+                        v[i] = x;
+                        b[i] = __popc((x - 1) & ~x);
                         x &= x - 1;
                     }
 #pragma unroll
-                    for (int i = 0; i < 4; i++) code[i] = b[i] != NONE ? lds_u8(evl + 32 * w + b[i]) : 0u;
+                    for (int i = 0; i < 4; i++) code[i] = event_code(evl + 32 * w + b[i], v[i]);
 #pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        const int pos = (int)(32 * w + b[i]);
-                        put_token(sa, code[i], (uint32_t)(pos - prev));
-                        prev = code[i] ? pos : prev;
-                    }
+                    for (int i = 0; i < 4; i++) put_event(sa, prev, v[i], code[i], b[i] + 32 * w);
                 }
             }
             if (tail >= 4) sts_u16(sa, (tail << 8) + (uint32_t)((int)(pe - p0) - prev));
@@ -731,10 +729,12 @@ constexpr uint64_t FUSED_MAX = 4ull << 20;
 constexpr uint64_t SMALL_ZERO = 48 * 1024;
 static_assert(64 + 8 * (FUSED_MAX / 1024 + 1) + 16 * (FUSED_MAX / 1024 / GS + 2) + 64 <= SMALL_ZERO, "small scratch");
 // A warp's time for a tile of 32 slices of 32 k bytes, in units of its fixed
-// part (measured, JSON: 25.7, 29.9, 34.4, 35.8 and 39.1 thousand cycles for
-// k = 4 to 8); a launch takes its rounds of tiles and half a round more, the
-// last one's share.
-constexpr double TILE_FIXED = 1.0, TILE_STEP = 0.265;
+// part, and the warps per SM past which more of them do not help (measured at
+// 20 warps, 512 MiB of JSON: 669, 616, 581, 584 and 637 us for k = 4 to 8; 192
+// MiB of C-like text: 380, 363, 342, 356, 360, and the same at 18); a launch
+// takes its rounds of tiles and half a round more, the last one's share.
+constexpr double TILE_FIXED = 1.0, TILE_STEP = 0.385;
+constexpr uint32_t USEFUL_WARPS = 18;
 
 using RowsKernel = void (*)(RParams);
 
@@ -755,9 +755,6 @@ RowsKernel rows_kernel(int nw, bool fused)
     default: return lex_rows<FORM, 8, false, BATCH>;
     }
 }
-constexpr uint32_t AREA[9] = {0, Geo<1>::WAREA, Geo<2>::WAREA, Geo<3>::WAREA, Geo<4>::WAREA,
-                              Geo<5>::WAREA, Geo<6>::WAREA, Geo<7>::WAREA, Geo<8>::WAREA};
-
 RowsKernel rows_kernel(int form, int nw, bool fused, bool batch = false)
 {
     if (batch) return rows_kernel<FORM_CLASS, true>(nw, false);
@@ -789,14 +786,15 @@ int allow_smem(lx_ctx *c, int form, int nw, bool fused, bool batch = false)
 // The slice length (32 nw bytes) for `tiles_of(nw)` tiles beside `fixed` bytes
 // of tables, among 1 .. most and multiples of `step` bytes; 0: none fits.
 template <class F>
-int choose_nw(const lx_ctx *c, uint32_t fixed, uint32_t want, int most, uint32_t step, F tiles_of)
+int choose_nw(const lx_ctx *c, int mode, uint32_t fixed, uint32_t want, int most, uint32_t step, F tiles_of)
 {
     double best = 0;
     int nw = 0;
     for (int k = 1; k <= most; k++) {
-        if (fixed + AREA[k] > SMEM_BUDGET) break;
+        const uint32_t area = warp_area(k, stage_for(k, mode));
+        if (fixed + area > SMEM_BUDGET) break;
         if (32 * k % step != 0) continue;
-        uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[k]);
+        uint32_t warps = std::min<uint32_t>(USEFUL_WARPS, (SMEM_BUDGET - fixed) / area);
         if (want) warps = std::min(warps, want);
         const uint64_t all = (uint64_t)warps * c->num_sms;
         const double cost = ((double)tiles_of(k) / (double)all + 0.5) * (TILE_FIXED + TILE_STEP * k);
@@ -816,8 +814,12 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGive
     const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16, want = warps_setting(c, ts, mode);
     const uint64_t n = L.P.n;
     L.fused = !given && n <= FUSED_MAX;
-    const int nw = choose_nw(c, fixed, want, L.fused ? 2 : 8, given ? given->step : 1,
-                             [&](int k) { return (n + 1024 * k - 1) / (1024 * k); });
+    // a small launch takes one tile of 1 KiB per SM, or tiles of 2 KiB (1 MiB of
+    // arith tokens 33 us in the former, 30 in the latter)
+    const int nw = L.fused ? (n <= 1024ull * c->num_sms ? 1 : 2)
+                           : choose_nw(c, mode, fixed, want, 8, given ? given->step : 1,
+                                       [&](int k) { return (n + 1024 * k - 1) / (1024 * k); });
+    if (L.fused && fixed + warp_area(nw, stage_for(nw, mode)) > SMEM_BUDGET) return LX_E_TOOBIG;
     if (!nw) return LX_E_TOOBIG;
     L.nw = nw;
     L.P.slice = 32 * nw;
@@ -825,11 +827,13 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGive
     const uint64_t tiles = (n + 1024 * nw - 1) / (1024 * nw);
     if (tiles > 0xFFFFFFF0ull) return LX_E_INVAL;
     L.P.n_tiles = (uint32_t)tiles;
-    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[nw]);
+    L.P.stage = stage_for(nw, mode);
+    const uint32_t area = warp_area(nw, L.P.stage);
+    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
     if (want) warps = std::min(warps, want);
     // few tiles: one CTA on every SM, no more warps than its share (sixteen stage the table)
     L.nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(16, (tiles + c->num_sms - 1) / c->num_sms));
-    L.smem = fixed + L.nwarps * AREA[nw];
+    L.smem = fixed + L.nwarps * area;
     L.grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, tiles);
     L.gsmem = fixed;
     return allow_smem(c, w.form, nw, L.fused);
@@ -1028,7 +1032,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         }
     if (!D) return LX_OK;
     // half a tile of every document is empty on average
-    const int nw = choose_nw(c, fixed, c->warps, 8, 1, [&](int k) { return bytes / (1024 * k) + (D + 1) / 2; });
+    const int nw = choose_nw(c, mode, fixed, c->warps, 8, 1, [&](int k) { return bytes / (1024 * k) + (D + 1) / 2; });
     if (!nw) return LX_ROWS;
     const uint32_t tile = 1024 * nw;
     std::vector<WDoc> hd;
@@ -1043,11 +1047,12 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         TT += (docs[i].n + tile - 1) / tile;
         if (TT > 0xFFFFFFF0ull) return LX_E_INVAL;
     }
-    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / AREA[nw]);
+    const uint32_t area = warp_area(nw, stage_for(nw, mode));
+    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
     if (c->warps) warps = std::min(warps, c->warps);
     const uint32_t n_tiles = (uint32_t)TT;
     const uint32_t nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(16, (TT + c->num_sms - 1) / c->num_sms));
-    const uint32_t smem = fixed + nwarps * AREA[nw], grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, TT);
+    const uint32_t smem = fixed + nwarps * area, grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, TT);
     int rc = allow_smem(c, FORM_CLASS, nw, false, true);
     if (rc != LX_OK) return rc;
 
@@ -1089,6 +1094,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         P.sets_off = c->wb_sets_off;
         P.guess = 32;
         P.slice = 32 * nw;
+        P.stage = stage_for(nw, mode);
         P.n_slices = 32ull * n_tiles;
         P.row_step = 1;
         P.out_kinds = d_kinds;

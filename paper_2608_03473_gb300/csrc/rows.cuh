@@ -30,6 +30,7 @@ struct RParams {
     uint64_t n;
     uint32_t lo;                   // 0..15
     uint32_t slice;                // bytes per slice
+    uint32_t stage;                // tokens a warp's stage holds
     const uint8_t *blob;           // walk table, then WalkTable::sync
     uint32_t blob_bytes, rows_bytes, row_shift, sync_bytes;   // multiples of 16 but the shift
     uint32_t p_start, p_pre, acc_off, kmap_off, cmap_off;
@@ -89,17 +90,26 @@ constexpr unsigned ERR_FAR = 8u;            // no synchronizing byte near a slic
 
 // A warp's shared memory: the slices' bytes and then, in their place, their
 // event codes, SLICE + 16 bytes per lane (the 16-byte stores and loads of eight
-// lanes then fall in different banks); the stage of STAGE tokens, 2 bytes each
+// lanes then fall in different banks); the stage of P.stage tokens, 2 bytes each
 // (event code << 8 | length); the mbarrier of the copies.
 template <int NW>   // event mask words per lane
 struct Geo {
     static constexpr uint32_t SLICE = 32 * NW;
     static constexpr uint32_t TILE = 32 * SLICE;
     static constexpr uint32_t STRIDE = SLICE + 16;
-    static constexpr uint32_t STAGE = NW < 3 ? TILE : 512 + 256 * NW;
-    static constexpr uint32_t WAREA = 32 * STRIDE + 2 * STAGE + 16;
-    static_assert(WAREA % 16 == 0, "geometry");
 };
+// Shared bytes of a warp with a stage of `stage` tokens (a multiple of 8).
+__host__ __device__ constexpr uint32_t warp_area(uint32_t nw, uint32_t stage)
+{
+    return 32 * (32 * nw + 16) + 2 * stage + 16;
+}
+// Tokens of the stage: what a tile of 1024 nw bytes seldom exceeds, so that
+// enough warps fit (a stage for every mode's tokens left 16 beside the C-like
+// set's table at nw = 6, one for the filtered modes' tokens leaves 18).
+constexpr uint32_t stage_for(int nw, int mode)
+{
+    return nw < 3 ? 1024 * nw : mode == LX_FULL_EXACT ? 352 * nw : 240 * nw;
+}
 
 // Shared addresses of the tables.
 struct REnv {
@@ -156,10 +166,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint64
     }
 }
 
-template <int FORM>
+// SPREAD: the class form's rows as stage_table<FORM, true> lays them out.
+template <int FORM, bool SPREAD = false>
 __device__ __forceinline__ uint32_t wstep(const REnv &E, uint32_t e, uint32_t b)
 {
-    const uint32_t a = FORM == FORM_BYTE ? ((e & ~0x1FEu) | (b << 1)) : ((e & ~0xFFu) | lds_u8(E.cmap + b));
+    const uint32_t a = FORM == FORM_BYTE ? ((e & ~0x1FEu) | (b << 1))
+                                         : ((e & ~0xFFu) | (lds_u8(E.cmap + b) ^ (SPREAD ? (e >> 6) & 0x7Cu : 0u)));
     return lds_u16(a);
 }
 __device__ __forceinline__ uint32_t acc_code(const REnv &E, uint32_t e)
@@ -200,22 +212,30 @@ __device__ __forceinline__ uint32_t wword(uint32_t &e, uint32_t w, uint32_t cm)
     return pk;
 }
 
-__device__ __forceinline__ uint32_t top_bit(uint32_t x)   // index of the highest one, NONE for 0
+// The code at shared address a where v != 0 (else undefined): lanes without an
+// event stay off the banks.
+__device__ __forceinline__ uint32_t event_code(uint32_t a, uint32_t v)
 {
-    uint32_t b;
-    asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(x));
-    return b;
+    uint32_t c;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u8 %0, [%1];\n\t}"
+                 : "=r"(c) : "r"(a), "r"(v));
+    return c;
 }
 
-// A kept token (code >= 4) of length d into the stage at sa, which advances.
-__device__ __forceinline__ void put_token(uint32_t &sa, uint32_t code, uint32_t d)
+// An event at position pos: where there is one (v != 0), a kept token (code >=
+// 4) from prev to pos goes into the stage at sa, which advances, and prev
+// moves on.
+__device__ __forceinline__ void put_event(uint32_t &sa, int &prev, uint32_t v, uint32_t code, uint32_t pos)
 {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 v;\n\t"
-                 "setp.gt.u32 p, %1, 3;\n\t"
-                 "mad.lo.u32 v, %1, 256, %2;\n\t"
-                 "@p st.shared.u16 [%0], v;\n\t"
-                 "@p add.u32 %0, %0, 2;\n\t}"
-                 : "+r"(sa) : "r"(code), "r"(d) : "memory");
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 d;\n\t"
+                 "setp.ne.u32 p, %2, 0;\n\t"
+                 "setp.gt.and.u32 q, %3, 3, p;\n\t"
+                 "sub.u32 d, %4, %1;\n\t"
+                 "mad.lo.u32 d, %3, 256, d;\n\t"
+                 "@q st.shared.u16 [%0], d;\n\t"
+                 "@q add.u32 %0, %0, 2;\n\t"
+                 "@p mov.u32 %1, %4;\n\t}"
+                 : "+r"(sa), "+r"(prev) : "r"(v), "r"(code), "r"(pos) : "memory");
 }
 
 __device__ __forceinline__ uint32_t kept_mask(uint32_t w)   // bit 7 of every byte >= 4 (a kept code)
@@ -229,8 +249,14 @@ __device__ __forceinline__ uint32_t event_mask(uint32_t w)  // bit 7 of every no
 
 // Stage the walk table (row offsets become shared addresses) with the PRE
 // row replaced by the synchronizing one; false where the 16-bit row
-// addresses would not reach every row.
-template <int FORM>
+// addresses would not reach every row.  Class-form rows start on 256-byte
+// boundaries, so a class has the same bank in every row and lanes that read
+// one class in different rows queue; SPREAD: the words of each row are XORed
+// with its number.  That takes a sixth off the wavefronts of the C-like set's
+// walk and two instructions more on each byte's chain: 6 % faster where six
+// chains hide them (cm_maps), nothing on C-like text and 12 % slower on a
+// batch in lex_rows, which therefore does without.
+template <int FORM, bool SPREAD = false>
 __device__ bool stage_table(const RParams &P, uint8_t *smem, REnv &E)
 {
     const uint32_t sbase = smem_u32(smem), tb = (sbase + 511u) & ~511u;
@@ -244,7 +270,15 @@ __device__ bool stage_table(const RParams &P, uint8_t *smem, REnv &E)
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
         uint4 v = __ldg(src + (i - pre < P.sync_bytes / 16 ? n + (i - pre) : i));
         if (i < r) v = make_uint4(__vadd2(v.x, tb2), __vadd2(v.y, tb2), __vadd2(v.z, tb2), __vadd2(v.w, tb2));
-        dst[i] = v;
+        if (SPREAD && FORM == FORM_CLASS && i < r) {   // word j of row q at j ^ (q mod 32), q as in the row's address
+            const uint32_t at = tb + 16 * i, x = (at >> 6) & 0x7Cu;
+            sts_u32(at ^ x, v.x);
+            sts_u32((at + 4) ^ x, v.y);
+            sts_u32((at + 8) ^ x, v.z);
+            sts_u32((at + 12) ^ x, v.w);
+        } else {
+            dst[i] = v;
+        }
     }
     E.tb = E.slow = tb;
     E.start = tb + P.p_start;
