@@ -1136,6 +1136,7 @@ extern "C" int lx_ctx_enable_timing(lx_ctx *c, int on)
 extern "C" int lx_ctx_last_kernel_ms(lx_ctx *c, float *ms)
 {
     if (!c || !ms || !c->ev[0]) return LX_E_INVAL;
+    cudaEventSynchronize(c->ev[1]);   // a call returns once its record is there, a moment before its event
     return cuda_err(cudaEventElapsedTime(ms, c->ev[0], c->ev[1]));
 }
 
@@ -1468,14 +1469,15 @@ extern "C" int lx_lex(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
                       static_cast<cudaStream_t>(stream));
 }
 
-// lx_lex_host splits inputs of at least 2 * HOST_PIECE bytes into up to
-// HOST_PIECES pieces at certified bytes (the planner of Section 6 on the
-// host: each equal-division target slides forward to the next byte of the
-// mode's cut set, within HOST_SLIDE bytes), so that the copy of one piece in,
-// the lexing of another and the copy of a third's tokens out overlap.  Each
-// piece is lexed by its own launch, in order on the caller's stream, its
-// output placed after the previous pieces' tokens (device-side totals).
+// lx_lex_host splits inputs of at least 2 * HOST_PIECE bytes (2 * ROWS_PIECE
+// on the row kernels) into up to HOST_PIECES pieces at certified bytes (the
+// planner of Section 6 on the host: each equal-division target slides forward
+// to the next byte of the mode's cut set, within HOST_SLIDE bytes), so that the
+// copy of one piece in, the lexing of another and the copy of a third's tokens
+// out overlap.  Each piece is lexed by its own launch, in order on the caller's
+// stream, its output placed after the previous pieces' tokens.
 constexpr uint64_t HOST_PIECE = 32ull << 20;
+constexpr uint64_t ROWS_PIECE = 12ull << 20;
 constexpr uint32_t HOST_PIECES = 8;
 constexpr uint64_t HOST_SLIDE = 4ull << 20;
 
@@ -1489,11 +1491,11 @@ __global__ void copy_record(const Result *src, Result *dst)
             reinterpret_cast<const volatile unsigned long long *>(src)[threadIdx.x];
 }
 
-static std::vector<uint64_t> host_pieces(const HostTable &h, const uint8_t *in, uint64_t n)
+static std::vector<uint64_t> host_pieces(const HostTable &h, const uint8_t *in, uint64_t n, uint64_t piece)
 {
     std::vector<uint64_t> b{0};
     const uint8_t *cert = h.blob.data() + h.cert_off;
-    uint32_t k = (uint32_t)std::min<uint64_t>(HOST_PIECES, n / HOST_PIECE);
+    uint32_t k = (uint32_t)std::min<uint64_t>(HOST_PIECES, n / piece);
     bool any = false;
     for (uint32_t x = 0; x < 256; x++) any |= cert[x] != 0;
     if (!any || k < 2) k = 1;
@@ -1560,7 +1562,9 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
     if (can_enumerate && !(warp ? warp_has_cuts(ts, mode) : mode_has_cuts(ts, mode)))
         return whole(true);   // no certified byte: the enumerative path
 
-    const std::vector<uint64_t> b = host_pieces(h, h_in, n);
+    // from entry rows (rows.cu) where the set has a synchronizing byte
+    const bool rows = can_enumerate && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode);
+    const std::vector<uint64_t> b = host_pieces(h, h_in, n, rows ? ROWS_PIECE : HOST_PIECE);
     const uint32_t K = (uint32_t)b.size() - 1;
     if (!c->s_in && (cudaStreamCreateWithFlags(&c->s_in, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaStreamCreateWithFlags(&c->s_out, cudaStreamNonBlocking) != cudaSuccess))
@@ -1572,6 +1576,11 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
             return LX_E_CUDA;
         c->ev_in.push_back(e1);
         c->ev_lex.push_back(e2);
+    }
+    if (rows) {
+        rc = lex_rows_host(c, ts, h_in, n, mode, h_kinds, h_lens, capacity, b.data(), K, n_tokens, consumed, st);
+        if (rc != LX_ROWS && rc != LX_FAR) return rc;
+        return whole(false);
     }
     if (warp) {
         rc = lex_warp_host(c, ts, h_in, n, mode, h_kinds, h_lens, capacity, b.data(), K, n_tokens, consumed, st,

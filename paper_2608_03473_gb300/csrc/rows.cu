@@ -864,16 +864,16 @@ void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
 }
 
 // The last CTA of a launch has written its record to pinned memory: a launch
-// that takes long (or failed) is waited for by the runtime.
+// that takes long (or failed) is waited for by the runtime, at `ev` if given.
 template <class F>
-int wait_record(cudaStream_t st, F there)
+int wait_record(cudaStream_t st, cudaEvent_t ev, F there)
 {
     const auto t0 = std::chrono::steady_clock::now();
     bool ok = there();
     for (uint32_t i = 1; !ok; i++, ok = there())
         if (i % 1024 == 0 && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(2)) break;
     if (!ok) {
-        const int rc = cuda_err(cudaStreamSynchronize(st));
+        const int rc = cuda_err(ev ? cudaEventSynchronize(ev) : cudaStreamSynchronize(st));
         if (rc != LX_OK) return rc;
         if (!there()) return LX_E_CUDA;
     }
@@ -903,22 +903,18 @@ void rows_table(const lx_tokenset *ts, int mode, const DeviceTables &dt, RParams
     P.cmap_off = w.cmap_off;
 }
 
-int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
-                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
-                    const RowsGiven *given)
+namespace {
+
+// One input's launch: its parameters and shape, with the scratch grown for it.
+int rows_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+                 uint32_t *d_lens, uint64_t capacity, const RowsGiven *given, RLaunch &L)
 {
-    if (n == 0) {
-        *n_tokens = 0;
-        *consumed = 0;
-        return LX_OK;
-    }
     const WalkTable &w = ts->walk[mode];
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != c->device) return LX_E_INVAL;
     DeviceTables dt;
     int rc = ensure_device_tables(ts, dev, &dt);
     if (rc != LX_OK) return rc;
-    RLaunch L;
     RParams &P = L.P;
     P = RParams{};
     P.lo = (uint32_t)(reinterpret_cast<uintptr_t>(d_in) & 15u);
@@ -947,11 +943,10 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     const uint64_t need = o_spill + 2ull * (32 * P.slice + 1) * L.grid * L.nwarps;
     void **buf = L.fused ? &c->small : &c->scratch;
     size_t *have = L.fused ? &c->small_bytes : &c->scratch_bytes;
-    if (*have < need) c->small_clean = L.fused ? false : c->small_clean;
+    if (L.fused && *have < need) c->small_clean = false;
     rc = grow(buf, have, need);
     if (rc != LX_OK) return rc;
     uint8_t *scr = static_cast<uint8_t *>(*buf);
-    static_assert(sizeof(RResult) == 32 && sizeof(HostRecord) <= LAUNCH_RECORD_BYTES, "record layout");
     P.res = reinterpret_cast<RResult *>(scr);
     P.tile_counter = reinterpret_cast<unsigned int *>(scr + sizeof(RResult));
     P.done = P.tile_counter + 1;
@@ -963,39 +958,157 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     P.row_step = given ? P.slice / given->step : 1;
     P.before = given ? given->error : nullptr;
     P.spill = reinterpret_cast<uint16_t *>(scr + o_spill);
-    P.host = static_cast<HostRecord *>(c->h_res);
-    P.seq = ++c->seq ? c->seq : ++c->seq;
     P.clean = L.fused;
     L.ggrid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (P.n_slices + GUESS_NT - 1) / GUESS_NT);
+    return LX_OK;
+}
+
+// Queue it on st; its record goes to `rec` (pinned).
+int rows_queue(lx_ctx *c, RLaunch &L, const RowsGiven *given, HostRecord *rec, cudaStream_t st)
+{
+    RParams &P = L.P;
+    P.host = rec;
+    P.seq = ++c->seq ? c->seq : ++c->seq;
     // a small launch finds its scratch zeroed by the one before
     if (given || (L.fused && !c->small_clean)) {
-        rc = cuda_err(cudaMemsetAsync(scr, 0, L.fused ? SMALL_ZERO : zero, st));
+        const int rc = cuda_err(cudaMemsetAsync(P.res, 0, L.fused ? SMALL_ZERO : P.zero_bytes, st));
         if (rc != LX_OK) return rc;
     }
-    volatile HostRecord *hr = P.host;
-    hr->seq = 0;
+    static_cast<volatile HostRecord *>(rec)->seq = 0;
     std::atomic_thread_fence(std::memory_order_seq_cst);
     if (L.fused) c->small_clean = false;   // until this launch has finished without an error
-    if (c->timing && !given) cudaEventRecord(c->ev[0], st);
     launch(L, given, st);
-    rc = cuda_err(cudaGetLastError());
-    if (c->timing) cudaEventRecord(c->ev[1], st);
+    return cuda_err(cudaGetLastError());
+}
+
+// Wait for its record: the tokens, con(w) and whether it failed.  `ev`: an event
+// behind it, where more work is queued on st.
+int rows_collect(lx_ctx *c, const RLaunch &L, cudaStream_t st, cudaEvent_t ev, uint64_t *tokens, uint64_t *consumed,
+                 bool *failed)
+{
+    const volatile HostRecord *hr = L.P.host;
+    const int rc = wait_record(st, ev, [&] { return hr->seq == L.P.seq; });
     if (rc != LX_OK) return rc;
-    rc = wait_record(st, [&] { return hr->seq == P.seq; });
-    if (rc != LX_OK) return rc;
-    const RResult r = static_cast<const HostRecord *>(c->h_res)->r;
+    const RResult r = L.P.host->r;
     if (L.fused && r.error == 0) c->small_clean = true;
     if (r.error == ERR_TIMEOUT) return LX_E_TIMEOUT;
     if ((r.error & ~ERR_TIMEOUT) == ERR_FAR) return LX_FAR;   // (waits end early once an error is flagged)
     if (r.error) return LX_ROWS;
-    uint64_t tokens = r.total, con = n;
-    if (r.inv_fail_pos) {
-        con = ~r.inv_fail_pos - P.lo;
-        tokens = ~r.inv_fail_tok;
+    *failed = r.inv_fail_pos != 0;
+    *tokens = *failed ? ~r.inv_fail_tok : r.total;
+    *consumed = (*failed ? ~r.inv_fail_pos : L.P.n) - L.P.lo;
+    return LX_OK;
+}
+
+}  // namespace
+
+int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
+                    uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
+                    const RowsGiven *given)
+{
+    static_assert(sizeof(RResult) == 32 && sizeof(HostRecord) <= LAUNCH_RECORD_BYTES, "record layout");
+    if (n == 0) {
+        *n_tokens = 0;
+        *consumed = 0;
+        return LX_OK;
     }
+    RLaunch L;
+    int rc = rows_prepare(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, given, L);
+    if (rc != LX_OK) return rc;
+    if (c->timing && !given) cudaEventRecord(c->ev[0], st);
+    rc = rows_queue(c, L, given, static_cast<HostRecord *>(c->h_res), st);
+    if (c->timing) cudaEventRecord(c->ev[1], st);
+    uint64_t tokens = 0, con = 0;
+    bool failed = false;
+    if (rc == LX_OK) rc = rows_collect(c, L, st, nullptr, &tokens, &con, &failed);
+    if (rc != LX_OK) return rc;
     *n_tokens = tokens;
     *consumed = con;
     return tokens > capacity ? LX_E_CAPACITY : LX_OK;
+}
+
+// Bound by the two copies (17 and about 24 MB for 80 MiB of JSON: 533 us when
+// they overlap).  Pieces of 12 MiB, at most eight (lex.cu: ROWS_PIECE): the
+// launches of a piece take a few microseconds of host time, the copy in of the
+// first and the copy out of the last overlap nothing.  JSON, kinds 2, against
+// the single-pass kernel in pieces of 32 MiB: 1.5 KB 60 -> 33 us, 1 MiB
+// 83 -> 53, 24 MiB 361 -> 277, 48 MiB 632 -> 497, 80 MiB 832 -> 756..790 (with
+// pieces of 8 MiB 814, of 16 MiB 783; tapered at both ends 790).
+int lex_rows_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in, uint64_t n, int mode, uint16_t *h_kinds,
+                  uint32_t *h_lens, uint64_t capacity, const uint64_t *b, uint32_t K, uint64_t *n_tokens,
+                  uint64_t *consumed, cudaStream_t st)
+{
+    auto al = [](uint64_t x, uint64_t a) { return (x + a - 1) / a * a; };
+    // device layout: piece i's bytes at a 16-byte aligned offset; its tokens
+    // (at most one per byte) in its own output range, 4-token aligned
+    std::vector<uint64_t> in_off(K), out_off(K), cap(K);
+    uint64_t in_total = 0, out_total = 0;
+    for (uint32_t i = 0; i < K; i++) {
+        const uint64_t len = b[i + 1] - b[i];
+        in_off[i] = in_total;
+        in_total = al(in_total + len, 16);
+        cap[i] = al(len + 1, 4);
+        out_off[i] = out_total;
+        out_total += cap[i];
+    }
+    int rc = grow(&c->d_in, &c->d_in_bytes, in_total + 16);
+    if (rc == LX_OK) rc = grow(&c->d_out, &c->d_out_bytes, 6 * out_total + 64);
+    if (rc == LX_OK) rc = grow_host(&c->h_scratch, &c->h_scratch_bytes, sizeof(HostRecord) * (size_t)K);
+    if (rc != LX_OK) return rc;
+    uint8_t *d_in = static_cast<uint8_t *>(c->d_in);
+    uint32_t *d_lens = static_cast<uint32_t *>(c->d_out);
+    uint16_t *d_kinds = reinterpret_cast<uint16_t *>(d_lens + out_total);
+    HostRecord *rec = static_cast<HostRecord *>(c->h_scratch);
+    // every piece's parameters twice: the scratch has grown for all of them
+    // before the first launch is queued
+    std::vector<RLaunch> L(K);
+    for (int pass = 0; pass < 2 && rc == LX_OK; pass++)
+        for (uint32_t i = 0; i < K && rc == LX_OK; i++)
+            rc = rows_prepare(c, ts, d_in + in_off[i], b[i + 1] - b[i], mode, d_kinds + out_off[i], d_lens + out_off[i],
+                              cap[i], nullptr, L[i]);
+    if (rc != LX_OK) return rc;
+    // one piece: all on the caller's stream
+    cudaStream_t si = K > 1 ? c->s_in : st, so = K > 1 ? c->s_out : st;
+    for (uint32_t i = 0; i < K && rc == LX_OK; i++) {
+        rc = cuda_err(cudaMemcpyAsync(d_in + in_off[i], h_in + b[i], b[i + 1] - b[i], cudaMemcpyHostToDevice, si));
+        if (rc == LX_OK && K > 1) rc = cuda_err(cudaEventRecord(c->ev_in[i], si));
+    }
+    // the launches, in order on the caller's stream (one scratch, reused)
+    if (c->timing) cudaEventRecord(c->ev[0], st);
+    for (uint32_t i = 0; i < K && rc == LX_OK; i++) {
+        if (K > 1) rc = cuda_err(cudaStreamWaitEvent(st, c->ev_in[i], 0));
+        if (rc == LX_OK) rc = rows_queue(c, L[i], nullptr, rec + i, st);
+        if (rc == LX_OK && K > 1) rc = cuda_err(cudaEventRecord(c->ev_lex[i], st));
+    }
+    if (c->timing) cudaEventRecord(c->ev[1], st);
+    // each piece's tokens out as soon as it is lexed, after the previous pieces'
+    uint64_t out = 0, con = n;
+    bool failed = false;
+    for (uint32_t i = 0; i < K && !failed && rc == LX_OK; i++) {
+        uint64_t m = 0, pc = 0;
+        rc = rows_collect(c, L[i], st, K > 1 ? c->ev_lex[i] : nullptr, &m, &pc, &failed);
+        if (rc != LX_OK) break;
+        if (failed) con = b[i] + pc;   // Corollary 1: the first failing piece ends the stream
+        const uint64_t lo = std::min(out, capacity), hi = std::min(out + m, capacity);
+        if (hi > lo) {
+            rc = cuda_err(cudaMemcpyAsync(h_lens + lo, d_lens + out_off[i], (hi - lo) * 4, cudaMemcpyDeviceToHost, so));
+            if (rc == LX_OK)
+                rc = cuda_err(cudaMemcpyAsync(h_kinds + lo, d_kinds + out_off[i], (hi - lo) * 2, cudaMemcpyDeviceToHost, so));
+        }
+        out += m;
+    }
+    int r2 = cuda_err(cudaStreamSynchronize(so));
+    if (rc == LX_OK) rc = r2;
+    if (K > 1) {
+        r2 = cuda_err(cudaStreamSynchronize(st));
+        if (rc == LX_OK) rc = r2;
+        r2 = cuda_err(cudaStreamSynchronize(si));
+        if (rc == LX_OK) rc = r2;
+    }
+    if (rc != LX_OK) return rc;
+    *n_tokens = out;
+    *consumed = con;
+    return out > capacity ? LX_E_CAPACITY : LX_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1142,7 +1255,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
     if (c->timing) cudaEventRecord(c->ev[0], st);
     rc = cuda_err(cudaGraphLaunch(c->b_exec, st));
     if (c->timing) cudaEventRecord(c->ev[1], st);
-    if (rc == LX_OK) rc = wait_record(st, [&] { return *seq == 1; });
+    if (rc == LX_OK) rc = wait_record(st, nullptr, [&] { return *seq == 1; });
     if (rc != LX_OK) return rc;
 
     const RResult r = *reinterpret_cast<const RResult *>(hs + h_down);

@@ -163,6 +163,14 @@ struct RowsGiven {
 int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
                     uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
                     const RowsGiven *given = nullptr);
+// lx_lex_host on the same kernels: the K pieces [b[i], b[i + 1]) of the host
+// input (cut at certified bytes) each copied in, lexed by its own launch into
+// its own output range, and copied out after the previous pieces' tokens.  Uses
+// the context's s_in / s_out streams and K of its events where K > 1; LX_ROWS
+// and LX_FAR as above (the host buffers then hold nothing defined).
+int lex_rows_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in, uint64_t n, int mode, uint16_t *h_kinds,
+                  uint32_t *h_lens, uint64_t capacity, const uint64_t *b, uint32_t K, uint64_t *n_tokens,
+                  uint64_t *consumed, cudaStream_t st);
 // lx_lex_batch in one launch from entry rows (rows.cu), with the context's
 // combined table (its key: part of the graph's); LX_ROWS, LX_FAR as above.
 int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_doc *docs, uint32_t n_docs, int mode,
