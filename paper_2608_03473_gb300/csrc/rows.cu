@@ -12,7 +12,8 @@
 //               certified bytes of the mode are among them), so a lane that
 //               starts a few bytes before the slice in the PRE row, which
 //               absorbs bytes up to the first synchronizing one, reaches the
-//               slice in the scanner's row.
+//               slice in the scanner's row.  (Small inputs, and large ones
+//               where 32 bytes nearly always suffice: lex_rows does it.)
 //   lex_rows    every warp claims tiles of 32 slices; lane i walks slice i
 //               from its entry row, stores the event codes in its part of
 //               the warp's event buffer, counts them, and turns them into
@@ -34,7 +35,7 @@
 // on past their lane's bytes to the next one: no lane walks another's bytes
 // (that tail was 16-26 % of the time), no halo, 16-byte event stores, and
 // token-driven instead of byte-driven emission (instructions per input byte
-// 1.02 -> 0.7).  A call: 512 MiB of JSON 1 003 -> 545 us, 192 MiB of C-like
+// 1.02 -> 0.7).  A call: 512 MiB of JSON 1 003 -> 520 us, 192 MiB of C-like
 // text 630 -> 334 us, 1 MiB of arith tokens 84 -> 30 us, 40 MiB not 16-byte
 // aligned (formerly the tile kernel) 333 -> 79 us.  What bounds it: the
 // load/store pipe, 66-80 % busy (1 460 wavefronts per 6 KiB tile of JSON: 614
@@ -175,6 +176,16 @@ __global__ void __launch_bounds__(GUESS_NT) row_guess(RParams P)
         if (p == 0) r = E.start - E.tb;
         if (p < n) P.rows[s] = (uint16_t)r;
     }
+}
+
+// The scratch of a lex_rows that finds its rows itself.
+__global__ void rows_zero(RParams P)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    uint4 *z = reinterpret_cast<uint4 *>(P.res);
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < P.zero_bytes / 16;
+         i += (uint64_t)gridDim.x * blockDim.x)
+        z[i] = make_uint4(0, 0, 0, 0);
 }
 
 // The slice [ps, pe) of a lane token by token, from the last event that its
@@ -413,7 +424,7 @@ __device__ void finish_launch(const RParams &P)
     }
 }
 
-template <int FORM, int NW, bool FUSED, bool BATCH>
+template <int FORM, int NW, bool FIND, bool BATCH>
 __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -422,7 +433,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     REnv E;
     bool go = stage_table<FORM>(P, smem, E);
-    if (!FUSED) asm volatile("griddepcontrol.wait;" ::: "memory");   // the rows and the zeroed scratch of row_guess
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the zeroed scratch and the rows of the kernel before
     if (!go && threadIdx.x == 0) atomicOr(P.error(), ERR_SMEM);   // (row_guess may have zeroed the first one)
     __syncthreads();
     const uint32_t area = ((E.tb + P.blob_bytes + 15u) & ~15u) + wid * WAREA;
@@ -478,21 +489,21 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
             __syncwarp();
             bulk_load(evl, in + p0, SLICE, mbar);
         }
-        uint32_t er;
-        if (FUSED) {
-            const uint64_t p = (uint64_t)tile * TILE + p0;
+        const uint64_t p = (uint64_t)tile * TILE + p0;
+        const bool near = FIND && whole && !P.n_pat;   // rows from the slices' own bytes
+        uint32_t er = 0, e;
+        uint4 g0, g1;
+        if (near) {
+            if (lane == 0 && tile) {
+                g0 = ldg16(in - 32);
+                g1 = ldg16(in - 16);
+            }
+        } else if (FIND) {
             er = guess_row<FORM>(guess_in(P), E, p, has && p > 0);
             if (p == 0) er = P.p_start;
-        } else {
-            er = has ? P.rows[((uint64_t)tile * 32 + lane) * P.row_step] : 0u;
+        } else if (has) {
+            er = P.rows[((uint64_t)tile * 32 + lane) * P.row_step];
         }
-        const bool act = has && er < ROW_DEAD;
-        const uint32_t e_in = er + E.tb, ps = max(p0, lo), pe = min(p0 + SLICE, nrel);
-        uint32_t e = e_in;
-
-        // walk the slice, its codes over its bytes.  (With 16-byte loads from
-        // global memory instead, 32 lines a load, the input alone took a quarter
-        // of the shared-memory and L1 pipe that bounds this kernel.)
         if (whole) {
             const bool there = mbar_wait(mbar, phase, P.timeout_ns);
             phase ^= 1u;
@@ -501,6 +512,41 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
                 mbar_wait(mbar, phase ^ 1u, P.timeout_ns);   // the copies must not land in a finished CTA
                 break;
             }
+        }
+        if (near) {   // as guess_row, from the end of the lane before's slice
+            if (lane) {
+                g0 = lds16(evl - STRIDE + SLICE - 32);
+                g1 = lds16(evl - STRIDE + SLICE - 16);
+            }
+            __syncwarp();   // (the walks below write over it)
+            e = p > 32 ? E.pre : E.start;
+            wword<FORM>(e, g0.x, E.cmap);
+            wword<FORM>(e, g0.y, E.cmap);
+            wword<FORM>(e, g0.z, E.cmap);
+            wword<FORM>(e, g0.w, E.cmap);
+            if (e == E.slow) e = E.pre;
+            wword<FORM>(e, g1.x, E.cmap);
+            wword<FORM>(e, g1.y, E.cmap);
+            wword<FORM>(e, g1.z, E.cmap);
+            wword<FORM>(e, g1.w, E.cmap);
+            if (e == E.slow) e = E.pre;
+            er = p ? (e & ~0xFFu) - E.tb : P.p_start;
+            const bool open = p && e >= E.pre;
+            if (__any_sync(0xffffffffu, open)) {   // no synchronizing byte there
+                GuessIn I = guess_in(P);
+                I.guess = 128;
+                const uint32_t r = guess_row<FORM>(I, E, p, open);
+                if (open) er = r;
+            }
+        }
+        const bool act = has && er < ROW_DEAD;
+        const uint32_t e_in = er + E.tb, ps = max(p0, lo), pe = min(p0 + SLICE, nrel);
+        e = e_in;
+
+        // walk the slice, its codes over its bytes.  (With 16-byte loads from
+        // global memory instead, 32 lines a load, the input alone took a quarter
+        // of the shared-memory and L1 pipe that bounds this kernel.)
+        if (whole) {
             if (act) {
                 uint4 A = lds16(evl);
 #pragma unroll 2
@@ -718,7 +764,8 @@ struct RLaunch {
     RParams P;
     uint32_t grid = 0, nwarps = 0, smem = 0;
     uint32_t ggrid = 0, gsmem = 0;
-    bool fused = false;
+    bool fused = false;   // its scratch is zero between launches
+    bool find = false;    // lex_rows finds its entry rows itself
     int form = FORM_BYTE, nw = 1;
 };
 
@@ -728,6 +775,17 @@ constexpr uint64_t FUSED_MAX = 4ull << 20;
 // words for FUSED_MAX / 1 KiB + 1 tiles, group words, the record.
 constexpr uint64_t SMALL_ZERO = 48 * 1024;
 static_assert(64 + 8 * (FUSED_MAX / 1024 + 1) + 16 * (FUSED_MAX / 1024 / GS + 2) + 64 <= SMALL_ZERO, "small scratch");
+// Where no word has to be searched for (n_pat = 0: the 32 bytes before a slice
+// nearly always synchronize, and they are in shared memory as the end of the
+// slice before), launches of three rounds of tiles and more find their rows
+// themselves too, at slice lengths that such launches have.  512 MiB of JSON
+// 546 -> 520 us, 256 MiB 306 -> 280, 64 MiB 109 -> 99; 256 MiB of arith tokens
+// 641 -> 615: row_guess reads 128 bytes of memory for each 32 that it walks.
+// In fewer rounds the rare lane that has to look 128 or 512 bytes back, one
+// byte in 90 cycles beside 19 other warps, is a round's time by itself: 20 MiB
+// of JSON 61 us with row_guess, 84 .. 93 without.
+constexpr int FIND_NW_MIN = 5, FIND_NW_MAX = 7;
+constexpr uint64_t FIND_ROUNDS = 3;
 // A warp's time for a tile of 32 slices of 32 k bytes, in units of its fixed
 // part, and the warps per SM past which more of them do not help (measured at
 // 20 warps, 512 MiB of JSON: 669, 616, 581, 584 and 637 us for k = 4 to 8; 192
@@ -740,10 +798,16 @@ using RowsKernel = void (*)(RParams);
 
 // The kernel of a table form and geometry, and its per-warp shared bytes.
 template <int FORM, bool BATCH>
-RowsKernel rows_kernel(int nw, bool fused)
+RowsKernel rows_kernel(int nw, bool find)
 {
     if constexpr (!BATCH)
-        if (fused) return nw == 1 ? lex_rows<FORM, 1, true, false> : lex_rows<FORM, 2, true, false>;
+        if (find) switch (nw) {
+            case 1: return lex_rows<FORM, 1, true, false>;
+            case 2: return lex_rows<FORM, 2, true, false>;
+            case 5: return lex_rows<FORM, 5, true, false>;
+            case 6: return lex_rows<FORM, 6, true, false>;
+            default: return lex_rows<FORM, FIND_NW_MAX, true, false>;
+            }
     switch (nw) {
     case 1: return lex_rows<FORM, 1, false, BATCH>;
     case 2: return lex_rows<FORM, 2, false, BATCH>;
@@ -755,10 +819,10 @@ RowsKernel rows_kernel(int nw, bool fused)
     default: return lex_rows<FORM, 8, false, BATCH>;
     }
 }
-RowsKernel rows_kernel(int form, int nw, bool fused, bool batch = false)
+RowsKernel rows_kernel(int form, int nw, bool find, bool batch = false)
 {
     if (batch) return rows_kernel<FORM_CLASS, true>(nw, false);
-    return form == FORM_BYTE ? rows_kernel<FORM_BYTE, false>(nw, fused) : rows_kernel<FORM_CLASS, false>(nw, fused);
+    return form == FORM_BYTE ? rows_kernel<FORM_BYTE, false>(nw, find) : rows_kernel<FORM_CLASS, false>(nw, find);
 }
 
 RowsKernel guess_kernel(int form, bool batch)
@@ -768,12 +832,12 @@ RowsKernel guess_kernel(int form, bool batch)
 }
 
 // Whether the kernels may use the shared memory they are launched with (once per context and kernel).
-int allow_smem(lx_ctx *c, int form, int nw, bool fused, bool batch = false)
+int allow_smem(lx_ctx *c, int form, int nw, bool find, bool batch = false)
 {
-    const uint64_t key = (2ull << 62) | ((uint64_t)batch << 9) | ((uint64_t)form << 8) | ((uint64_t)fused << 7) | (uint64_t)nw;
+    const uint64_t key = (2ull << 62) | ((uint64_t)batch << 9) | ((uint64_t)form << 8) | ((uint64_t)find << 7) | (uint64_t)nw;
     for (auto &kv : c->occupancy)
         if (kv.first == key) return LX_OK;
-    cudaError_t e = cudaFuncSetAttribute(rows_kernel(form, nw, fused, batch),
+    cudaError_t e = cudaFuncSetAttribute(rows_kernel(form, nw, find, batch),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(guess_kernel(form, batch), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -836,16 +900,17 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGive
     L.smem = fixed + L.nwarps * area;
     L.grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, tiles);
     L.gsmem = fixed;
-    return allow_smem(c, w.form, nw, L.fused);
+    L.find = L.fused || (!given && !L.P.n_pat && nw >= FIND_NW_MIN && nw <= FIND_NW_MAX &&
+                         tiles >= FIND_ROUNDS * L.grid * L.nwarps);
+    return allow_smem(c, w.form, nw, L.find);
 }
 
 void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
 {
-    if (!L.fused && !given) {
-        guess_kernel(L.form, false)<<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
-    }
+    if (!L.find && !given) guess_kernel(L.form, false)<<<L.ggrid, GUESS_NT, L.gsmem, st>>>(L.P);
+    else if (L.find && !L.fused) rows_zero<<<32, 256, 0, st>>>(L.P);
     if (L.fused || given) {
-        rows_kernel(L.form, L.nw, L.fused)<<<L.grid, 32 * L.nwarps, L.smem, st>>>(L.P);
+        rows_kernel(L.form, L.nw, L.find)<<<L.grid, 32 * L.nwarps, L.smem, st>>>(L.P);
         return;
     }
     // lex_rows may start, and stage its table, while the last CTAs of row_guess
@@ -860,7 +925,7 @@ void launch(const RLaunch &L, const RowsGiven *given, cudaStream_t st)
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, rows_kernel(L.form, L.nw, L.fused), L.P);
+    cudaLaunchKernelEx(&cfg, rows_kernel(L.form, L.nw, L.find), L.P);
 }
 
 // The last CTA of a launch has written its record to pinned memory: a launch
@@ -921,14 +986,14 @@ int rows_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     P.in = d_in - P.lo;
     P.n = n + P.lo;
     L.form = w.form;
-    rc = shape(c, ts, mode, L, given);
-    if (rc == LX_E_TOOBIG) return LX_ROWS;
-    if (rc != LX_OK) return rc;
-    rows_table(ts, mode, dt, P);
     P.guess = 32;
     if (w.n_sync <= 4)   // few byte values synchronize: they are searched for
         for (uint32_t b = 0; b < 256; b++)
             if (w.sync[w.form == FORM_BYTE ? b : ts->byte_class[b]] != w.p_pre) P.pat[P.n_pat++] = b * 0x01010101u;
+    rc = shape(c, ts, mode, L, given);
+    if (rc == LX_E_TOOBIG) return LX_ROWS;
+    if (rc != LX_OK) return rc;
+    rows_table(ts, mode, dt, P);
     P.out_kinds = d_kinds;
     P.out_lens = d_lens;
     P.cap = capacity;
@@ -939,7 +1004,7 @@ int rows_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
     const uint64_t groups = (P.n_tiles + GS - 1) / GS;
     const uint64_t o_g = 64 + 8ull * P.n_tiles, o_i = o_g + 8 * groups, zero = (o_i + 8 * groups + 15) & ~15ull;
-    const uint64_t o_rows = L.fused ? SMALL_ZERO : al(zero), o_spill = al(o_rows + (L.fused || given ? 0 : 2 * P.n_slices));
+    const uint64_t o_rows = L.fused ? SMALL_ZERO : al(zero), o_spill = al(o_rows + (L.find || given ? 0 : 2 * P.n_slices));
     const uint64_t need = o_spill + 2ull * (32 * P.slice + 1) * L.grid * L.nwarps;
     void **buf = L.fused ? &c->small : &c->scratch;
     size_t *have = L.fused ? &c->small_bytes : &c->scratch_bytes;

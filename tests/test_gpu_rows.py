@@ -134,3 +134,26 @@ def test_random_automata(env):
         for n in (777, 9000):
             w = bytes(rng.choice(b"abc") for _ in range(n))
             check(lg, ctx, ts, dfa, [], w, 0, off=rng.randrange(16))
+
+
+@pytest.mark.parametrize("name,mode,off,size", [("json", 2, 13, 64 << 20), ("json", 0, 0, (90 << 20) + 1001), ("arith", 0, 5, 72 << 20)])
+def test_rows_found_by_the_lexing_kernel(env, name, mode, off, size):
+    # csrc/rows.cu: FIND_ROUNDS; strings, spaces and digits for which a lane
+    # looks 32, 128 and 512 bytes back, and an error near the end
+    lg, ctx = env
+    dfa, disc = T.tokenset(name), T.discarded_kinds(name)
+    base = corpus.generate(name, size, seed=314)
+    rng = random.Random(8)
+    if name == "json":
+        nl = np.flatnonzero(base == 10)
+        parts, at = [], 0
+        for i in range(400):
+            cut = int(nl[(i + 1) * nl.size // 402]) + 1
+            length = rng.choice([20, 31, 32, 33, 60, 100, 127, 128, 129, 200, 250, 300])
+            parts += [base[at:cut].tobytes(), b'"' + b"z" * length + b'"\n' + b" " * rng.randrange(200)]
+            at = cut
+        base = np.frombuffer(b"".join(parts) + base[at:].tobytes(), np.uint8)
+    check(lg, ctx, compiled(lg, name), dfa, disc, base, mode, off=off)
+    bad = base.copy()
+    bad[size - 5000] = ord("?")
+    check(lg, ctx, compiled(lg, name), dfa, disc, bad, mode, off=off)
