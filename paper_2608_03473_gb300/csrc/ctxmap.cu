@@ -16,7 +16,7 @@
 //               chains, one class lookup for all): the context left in per
 //               candidate, as eight 4-bit indexes, and the row at every
 //               128-byte boundary passed.  A warp composes its tile's 32 maps;
-//   cm_top      one CTA composes the tiles' maps: each tile's true entry;
+//   cm_fold, cm_top   the tiles' maps composed: each tile's true entry;
 //   cm_rows     the true row at every slice boundary, for lex_rows.
 // Backtracking inside a slice is replayed (hard_run); a candidate that fails,
 // or that would have to backtrack to before its slice, is dead (15).  Where
@@ -63,6 +63,7 @@ struct CParams {
     uint8_t *starts;           // per slice: its start's offset, NO_START
     uint32_t *pmap;            // per slice: map of the slices before it in its tile
     uint32_t *tmap;            // per tile: its 32 slices' map
+    uint32_t *bmap;            // per TOP_NT tiles: their map
     uint8_t *tent;             // per tile: context index at its first start
     uint16_t *rf;              // per slice boundary and candidate of the start before it: row there (0: dead)
     uint32_t n_tiles;
@@ -428,42 +429,54 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
     }
 }
 
-// Every tile's true entry: each thread composes a run of tiles, the block
-// scans the runs' maps, each thread follows its run from the true entry.
-__global__ void __launch_bounds__(TOP_NT) cm_top(CParams P)
+// Inclusive compositions of the block's words, thread by thread.
+__device__ __forceinline__ uint32_t block_compose(uint32_t x, uint32_t *sh)
 {
-    __shared__ uint32_t sh[32];
-    const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const uint32_t per = (P.n_tiles + TOP_NT - 1) / TOP_NT;
-    const uint32_t t0 = min(P.n_tiles, t * per), t1 = min(P.n_tiles, t0 + per);
-    uint32_t m = IDENT;
-#pragma unroll 8
-    for (uint32_t i = t0; i < t1; i++) m = compose(m, __ldg(P.tmap + i));
-    uint32_t incl = m;
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (uint32_t o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl = compose(y, incl);
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x = compose(y, x);
     }
-    if (lane == 31) sh[w] = incl;
+    if (lane == 31) sh[w] = x;
     __syncthreads();
     if (w == 0) {
-        uint32_t x = sh[lane];
+        uint32_t v = sh[lane];
         for (uint32_t o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x = compose(y, x);
+            const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v = compose(y, v);
         }
-        sh[lane] = x;
+        sh[lane] = v;
     }
     __syncthreads();
-    uint32_t excl = __shfl_up_sync(0xffffffffu, incl, 1);
-    if (lane == 0) excl = IDENT;
-    if (w > 0) excl = compose(sh[w - 1], excl);
-    uint32_t k = map_at(excl, 0);   // the input begins at BOUNDARY
-#pragma unroll 8
-    for (uint32_t i = t0; i < t1; i++) {
-        P.tent[i] = (uint8_t)k;
-        k = map_at(__ldg(P.tmap + i), k);
-    }
+    return w ? compose(sh[w - 1], x) : x;
+}
+
+// Every tile's true entry, in two launches: the maps of TOP_NT tiles composed
+// by a block (cm_fold), then each block composes those of the blocks before it
+// and follows its tiles from BOUNDARY at the input's start (cm_top).  (One
+// block over all tiles took 21 us at 96 MiB and 40 at 160, on one SM.)
+__global__ void __launch_bounds__(TOP_NT) cm_fold(CParams P)
+{
+    __shared__ uint32_t sh[32];
+    const uint32_t t = blockIdx.x * TOP_NT + threadIdx.x;
+    const uint32_t m = block_compose(t < P.n_tiles ? __ldg(P.tmap + t) : IDENT, sh);
+    if (threadIdx.x == TOP_NT - 1) P.bmap[blockIdx.x] = m;
+}
+
+__global__ void __launch_bounds__(TOP_NT) cm_top(CParams P)
+{
+    __shared__ uint32_t sh[32], sh2[32], first;
+    const uint32_t per = (blockIdx.x + TOP_NT - 1) / TOP_NT;   // blocks before this one, for each thread
+    const uint32_t b0 = min(blockIdx.x, threadIdx.x * per), b1 = min(blockIdx.x, b0 + per);
+    uint32_t m = IDENT;
+    for (uint32_t i = b0; i < b1; i++) m = compose(m, __ldg(P.bmap + i));
+    m = block_compose(m, sh);
+    if (threadIdx.x == TOP_NT - 1) first = m;
+    const uint32_t t = blockIdx.x * TOP_NT + threadIdx.x;
+    const uint32_t incl = block_compose(t < P.n_tiles ? __ldg(P.tmap + t) : IDENT, sh2);   // (its barriers publish `first`)
+    const uint32_t k = map_at(incl, map_at(first, 0));
+    if (t == 0) P.tent[0] = 0;
+    if (t + 1 < P.n_tiles) P.tent[t + 1] = (uint8_t)k;
 }
 
 // The true row at every slice boundary: each slice's start hands out those up
@@ -595,7 +608,8 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const size_t o_cnt = 64, o_rows = 256, o_starts = al(o_rows + 2 * S), o_pmap = al(o_starts + S);
     const size_t o_rf = al(o_pmap + 4 * S), o_tmap = al(o_rf + 2 * KMAX * S), o_tent = al(o_tmap + 4 * T);
     const size_t o_cs = al(o_tent + T), o_ci = al(o_cs + 8 * T), o_cur = al(o_ci + 4 * T), o_nxt = al(o_cur + T);
-    const size_t o_guess = al(o_nxt + T), total = al(o_guess + 2 * T);
+    const size_t o_guess = al(o_nxt + T), o_bmap = al(o_guess + 2 * T);
+    const size_t total = al(o_bmap + 4 * ((T + TOP_NT - 1) / TOP_NT));
     rc = grow(&c->e_dev, &c->e_dev_bytes, total);
     if (rc != LX_OK) return rc;
     uint8_t *d = static_cast<uint8_t *>(c->e_dev);
@@ -607,6 +621,7 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     P.rf = reinterpret_cast<uint16_t *>(d + o_rf);
     P.tmap = reinterpret_cast<uint32_t *>(d + o_tmap);
     P.tent = d + o_tent;
+    P.bmap = reinterpret_cast<uint32_t *>(d + o_bmap);
     P.cstart = reinterpret_cast<uint64_t *>(d + o_cs);
     P.cinfo = reinterpret_cast<uint32_t *>(d + o_ci);
     P.cur = d + o_cur;
@@ -620,7 +635,9 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const uint32_t mgrid = (uint32_t)std::min<uint64_t>(2ull * c->num_sms, (tiles + MAP_NT / 32 - 1) / (MAP_NT / 32));
     if (w.form == FORM_BYTE) cm_maps<FORM_BYTE><<<mgrid, MAP_NT, smem, st>>>(P);
     else cm_maps<FORM_CLASS><<<mgrid, MAP_NT, smem, st>>>(P);
-    cm_top<<<1, TOP_NT, 0, st>>>(P);
+    const uint32_t blocks = (P.n_tiles + TOP_NT - 1) / TOP_NT;
+    cm_fold<<<blocks, TOP_NT, 0, st>>>(P);
+    cm_top<<<blocks, TOP_NT, 0, st>>>(P);
     cm_rows<<<(uint32_t)std::min<uint64_t>(8ull * c->num_sms, (32 * tiles + CM_NT - 1) / CM_NT), CM_NT, 0, st>>>(P);
     unsigned int h[ROUNDS + 1] = {0};
     if (spec) {

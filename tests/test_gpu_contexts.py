@@ -119,3 +119,16 @@ def test_speculative_counts(env):
         inside = [j for j in range(1, -(-w.size // 4096)) if len(code) + 2 <= j * 4096 < len(code) + chunks * 4096]
         assert st["chunks"] == -(-w.size // 4096) and not st["judged"]
         assert st["rescanned"] >= len(inside) and st["rounds"] >= 1 + len(inside)
+
+
+@pytest.mark.parametrize("tiles", [1023, 1024, 1025, 2049])
+def test_tile_maps_across_blocks(env, tiles):
+    # csrc/ctxmap.cu: cm_fold, cm_top compose 1024 tiles a block
+    lg, ctx = env
+    dfa, disc = T.tokenset("clike_block"), T.discarded_kinds("clike_block")
+    ts = lg.lx_compile_tokenset(dfa, disc)
+    w = corpus.generate("clike_block", tiles * 4096 - 9, seed=403).copy()
+    w[500:502] = np.frombuffer(b"/*", np.uint8)   # at the latest the next "*/" closes it
+    check(lg, ctx, ts, dfa, disc, w, 2)
+    w = np.frombuffer(b"/* " + b"in a comment\n" * (tiles * 4096 // 13) + b"*/ int a;\n", np.uint8)
+    check(lg, ctx, ts, dfa, disc, w, 0)
