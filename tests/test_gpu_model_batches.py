@@ -68,3 +68,47 @@ def test_step_equals_its_gradient(lg):
     step = (m.get_params() - p0)[big]
     assert big.sum() > 1000 and np.all(np.sign(step) == -np.sign(g[big]))
     assert np.max(np.abs(np.abs(step) - 1e-3)) < 1e-5
+
+
+@pytest.mark.parametrize("chunks,hidden", [(2, 64), (63, 33), (64, 64), (65, 64), (1001, 100), (24579, 64)])
+def test_predictions_of_a_speculative_call(lg, chunks, hidden):
+    # a model whose argmax (by lx_model_forward, other kernels) is the true
+    # context at the chunk starts of a text of three chunks, repeated: nothing
+    # is scanned again
+    import torch
+    from lexinputs import tokensets as T
+    ts = lg.lx_compile_tokenset(T.tokenset("clike_block"), T.discarded_kinds("clike_block"))
+    _, blob, t = lg.lx_tokenset_scan_table(ts)
+    cbeg = blob[t["cbeg_off"]:t["cbeg_off"] + 514].view(np.uint16).astype(np.int64)
+    cands = blob[t["cand_off"]:t["cand_off"] + 2 * int(cbeg[256])].view(np.uint16).astype(np.int64)
+    text = corpus.generate("clike_block", 60_000, seed=31)
+    text = text[:int(np.flatnonzero(text[:3 * 4096 - 40] == 10)[-1]) + 1]
+    text = np.concatenate([text, np.full(3 * 4096 - text.size, ord(" "), np.uint8)])
+    w = np.resize(text, chunks * 4096 - 100)
+    d = torch.from_numpy(w.copy()).cuda()
+    ctx = lg.lx_ctx_create()
+    rc, starts, labels = lg.lx_chunk_contexts(ctx, ts, d)
+    assert rc == 0
+    starts, labels = starts.cpu().numpy(), labels.cpu().numpy().view(np.uint16).astype(np.int64)
+    assert starts.size == chunks and (starts >= 0).all()
+    some = np.arange(1, min(chunks, 7))
+    for seed in range(1, 2000):
+        m = lg.Model(t["S"] + 1, hidden=hidden, seed=seed)
+        z = m.forward(m.windows(d, torch.from_numpy(starts[some].astype(np.int64)).cuda())).cpu().numpy()
+        for j, v in zip(some, z):
+            b = int(w[starts[j] - 1])
+            c = np.append(np.sort(cands[cbeg[b]:cbeg[b + 1]]), t["S"])
+            order = np.argsort(-v[c])
+            best = c[order[0]]
+            if (lg.CTX_BOUNDARY if best == t["S"] else best) != labels[j] or (
+                    order.size > 1 and v[c[order[0]]] - v[c[order[1]]] < 1e-4):
+                break
+        else:
+            break
+    else:
+        pytest.fail("no seed predicts the text")
+    k = torch.zeros(w.size, dtype=torch.int16, device="cuda")
+    l = torch.zeros(w.size, dtype=torch.int32, device="cuda")
+    rc, nt, con, st = lg.lx_lex_speculative(ctx, ts, m, d, 0, k, l)
+    assert rc == 0 and con == w.size
+    assert (st["chunks"], st["rescanned"], st["rounds"]) == (chunks, 0, 1)
