@@ -131,19 +131,21 @@ def measured_peak_gbs():
 
 
 def profiled_traffic(workload_key):
-    """DRAM bytes of one launch from the committed ncu summary, or None when
-    the kernel source changed since the counters were taken."""
+    """DRAM bytes of one step's kernels from the committed ncu summaries, or
+    None when the kernel source changed since the counters were taken: the
+    entry-row kernels' first, then the warp-tile kernel's."""
     import hashlib
     import re
-    try:
-        src = open(os.path.join(ROOT, "paper_2608_03473_gb300", "csrc", "lexwarp.cu"), "rb").read()
-        text = open(os.path.join(ROOT, "profiles", "lex_warps_dram_512mib.md")).read()
-    except OSError:
-        return None
-    h = hashlib.sha256(src).hexdigest()
-    for key, val, sha in re.findall(r"<!-- traffic (\S+) (\d+) ([0-9a-f]{64}) -->", text):
-        if key == workload_key and sha == h:
-            return int(val)
+    for source, profile in (("rows.cu", "lex_rows_dram_512mib.md"), ("lexwarp.cu", "lex_warps_dram_512mib.md")):
+        try:
+            src = open(os.path.join(ROOT, "paper_2608_03473_gb300", "csrc", source), "rb").read()
+            text = open(os.path.join(ROOT, "profiles", profile)).read()
+        except OSError:
+            continue
+        h = hashlib.sha256(src).hexdigest()
+        for key, val, sha in re.findall(r"<!-- traffic (\S+) (\d+) ([0-9a-f]{64}) -->", text):
+            if key == workload_key and sha == h:
+                return int(val)
     return None
 
 
@@ -454,7 +456,7 @@ def run_batch(args, rank, world, local):
             "roofline": {"bound": "hbm", "achieved": alg / (g_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / (g_ms / 1e3) / 1e9 / peak, "traffic": None,
                          "peak_source": f"{peak_src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                         "kernel": "lex_warps<class form, batch> (one launch over every document, the "
+                         "kernel": "row_guess + lex_rows<class form, batch> (over every document, the "
                                    "tables of both token sets resident, in one CUDA graph)",
                          "kernel_ms": g_ms, "algorithmic_bytes": alg},
             "separate_calls": {"value": total / sep_s / 1e9, "unit": "GB/s", "ms": 1e3 * sep_s,
@@ -465,7 +467,7 @@ def run_batch(args, rank, world, local):
             "e2e": {"value": world * total / (e2e_ms / 1e3) / 1e9, "unit": "GB/s", "h2d_bytes_per_step": total,
                     "d2h_bytes_per_step": 6 * n_tok, "ms_per_step": e2e_ms,
                     "api": "torch pinned copies + lx_lex_batch"},
-            "gpu_launches": 2 * args.steps,   # the tile map and the batch kernel per graph replay
+            "gpu_launches": 3 * args.steps,   # the tile map, row_guess and lex_rows per graph replay
             "clocks": clocks,
             "bit_exact": True if args.check else None,
         }), flush=True)
@@ -694,8 +696,8 @@ def main():
                          "frac": achieved / peak,
                          "traffic": profiled_traffic(workload_name(args.workload, args.size_mib)),
                          "peak_source": f"{peak_src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                         "kernel": "en_plan + model + sp_scan/sp_fix rounds + sp_offsets + en_emit" if refused
-                         else ("lex_warps (warp-tile kernel)" if lg.lx_tokenset_walk_table(ts, mode)[0] == 0
+                         "kernel": "cm_starts + cm_maps + cm_fold/cm_top + cm_rows + model + cm_round rounds + lex_rows" if refused
+                         else ("row_guess or rows_zero + lex_rows (entry rows)" if lg.lx_tokenset_walk_table(ts, mode)[0] == 0
                                else "lex_tiles"),
                          "kernel_ms": k_ms,
                          "algorithmic_bytes": alg_bytes, "frac_of_nominal_8tbs": achieved / 8000.0},
@@ -703,7 +705,7 @@ def main():
             "e2e": {"value": e2e_value, "unit": "GB/s", "h2d_bytes_per_step": n, "d2h_bytes_per_step": 6 * nt + 32,
                     "ms_per_step": e2e_ms,
                     "api": "torch pinned copies + lx_lex_speculative" if refused else "lx_lex_host"},
-            "gpu_launches": (None if refused else args.steps),
+            "gpu_launches": (None if refused else (1 if n <= 4 * MiB else 2) * args.steps),   # lex_rows, row_guess or rows_zero
             "clocks": clocks,
             "bit_exact": bit_exact,
         }
@@ -762,9 +764,9 @@ def main():
             line["speculative_no_model"] = {"kernel_ms": statistics.median(nm_ms),
                                             "value": n / (statistics.median(nm_ms) / 1e3) / 1e9, "unit": "GB/s",
                                             "rounds": nm_st.get("rounds"), "rescanned": nm_st.get("rescanned")}
-            # en_plan, sp_init, so_block, so_top, so_out, sp_copy; sp_scan + sp_fix per round; per
-            # batch of 16 384 windows: k_windows, two k_gemm_rb, k_argmax
-            launches = 6 + 2 * (spec_stats.get("rounds") or 1) + (n // 4096 + 16383) // 16384 * 4
+            # cm_starts, cm_maps, cm_fold, cm_top, cm_rows, cm_guess, 8 cm_round, cm_judge, lex_rows; per
+            # batch of up to 24 576 windows: k_windows, k_conv_pool2, two k_gemm_rb, k_argmax
+            launches = 16 + ((n + 4095) // 4096 + 24575) // 24576 * 5
             line["gpu_launches"] = launches * args.steps
         print(json.dumps(line), flush=True)
     if world > 1:

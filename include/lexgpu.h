@@ -250,11 +250,14 @@ int lx_ctx_last_kernel_ms(lx_ctx *ctx, float *ms);
 
 /*
  * lx_ctx_set_kernel -- which kernel lx_lex uses on this context.
- *   LX_KERNEL_AUTO (default): the warp-tile kernel (every warp owns 6144-byte
- *     tiles, event codes in the walk table) when the token set has an
- *     event-code walk table for the mode (lx_tokenset_walk_table) and d_in is
- *     16-byte aligned; the tile kernel (CTAs of 256 threads over 17408-byte
- *     tiles, per-lane token records) otherwise;
+ *   LX_KERNEL_AUTO (default): the entry-row kernels (event codes in the walk
+ *     table; every 32 to 256 bytes lexed from the row the scanner is in
+ *     there) when the token set has an event-code walk table for the mode
+ *     (lx_tokenset_walk_table) and a byte after which every run is in one
+ *     row; for inputs they refuse, and other sets, the warp-tile kernel (every
+ *     warp owns 6144-byte tiles) when there is a walk table and d_in is 16-byte
+ *     aligned; the tile kernel (CTAs of 256 threads over 17408-byte tiles,
+ *     per-lane token records) otherwise;
  *   LX_KERNEL_TILE: always the tile kernel;
  *   LX_KERNEL_WARP: always the warp-tile kernel; lx_lex returns LX_E_INVAL
  *     for a call it cannot serve.
@@ -317,8 +320,7 @@ int lx_ctx_debug_withhold(lx_ctx *ctx, uint32_t tile);
  * in order (Section 6).  By Theorem 1 (exact cuts) the result equals the
  * serial tok(w); by Theorem 3 (modulo cuts) it equals pi_I(tok(w)).
  *
- *   d_in       device, n bytes, read only.  16-byte alignment enables the
- *              bulk-copy (TMA) staging path; other alignments are accepted.
+ *   d_in       device, n bytes, read only; any alignment.
  *   mode       LX_FULL_EXACT, LX_FILTERED_EXACT or LX_FILTERED_MODULO.
  *   d_kinds    device, capacity entries: token kind of each emitted token.
  *   d_lens     device, capacity entries: its length in bytes.
@@ -331,8 +333,8 @@ int lx_ctx_debug_withhold(lx_ctx *ctx, uint32_t tile);
  *              pi_I: every serial token ends at or before con(w), so the
  *              one-cut argument of Theorem 3 covers every cut below it and
  *              the chunk holding con(w) halts there).
- *   stream     cudaStream_t.  The call synchronizes this stream once, to
- *              read back the 32-byte result record.
+ *   stream     cudaStream_t.  The call waits for its work on this stream
+ *              (its result record, in pinned host memory).
  * Errors: LX_E_INVAL, LX_E_MODE (LX_FULL_EXACT needs exact cuts: modulo
  * cuts only preserve pi_I, Theorem 3), LX_E_CAPACITY (entries beyond
  * capacity are not written), LX_E_TOOBIG, LX_E_CUDA, LX_E_TIMEOUT, LX_E_NOMEM.
@@ -367,14 +369,15 @@ int lx_lex_async(lx_ctx *ctx, const lx_tokenset *ts, const uint8_t *d_in, uint64
  * lx_lex_host -- lx_lex on HOST buffers: copies h_in to the device, lexes it
  * and copies the tokens back into h_kinds / h_lens (host, capacity entries),
  * using device buffers owned by the context.  Same results and errors as
- * lx_lex.  Inputs of 64 MiB or more with a non-empty cut set are split on the
- * host into up to 8 pieces at certified bytes (the planner of Section 6) and
- * piece copies overlap the lexing of other pieces (two context-owned copy
- * streams; the launches run in order on `stream`).  On the warp-tile kernel
+ * lx_lex.  Inputs of 24 MiB or more (64 MiB where the entry-row kernels do
+ * not apply) with a non-empty cut set are split on the host into up to 8
+ * pieces at certified bytes (the planner of Section 6) and piece copies
+ * overlap the lexing of other pieces (two context-owned copy streams; the
+ * launches run in order on `stream`).  On the entry-row and warp-tile kernels
  * each piece is copied to a 16-byte aligned place and lexed into its own
  * output range, and its tokens are copied out behind the previous pieces';
- * if some piece's certified bytes lie too far apart, or its backtracking
- * runs past the step budget (failed lookahead), the whole input is copied
+ * if some piece is refused (entry rows that do not fit, certified bytes too
+ * far apart, backtracking past the step budget), the whole input is copied
  * in again and lexed by lx_lex's plan.  Host buffers should be pinned for
  * full copy speed.  Returns after all copies have completed.
  */
@@ -423,11 +426,13 @@ int lx_autotune(lx_ctx *ctx, const lx_tokenset *ts, int mode, const uint8_t *d_s
  *
  * The input is split every 4096 bytes, each start placed within the first
  * 256 bytes of its target right after the byte with the fewest possible entry
- * contexts (at most 8: BOUNDARY or a state delta+(q, b) of Q+).  Every chunk
- * is scanned from every candidate context (counting kept tokens, recording
- * the context at the next start); the chain of exit contexts from BOUNDARY at
- * offset 0 then fixes each chunk's true context and output offset, and each
- * chunk is scanned once more to write its tokens.  Output and errors as
+ * contexts (at most 8: BOUNDARY or a state delta+(q, b) of Q+), and every 128
+ * bytes in between likewise.  Each stretch is walked from every candidate
+ * context to the next start; the chain of exit contexts from BOUNDARY at
+ * offset 0 then fixes the scanner's row every 128 bytes, from which the
+ * entry-row kernel lexes.  Without a walk table, or where a run dies that
+ * the true scan follows, every chunk is scanned from every candidate (counting
+ * kept tokens) and once more to write its tokens.  Output and errors as
  * lx_lex: tok(w) with LX_FULL_EXACT, pi_I(tok(w)) with either filtered mode
  * (the certificates play no part), con(w) in *consumed (Corollary 1).
  * Works for any token set; LX_E_TOOBIG when its plain DFA table exceeds the
@@ -524,10 +529,12 @@ int lx_model_train_step(lx_model *m, const uint16_t *d_windows, const uint16_t *
  * which one more round rescans the chunks whose entry it changed.  stats
  * (optional): chunk targets, rounds that scanned chunks (the first, the
  * fix-up rounds that changed an entry, and the round after the judge), chunks
- * scanned again after the first round, judged = 1 when the judge ran.  Each
- * scan also stages the chunk's kept tokens in context scratch (6 bytes of
- * device memory per input byte), so that the settled chunks are copied to the
- * output rather than scanned again.
+ * scanned again after the first round, judged = 1 when the judge ran.  Where
+ * lx_lex_enumerative walks from every candidate context, the rounds run on
+ * the chunks' entry-to-exit maps and nothing is scanned again; the stats are
+ * the same.  Otherwise each scan also stages the chunk's kept tokens in
+ * context scratch (6 bytes of device memory per input byte), so that the
+ * settled chunks are copied to the output.
  */
 typedef struct {
     uint64_t chunks;
@@ -548,8 +555,8 @@ int lx_lex_speculative(lx_ctx *ctx, const lx_tokenset *ts, lx_model *model, cons
  * token set in sets[0 .. n_sets).  Every document is lexed exactly as
  * lx_lex would lex it alone (cuts at the mode's certificates of its own
  * token set, Theorems 1 and 3; failures per Corollary 1).
- * One launch (the default): the warp-tile kernel runs over the tiles of all
- * documents in their order in docs[], the class-form walk tables of all the
+ * One launch (the default): the entry-row kernels (or, for what they refuse,
+ * the warp-tile kernel) run over the tiles of all documents in their order in docs[], the class-form walk tables of all the
  * sets side by side in shared memory (their rows must share the 16-bit
  * shared-address window, about 250 rows of 256 bytes in all), each tile
  * taking its document's table; the output stream d_kinds / d_lens (capacity

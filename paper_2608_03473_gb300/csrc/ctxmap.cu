@@ -22,13 +22,15 @@
 // or that would have to backtrack to before its slice, is dead (15).  Where
 // the true chain dies without a lexing failure, lex_rows finds rows that do
 // not fit and the caller takes the chunks of enumerate.cu.
-// cm_spec plays the speculative path's rounds on the chunks' maps.
+// cm_guess, cm_round and cm_judge play the speculative path's rounds on the
+// chunks' maps.
 //
-// 96 MiB of the refused C-like set, filtered: 7 143 -> 635 us a call (starts
-// 32, maps 420, top 20, rows 9, lex_rows 150); 160 MiB through the speculative
-// call with a model 11.4 -> 1.96 ms, half of it the model.  cm_maps is bound by
-// the shared-memory pipe: fifteen wavefronts a byte step (six rows and the
-// class map, lanes in unrelated rows two to four apart).
+// 96 MiB of the refused C-like set, filtered: 7 143 -> 560 us a call (starts
+// 32, maps 375, fold and top 7, rows 9, lex_rows 135); 160 MiB through the
+// speculative call with a model 11.4 -> 1.25 ms (maps 520, the model 300,
+// lex_rows 215).  cm_maps is bound by the shared-memory pipe: fifteen wavefronts
+// a byte step (six rows and the class map, lanes in unrelated rows two to four
+// apart; rows spread over the banks took it from 420 to 375).
 
 #include <cuda_runtime.h>
 

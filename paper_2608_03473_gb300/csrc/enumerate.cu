@@ -24,6 +24,8 @@
 //   (4) emit:      per chunk, scan once more from its true context and write
 //                  its tokens at its offset.
 // The result is tok(w) (or pi_I(tok(w))) and con(w) exactly.
+// ctxmap.cu does the same with a lane per 128 bytes and is taken first; these
+// kernels remain for automata without a walk table and for inputs it refuses.
 
 #include <cuda_runtime.h>
 

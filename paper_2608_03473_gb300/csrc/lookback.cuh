@@ -24,7 +24,7 @@ namespace lx {
 
 constexpr uint32_t GS = 256;                  // tiles per look-back group
 constexpr unsigned ERR_TIMEOUT_BIT = 1u;      // the error word's "a wait ran out" bit
-constexpr int GW_SHIFT = 54;                  // a group word: tiles that have published << 57 | their counts
+constexpr int GW_SHIFT = 54;                  // a group word: tiles that have published << 54 | their counts
 constexpr int LB_IN = GS / 32;                // status words per lane of a tile's own group
 
 // Polls back off exponentially (64 ns doubling to 4 us): while one slow tile
@@ -83,9 +83,9 @@ __device__ bool wait_for(const PT &P, Waiter &W, F done)
 
 // The output offset of `tile` and the status word of the tile before it (0
 // for tile 0); false when a wait ran out of time.  A wait polls one word, by
-// lane 0, and then reads the round again: thousands of waiting warps that
-// re-read whole rounds crowd the L2 lines every warp reads (512 MiB of JSON in
-// tiles of 4 KiB then took 2.2 ms, 0.7 with single words).
+// lane 0, and then reads the round again.  (Groups of 256 tiles: with 64, the
+// group words of a 4 KiB-tile launch are read so often that 512 MiB of JSON took
+// 2.2 ms instead of 0.73.)
 template <class PT>
 __device__ __forceinline__ bool resolve_tile(const PT &P, uint32_t tile, uint64_t &G, unsigned long long &before)
 {
