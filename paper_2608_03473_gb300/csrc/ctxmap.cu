@@ -634,9 +634,15 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const uint32_t wpb = CM_NT / 32, grid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (tiles + wpb - 1) / wpb);
     const uint32_t smem = 512 + R.blob_bytes + 16;
     cm_starts<<<grid, CM_NT, 0, st>>>(P);
-    const uint32_t mgrid = (uint32_t)std::min<uint64_t>(2ull * c->num_sms, (tiles + MAP_NT / 32 - 1) / (MAP_NT / 32));
-    if (w.form == FORM_BYTE) cm_maps<FORM_BYTE><<<mgrid, MAP_NT, smem, st>>>(P);
-    else cm_maps<FORM_CLASS><<<mgrid, MAP_NT, smem, st>>>(P);
+    // as many warps as make the last round of tiles a full one (every warp takes
+    // tiles in turn, and a round's time is its warps' share of the shared-memory
+    // pipe): 96 MiB are 4.04 rounds of 40 warps per SM, or 5 of 34
+    const uint32_t ctas = 2 * c->num_sms, rounds = (P.n_tiles + ctas * (MAP_NT / 32) - 1) / (ctas * (MAP_NT / 32));
+    const uint32_t mwarps = (P.n_tiles + ctas * rounds - 1) / (ctas * rounds);
+    const uint32_t mnt = 32 * std::max(mwarps, std::min(16u, (uint32_t)MAP_NT / 32));   // (sixteen stage the table)
+    const uint32_t mgrid = std::min(ctas, (P.n_tiles + mnt / 32 - 1) / (mnt / 32));
+    if (w.form == FORM_BYTE) cm_maps<FORM_BYTE><<<mgrid, mnt, smem, st>>>(P);
+    else cm_maps<FORM_CLASS><<<mgrid, mnt, smem, st>>>(P);
     const uint32_t blocks = (P.n_tiles + TOP_NT - 1) / TOP_NT;
     cm_fold<<<blocks, TOP_NT, 0, st>>>(P);
     cm_top<<<blocks, TOP_NT, 0, st>>>(P);
