@@ -25,9 +25,9 @@
 // cm_guess, cm_round and cm_judge play the speculative path's rounds on the
 // chunks' maps.
 //
-// 96 MiB of the refused C-like set, filtered: 7 143 -> 560 us a call (starts
-// 32, maps 375, fold and top 7, rows 9, lex_rows 135); 160 MiB through the
-// speculative call with a model 11.4 -> 1.25 ms (maps 520, the model 300,
+// 96 MiB of the refused C-like set, filtered: 7 143 -> 542 us a call (starts
+// 32, maps 340, fold and top 7, rows 9, lex_rows 135); 160 MiB through the
+// speculative call with a model 11.4 -> 1.20 ms (maps 480, the model 300,
 // lex_rows 215).  cm_maps is bound by the shared-memory pipe: fifteen wavefronts
 // a byte step (six rows and the class map, lanes in unrelated rows two to four
 // apart; rows spread over the banks took it from 420 to 375).
@@ -56,6 +56,7 @@ constexpr int MAP_NT = 640;        // two CTAs of 20 warps per SM
 constexpr int TOP_NT = 1024;
 constexpr uint32_t FAR_TILES = 4;  // tiles searched for the next start
 constexpr uint64_t NOPOS64 = ~0ull;
+constexpr int CLAIM = 12;          // P.counts: the tiles cm_maps has given out
 constexpr int ROUNDS = 8;          // speculative fix-up rounds (enumerate.cu: SPEC_ROUNDS)
 
 struct CParams {
@@ -282,10 +283,14 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
     __syncthreads();
     hard_rows(P, smem, E);
     __syncthreads();
-    const uint32_t lane = threadIdx.x & 31, nw = gridDim.x * (blockDim.x / 32);
+    const uint32_t lane = threadIdx.x & 31;
     const uint8_t *in = P.R.in;
     const uint64_t n = P.R.n;
-    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) / 32; t < P.n_tiles; t += nw) {
+    for (;;) {
+        uint32_t t = 0;
+        if (lane == 0) t = atomicAdd(P.counts + CLAIM, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= P.n_tiles) break;
         const uint64_t T0 = (uint64_t)t * CT, sl = (uint64_t)t * 32 + lane;
         const uint32_t so = sl < P.R.n_slices ? P.starts[sl] : NO_START;
         const bool has = so != NO_START;
@@ -634,9 +639,10 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const uint32_t wpb = CM_NT / 32, grid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (tiles + wpb - 1) / wpb);
     const uint32_t smem = 512 + R.blob_bytes + 16;
     cm_starts<<<grid, CM_NT, 0, st>>>(P);
-    // as many warps as make the last round of tiles a full one (every warp takes
-    // tiles in turn, and a round's time is its warps' share of the shared-memory
-    // pipe): 96 MiB are 4.04 rounds of 40 warps per SM, or 5 of 34
+    // as many warps as make the last round of tiles a full one (a round's time is
+    // its warps' share of the shared-memory pipe): 96 MiB are 4.04 rounds of 40
+    // warps per SM, or 5 of 34, 597 -> 572 us a call.  The warps claim their tiles
+    // (by turns they took 8 % longer: 542 us so).
     const uint32_t ctas = 2 * c->num_sms, rounds = (P.n_tiles + ctas * (MAP_NT / 32) - 1) / (ctas * (MAP_NT / 32));
     const uint32_t mwarps = (P.n_tiles + ctas * rounds - 1) / (ctas * rounds);
     const uint32_t mnt = 32 * std::max(mwarps, std::min(16u, (uint32_t)MAP_NT / 32));   // (sixteen stage the table)
