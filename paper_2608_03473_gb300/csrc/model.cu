@@ -494,8 +494,9 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
     __syncthreads();
     for (uint32_t i = tid; i < MG * MW * MD; i += MG_NT) {
         const uint32_t t = i / MD;   // window * 64 + position
+        if (b0 + t / MW >= B) break;   // past the batch there is no window (and 0 times an infinite weight is not 0)
         const float v = half0[i] + half1[i];
-        if (v != 0.0f) atomicAdd(&ge[win[(size_t)b0 * MW + t] * MD + i % MD], v);   // 0 past the batch
+        if (v != 0.0f) atomicAdd(&ge[win[(size_t)b0 * MW + t] * MD + i % MD], v);
     }
     __syncthreads();
     for (uint32_t i = tid; i < MF * MK * MD; i += MG_NT) {   // i = (k, d) * MF + f
