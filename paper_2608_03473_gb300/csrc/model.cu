@@ -304,6 +304,8 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         a.z = fmaf(w, v.z, a.z);
         a.w = fmaf(w, v.w, a.w);
     };
+    // NaN stays (fmaxf would make it 0, and a diverged model's loss finite)
+    auto relu = [](float a) { return a <= 0.0f ? 0.0f : a; };
     auto add4 = [](float4 a, const float4 &v) { return make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w); };
     // a1 = m W1 + b1, the sum over k in parts
     for (uint32_t q = tid; q < MG_KP * H; q += MG_NT) {
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         const float b = to_f(b1[j]);
         a = make_float4(a.x + b, a.y + b, a.z + b, a.w + b);
         sa1[j] = a;
-        a = make_float4(fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f), fmaxf(a.z, 0.0f), fmaxf(a.w, 0.0f));
+        a = make_float4(relu(a.x), relu(a.y), relu(a.z), relu(a.w));
         sh1[j] = a;
         if (ok[0]) h1o[(size_t)(b0 + 0) * H + j] = a.x;
         if (ok[1]) h1o[(size_t)(b0 + 1) * H + j] = a.y;
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         for (uint32_t c = lane; c < C; c += 32) sm[L.z + MG * c + wid] = 0.0f;
     }
     __syncthreads();
-    // dh1 = dz W2^T where a1 > 0: a warp per row of W2
+    // dh1 = dz W2^T where a1 > 0 (or NaN): a warp per row of W2
     for (uint32_t j = wid; j < H; j += MG_NT / 32) {
         float4 a = make_float4(0, 0, 0, 0);
         for (uint32_t c = lane; c < C; c += 32) fma4(a, to_f(w2[(size_t)j * C + c]), sz[c]);
@@ -378,8 +380,8 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         }
         if (lane == 0) {
             const float4 s = sa1[j];
-            a = make_float4(s.x > 0.0f ? a.x : 0.0f, s.y > 0.0f ? a.y : 0.0f, s.z > 0.0f ? a.z : 0.0f,
-                            s.w > 0.0f ? a.w : 0.0f);
+            a = make_float4(s.x <= 0.0f ? 0.0f : a.x, s.y <= 0.0f ? 0.0f : a.y, s.z <= 0.0f ? 0.0f : a.z,
+                            s.w <= 0.0f ? 0.0f : a.w);
             sdh[j] = a;
             if (ok[0]) dho[(size_t)(b0 + 0) * H + j] = a.x;
             if (ok[1]) dho[(size_t)(b0 + 1) * H + j] = a.y;

@@ -46,3 +46,46 @@ def test_rows_of_other_bytes_take_nothing(lg, n):
     rows = g[:OM.ROWS * OM.D].reshape(OM.ROWS, OM.D)
     others = np.setdiff1d(np.arange(OM.ROWS), win)
     assert others.size > 100 and np.all(rows[others] == 0)
+
+
+WIDE = 257   # past the sizes of the one-kernel form: the layers' kernels one by one
+
+
+def widened(p):
+    """The same function with WIDE hidden units: the rest of weight zero."""
+    emb, wc, bc, w1, b1, w2, b2 = p
+    return np.concatenate([emb, wc, bc, np.pad(w1.reshape(-1, H), ((0, 0), (0, WIDE - H))).ravel(),
+                           np.pad(b1, (0, WIDE - H)), np.pad(w2.reshape(H, C), ((0, WIDE - H), (0, 0))).ravel(), b2])
+
+
+def narrowed(g):
+    emb, wc, bc, w1, b1, w2, b2 = np.split(g, np.cumsum(OM.sizes(WIDE, C))[:-1])
+    return [emb, wc, bc, w1.reshape(-1, WIDE)[:, :H].ravel(), b1[:H], w2.reshape(WIDE, C)[:H].ravel(), b2]
+
+
+def check_against_the_layers(lg, p, n):
+    """Gradient and loss equal those of the general kernels: NaN and infinities
+    in the same places, finite values within the tolerance of the FP32 sums."""
+    win, dw, dy = batch(n, 100 + n)
+    m, wide = lg.Model(C, hidden=H), lg.Model(C, hidden=WIDE)
+    m.set_params(np.concatenate(p))
+    wide.set_params(widened(p))
+    g, loss = m.gradient(dw, dy)
+    rg, rl = wide.gradient(dw, dy)
+    assert np.isnan(loss) == np.isnan(rl) and (np.isnan(rl) or abs(loss - rl) < 1e-4 * (1 + abs(rl)))
+    for i, (a, b) in enumerate(zip(np.split(g, np.cumsum(OM.sizes(H, C))[:-1]), narrowed(rg))):
+        assert np.array_equal(np.isnan(a), np.isnan(b)), i
+        assert np.array_equal(np.isinf(a), np.isinf(b)), i
+        ok = np.isfinite(b)
+        if ok.any():
+            assert np.max(np.abs(a[ok] - b[ok])) < 1e-5 + 1e-3 * np.max(np.abs(b[ok])), i
+    return loss
+
+
+@pytest.mark.parametrize("n", [1, 4, 6, 65])
+@pytest.mark.parametrize("block,at,value", [(3, 5 * H + 3, np.nan), (4, 3, np.nan), (5, 3 * C + 2, np.nan), (6, 2, np.nan),
+                                            (4, 3, np.inf), (4, 3, -np.inf), (5, 3 * C + 2, np.inf)])
+def test_dense_layers_keep_nan(lg, block, at, value, n):
+    loss = check_against_the_layers(lg, parameters(block, at, value), n)
+    if np.isnan(value):
+        assert np.isnan(loss)
