@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
     // the convolution's part of shared memory
     float *hs = sm + L.part, *da = hs + MG * MHR * MD, *pw = da + MG * MHR * DA_LD;
     float *swc = pw + (MG_NT / 32) * MF * MK * MD, *ge = swc + MF * MK * MD;
-    for (uint32_t i = tid; i < MG * MHR * DA_LD; i += MG_NT) da[i] = 0.0f;
+    for (uint32_t i = tid; i < MG * MHR * DA_LD; i += MG_NT) da[i] = -0.0f;   // no maximum there
     for (uint32_t i = tid; i < MF * MK * MD; i += MG_NT) swc[i] = to_f(wc[i]);
     for (uint32_t i = tid; i < MROWS * MD; i += MG_NT) ge[i] = 0.0f;
     __syncthreads();
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
 #pragma unroll
         for (uint32_t i = 0; i < MG * MIN_ / MG_NT; i++) {
             const uint32_t q = tid + i * MG_NT, w = q / MIN_, r = q % MIN_, u = r / MF, f = r % MF;
-            if (av[i] & 4u) da[(w * MHR + MPAD + MPOOL * u + (av[i] & 3u)) * DA_LD + f] = sm[L.mo + MG * r + w];
+            if (av[i] & 4u) da[(w * MHR + MPAD + MPOOL * u + (av[i] & 3u)) * DA_LD + f] = sm[L.mo + MG * r + w] + 0.0f;   // (-0 -> 0)
         }
     }
     __syncthreads();
@@ -449,7 +449,8 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
 #pragma unroll
             for (uint32_t i = 0; i < UP; i++) {
                 const uint32_t u = u0 + i, ar = av[i];
-                const float g = (ar & 4u) ? sm[L.mo + MG * (u * MF + lane) + w] : 0.0f;
+                if (!(ar & 4u)) continue;   // (0 times an infinite embedding is not 0)
+                const float g = sm[L.mo + MG * (u * MF + lane) + w];
                 sb += g;
                 const float *h = hs + (w * MHR + MPOOL * u + (ar & 3u)) * MD;   // row t - 2
 #pragma unroll
@@ -478,6 +479,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
 #pragma unroll 4
             for (uint32_t f = part * (MF / FP); f < (part + 1) * (MF / FP); f++) {
                 const float gv = g[f];
+                if (__float_as_uint(gv) == 0x80000000u) continue;   // -0: no maximum (0 times an infinite weight is not 0)
                 const float4 p = *reinterpret_cast<const float4 *>(swc + (f * MK + k) * MD);
                 const float4 q = *reinterpret_cast<const float4 *>(swc + (f * MK + k) * MD + 4);
                 const float v[MD] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};

@@ -89,3 +89,14 @@ def test_dense_layers_keep_nan(lg, block, at, value, n):
     loss = check_against_the_layers(lg, parameters(block, at, value), n)
     if np.isnan(value):
         assert np.isnan(loss)
+
+
+@pytest.mark.parametrize("n", [1, 4, 6, 65])
+@pytest.mark.parametrize("block,at,value", [(0, 32 * 8 + 1, np.nan), (0, 101 * 8, np.inf), (0, 101 * 8 + 5, -np.inf),
+                                            (1, 77, np.nan), (1, 77, np.inf), (1, 78, -np.inf), (2, 3, np.nan),
+                                            (2, 3, np.inf), (2, 3, -np.inf)])
+def test_inactive_positions_add_nothing(lg, block, at, value, n):
+    # embedding, filters, their bias: a convolution output of NaN is no maximum
+    loss = check_against_the_layers(lg, parameters(block, at, value), n)
+    if np.isnan(value):
+        assert np.isfinite(loss)
