@@ -312,6 +312,22 @@ int lx_ctx_set_warp_geometry(lx_ctx *ctx, int geometry);
 int lx_ctx_debug_withhold(lx_ctx *ctx, uint32_t tile);
 
 /*
+ * lx_ctx_debug_counts -- which kernels the calls on this context have run so
+ * far (test hook: every route gives the same tokens).  One count per attempt,
+ * whether the input was lexed by it or handed on.
+ */
+typedef struct {
+    uint64_t rows;      /* entry-row kernels, with rows they found themselves   */
+    uint64_t warps;     /* warp-tile kernel                                     */
+    uint64_t tiles;     /* tile kernel                                          */
+    uint64_t contexts;  /* contexts of 128-byte slices, then entry-row kernel   */
+    uint64_t chunks;    /* chunks of 4096 bytes scanned by lx_lex_enumerative,
+                           lx_lex_speculative or a call that uses them          */
+    uint64_t graphs;    /* batch graphs captured                                */
+} lx_debug_counts;
+int lx_ctx_debug_counts(const lx_ctx *ctx, lx_debug_counts *out);
+
+/*
  * lx_lex -- lex n bytes at d_in (device) on the context's device.
  *
  * The input is cut before occurrences of the certified bytes that `mode`

@@ -58,7 +58,8 @@ EXPORTED = (
     "lx_liveness",
     "lx_tokenset_free",
     "lx_ctx_create", "lx_ctx_free", "lx_ctx_set_timeout_ms", "lx_ctx_enable_timing", "lx_ctx_last_kernel_ms",
-    "lx_ctx_set_config", "lx_ctx_get_config", "lx_autotune", "lx_ctx_debug_withhold", "lx_ctx_set_kernel",
+    "lx_ctx_set_config", "lx_ctx_get_config", "lx_autotune", "lx_ctx_debug_withhold", "lx_ctx_debug_counts",
+    "lx_ctx_set_kernel",
     "lx_ctx_set_warps", "lx_ctx_set_warp_geometry", "lx_lex_async",
     "lx_lex", "lx_lex_host", "lx_lex_noalloc", "lx_lex_batch", "lx_lex_enumerative", "lx_chunk_contexts",
     "lx_lex_speculative", "lx_model_create", "lx_model_free", "lx_model_info", "lx_model_get_params",
@@ -125,6 +126,7 @@ def load_library(path: Optional[str] = None):
             "lx_ctx_last_kernel_ms": (i32, [vp, vp]),
             "lx_ctx_set_config": (i32, [vp, vp, i32, u32, u32, u32]),
             "lx_ctx_debug_withhold": (i32, [vp, u32]),
+            "lx_ctx_debug_counts": (i32, [vp, vp]),
             "lx_ctx_set_kernel": (i32, [vp, i32]),
             "lx_ctx_set_warps": (i32, [vp, u32]),
             "lx_ctx_set_warp_geometry": (i32, [vp, i32]),
@@ -703,3 +705,16 @@ def lx_ctx_debug_withhold(ctx: Ctx, tile: int) -> int:
     """Failure-detection test hook: tile ``tile`` never publishes its
     look-back aggregate (0xFFFFFFFF: off)."""
     return load_library().lx_ctx_debug_withhold(ctx.handle, int(tile) & 0xFFFFFFFF)
+
+
+class _DebugCounts(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_uint64) for k in ("rows", "warps", "tiles", "contexts", "chunks", "graphs")]
+
+
+def lx_ctx_debug_counts(ctx: Ctx) -> dict:
+    """Route test hook: how often calls on the context have run each kernel."""
+    out = _DebugCounts()
+    rc = load_library().lx_ctx_debug_counts(ctx.handle, ctypes.byref(out))
+    if rc != LX_OK:
+        raise LexError(rc, "lx_ctx_debug_counts")
+    return {k: int(getattr(out, k)) for k, _ in out._fields_}

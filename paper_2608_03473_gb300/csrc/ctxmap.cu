@@ -635,6 +635,7 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     P.nxt = d + o_nxt;
     rc = cuda_err(cudaMemsetAsync(d, 0, 256, st));
     if (rc != LX_OK) return rc;
+    c->counts.contexts++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     const uint32_t wpb = CM_NT / 32, grid = (uint32_t)std::min<uint64_t>(4ull * c->num_sms, (tiles + wpb - 1) / wpb);
     const uint32_t smem = 512 + R.blob_bytes + 16;

@@ -1211,6 +1211,7 @@ int lx::lex_enumerative_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *
     }
     rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R);
     if (rc != LX_OK || n == 0) return rc;
+    c->counts.chunks++;
     if (c->timing) cudaEventRecord(c->ev[0], R.s);
     if (guard && (rc = en_guard(c, ts, R)) != LX_OK) return rc;
     for (;;) {
@@ -1279,6 +1280,7 @@ extern "C" int lx_lex_speculative(lx_ctx *c, const lx_tokenset *ts, lx_model *mo
     rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R, true);
     if (rc != LX_OK || n == 0) return rc;
     if (model && model_contexts(model) != ts->scan.S + 1) return LX_E_INVAL;
+    c->counts.chunks++;
     if (c->timing) cudaEventRecord(c->ev[0], R.s);
     for (;;) {
         rc = spec_pipeline(c, R, model, capacity, n_tokens, consumed, stats);

@@ -1180,6 +1180,13 @@ extern "C" int lx_ctx_debug_withhold(lx_ctx *c, uint32_t tile)
     return LX_OK;
 }
 
+extern "C" int lx_ctx_debug_counts(const lx_ctx *c, lx_debug_counts *out)
+{
+    if (!c || !out) return LX_E_INVAL;
+    *out = c->counts;
+    return LX_OK;
+}
+
 extern "C" int lx_ctx_set_timeout_ms(lx_ctx *c, uint32_t ms)
 {
     if (!c || ms == 0) return LX_E_INVAL;
@@ -1428,6 +1435,7 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
 
     rc = cuda_err(cudaMemsetAsync(c->scratch, 0, need, st));
     if (rc != LX_OK) return rc;
+    c->counts.tiles++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     launch_tiles(form, grid, L.total, st, P);
     rc = cuda_err(cudaGetLastError());
@@ -1628,6 +1636,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         if (rc != LX_OK) return rc;
     }
     // the launches, in order on the caller's stream
+    c->counts.tiles++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     uint64_t tile_off = 0;
     for (uint32_t i = 0; i < K; i++) {
@@ -1903,7 +1912,9 @@ extern "C" int lx_lex_batch(lx_ctx *c, const lx_tokenset *const *sets, uint32_t 
             return LX_E_CUDA;
         }
         c->b_key = key;
+        c->counts.graphs++;
     }
+    c->counts.tiles++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     int rc = cuda_err(cudaGraphLaunch(c->b_exec, st));
     if (c->timing) cudaEventRecord(c->ev[1], st);

@@ -1275,6 +1275,7 @@ int lex_warp_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     if (rc != LX_OK) return rc;
     rc = cuda_err(cudaMemsetAsync(c->scratch, 0, L.need, st));
     if (rc != LX_OK) return rc;
+    c->counts.warps++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     warp_launch(L, st);
     rc = cuda_err(cudaGetLastError());
@@ -1312,6 +1313,7 @@ int lex_warp_async(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64
     if (rc != LX_OK) return rc;
     rc = cuda_err(cudaMemsetAsync(c->scratch, 0, L.need, st));
     if (rc != LX_OK) return rc;
+    c->counts.warps++;
     warp_launch(L, st);
     as_finish<<<1, 32, 0, st>>>(L.P.res, n, capacity, d_result);
     return cuda_err(cudaGetLastError());
@@ -1378,6 +1380,7 @@ int lex_warp_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in, uint64_
         if (rc != LX_OK) return rc;
     }
     // the launches, in order on the caller's stream (one scratch, reused)
+    c->counts.warps++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     for (uint32_t i = 0; i < K; i++) {
         rc = warp_prepare(c, ts, d_in + in_off[i], b[i + 1] - b[i], mode, d_kinds + out_off[i], d_lens + out_off[i],
@@ -1654,7 +1657,9 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
             return LX_E_CUDA;
         }
         c->b_key = gkey;
+        c->counts.graphs++;
     }
+    c->counts.warps++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     rc = cuda_err(cudaGraphLaunch(c->b_exec, st));
     if (c->timing) cudaEventRecord(c->ev[1], st);

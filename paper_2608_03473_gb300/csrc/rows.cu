@@ -1080,6 +1080,7 @@ int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
     RLaunch L;
     int rc = rows_prepare(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, given, L);
     if (rc != LX_OK) return rc;
+    if (!given) c->counts.rows++;
     if (c->timing && !given) cudaEventRecord(c->ev[0], st);
     rc = rows_queue(c, L, given, static_cast<HostRecord *>(c->h_res), st);
     if (c->timing) cudaEventRecord(c->ev[1], st);
@@ -1139,6 +1140,7 @@ int lex_rows_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in, uint64_
         if (rc == LX_OK && K > 1) rc = cuda_err(cudaEventRecord(c->ev_in[i], si));
     }
     // the launches, in order on the caller's stream (one scratch, reused)
+    c->counts.rows++;
     if (c->timing) cudaEventRecord(c->ev[0], st);
     for (uint32_t i = 0; i < K && rc == LX_OK; i++) {
         if (K > 1) rc = cuda_err(cudaStreamWaitEvent(st, c->ev_in[i], 0));
@@ -1313,7 +1315,9 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
             return LX_E_CUDA;
         }
         c->b_key = gkey;
+        c->counts.graphs++;
     }
+    c->counts.rows++;
     volatile unsigned long long *seq = reinterpret_cast<volatile unsigned long long *>(hs + h_down + down);
     *seq = 0;
     std::atomic_thread_fence(std::memory_order_seq_cst);

@@ -1,0 +1,164 @@
+"""Which kernels serve a call (lx_ctx_debug_counts), together with its tokens:
+every route ends in another exact one, so that results alone do not show that
+the first was taken.  And the kernels that only serve what others hand on, on
+inputs that reach them: the tile kernel's configurations (LX_KERNEL_TILE) and
+the 4096-byte chunks (tokens with failed lookahead on the edge of a slice)."""
+
+import numpy as np
+import pytest
+
+import oracle
+from lexinputs import corpus
+from lexinputs import tokensets as T
+
+pytestmark = pytest.mark.gpu
+CH = 4096
+
+
+@pytest.fixture(scope="module")
+def lg(lexlib):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return lexlib
+
+
+def tset(lg, name):
+    return lg.lx_compile_tokenset(T.tokenset(name), T.discarded_kinds(name))
+
+
+def expected(name, w, mode):
+    dfa = T.tokenset(name)
+    k, l, con = oracle.lex(dfa, w)
+    if mode:
+        k, l = oracle.discard(k, l, T.discarded_kinds(name), dfa.n_kinds)
+    return k, l, con
+
+
+def ran(lg, ctx, before):
+    """The kernels run since `before` (counts that moved)."""
+    after = lg.lx_ctx_debug_counts(ctx)
+    return {k: after[k] - before[k] for k in after if after[k] != before[k]}
+
+
+def call(lg, ctx, name, w, mode, fn, off=0, ts=None):
+    """fn(ts, d, k, l) -> (rc, tokens, consumed); checks the tokens, returns the route."""
+    import torch
+    w = np.frombuffer(bytes(w), np.uint8) if isinstance(w, (bytes, bytearray)) else np.ascontiguousarray(w)
+    d = torch.zeros(w.size + 32, dtype=torch.uint8, device="cuda")[off:off + w.size]
+    d.copy_(torch.from_numpy(w.copy()))
+    k = torch.zeros(w.size + 1, dtype=torch.int16, device="cuda")
+    l = torch.zeros(w.size + 1, dtype=torch.int32, device="cuda")
+    before = lg.lx_ctx_debug_counts(ctx)
+    rc, nt, con = fn(ts or tset(lg, name), d, k, l)[:3]
+    ek, el, econ = expected(name, w, mode)
+    assert rc == 0, lg.lx_strerror(rc)
+    assert (nt, con) == (ek.size, econ)
+    assert np.array_equal(k[:nt].cpu().numpy().view(np.uint16).astype(np.int64), ek)
+    assert np.array_equal(l[:nt].cpu().numpy().view(np.uint32).astype(np.int64), el)
+    return ran(lg, ctx, before)
+
+
+# failed lookahead every few bytes, at all phases of a slice: "1e" before a letter
+LOOKAHEAD = b"1en a; " * 900
+
+
+def after_text(name, n):
+    """n bytes: text, then lookahead that the entry-row kernels hand on."""
+    return (corpus.generate(name, max(n - len(LOOKAHEAD), 64), seed=71).tobytes() + LOOKAHEAD)[:n]
+
+
+@pytest.mark.parametrize("off", [0, 5])
+@pytest.mark.parametrize("name,mode", [("json", 2), ("json", 1), ("json", 0), ("clike", 2), ("clike", 0), ("arith", 0)])
+def test_lex(lg, name, mode, off):
+    ctx = lg.lx_ctx_create()
+    for n in (1500, 5 << 20):   # one launch, and two
+        w = corpus.generate(name, n, seed=72)
+        assert call(lg, ctx, name, w, mode, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, mode, k, l), off) == {"rows": 1}
+
+
+def test_lex_handed_on(lg):
+    # over a, a+b and ; : an a that no b follows is found by lookahead to the next ';'
+    w = (b"ab;" * 5 + b"a" * 40 + b";") * 2000
+    for off, route in ((0, "warps"), (3, "tiles")):
+        ctx = lg.lx_ctx_create()
+        for n in (5000, len(w)):
+            assert call(lg, ctx, "lookahead", w[:n], 0, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 0, k, l),
+                        off) == {"rows": 1, route: 1}
+
+
+def test_kernel_setting(lg):
+    for kernel, route in ((lg.LX_KERNEL_TILE, "tiles"), (lg.LX_KERNEL_WARP, "warps")):
+        ctx = lg.lx_ctx_create()
+        assert lg.lx_ctx_set_kernel(ctx, kernel) == 0
+        w = corpus.generate("json", 200_000, seed=73)
+        assert call(lg, ctx, "json", w, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l)) == {route: 1}
+
+
+@pytest.mark.parametrize("name", ["json", "clike"])
+def test_every_tile_configuration(lg, name):
+    ctx, ts = lg.lx_ctx_create(), tset(lg, name)
+    assert lg.lx_ctx_set_kernel(ctx, lg.LX_KERNEL_TILE) == 0
+    w = corpus.generate(name, 1 << 20, seed=74)
+    for cls in (0, 1):
+        for ks in (16, 24, 40, 96):
+            for ctas in (0, 1):
+                assert lg.lx_ctx_set_config(ctx, ts, 2, ks, ctas, cls) == 0
+                assert call(lg, ctx, name, w, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l),
+                            ts=ts) == {"tiles": 1}
+
+
+def test_host(lg):
+    import torch
+    ctx, ts = lg.lx_ctx_create(), tset(lg, "json")
+    for n in (1500, 25 << 20):
+        w = corpus.generate("json", n, seed=75)
+        k, l = torch.zeros(n, dtype=torch.int16), torch.zeros(n, dtype=torch.int32)
+        before = lg.lx_ctx_debug_counts(ctx)
+        rc, nt, con = lg.lx_lex_host(ctx, ts, torch.from_numpy(w.copy()), 2, k, l)
+        ek, el, econ = expected("json", w, 2)
+        assert rc == 0 and (nt, con) == (ek.size, econ) and np.array_equal(l[:nt].numpy().astype(np.int64), el)
+        assert ran(lg, ctx, before) == {"rows": 1}
+
+
+def test_batch(lg):
+    import torch
+    names = ["json", "clike"]
+    ctx, sets = lg.lx_ctx_create(), [tset(lg, n) for n in names]
+    docs = [(i % 2, corpus.generate(names[i % 2], n, seed=76 + i)) for i, n in enumerate((100, 9000, 40000, 7, 70000))]
+    d = [torch.from_numpy(w.copy()).cuda() for _, w in docs]
+    k = torch.zeros(200_000, dtype=torch.int16, device="cuda")
+    l = torch.zeros(200_000, dtype=torch.int32, device="cuda")
+    for want in ({"rows": 1, "graphs": 1}, {"rows": 1}):
+        before = lg.lx_ctx_debug_counts(ctx)
+        rc, total, res = lg.lx_lex_batch(ctx, sets, [(x, s) for x, (s, _) in zip(d, docs)], 2, k, l)
+        assert rc == 0 and ran(lg, ctx, before) == want
+        for (s, w), (off, nt, con) in zip(docs, res):
+            ek, el, econ = expected(names[s], w, 2)
+            assert (nt, con) == (ek.size, econ)
+            assert np.array_equal(l[off:off + nt].cpu().numpy().astype(np.int64), el)
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("n", [6400, 2 * CH - 1, 2 * CH, 2 * CH + 1, 3 * CH + 255, 70001, 300 * CH + 17])
+def test_enumerative(lg, n, mode):
+    ctx = lg.lx_ctx_create()
+    for off in (0, 9):
+        w = corpus.generate("clike_block", n, seed=77)
+        enum = lambda ts, d, k, l: lg.lx_lex_enumerative(ctx, ts, d, mode, k, l)   # noqa: E731
+        assert call(lg, ctx, "clike_block", w, mode, enum, off) == {"contexts": 1}
+        # the chunks
+        assert call(lg, ctx, "clike_block", after_text("clike_block", n), mode, enum, off) == {"contexts": 1, "chunks": 1}
+
+
+@pytest.mark.parametrize("with_model", [False, True])
+@pytest.mark.parametrize("n", [6400, 2 * CH - 1, 2 * CH + 1, 70001, 300 * CH + 17])
+def test_speculative(lg, n, with_model):
+    ctx, ts = lg.lx_ctx_create(), tset(lg, "clike_block")
+    model = lg.Model(lg.lx_tokenset_scan_table(ts)[2]["S"] + 1, hidden=16, seed=5) if with_model else None
+    spec = lambda ts, d, k, l: lg.lx_lex_speculative(ctx, ts, model, d, 0, k, l)   # noqa: E731
+    w = corpus.generate("clike_block", n, seed=78)
+    assert call(lg, ctx, "clike_block", w, 0, spec, ts=ts) == {"contexts": 1}
+    # the chunks: addresses that are not 16-byte aligned, and lookahead
+    assert call(lg, ctx, "clike_block", w, 0, spec, off=5, ts=ts) == {"chunks": 1}
+    assert call(lg, ctx, "clike_block", after_text("clike_block", n), 0, spec, ts=ts) == {"contexts": 1, "chunks": 1}
