@@ -61,7 +61,6 @@ constexpr int ROUNDS = 8;          // speculative fix-up rounds (enumerate.cu: S
 
 struct CParams {
     RParams R;                 // input, table, and the record whose error word the kernels flag
-    uint32_t noacc_off;        // u8 per row behind the synchronizing rows: no accepting row on any way to it
     const uint16_t *cbeg, *cand;   // scan table: candidate states after every byte
     uint8_t *starts;           // per slice: its start's offset, NO_START
     uint32_t *pmap;            // per slice: map of the slices before it in its tile
@@ -233,7 +232,7 @@ __device__ __noinline__ uint32_t hard_run(const CParams &P, const REnv &E, uint6
 // accepting prefix.
 __device__ void hard_rows(const CParams &P, uint8_t *smem, const REnv &E)
 {
-    const uint8_t *noacc = P.R.blob + P.noacc_off, *acc = P.R.blob + P.R.acc_off;
+    const uint8_t *noacc = P.R.blob + P.R.noacc_off, *acc = P.R.blob + P.R.acc_off;
     uint32_t *tab = reinterpret_cast<uint32_t *>(smem + (E.tb - smem_u32(smem)));
     const uint32_t pre = P.R.p_pre >> E.shift, start = P.R.p_start >> E.shift, h = E.pre * 0x10001u, sl = E.slow * 0x10001u;
     for (uint32_t i = threadIdx.x; i < P.R.rows_bytes / 4; i += blockDim.x) {
@@ -606,7 +605,6 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const uint64_t tiles = (R.n + CT - 1) / CT;
     if (tiles > 0xFFFFFFF0ull) return LX_E_INVAL;
     P.n_tiles = (uint32_t)tiles;
-    P.noacc_off = R.blob_bytes + R.sync_bytes;
     const uint8_t *scan = static_cast<const uint8_t *>(dt.d_scan);
     P.cbeg = reinterpret_cast<const uint16_t *>(scan + ts->scan.cbeg_off);
     P.cand = reinterpret_cast<const uint16_t *>(scan + ts->scan.cand_off);
@@ -676,7 +674,8 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     }
     rc = cuda_err(cudaGetLastError());
     if (rc != LX_OK) return rc;
-    const RowsGiven given{R.rows, CL, R.res ? &R.res->error : nullptr};
+    // (spec: a token that fails past its chunk ends the chunk's scan, which the maps do not show; the chunks count it)
+    const RowsGiven given{R.rows, CL, &R.res->error, !spec};
     rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st, &given);
     if (spec && (rc == LX_OK || rc == LX_E_CAPACITY)) {
         // as the rounds of enumerate.cu count: a changed entry is scanned in

@@ -1450,7 +1450,7 @@ namespace {
 // the WSet array.
 struct Combined {
     std::vector<uint8_t> blob;
-    uint32_t rows_bytes = 0, acc_off = 0, sets_off = 0;
+    uint32_t bytes = 0, rows_bytes = 0, acc_off = 0, sets_off = 0;   // bytes: of one table
     bool sync = true;   // every set has a synchronizing byte
 };
 
@@ -1517,6 +1517,11 @@ int combine(const lx_tokenset *const *sets, uint32_t n_sets, int mode, Combined 
         uint16_t *pre = reinterpret_cast<uint16_t *>(out.blob.data() + bytes + base[s] + w[s]->p_pre);
         for (uint32_t k = 0; k < 128; k++) pre[k] = (uint16_t)(w[s]->sync[k] + base[s]);
     }
+    // and the rows' noacc bytes
+    out.bytes = (uint32_t)bytes;
+    out.blob.resize(2 * bytes + n_rows);
+    for (uint32_t s = 0; s < n_sets; s++)
+        std::memcpy(out.blob.data() + 2 * bytes + (base[s] >> 8), w[s]->noacc.data(), w[s]->n_rows);
     return LX_OK;
 }
 
@@ -1542,7 +1547,7 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
         r2 = cuda_err(cudaMemcpy(c->wb_dev, cb.blob.data(), cb.blob.size(), cudaMemcpyHostToDevice));
         if (r2 != LX_OK) return r2;
         c->wb_key = key;
-        c->wb_blob_bytes = (uint32_t)(cb.blob.size() / 2);
+        c->wb_blob_bytes = cb.bytes;
         c->wb_sync = cb.sync;
         c->wb_rows = cb.rows_bytes;
         c->wb_acc_off = cb.acc_off;

@@ -29,7 +29,12 @@
 // lexes the input another way; what was written is overwritten.
 //
 // Backtracking inside a slice (SLOW) is replayed by its lane (relex), and the
-// first lexing failure ends the stream (Corollary 1).
+// first lexing failure ends the stream (Corollary 1); a token that fails in a
+// later slice than its own, with no accepting prefix (WalkTable::noacc: an open
+// string at the input's end), fails at the last event before.  Handing such
+// inputs on took two passes: JSON cut inside a string 107 -> 32 us a call at
+// 1.5 KB, 309 -> 135 at 64 MiB; for it, a register or two of spills more: 512
+// MiB of JSON 519.8 -> 522.2 us, 512 documents 362.7 -> 367.4.
 //
 // Against the chunks of lexwarp.cu, which start at a certified byte and run
 // on past their lane's bytes to the next one: no lane walks another's bytes
@@ -192,12 +197,14 @@ __global__ void rows_zero(RParams P)
 // walk stored (or from the entry row): the walk ran into SLOW, or the input
 // ends at pe in a row that does not accept.  Codes go to ev + position - p0.
 // Sets the exit row, the code that ends at pe == end of input (tail), a
-// failure offset, or `back` where the token in progress at ps does not
-// accept in the slice (it has to be replayed from before it).
+// failure (twice its offset; twice ps + 1 where the token began before the
+// slice and has no accepting prefix: an open string at the input's end, a
+// control byte inside one), or `back` where the token in progress at ps does
+// not accept in the slice but did before it (it has to be replayed from there).
 template <int FORM>
-__device__ __noinline__ void relex(const REnv &E, const uint8_t *in, uint32_t ev, uint32_t p0, uint32_t ps, uint32_t pe,
-                                   uint32_t e_in, bool at_end, uint32_t *exit, uint32_t *tail, uint32_t *fail,
-                                   bool *back)
+__device__ __noinline__ void relex(const REnv &E, const uint8_t *noacc, const uint8_t *in, uint32_t ev, uint32_t p0,
+                                   uint32_t ps, uint32_t pe, uint32_t e_in, bool at_end, uint32_t *exit, uint32_t *tail,
+                                   uint32_t *fail, bool *back)
 {
     uint32_t tok = ps, q = e_in, r = NONE, rc = 0, k;
     bool own = false;   // a token start lies in the slice
@@ -248,7 +255,8 @@ __device__ __noinline__ void relex(const REnv &E, const uint8_t *in, uint32_t ev
             continue;
         }
         if (r == NONE) {
-            if (own) *fail = tok;
+            if (own) *fail = 2 * tok;
+            else if (noacc && __ldg(noacc + ((e_in - E.tb) >> E.shift))) *fail = 2 * ps + 1;
             else *back = true;
             return;
         }
@@ -260,14 +268,17 @@ __device__ __noinline__ void relex(const REnv &E, const uint8_t *in, uint32_t ev
     }
 }
 
+// A failure of a token that began in an earlier tile (as a position in a tile).
+constexpr uint32_t FAIL_BEFORE = NONE - 1;
+
 // A tile whose tokens wait in the warp's stage for their output offset.
 struct Pending {
     uint32_t tile;      // NONE: nothing pending
     uint32_t staged;    // kept tokens
     uint32_t split;     // of them in the shared stage (the rest: spill slot)
     uint32_t entry;     // entry row of its first lane
+    uint32_t fail;      // failure position in the tile, or NONE, or FAIL_BEFORE
     uint32_t open;      // its first event ended a kept token that began in an earlier tile
-    uint32_t fail;      // failure position in the tile, or NONE
     uint32_t lidx, llen;   // per lane: a token whose length the stage does not hold
     uint32_t doc, dtile, kmap;   // batches: its document, its index there, its set's kind map
 };
@@ -339,7 +350,7 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
             if (lane == 0) atomicOr(P.error(), ERR_ROWS);
             return false;
         }
-        if (D.open) {   // where the open token began: the last event before the tile (every earlier tile has published)
+        if (D.open || D.fail == FAIL_BEFORE) {   // where that token began: the last event before the tile (every earlier tile has published)
             bool good = true;
             if (lane == 0) {
                 Waiter W;
@@ -359,7 +370,8 @@ __device__ bool finish_tile(const RParams &P, const REnv &E, const Pending &D, u
         unsigned long long *fp = BATCH ? &P.dres[D.doc].inv_fail_pos : &P.res->inv_fail_pos;
         unsigned long long *ft = BATCH ? &P.dres[D.doc].inv_fail_tok : &P.res->inv_fail_tok;
         if (D.fail != NONE) {
-            atomicMax(fp, ~(unsigned long long)((uint64_t)dtile * TILE + D.fail));
+            const uint64_t f = (uint64_t)dtile * TILE;
+            atomicMax(fp, ~(unsigned long long)(D.fail == FAIL_BEFORE ? f - carry : f + D.fail));
             atomicMax(ft, ~(unsigned long long)(G + D.staged));
         }
         if (BATCH) {
@@ -581,8 +593,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         bool back = has && er == ROW_UNKNOWN;
         if (at_end && e != E.slow && e < E.pre) tail = acc_code(E, e);
         if (act && (e == E.slow || (at_end && !tail)))
-            relex<FORM>(E, in, evl, p0, ps, pe, e_in, at_end, &exit, &tail, &fail, &back);
-        const uint32_t fmin = __reduce_min_sync(0xffffffffu, fail);
+            relex<FORM>(E, P.noacc_off ? P.blob + P.noacc_off : nullptr, in, evl, p0, ps, pe, e_in, at_end, &exit, &tail, &fail, &back);
+        const uint32_t fmin2 = __reduce_min_sync(0xffffffffu, fail), fmin = fmin2 >> 1;   // (NONE: past every position)
         {
             const uint32_t ner = __shfl_down_sync(0xffffffffu, er, 1);
             bool bad = back;
@@ -618,7 +630,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
             }
         }
         cnt >>= 7;
-        if (fmin != NONE) {   // nothing after the failure counts
+        if (fmin2 != NONE) {   // nothing after the failure counts
             cnt = 0;
 #pragma unroll
             for (uint32_t w = 0; w < NW; w++) {
@@ -648,8 +660,12 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         const uint32_t total = __shfl_sync(0xffffffffu, excl, 31);
         excl -= cnt;
         const uint32_t xr = __shfl_sync(0xffffffffu, exit, 31);   // 0 where the input ended or failed
-        const uint32_t x31 = __shfl_sync(0xffffffffu, (act && !at_end && fmin == NONE) ? 1u : 0u, 31) ? xr - E.tb : 0u;
+        const uint32_t x31 = __shfl_sync(0xffffffffu, (act && !at_end && fmin2 == NONE) ? 1u : 0u, 31) ? xr - E.tb : 0u;
         publish_word(P, tile, ((unsigned long long)x31 << 32) | ((unsigned long long)last1 << 16) | total);
+
+        uint32_t pfail = fmin2 == NONE ? NONE : fmin;
+        if (fmin2 != NONE && (fmin2 & 1u))   // a token that fails in a later slice than its own began at the last event before it
+            pfail = last1 ? last1 - 1 : dtile == 0 ? lo : FAIL_BEFORE;
 
         // the previous tile's output: its predecessors have had a whole tile to publish
         if (pend.tile != NONE) {
@@ -663,7 +679,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         // (e) the kept events into the stage, in order
         pend.tile = tile;
         pend.staged = total;
-        pend.fail = fmin;
+        pend.fail = pfail;
         pend.entry = __shfl_sync(0xffffffffu, er, 0);
         pend.lidx = NONE;
         pend.llen = 0;
@@ -966,6 +982,7 @@ void rows_table(const lx_tokenset *ts, int mode, const DeviceTables &dt, RParams
     P.acc_off = w.acc_off;
     P.kmap_off = w.kmap_off;
     P.cmap_off = w.cmap_off;
+    P.noacc_off = P.blob_bytes + P.sync_bytes;
 }
 
 namespace {
@@ -994,6 +1011,7 @@ int rows_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     if (rc == LX_E_TOOBIG) return LX_ROWS;
     if (rc != LX_OK) return rc;
     rows_table(ts, mode, dt, P);
+    if (given && !given->open) P.noacc_off = 0;
     P.out_kinds = d_kinds;
     P.out_lens = d_lens;
     P.cap = capacity;
@@ -1271,6 +1289,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         P.rows_bytes = c->wb_rows;
         P.row_shift = 8;
         P.acc_off = c->wb_acc_off;
+        P.noacc_off = c->wb_blob_bytes;
         P.sets_off = c->wb_sets_off;
         P.guess = 32;
         P.slice = 32 * nw;

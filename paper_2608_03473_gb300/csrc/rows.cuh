@@ -34,6 +34,7 @@ struct RParams {
     const uint8_t *blob;           // walk table, then WalkTable::sync
     uint32_t blob_bytes, rows_bytes, row_shift, sync_bytes;   // multiples of 16 but the shift
     uint32_t p_start, p_pre, acc_off, kmap_off, cmap_off;
+    uint32_t noacc_off;            // u8 per row (WalkTable::noacc), in global memory only; 0: failures in an earlier slice are not taken
     uint32_t guess;                // bytes walked before a slice at first
     uint16_t *rows;                // entry row of every slice (relative address)
     uint32_t row_step;             // rows per slice of lex_rows

@@ -160,6 +160,7 @@ struct RowsGiven {
     uint16_t *rows;
     uint32_t step;
     const unsigned int *error;
+    bool open;   // whether a token may fail in a later slice than its own
 };
 int lex_rows_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
                     uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,

@@ -162,3 +162,62 @@ def test_speculative(lg, n, with_model):
     # the chunks: addresses that are not 16-byte aligned, and lookahead
     assert call(lg, ctx, "clike_block", w, 0, spec, off=5, ts=ts) == {"chunks": 1}
     assert call(lg, ctx, "clike_block", after_text("clike_block", n), 0, spec, ts=ts) == {"contexts": 1, "chunks": 1}
+
+
+def open_ended(name, n, cut, seed):
+    """A text whose last token, begun `cut` bytes before the end, has no accepting prefix."""
+    base = corpus.generate(name, n, seed=seed)
+    base = base[:int(np.flatnonzero(base == 10)[-1]) + 1].tobytes() if n else b""
+    return base + b'"' + b"text " * (cut // 5) + b"x" * (cut % 5)
+
+
+# a token that fails without an accepting prefix, begun in an earlier slice, in
+# an earlier tile, many tiles before or with the input, is a lexing error at its
+# start, not a reason to lex the input another way
+@pytest.mark.parametrize("n,cut", [(0, 40), (0, 9000), (1000, 33), (1400, 700), (300_000, 2100), (300_000, 70_000),
+                                   (5 << 20, 400), (5 << 20, 30_000)])
+def test_open_token(lg, n, cut):
+    ctx = lg.lx_ctx_create()
+    for name in ("json", "clike"):
+        if name == "clike" and cut > 8000:
+            continue   # its rows are found at newlines
+        w = open_ended(name, n, cut, 81)
+        for off in (0, 5):
+            for v in (w, w + b"\n" + corpus.generate(name, 3000, seed=82).tobytes()):   # (a raw newline ends no string)
+                assert call(lg, ctx, name, v, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l), off) == {"rows": 1}
+
+
+def test_open_token_in_a_batch(lg):
+    import torch
+    names = ["clike", "json"]
+    ctx, sets = lg.lx_ctx_create(), [tset(lg, n) for n in names]
+    rng = np.random.default_rng(83)
+    docs = [(i % 2, np.frombuffer(open_ended(names[i % 2], int(rng.integers(0, 60_000)), int(rng.integers(1, 3000)), 84 + i),
+                                  np.uint8)) for i in range(40)]
+    d = [torch.from_numpy(w.copy()).cuda() for _, w in docs]
+    size = sum(w.size for _, w in docs)
+    k = torch.zeros(size, dtype=torch.int16, device="cuda")
+    l = torch.zeros(size, dtype=torch.int32, device="cuda")
+    before = lg.lx_ctx_debug_counts(ctx)
+    rc, total, res = lg.lx_lex_batch(ctx, sets, [(x, s) for x, (s, _) in zip(d, docs)], 2, k, l)
+    assert rc == 0 and ran(lg, ctx, before) == {"rows": 1, "graphs": 1}
+    for (s, w), (off, nt, con) in zip(docs, res):
+        ek, el, econ = expected(names[s], w, 2)
+        assert (nt, con) == (ek.size, econ)
+        assert np.array_equal(l[off:off + nt].cpu().numpy().astype(np.int64), el)
+
+
+@pytest.mark.parametrize("n,cut", [(0, 300), (5000, 400), (300_000, 150), (300_000, 9000)])
+def test_open_token_from_contexts(lg, n, cut):
+    ctx, ts = lg.lx_ctx_create(), tset(lg, "clike_block")
+    w = open_ended("clike_block", n, cut, 85)
+    assert call(lg, ctx, "clike_block", w, 2, lambda ts, d, k, l: lg.lx_lex_enumerative(ctx, ts, d, 2, k, l),
+                9) == {"contexts": 1}
+    stats = []
+    for off, route in ((0, {"contexts": 1, "chunks": 1}), (5, {"chunks": 1})):
+        def spec(ts, d, k, l):
+            rc, nt, con, st = lg.lx_lex_speculative(ctx, ts, None, d, 2, k, l)
+            stats.append(st)
+            return rc, nt, con
+        assert call(lg, ctx, "clike_block", w, 2, spec, off, ts=ts) == route
+    assert stats[0] == stats[1]   # the counts of the rounds are the chunks'
