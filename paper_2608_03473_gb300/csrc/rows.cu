@@ -85,8 +85,11 @@ __device__ __forceinline__ bool has_sync(const GuessIn &P, const uint4 &c)
 // where few byte values synchronize (compared a word at a time, which takes
 // no table lookups), else from `guess` bytes before, four times as many where
 // none of them synchronizes; at most GUESS_MAX bytes back, and from START where
-// the input begins there.  SLOW looks for the next synchronizing byte (the
-// row need not be right).  All lanes of a warp call it together.
+// the input begins there.  After SLOW (a token that backtracks) the next
+// synchronizing byte is looked for; where none follows the row is lost, since
+// a walk from farther back comes to the same place (looking there all the same
+// took 1 ms of 64 MiB of C-like text with one line of them).  All lanes of a
+// warp call it together.
 template <int FORM>
 __device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool has)
 {
@@ -109,7 +112,7 @@ __device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool 
             w += back;
         }
     }
-    bool todo = has;
+    bool todo = has, lost = false;
     while (__any_sync(0xffffffffu, todo)) {
         if (todo) {
             uint64_t a = p > w ? p - w : 0;
@@ -127,13 +130,14 @@ __device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool 
                 wword<FORM>(e, c.y, E.cmap);
                 wword<FORM>(e, c.z, E.cmap);
                 wword<FORM>(e, c.w, E.cmap);
-                if (e == E.slow) e = E.pre;
+                if (e == E.slow) e = E.pre, lost = true;
             }
-            todo = e >= E.pre && w < GUESS_MAX && w < p;
+            todo = e >= E.pre && w < GUESS_MAX && w < p && !lost;
         }
         w *= 4;
     }
-    return e >= E.pre || e == E.slow ? ROW_UNKNOWN : (e & ~0xFFu) - E.tb;
+    if (e >= E.pre || e == E.slow) return lost ? ROW_LOST : ROW_UNKNOWN;
+    return (e & ~0xFFu) - E.tb;
 }
 
 __device__ __forceinline__ GuessIn guess_in(const RParams &P)
@@ -590,7 +594,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
         // the lane's end: backtracking, the end of the input, the exit row
         const bool at_end = act && pe == nrel;
         uint32_t tail = 0, fail = NONE, exit = e & ~0xFFu;   // without the event code
-        bool back = has && er == ROW_UNKNOWN;
+        bool back = has && er >= ROW_LOST;
         if (at_end && e != E.slow && e < E.pre) tail = acc_code(E, e);
         if (act && (e == E.slow || (at_end && !tail)))
             relex<FORM>(E, P.noacc_off ? P.blob + P.noacc_off : nullptr, in, evl, p0, ps, pe, e_in, at_end, &exit, &tail, &fail, &back);

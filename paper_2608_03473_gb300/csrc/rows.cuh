@@ -79,7 +79,8 @@ namespace {   // each translation unit its own copy
 constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t BIG = 0x7FFFFFFFu;
 constexpr uint32_t ROW_UNKNOWN = 0xFFFFu;   // entry row: none found (rows are at even addresses)
-constexpr uint32_t ROW_DEAD = 0xFFFEu;      // entry row: after the first failure
+constexpr uint32_t ROW_LOST = 0xFFFEu;      // entry row: a token before it backtracks
+constexpr uint32_t ROW_DEAD = 0xFFFDu;      // entry row: after the first failure
 constexpr int MAX_WARPS = 20;               // warps per CTA at most
 constexpr uint32_t LEN_MAX = 511;           // a stage entry's length field; this value: kept aside
 constexpr uint32_t GUESS_MAX = 8192;        // bytes before a slice searched for a synchronizing byte

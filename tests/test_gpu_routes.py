@@ -87,6 +87,17 @@ def test_lex_handed_on(lg):
                         off) == {"rows": 1, route: 1}
 
 
+def test_backtracking_is_not_far(lg):
+    # rows behind a token that backtracks are lost, however near the newline before it is: the old plan
+    # at once, not the contexts (and then the chunks) for inputs without a newline for 8 KiB
+    w = b"int a = 1en ; int b = 0;\n" * 3000
+    for off, route in ((0, "warps"), (3, "tiles")):
+        ctx = lg.lx_ctx_create()
+        for n in (5000, len(w)):
+            assert call(lg, ctx, "clike", w[:n], 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l),
+                        off) == {"rows": 1, route: 1}
+
+
 def test_kernel_setting(lg):
     for kernel, route in ((lg.LX_KERNEL_TILE, "tiles"), (lg.LX_KERNEL_WARP, "warps")):
         ctx = lg.lx_ctx_create()
