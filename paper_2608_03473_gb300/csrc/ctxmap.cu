@@ -54,7 +54,11 @@ constexpr uint32_t NO_START = 255;
 constexpr int CM_NT = 512;
 constexpr int MAP_NT = 640;        // two CTAs of 20 warps per SM
 constexpr int TOP_NT = 1024;
-constexpr uint32_t FAR_TILES = 4;  // tiles searched for the next start
+// Tiles searched for the next start: one lane walks all bytes up to it, 70 ns
+// each (64 MiB of C-like text with one line of 30 KiB, which has no start: 2.4
+// ms; 14.1 through the chunks of enumerate.cu, where four tiles sent it).
+constexpr uint32_t FAR_TILES = 16;
+constexpr uint64_t HARD_MAX = 64 * 4 * CT + 4096;   // steps of a stretch replayed with backtracking, at most
 constexpr uint64_t NOPOS64 = ~0ull;
 constexpr int CLAIM = 12;          // P.counts: the tiles cm_maps has given out
 constexpr int ROUNDS = 8;          // speculative fix-up rounds (enumerate.cu: SPEC_ROUNDS)
@@ -201,7 +205,7 @@ __device__ __noinline__ uint32_t hard_run(const CParams &P, const REnv &E, uint6
 {
     uint32_t q = row;
     uint64_t r = acc_code(E, q) && q != E.start ? s : NOPOS64, p = s;
-    for (uint64_t steps = 64 * (ne - s) + 4096; p < ne; steps--) {
+    for (uint64_t steps = min(64 * (ne - s) + 4096, HARD_MAX); p < ne; steps--) {
         if (steps == 0) {   // repeated failed lookahead: left to the guarded scans
             atomicOr(P.R.error(), ERR_ROWS);
             return E.slow;
@@ -317,7 +321,7 @@ __global__ void __launch_bounds__(MAP_NT, 2) cm_maps(CParams P)
                         found = true;
                     }
                 }
-                if (!found && lane == 0) atomicOr(P.R.error(), ERR_ROWS);   // starts too far apart
+                if (!found && lane == 0) atomicOr(P.R.error(), ERR_FAR);   // starts too far apart
                 if (!found) far = T0;   // walk nothing
             }
             ne = above ? T0 + src * CL + o : far;

@@ -1197,17 +1197,17 @@ int spec_pipeline(lx_ctx *c, EnRun &R, lx_model *model, uint64_t capacity, uint6
 
 int lx::lex_enumerative_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode,
                                uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens,
-                               uint64_t *consumed, cudaStream_t stream, bool guard)
+                               uint64_t *consumed, cudaStream_t stream, bool guard, bool chunks)
 {
     if (!n_tokens || !consumed) return LX_E_INVAL;
     *n_tokens = 0;
     *consumed = 0;
     EnRun R;
     int rc;
-    if (!guard && n && en_args(c, ts, d_in, n, mode, d_kinds, d_lens, capacity) == LX_OK && contexts_path_ok(ts, mode)) {
+    if (!chunks && n && en_args(c, ts, d_in, n, mode, d_kinds, d_lens, capacity) == LX_OK && contexts_path_ok(ts, mode)) {
         rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, stream, nullptr,
                                  nullptr);
-        if (rc != LX_ROWS) return rc;
+        if (rc != LX_ROWS && rc != LX_FAR) return rc;
     }
     rc = en_setup(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, stream, R);
     if (rc != LX_OK || n == 0) return rc;
@@ -1229,7 +1229,7 @@ extern "C" int lx_lex_enumerative(lx_ctx *c, const lx_tokenset *ts, const uint8_
                                   uint64_t *consumed, void *stream)
 {
     return lex_enumerative_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed,
-                                  static_cast<cudaStream_t>(stream), false);
+                                  static_cast<cudaStream_t>(stream), false, false);
 }
 
 extern "C" int lx_chunk_contexts(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n,
@@ -1272,7 +1272,7 @@ extern "C" int lx_lex_speculative(lx_ctx *c, const lx_tokenset *ts, lx_model *mo
         lx_spec_stats sp{0, 0, 0, 0};
         rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed,
                                  static_cast<cudaStream_t>(stream), model, &sp);
-        if (rc != LX_ROWS) {
+        if (rc != LX_ROWS && rc != LX_FAR) {
             if (stats) *stats = sp;
             return rc;
         }

@@ -1358,23 +1358,31 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     const bool can_enumerate = !force && c->kernel == LX_KERNEL_AUTO && ts->scan.status == LX_OK;
     const lx_tuned *tu = tuned_for(c, ts, mode);
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;
+    bool no_contexts = false;   // the contexts' rows do not fit either
     if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
-        const int rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
-        if (rc == LX_FAR)   // contexts are enumerated instead
-            return lx_lex_enumerative(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        int rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        if (rc == LX_FAR) {   // contexts are enumerated instead, of chunks where their starts are far apart as well
+            rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st, nullptr,
+                                     nullptr);
+            if (rc == LX_FAR)
+                return lex_enumerative_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st,
+                                              false, true);
+            no_contexts = true;
+        }
         if (rc != LX_ROWS) return rc;
     }
     const bool warp_ok = !force && c->kernel != LX_KERNEL_TILE && warp_path_ok(ts, mode, d_in);
     // the tile kernel cuts at single certified bytes only; the warp kernel also at windows
     const bool warp_windows = warp_ok && !mode_has_cuts(ts, mode) && warp_has_cuts(ts, mode);
     if (can_enumerate && !mode_has_cuts(ts, mode) && !warp_windows)
-        return lx_lex_enumerative(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        return lex_enumerative_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st, false,
+                                      no_contexts);
     if (warp_ok && (!tuned_tile || warp_windows)) {
         const int rc = lex_warp_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st,
                                        can_enumerate ? SPARSE_LIMIT : 0);
         if (rc != LX_SPARSE && rc != LX_LOOKAHEAD) return rc;
         return lex_enumerative_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st,
-                                      rc == LX_LOOKAHEAD);
+                                      rc == LX_LOOKAHEAD, rc == LX_LOOKAHEAD || no_contexts);
     }
     if (!force && c->kernel == LX_KERNEL_WARP && n) return LX_E_INVAL;   // asked for, not available here
     if (ts->tab[mode].status != LX_OK) return ts->tab[mode].status;

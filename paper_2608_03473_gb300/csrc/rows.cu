@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 1) lex_rows(RParams P)
     fence_proxy_async();
     __syncwarp();
     if (P.before && *P.before != 0) {   // no rows to start from
-        if (threadIdx.x == 0) atomicOr(P.error(), ERR_ROWS);
+        if (threadIdx.x == 0) atomicOr(P.error(), *P.before == ERR_FAR ? ERR_FAR : ERR_ROWS);
         go = false;
     }
 

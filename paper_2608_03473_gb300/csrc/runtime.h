@@ -150,7 +150,8 @@ bool warp_path_ok(const lx_tokenset *ts, int mode, const uint8_t *d_in);
 // lx_lex, any input alignment), for token sets with a synchronizing byte.
 // LX_ROWS: the entry rows were not found or do not fit together; the caller
 // lexes the input another way.
-// LX_FAR: only because synchronizing bytes lie too far apart.
+// LX_FAR: only because synchronizing bytes (or, with rows given, the starts
+// from which they were found) lie too far apart.
 constexpr int LX_ROWS = -102;   // internal statuses, never returned by the C ABI
 constexpr int LX_FAR = -103;
 bool rows_path_ok(const lx_tokenset *ts, int mode);
@@ -181,6 +182,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
 // lex_rows_device with the entry rows found by enumerating contexts (ctxmap.cu): any
 // token set with a walk and a scan table.  With `spec`, the speculative path's
 // predictions and rounds as well (model: nullptr for BOUNDARY everywhere).
+// LX_ROWS, LX_FAR as above.
 bool contexts_path_ok(const lx_tokenset *ts, int mode);
 int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
                         uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
@@ -208,10 +210,11 @@ int lex_warp_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint6
 // failed-lookahead guard.  Never returned by the C ABI.
 constexpr int LX_LOOKAHEAD = -101;
 // lx_lex_enumerative (enumerate.cu) with the failed-lookahead guard from the
-// start when `guard` (the caller saw a scan run past its budget already).
+// start when `guard` (the caller saw a scan run past its budget already), on
+// the chunks at once when `chunks` (the contexts of ctxmap.cu do not serve it).
 int lex_enumerative_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode,
                            uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens,
-                           uint64_t *consumed, cudaStream_t stream, bool guard);
+                           uint64_t *consumed, cudaStream_t stream, bool guard, bool chunks);
 // The guard's prepass (liveness.cu): the liveness automaton's state at every
 // offset 0..n of the input into d_out[n + 1] (nullptr: the context's scratch);
 // *live receives the array, *member the automaton's member bitsets on the

@@ -98,6 +98,32 @@ def test_backtracking_is_not_far(lg):
                         off) == {"rows": 1, route: 1}
 
 
+@pytest.mark.parametrize("length,route", [(3000, {"rows": 1}), (9000, {"rows": 1, "contexts": 1}),
+                                          (17_000, {"rows": 1, "contexts": 1}), (60_000, {"rows": 1, "contexts": 1}),
+                                          (80_000, {"rows": 1, "contexts": 1, "chunks": 1})])
+def test_long_lines(lg, length, route):
+    # C-like text synchronizes at newlines, and a comment's bytes have too many contexts for a start
+    base = corpus.generate("clike", 200_000, seed=79)
+    at = int(np.flatnonzero(base[:100_000] == 10)[-1]) + 1
+    line = np.frombuffer(b"//" + b"c" * length + b"\n", np.uint8)
+    w = np.concatenate([base[:at], line, base[at:]])
+    for off in (0, 7):
+        ctx = lg.lx_ctx_create()
+        assert call(lg, ctx, "clike", w, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l), off) == route
+
+
+def test_far_rows_that_backtrack(lg):
+    # a long line and, in another tile's reach, tokens that backtrack across slices: neither the rows nor the
+    # contexts serve it, the warp-tile kernel does
+    base = corpus.generate("clike", 200_000, seed=80)
+    at = int(np.flatnonzero(base[:100_000] == 10)[-1]) + 1
+    w = np.concatenate([base[:at], np.frombuffer(b"//" + b"c" * 9000 + b"\n", np.uint8), base[at:],
+                        np.frombuffer(b"\n" + b"int a = 1en ; int b = 0;\n" * 4000, np.uint8)])
+    ctx = lg.lx_ctx_create()
+    got = call(lg, ctx, "clike", w, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l))
+    assert got in ({"rows": 1, "contexts": 1, "warps": 1}, {"rows": 1, "warps": 1})   # (which tile is met first)
+
+
 def test_kernel_setting(lg):
     for kernel, route in ((lg.LX_KERNEL_TILE, "tiles"), (lg.LX_KERNEL_WARP, "warps")):
         ctx = lg.lx_ctx_create()
@@ -160,6 +186,23 @@ def test_enumerative(lg, n, mode):
         assert call(lg, ctx, "clike_block", w, mode, enum, off) == {"contexts": 1}
         # the chunks
         assert call(lg, ctx, "clike_block", after_text("clike_block", n), mode, enum, off) == {"contexts": 1, "chunks": 1}
+
+
+@pytest.mark.parametrize("tiles", [1, 3, 5, 9, 14])
+def test_counts_across_tiles_without_a_start(lg, tiles):
+    # bytes with too many contexts for a start in whole tiles: the rounds count as the chunks' do (unaligned)
+    ts, ctx = tset(lg, "clike_block"), lg.lx_ctx_create()
+    base = corpus.generate("clike_block", 60_000, seed=86)
+    at = int(np.flatnonzero(base[:30_000] == 10)[-1]) + 1
+    w = np.concatenate([base[:at], np.frombuffer(b"//" + b"c" * (tiles * CH + 100) + b"\n", np.uint8), base[at:]])
+    stats = []
+    for off, route in ((0, {"contexts": 1}), (5, {"chunks": 1})):
+        def spec(ts, d, k, l):
+            rc, nt, con, st = lg.lx_lex_speculative(ctx, ts, None, d, 0, k, l)
+            stats.append(st)
+            return rc, nt, con
+        assert call(lg, ctx, "clike_block", w, 0, spec, off, ts=ts) == route
+    assert stats[0] == stats[1]
 
 
 @pytest.mark.parametrize("with_model", [False, True])
