@@ -1346,10 +1346,11 @@ static bool warp_has_cuts(const lx_tokenset *ts, int mode)
     return mode_has_cuts(ts, mode) || (ts->walk[mode].status == LX_OK && ts->walk[mode].n_ctx > 0);
 }
 
-// Launch the tile kernel and read back its result record.
+// Lex on the device by the plan below.  `refused`: what the entry-row kernels
+// returned for this input already (LX_ROWS or LX_FAR).
 static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode,
                       uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens,
-                      uint64_t *consumed, cudaStream_t st, const LaunchCfg *force = nullptr)
+                      uint64_t *consumed, cudaStream_t st, const LaunchCfg *force = nullptr, int refused = LX_OK)
 {
     // Hybrid plan (Section 9): certified cuts where certified bytes occur;
     // where the mode certifies no byte, or certified bytes turn out too far
@@ -1360,7 +1361,9 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;
     bool no_contexts = false;   // the contexts' rows do not fit either
     if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
-        int rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+        int rc = refused;
+        if (rc == LX_OK)
+            rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
         if (rc == LX_FAR) {   // contexts are enumerated instead, of chunks where their starts are far apart as well
             rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st, nullptr,
                                      nullptr);
@@ -1548,8 +1551,8 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
     if (rc == LX_OK) rc = grow(&c->d_out, &c->d_out_bytes, capacity ? capacity * 6 + 16 : 16);
     if (rc != LX_OK) return rc;
     cudaStream_t st0 = static_cast<cudaStream_t>(stream);
-    // the whole input in, one device-side call, the tokens out
-    auto whole = [&](bool enumerate) -> int {
+    // the whole input in, one device-side call, the tokens out (refused: as lex_device)
+    auto whole = [&](bool enumerate, int refused = LX_OK) -> int {
         int r = grow(&c->d_in, &c->d_in_bytes, n);
         if (r == LX_OK) r = grow(&c->d_out, &c->d_out_bytes, capacity ? capacity * 6 + 16 : 16);
         if (r == LX_OK) r = cuda_err(cudaMemcpyAsync(c->d_in, h_in, n, cudaMemcpyHostToDevice, st0));
@@ -1559,7 +1562,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         const uint8_t *di = static_cast<const uint8_t *>(c->d_in);
         uint64_t nt = 0, con = 0;
         r = enumerate ? lx_lex_enumerative(c, ts, di, n, mode, dk, dl, capacity, &nt, &con, stream)
-                      : lex_device(c, ts, di, n, mode, dk, dl, capacity, &nt, &con, st0);
+                      : lex_device(c, ts, di, n, mode, dk, dl, capacity, &nt, &con, st0, nullptr, refused);
         if (r != LX_OK && r != LX_E_CAPACITY) return r;
         const uint64_t m = std::min(nt, capacity);
         int r2 = LX_OK;
@@ -1580,23 +1583,30 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
 
     // from entry rows (rows.cu) where the set has a synchronizing byte
     const bool rows = can_enumerate && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode);
-    const std::vector<uint64_t> b = host_pieces(h, h_in, n, rows ? ROWS_PIECE : HOST_PIECE);
-    const uint32_t K = (uint32_t)b.size() - 1;
+    std::vector<uint64_t> b = host_pieces(h, h_in, n, rows ? ROWS_PIECE : HOST_PIECE);
+    uint32_t K = (uint32_t)b.size() - 1;
     if (!c->s_in && (cudaStreamCreateWithFlags(&c->s_in, cudaStreamNonBlocking) != cudaSuccess ||
                      cudaStreamCreateWithFlags(&c->s_out, cudaStreamNonBlocking) != cudaSuccess))
         return LX_E_CUDA;
-    while (c->ev_in.size() < K) {
-        cudaEvent_t e1 = nullptr, e2 = nullptr;
-        if (cudaEventCreateWithFlags(&e1, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&e2, cudaEventDisableTiming) != cudaSuccess)
-            return LX_E_CUDA;
-        c->ev_in.push_back(e1);
-        c->ev_lex.push_back(e2);
-    }
+    auto events = [&](uint32_t pieces) -> bool {
+        while (c->ev_in.size() < pieces) {
+            cudaEvent_t e1 = nullptr, e2 = nullptr;
+            if (cudaEventCreateWithFlags(&e1, cudaEventDisableTiming) != cudaSuccess ||
+                cudaEventCreateWithFlags(&e2, cudaEventDisableTiming) != cudaSuccess)
+                return false;
+            c->ev_in.push_back(e1);
+            c->ev_lex.push_back(e2);
+        }
+        return true;
+    };
+    if (!events(K)) return LX_E_CUDA;
     if (rows) {
         rc = lex_rows_host(c, ts, h_in, n, mode, h_kinds, h_lens, capacity, b.data(), K, n_tokens, consumed, st);
-        if (rc != LX_ROWS && rc != LX_FAR) return rc;
-        return whole(false);
+        if (rc == LX_FAR) return whole(false, rc);
+        if (rc != LX_ROWS) return rc;
+        b = host_pieces(h, h_in, n, HOST_PIECE);   // the warp-tile kernel's
+        K = (uint32_t)b.size() - 1;
+        if (!events(K)) return LX_E_CUDA;
     }
     if (warp) {
         rc = lex_warp_host(c, ts, h_in, n, mode, h_kinds, h_lens, capacity, b.data(), K, n_tokens, consumed, st,
@@ -1604,7 +1614,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         if (rc != LX_SPARSE && rc != LX_LOOKAHEAD) return rc;
         // certified bytes too far apart, or failed lookahead, in some piece:
         // the whole input through lx_lex's plan
-        return whole(false);
+        return whole(false, rows ? LX_ROWS : LX_OK);
     }
     uint32_t *d_lens = static_cast<uint32_t *>(c->d_out);
     uint16_t *d_kinds = reinterpret_cast<uint16_t *>(d_lens + capacity);

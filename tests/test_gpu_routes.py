@@ -158,6 +158,31 @@ def test_host(lg):
         assert ran(lg, ctx, before) == {"rows": 1}
 
 
+def handed_on(n, what):
+    if what == "far":
+        w = corpus.generate("clike", n, seed=87)
+        at = int(np.flatnonzero(w[:n // 2] == 10)[-1]) + 1
+        return "clike", 2, np.concatenate([w[:at], np.frombuffer(b"//" + b"c" * 9000 + b"\n", np.uint8), w[at:]])
+    unit = b"ab;" * 5 + b"a" * 40 + b";"
+    return "lookahead", 0, np.frombuffer(unit * (n // len(unit)), np.uint8)
+
+
+@pytest.mark.parametrize("n", [20_000, 25 << 20])
+@pytest.mark.parametrize("what,route", [("far", {"rows": 1, "contexts": 1}), ("backtracks", {"rows": 1, "warps": 1})])
+def test_host_handed_on(lg, n, what, route):
+    # one attempt on the rows, then what serves the input (refused once, the input was tried once more there)
+    import torch
+    name, mode, w = handed_on(n, what)
+    ctx, ts = lg.lx_ctx_create(), tset(lg, name)
+    k, l = torch.zeros(w.size, dtype=torch.int16), torch.zeros(w.size, dtype=torch.int32)
+    before = lg.lx_ctx_debug_counts(ctx)
+    rc, nt, con = lg.lx_lex_host(ctx, ts, torch.from_numpy(w.copy()), mode, k, l)
+    ek, el, econ = expected(name, w, mode)
+    assert rc == 0 and (nt, con) == (ek.size, econ)
+    assert np.array_equal(l[:nt].numpy().astype(np.int64), el) and np.array_equal(k[:nt].numpy().astype(np.int64), ek)
+    assert ran(lg, ctx, before) == route
+
+
 def test_batch(lg):
     import torch
     names = ["json", "clike"]
