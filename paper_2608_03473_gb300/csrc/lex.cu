@@ -1102,6 +1102,7 @@ extern "C" void lx_ctx_free(lx_ctx *c)
     cudaDeviceSynchronize();
     if (c->scratch) cudaFree(c->scratch);
     if (c->b_exec) cudaGraphExecDestroy(c->b_exec);
+    if (c->r_exec) cudaGraphExecDestroy(c->r_exec);
     if (c->b_stream) cudaStreamDestroy(c->b_stream);
     if (c->b_dev) cudaFree(c->b_dev);
     if (c->e_dev) cudaFree(c->e_dev);

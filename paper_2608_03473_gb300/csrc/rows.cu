@@ -1280,10 +1280,10 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
                                   (uint64_t)(uintptr_t)hs, c->timeout_ns, grid, nwarps, (uint64_t)nw,
                                   (uint64_t)(uintptr_t)c->wb_dev};
     gkey.insert(gkey.end(), sets_key.begin(), sets_key.end());
-    if (moved || gkey != c->b_key || !c->b_exec) {
-        if (c->b_exec) cudaGraphExecDestroy(c->b_exec);
-        c->b_exec = nullptr;
-        c->b_key.clear();
+    if (moved || gkey != c->r_key || !c->r_exec) {
+        if (c->r_exec) cudaGraphExecDestroy(c->r_exec);
+        c->r_exec = nullptr;
+        c->r_key.clear();
         if (!c->b_stream && cudaStreamCreateWithFlags(&c->b_stream, cudaStreamNonBlocking) != cudaSuccess)
             return LX_E_CUDA;
         cudaStream_t cs = c->b_stream;
@@ -1330,14 +1330,14 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         rows_kernel(FORM_CLASS, nw, false, true)<<<grid, 32 * nwarps, smem, cs>>>(P);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(cs, &graph);
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->b_exec, graph, 0);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->r_exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
-            c->b_exec = nullptr;
+            c->r_exec = nullptr;
             cudaGetLastError();
             return LX_E_CUDA;
         }
-        c->b_key = gkey;
+        c->r_key = gkey;
         c->counts.graphs++;
     }
     c->counts.rows++;
@@ -1345,7 +1345,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
     *seq = 0;
     std::atomic_thread_fence(std::memory_order_seq_cst);
     if (c->timing) cudaEventRecord(c->ev[0], st);
-    rc = cuda_err(cudaGraphLaunch(c->b_exec, st));
+    rc = cuda_err(cudaGraphLaunch(c->r_exec, st));
     if (c->timing) cudaEventRecord(c->ev[1], st);
     if (rc == LX_OK) rc = wait_record(st, nullptr, [&] { return *seq == 1; });
     if (rc != LX_OK) return rc;

@@ -46,6 +46,10 @@ struct lx_ctx {
     cudaStream_t b_stream = nullptr;
     cudaGraphExec_t b_exec = nullptr;
     std::vector<uint64_t> b_key;
+    // the same for batches from entry rows (rows.cu): a batch that they refuse
+    // keeps both
+    cudaGraphExec_t r_exec = nullptr;
+    std::vector<uint64_t> r_key;
     // lx_lex_enumerative: device scratch
     void *e_dev = nullptr;
     size_t e_dev_bytes = 0;

@@ -266,6 +266,38 @@ def test_open_token(lg, n, cut):
                 assert call(lg, ctx, name, v, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l), off) == {"rows": 1}
 
 
+def test_batches_handed_on_keep_their_graphs(lg):
+    # a batch that the rows refuse (tokens that backtrack across slices) has two graphs, each captured once:
+    # alone again and again, and in turn with one that they take
+    import torch
+    names = ["json", "clike"]
+    ctx, sets = lg.lx_ctx_create(), [tset(lg, n) for n in names]
+    json = corpus.generate("json", 30_000, seed=88)
+    some = np.frombuffer(b"int a = 1en ; int b = 0;\n" * 700, np.uint8)
+    good = np.frombuffer(b"int a = 1e1 ; int b = 0;\n" * 700, np.uint8)
+    k = torch.zeros(80_000, dtype=torch.int16, device="cuda")
+    l = torch.zeros(80_000, dtype=torch.int32, device="cuda")
+
+    def batch(second):
+        d = [torch.from_numpy(w.copy()).cuda() for w in (json, second, json)]
+        before = lg.lx_ctx_debug_counts(ctx)
+        rc, total, res = lg.lx_lex_batch(ctx, sets, list(zip(d, (0, 1, 0))), 2, k, l)
+        assert rc == 0
+        for (nm, w), (off, nt, con) in zip((("json", json), ("clike", second), ("json", json)), res):
+            ek, el, econ = expected(nm, w, 2)
+            assert (nt, con) == (ek.size, econ)
+            assert np.array_equal(l[off:off + nt].cpu().numpy().astype(np.int64), el)
+        return ran(lg, ctx, before)
+
+    first = batch(some)
+    assert first["rows"] == 1 and first["warps"] == 1 and first["graphs"] <= 3   # (a buffer that grows moves both)
+    batch(some)
+    for _ in range(3):
+        assert "graphs" not in batch(some)
+        assert batch(good) == {"rows": 1}
+        assert batch(some) == {"rows": 1, "warps": 1}
+
+
 def test_open_token_in_a_batch(lg):
     import torch
     names = ["clike", "json"]
