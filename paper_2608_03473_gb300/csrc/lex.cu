@@ -1347,6 +1347,33 @@ static bool warp_has_cuts(const lx_tokenset *ts, int mode)
     return mode_has_cuts(ts, mode) || (ts->walk[mode].status == LX_OK && ts->walk[mode].n_ctx > 0);
 }
 
+// The refusals of a set and mode (not kept for sets that had none).
+static Refusals *refusals_for(lx_ctx *c, const lx_tokenset *ts, int mode)
+{
+    for (auto &kv : c->refusals)
+        if (kv.first == ts->serial * 8 + (uint64_t)mode) return &kv.second;
+    return nullptr;
+}
+
+static bool rows_skipped(lx_ctx *c, const lx_tokenset *ts, int mode)
+{
+    Refusals *r = refusals_for(c, ts, mode);
+    return r && r->skips();
+}
+
+// After an attempt: its status (LX_FAR is no refusal: the contexts serve it best).
+static void note_rows(lx_ctx *c, const lx_tokenset *ts, int mode, int rc)
+{
+    if (rc != LX_ROWS && rc != LX_OK && rc != LX_E_CAPACITY) return;
+    Refusals *r = refusals_for(c, ts, mode);
+    if (!r && rc != LX_ROWS) return;
+    if (!r) {
+        c->refusals.emplace_back(ts->serial * 8 + (uint64_t)mode, Refusals());
+        r = &c->refusals.back().second;
+    }
+    r->note(rc == LX_ROWS);
+}
+
 // Lex on the device by the plan below.  `refused`: what the entry-row kernels
 // returned for this input already (LX_ROWS or LX_FAR).
 static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode,
@@ -1363,8 +1390,12 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     bool no_contexts = false;   // the contexts' rows do not fit either
     if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
         int rc = refused;
-        if (rc == LX_OK)
+        if (rc == LX_OK && rows_skipped(c, ts, mode)) {
+            rc = LX_ROWS;
+        } else if (rc == LX_OK) {
             rc = lex_rows_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st);
+            note_rows(c, ts, mode, rc);
+        }
         if (rc == LX_FAR) {   // contexts are enumerated instead, of chunks where their starts are far apart as well
             rc = lex_contexts_device(c, ts, d_in, n, mode, d_kinds, d_lens, capacity, n_tokens, consumed, st, nullptr,
                                      nullptr);
@@ -1583,7 +1614,8 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         return whole(true);   // no certified byte: the enumerative path
 
     // from entry rows (rows.cu) where the set has a synchronizing byte
-    const bool rows = can_enumerate && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode);
+    const bool rows_ok = can_enumerate && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode);
+    const bool rows = rows_ok && !rows_skipped(c, ts, mode);
     std::vector<uint64_t> b = host_pieces(h, h_in, n, rows ? ROWS_PIECE : HOST_PIECE);
     uint32_t K = (uint32_t)b.size() - 1;
     if (!c->s_in && (cudaStreamCreateWithFlags(&c->s_in, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1603,6 +1635,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
     if (!events(K)) return LX_E_CUDA;
     if (rows) {
         rc = lex_rows_host(c, ts, h_in, n, mode, h_kinds, h_lens, capacity, b.data(), K, n_tokens, consumed, st);
+        note_rows(c, ts, mode, rc);
         if (rc == LX_FAR) return whole(false, rc);
         if (rc != LX_ROWS) return rc;
         b = host_pieces(h, h_in, n, HOST_PIECE);   // the warp-tile kernel's
@@ -1615,7 +1648,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         if (rc != LX_SPARSE && rc != LX_LOOKAHEAD) return rc;
         // certified bytes too far apart, or failed lookahead, in some piece:
         // the whole input through lx_lex's plan
-        return whole(false, rows ? LX_ROWS : LX_OK);
+        return whole(false, rows_ok ? LX_ROWS : LX_OK);
     }
     uint32_t *d_lens = static_cast<uint32_t *>(c->d_out);
     uint16_t *d_kinds = reinterpret_cast<uint16_t *>(d_lens + capacity);

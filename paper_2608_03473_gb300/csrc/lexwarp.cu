@@ -1547,6 +1547,7 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
         r2 = cuda_err(cudaMemcpy(c->wb_dev, cb.blob.data(), cb.blob.size(), cudaMemcpyHostToDevice));
         if (r2 != LX_OK) return r2;
         c->wb_key = key;
+        c->wb_refusals = Refusals();
         c->wb_blob_bytes = cb.bytes;
         c->wb_sync = cb.sync;
         c->wb_rows = cb.rows_bytes;
@@ -1555,8 +1556,11 @@ int lex_batch_warp(lx_ctx *c, const lx_tokenset *const *sets, uint32_t n_sets, c
     }
 
     // from entry rows (rows.cu) where every set synchronizes
-    if (c->kernel == LX_KERNEL_AUTO && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && c->wb_sync) {
+    if (c->kernel == LX_KERNEL_AUTO && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && c->wb_sync &&
+        !c->wb_refusals.skips()) {
         const int rc = lex_batch_rows(c, key, docs, n_docs, mode, d_kinds, d_lens, capacity, results, n_total, st);
+        if (rc == LX_OK || rc == LX_E_CAPACITY || rc == LX_ROWS || rc == LX_FAR)
+            c->wb_refusals.note(rc == LX_ROWS || rc == LX_FAR);
         if (rc != LX_ROWS && rc != LX_FAR) return rc;
         for (uint32_t i = 0; i < n_docs; i++) results[i] = lx_doc_result{0, 0, 0};
         *n_total = 0;

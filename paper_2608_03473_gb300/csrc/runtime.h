@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <utility>
 #include <vector>
@@ -25,6 +26,29 @@ struct lx_tuned {
 
 // Bytes of the pinned buffer for a kernel's launch record (lx_ctx::h_res).
 constexpr size_t LAUNCH_RECORD_BYTES = 64;
+
+// Inputs of one kind that the entry-row kernels refuse one after the other
+// (tokens that backtrack across slices) are not tried each time: a refused
+// attempt costs up to a pass (64 MiB of C-like text with a line of them 1.55
+// ms a call, 1.35 without).  After the second refusal in a row one call goes
+// without, then 3, 7 and at most 15 between attempts; one that is taken ends
+// it, so that inputs refused now and then are all tried.
+struct Refusals {
+    uint32_t streak = 0, skip = 0;
+    bool skips()   // whether this call goes without an attempt
+    {
+        if (skip) {
+            skip--;
+            return true;
+        }
+        return false;
+    }
+    void note(bool refused)
+    {
+        streak = refused ? std::min(streak + 1, 5u) : 0u;
+        skip = streak ? (1u << (streak - 1)) - 1 : 0u;
+    }
+};
 
 struct lx_ctx {
     int device = 0;
@@ -84,6 +108,9 @@ struct lx_ctx {
     // the warp-tile kernel's per-warp spill slots (kept tokens of a tile beyond its shared stage)
     void *w_spill = nullptr;
     size_t w_spill_bytes = 0;
+    // refusals per (token set serial * 8 + mode), and of the batches of wb_key
+    std::vector<std::pair<uint64_t, Refusals>> refusals;
+    Refusals wb_refusals;
     // rows.cu: the scratch of small launches (its first part is zero between
     // them while small_clean), and the last launch's sequence number
     void *small = nullptr;

@@ -293,9 +293,16 @@ def test_batches_handed_on_keep_their_graphs(lg):
     assert first["rows"] == 1 and first["warps"] == 1 and first["graphs"] <= 3   # (a buffer that grows moves both)
     batch(some)
     for _ in range(3):
-        assert "graphs" not in batch(some)
+        while "rows" not in batch(some):   # (refused repeatedly, not every call tries)
+            pass
+        while "rows" not in batch(good):
+            pass
         assert batch(good) == {"rows": 1}
         assert batch(some) == {"rows": 1, "warps": 1}
+        assert batch(good) == {"rows": 1}
+        assert batch(some) == {"rows": 1, "warps": 1}
+        assert batch(some) == {"rows": 1, "warps": 1}
+        assert batch(some) == {"warps": 1}
 
 
 def test_open_token_in_a_batch(lg):
@@ -332,3 +339,35 @@ def test_open_token_from_contexts(lg, n, cut):
             return rc, nt, con
         assert call(lg, ctx, "clike_block", w, 2, spec, off, ts=ts) == route
     assert stats[0] == stats[1]   # the counts of the rounds are the chunks'
+
+
+@pytest.mark.parametrize("kind", ["device", "host", "batch"])
+def test_repeated_refusals(lg, kind):
+    # 1, 3, 7, 15, 15 calls without an attempt after the second refusal in a row and those that follow; a
+    # taken input ends it
+    import torch
+    some = np.frombuffer(b"int a = 1en ; int b = 0;\n" * 300, np.uint8)
+    good = np.frombuffer(b"int a = 1e1 ; int b = 0;\n" * 300, np.uint8)
+    ctx, ts = lg.lx_ctx_create(), tset(lg, "clike")
+    dev = "cpu" if kind == "host" else "cuda"
+    k = torch.zeros(some.size, dtype=torch.int16, device=dev)
+    l = torch.zeros(some.size, dtype=torch.int32, device=dev)
+    want = {id(w): expected("clike", w, 2) for w in (some, good)}
+    data = {id(w): torch.from_numpy(w.copy()).to(dev) for w in (some, good)}
+
+    def tried(w):
+        before = lg.lx_ctx_debug_counts(ctx)
+        if kind == "batch":
+            rc, _, ((off, nt, con),) = lg.lx_lex_batch(ctx, [ts], [(data[id(w)], 0)], 2, k, l)
+        else:
+            rc, nt, con = (lg.lx_lex if kind == "device" else lg.lx_lex_host)(ctx, ts, data[id(w)], 2, k, l)
+        ek, el, econ = want[id(w)]
+        assert rc == 0 and (nt, con) == (ek.size, econ) and np.array_equal(l[:nt].cpu().numpy().astype(np.int64), el)
+        route = ran(lg, ctx, before)
+        assert ("warps" in route) == (w is some or "rows" not in route)
+        return route.get("rows", 0)
+
+    calls = [tried(some) for _ in range(2 + 1 + 1 + 3 + 1 + 7 + 1 + 15 + 1 + 15 + 1)]
+    assert calls == [1, 1, 0, 1, 0, 0, 0, 1] + [0] * 7 + [1] + [0] * 15 + [1] + [0] * 15 + [1]
+    assert [tried(good) for _ in range(17)] == [0] * 15 + [1, 1]
+    assert [tried(w) for w in (some, good, some, good, some, some, good, good)] == [1, 1, 1, 1, 1, 1, 0, 1]
