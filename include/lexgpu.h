@@ -421,9 +421,11 @@ int lx_lex_host(lx_ctx *ctx, const lx_tokenset *ts, const uint8_t *h_in, uint64_
  * with the largest and the smallest CTA count, on `d_sample` (a device buffer representative
  * of the inputs to come, n bytes; outputs go to d_kinds / d_lens), then the
  * warp-tile kernel (where it applies to the sample) at 4, 8, 12, 16 and 20
- * warps per CTA; checks that all give the same result, keeps the fastest
- * tile configuration and, for lx_lex on LX_KERNEL_AUTO, the faster kernel
- * with its warps per CTA (lx_ctx_set_warps overrides the latter; setting a
+ * warps per CTA and the entry-row kernels (where they apply and do not refuse
+ * the sample); checks that all give the same result, keeps the fastest tile
+ * configuration, the warp-tile kernel's warps (lx_ctx_set_warps overrides
+ * them) and, for lx_lex and lx_lex_host on LX_KERNEL_AUTO, whether the
+ * entry-row kernels come first or one of the others was faster (setting a
  * configuration by hand clears the choice).  Synchronizes `stream`.
  * The tile configuration also applies to lx_lex_batch groups of that token set.
  */

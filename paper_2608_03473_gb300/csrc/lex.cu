@@ -1347,6 +1347,15 @@ static bool warp_has_cuts(const lx_tokenset *ts, int mode)
     return mode_has_cuts(ts, mode) || (ts->walk[mode].status == LX_OK && ts->walk[mode].n_ctx > 0);
 }
 
+// Whether the entry-row kernels come first on LX_KERNEL_AUTO: where the set has
+// them, no geometry of the warp-tile kernel is asked for, and lx_autotune did
+// not find another kernel faster.
+static bool rows_chosen(const lx_ctx *c, const lx_tokenset *ts, int mode)
+{
+    const lx_tuned *t = tuned_for(c, ts, mode);
+    return c->warp_geometry == LX_WARP_GEOMETRY_AUTO && (!t || t->kernel == LX_KERNEL_AUTO) && rows_path_ok(ts, mode);
+}
+
 // The refusals of a set and mode (not kept for sets that had none).
 static Refusals *refusals_for(lx_ctx *c, const lx_tokenset *ts, int mode)
 {
@@ -1388,7 +1397,7 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
     const lx_tuned *tu = tuned_for(c, ts, mode);
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;
     bool no_contexts = false;   // the contexts' rows do not fit either
-    if (can_enumerate && !tuned_tile && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode)) {
+    if (can_enumerate && rows_chosen(c, ts, mode)) {
         int rc = refused;
         if (rc == LX_OK && rows_skipped(c, ts, mode)) {
             rc = LX_ROWS;
@@ -1614,7 +1623,7 @@ extern "C" int lx_lex_host(lx_ctx *c, const lx_tokenset *ts, const uint8_t *h_in
         return whole(true);   // no certified byte: the enumerative path
 
     // from entry rows (rows.cu) where the set has a synchronizing byte
-    const bool rows_ok = can_enumerate && c->warp_geometry == LX_WARP_GEOMETRY_AUTO && rows_path_ok(ts, mode);
+    const bool rows_ok = can_enumerate && rows_chosen(c, ts, mode);
     const bool rows = rows_ok && !rows_skipped(c, ts, mode);
     std::vector<uint64_t> b = host_pieces(h, h_in, n, rows ? ROWS_PIECE : HOST_PIECE);
     uint32_t K = (uint32_t)b.size() - 1;
@@ -2153,6 +2162,27 @@ extern "C" int lx_autotune(lx_ctx *c, const lx_tokenset *ts, int mode, const uin
         }
     }
     c->warps = saved_warps;
+    // the entry-row kernels, when they apply and do not refuse the sample
+    float best_r = 1e30f;
+    if (rc == LX_OK && ts->scan.status == LX_OK && rows_path_ok(ts, mode)) {
+        uint64_t nt = 0, con = 0;
+        float total = 0.0f;
+        int r = LX_OK;
+        for (int rep = 0; rep < 4 && r == LX_OK; rep++) {
+            cudaEventRecord(e0, st);
+            r = lex_rows_device(c, ts, d_sample, n, mode, d_kinds, d_lens, capacity, &nt, &con, st);
+            cudaEventRecord(e1, st);
+            if (r == LX_E_CAPACITY) r = LX_OK;
+            if (r != LX_OK) break;
+            cudaEventSynchronize(e1);
+            float ms = 0.0f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (rep) total += ms;
+        }
+        if (r == LX_OK && (nt != ref_tokens || con != ref_con)) r = LX_E_CUDA;
+        if (r == LX_OK) best_r = total / 3;
+        else if (r != LX_ROWS && r != LX_FAR) rc = r;
+    }
     c->timing = timing;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -2163,6 +2193,10 @@ extern "C" int lx_autotune(lx_ctx *c, const lx_tokenset *ts, int mode, const uin
             t.kernel = best_nw && best_w < best ? LX_KERNEL_WARP : LX_KERNEL_TILE;
             t.warps = best_nw;
             if (t.kernel == LX_KERNEL_WARP) t.ms = best_w;
+            if (best_r <= t.ms) {   // (what they refuse later takes the plan without a choice)
+                t.kernel = LX_KERNEL_AUTO;
+                t.ms = best_r;
+            }
         }
     return LX_OK;
 }

@@ -870,7 +870,7 @@ int allow_smem(lx_ctx *c, int form, int nw, bool find, bool batch = false)
 // The slice length (32 nw bytes) for `tiles_of(nw)` tiles beside `fixed` bytes
 // of tables, among 1 .. most and multiples of `step` bytes; 0: none fits.
 template <class F>
-int choose_nw(const lx_ctx *c, int mode, uint32_t fixed, uint32_t want, int most, uint32_t step, F tiles_of)
+int choose_nw(const lx_ctx *c, int mode, uint32_t fixed, int most, uint32_t step, F tiles_of)
 {
     double best = 0;
     int nw = 0;
@@ -878,8 +878,7 @@ int choose_nw(const lx_ctx *c, int mode, uint32_t fixed, uint32_t want, int most
         const uint32_t area = warp_area(k, stage_for(k, mode));
         if (fixed + area > SMEM_BUDGET) break;
         if (32 * k % step != 0) continue;
-        uint32_t warps = std::min<uint32_t>(USEFUL_WARPS, (SMEM_BUDGET - fixed) / area);
-        if (want) warps = std::min(warps, want);
+        const uint32_t warps = std::min<uint32_t>(USEFUL_WARPS, (SMEM_BUDGET - fixed) / area);
         const uint64_t all = (uint64_t)warps * c->num_sms;
         const double cost = ((double)tiles_of(k) / (double)all + 0.5) * (TILE_FIXED + TILE_STEP * k);
         if (!nw || cost < best) {
@@ -895,13 +894,13 @@ int choose_nw(const lx_ctx *c, int mode, uint32_t fixed, uint32_t want, int most
 int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGiven *given)
 {
     const WalkTable &w = ts->walk[mode];
-    const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16, want = warps_setting(c, ts, mode);
+    const uint32_t fixed = 512 + (uint32_t)w.blob.size() + 16;
     const uint64_t n = L.P.n;
     L.fused = !given && n <= FUSED_MAX;
     // a small launch takes one tile of 1 KiB per SM, or tiles of 2 KiB (1 MiB of
     // arith tokens 33 us in the former, 30 in the latter)
     const int nw = L.fused ? (n <= 1024ull * c->num_sms ? 1 : 2)
-                           : choose_nw(c, mode, fixed, want, 8, given ? given->step : 1,
+                           : choose_nw(c, mode, fixed, 8, given ? given->step : 1,
                                        [&](int k) { return (n + 1024 * k - 1) / (1024 * k); });
     if (L.fused && fixed + warp_area(nw, stage_for(nw, mode)) > SMEM_BUDGET) return LX_E_TOOBIG;
     if (!nw) return LX_E_TOOBIG;
@@ -913,8 +912,7 @@ int shape(lx_ctx *c, const lx_tokenset *ts, int mode, RLaunch &L, const RowsGive
     L.P.n_tiles = (uint32_t)tiles;
     L.P.stage = stage_for(nw, mode);
     const uint32_t area = warp_area(nw, L.P.stage);
-    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
-    if (want) warps = std::min(warps, want);
+    const uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
     // few tiles: one CTA on every SM, no more warps than its share (sixteen stage the table)
     L.nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(16, (tiles + c->num_sms - 1) / c->num_sms));
     L.smem = fixed + L.nwarps * area;
@@ -1234,7 +1232,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         }
     if (!D) return LX_OK;
     // half a tile of every document is empty on average
-    const int nw = choose_nw(c, mode, fixed, c->warps, 8, 1, [&](int k) { return bytes / (1024 * k) + (D + 1) / 2; });
+    const int nw = choose_nw(c, mode, fixed, 8, 1, [&](int k) { return bytes / (1024 * k) + (D + 1) / 2; });
     if (!nw) return LX_ROWS;
     const uint32_t tile = 1024 * nw;
     std::vector<WDoc> hd;
@@ -1250,8 +1248,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
         if (TT > 0xFFFFFFF0ull) return LX_E_INVAL;
     }
     const uint32_t area = warp_area(nw, stage_for(nw, mode));
-    uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
-    if (c->warps) warps = std::min(warps, c->warps);
+    const uint32_t warps = std::min<uint32_t>(MAX_WARPS, (SMEM_BUDGET - fixed) / area);
     const uint32_t n_tiles = (uint32_t)TT;
     const uint32_t nwarps = (uint32_t)std::min<uint64_t>(warps, std::max<uint64_t>(16, (TT + c->num_sms - 1) / c->num_sms));
     const uint32_t smem = fixed + nwarps * area, grid = (uint32_t)std::min<uint64_t>((uint64_t)c->num_sms, TT);

@@ -20,7 +20,9 @@ struct lx_tuned {
     int mode;
     uint32_t ks, ctas, cls;   // cls: class-indexed table
     float ms;   // measured by lx_autotune (0 when set by hand)
-    int kernel = 0;           // LX_KERNEL_TILE or _WARP when lx_autotune chose one (0: not chosen)
+    // what lx_autotune found fastest: LX_KERNEL_TILE or _WARP; LX_KERNEL_AUTO
+    // where the entry-row kernels were, or nothing was chosen
+    int kernel = 0;
     uint32_t warps = 0;       // warps per CTA it chose for the warp-tile kernel (0: as many as fit)
 };
 
@@ -218,7 +220,8 @@ bool contexts_path_ok(const lx_tokenset *ts, int mode);
 int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t n, int mode, uint16_t *d_kinds,
                         uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens, uint64_t *consumed, cudaStream_t st,
                         lx_model *model, lx_spec_stats *spec);
-// Warps per CTA for the warp-tile kernel on (ts, mode): the context's
+// Warps per CTA of the warp-tile kernel (not of the entry-row kernels, whose
+// shared memory differs: they take what fits) on (ts, mode): the context's
 // setting, else lx_autotune's choice, else 0 (as many as fit).
 uint32_t warps_setting(const lx_ctx *c, const lx_tokenset *ts, int mode);
 // lx_lex_async (lexwarp.cu): the warp-tile kernel and a status kernel that

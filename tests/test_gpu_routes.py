@@ -371,3 +371,28 @@ def test_repeated_refusals(lg, kind):
     assert calls == [1, 1, 0, 1, 0, 0, 0, 1] + [0] * 7 + [1] + [0] * 15 + [1] + [0] * 15 + [1]
     assert [tried(good) for _ in range(17)] == [0] * 15 + [1, 1]
     assert [tried(w) for w in (some, good, some, good, some, some, good, good)] == [1, 1, 1, 1, 1, 1, 0, 1]
+
+
+@pytest.mark.parametrize("off", [0, 5])
+def test_autotune_times_every_kernel(lg, off):
+    # large enough that the entry-row kernels win by far; a sample that they refuse switches them off
+    import torch
+    w = corpus.generate("clike", 24 << 20, seed=89)
+    refused = np.frombuffer(b"int a = 1en ; int b = 0;\n" * 20_000, np.uint8)
+    for sample, rows in ((w, True), (refused, False)):
+        ctx, ts = lg.lx_ctx_create(), tset(lg, "clike")
+        d = torch.zeros(sample.size + 16, dtype=torch.uint8, device="cuda")[off:off + sample.size]
+        d.copy_(torch.from_numpy(sample.copy()))
+        k = torch.zeros(sample.size, dtype=torch.int16, device="cuda")
+        l = torch.zeros(sample.size, dtype=torch.int32, device="cuda")
+        assert lg.lx_autotune(ctx, ts, 2, d, k, l) == 0
+        assert lg.lx_ctx_get_config(ctx, ts, 2)[3] > 0
+        small = w[:300_000]
+        route = call(lg, ctx, "clike", small, 2, lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, 2, k, l), off, ts=ts)
+        assert ("rows" in route) == rows and sum(route.values()) == 1
+        h = torch.from_numpy(small.copy())
+        before = lg.lx_ctx_debug_counts(ctx)
+        rc, nt, con = lg.lx_lex_host(ctx, ts, h, 2, torch.zeros(small.size, dtype=torch.int16),
+                                     torch.zeros(small.size, dtype=torch.int32))
+        assert rc == 0 and (nt, con) == (expected("clike", small, 2)[0].size, expected("clike", small, 2)[2])
+        assert ("rows" in ran(lg, ctx, before)) == rows   # the same choice
