@@ -61,7 +61,7 @@ struct lx_model {
     float *act = nullptr;
     size_t act_floats = 0;
     uint16_t *win = nullptr;
-    bool mg_ready = false;          // k_mlp_grad may use its shared memory
+    bool mg_ready = false;          // k_mlp_grad may use its shared memory, k_outer its clusters
     float *h_g = nullptr;           // pinned: the gradient and the loss on their way to the caller
     int device = -1;
 };
@@ -513,12 +513,33 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         if (ge[i] != 0.0f) atomicAdd(&gemb[i], ge[i]);
 }
 
-// Weight gradients: G[M x N] += A^T D over a slice of the batch, A [B][M], D
-// [B][N], and the column sums of D (the bias) from the first row of tiles.  64
-// x 64 tiles, 4 x 4 per thread; blockIdx.z: which of the two layers.
-constexpr uint32_t OT = 64, OK = 16, OSLICE = 64;
+// Weight gradients: G[M x N] = A^T D, A [B][M], D [B][N], and the column sums of
+// D (the bias) from the first row of tiles.  64 x 64 tiles, 4 x 4 per thread;
+// blockIdx.z: which of the two layers.  A cluster of CTAs shares a tile, each
+// one slice of the batch; their sums are added in the order of the slices,
+// each CTA its part of the tile from all of them, so that a gradient is the
+// same each time (adding them to G as they came was not).
+constexpr uint32_t OT = 64, OK = 16, OSLICE = 64, OCLUSTER = 16;
 
-__global__ void __launch_bounds__(256) k_outer(uint32_t B, const float *A0, const float *D0, uint32_t M0, uint32_t N0,
+// The address of this CTA's shared word `a` in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 cluster_ld(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const float *A0, const float *D0, uint32_t M0, uint32_t N0,
                                                float *G0, float *s0, const float *A1, const float *D1, uint32_t M1,
                                                uint32_t N1, float *G1, float *s1)
 {
@@ -527,10 +548,10 @@ __global__ void __launch_bounds__(256) k_outer(uint32_t B, const float *A0, cons
     float *G = one ? G1 : G0, *cs = one ? s1 : s0;
     const uint32_t M = one ? M1 : M0, N = one ? N1 : N0;
     const uint32_t nt = (N + OT - 1) / OT, m0 = (blockIdx.x / nt) * OT, n0 = (blockIdx.x % nt) * OT;
-    if (m0 >= M) return;
-    __shared__ __align__(16) float As[OK][OT], Ds[OK][OT];
+    if (m0 >= M) return;   // (the whole cluster)
+    __shared__ __align__(16) float As[OK][OT], Ds[OK][OT], part[OT * OT + OT];
     const uint32_t tid = threadIdx.x, tx = tid & 15u, ty = tid >> 4;
-    const uint32_t k0 = blockIdx.y * OSLICE, k1 = min(B, k0 + OSLICE);
+    const uint32_t k0 = min(B, blockIdx.y * slice), k1 = min(B, k0 + slice);
     float acc[4][4], sum = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; i++)
@@ -560,11 +581,26 @@ __global__ void __launch_bounds__(256) k_outer(uint32_t B, const float *A0, cons
     }
 #pragma unroll
     for (int i = 0; i < 4; i++)
+        *reinterpret_cast<float4 *>(&part[(4 * ty + i) * OT + 4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (tid < OT) part[OT * OT + tid] = sum;
+    cluster_sync();
+    const uint32_t S = gridDim.y, base = (uint32_t)__cvta_generic_to_shared(part);   // the cluster's CTAs: all slices
+    const uint32_t words = OT * OT + (m0 == 0 ? OT : 0);
+    for (uint32_t i = 4 * (blockIdx.y * 256 + tid); i < words; i += S * 1024) {
+        float4 x[OCLUSTER];   // all loads first
 #pragma unroll
-        for (int j = 0; j < 4; j++)
-            if (m0 + 4 * ty + i < M && n0 + 4 * tx + j < N)
-                atomicAdd(&G[(size_t)(m0 + 4 * ty + i) * N + n0 + 4 * tx + j], acc[i][j]);
-    if (m0 == 0 && tid < OT && n0 + tid < N) atomicAdd(&cs[n0 + tid], sum);
+        for (uint32_t q = 0; q < OCLUSTER; q++)
+            x[q] = q < S ? cluster_ld(cluster_addr(base + 4 * i, q)) : make_float4(0, 0, 0, 0);
+        float v[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (uint32_t q = 0; q < OCLUSTER; q++) v[0] += x[q].x, v[1] += x[q].y, v[2] += x[q].z, v[3] += x[q].w;
+        float *to = i < OT * OT ? G + (size_t)(m0 + i / OT) * N : cs;
+        if (i < OT * OT && m0 + i / OT >= M) continue;
+#pragma unroll
+        for (uint32_t j = 0; j < 4; j++)
+            if (n0 + i % OT + j < N) to[n0 + i % OT + j] = v[j];
+    }
+    cluster_sync();   // (until the others have read this CTA's sums)
 }
 
 // Backward through pooling and the convolution's weights: each thread one
@@ -893,6 +929,8 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
         if (!m->mg_ready) {   // once per model; the largest sizes', which all models share
             rc = cuda_err(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                4 * MgSmem(MG_MAXH, MG_MAXC).total));
+            if (rc == LX_OK)
+                rc = cuda_err(cudaFuncSetAttribute(k_outer, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             if (rc != LX_OK) return rc;
             m->mg_ready = true;
         }
@@ -902,9 +940,25 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
                                                          w + m->o_w1, w + m->o_b1, w + m->o_w2, w + m->o_b2, h1, dz, dh1,
                                                          g + m->o_emb, g + m->o_wc, g + m->o_bc, g + m->n_params);
         const uint32_t t1 = (MIN_ / OT) * ((H + OT - 1) / OT), t2n = ((H + OT - 1) / OT) * ((C + OT - 1) / OT);
-        k_outer<<<dim3(std::max(t1, t2n), (B + OSLICE - 1) / OSLICE, 2), 256, 0, s>>>(
-            B, mo, dh1, MIN_, H, g + m->o_w1, g + m->o_b1, h1, dz, H, C, g + m->o_w2, g + m->o_b2);
-        rc = cuda_err(cudaGetLastError());
+        // slices of 64 windows, of more where that makes over 16 (8 192 windows: 432 -> 446 us; up to 2 048 as before)
+        uint32_t slices = 1;
+        while (slices < OCLUSTER && slices * OSLICE < B) slices *= 2;
+        const uint32_t slice = ((B + slices - 1) / slices + OK - 1) / OK * OK;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(std::max(t1, t2n), slices, 2);
+        cfg.blockDim = dim3(256);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1] = {};
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1;
+        at[0].val.clusterDim.y = slices;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        rc = cuda_err(cudaLaunchKernelEx(&cfg, k_outer, B, slice, (const float *)mo, (const float *)dh1, (uint32_t)MIN_, H,
+                                         g + m->o_w1, g + m->o_b1, (const float *)h1, (const float *)dz, H, C, g + m->o_w2,
+                                         g + m->o_b2));
+        if (rc == LX_OK) rc = cuda_err(cudaGetLastError());
         if (rc == LX_OK && h_loss) {
             rc = cuda_err(cudaMemcpyAsync(h_loss, g + m->n_params, sizeof(float), cudaMemcpyDeviceToHost, s));
             if (rc == LX_OK) rc = cuda_err(cudaStreamSynchronize(s));
