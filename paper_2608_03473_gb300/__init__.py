@@ -379,8 +379,12 @@ def lx_ctx_last_kernel_ms(ctx: Ctx) -> float:
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
-        # the raw handle: building a Stream object takes 4.6 us, a fifth of a small call
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        # the raw handle, where this torch has the (undocumented) calls: building
+        # a Stream object takes 4.6 us, a fifth of a small call
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            return torch.cuda.current_stream().cuda_stream
     return int(getattr(stream, "cuda_stream", stream))
 
 
