@@ -130,19 +130,32 @@ def measured_peak_gbs():
         return 6800.0, "fallback"
 
 
+# The device code of each kernel that has a committed DRAM profile: its file and
+# the headers that hold parts of it.
+PROFILED = {"lex_rows_dram_512mib.md": ("rows.cu", "rows.cuh", "lookback.cuh", "devutil.cuh"),
+            "lex_warps_dram_512mib.md": ("lexwarp.cu", "lookback.cuh", "devutil.cuh")}
+
+
+def kernel_hash(profile):
+    """SHA-256 of the profiled kernel's files, one after the other."""
+    import hashlib
+    h = hashlib.sha256()
+    for f in PROFILED[profile]:
+        h.update(open(os.path.join(ROOT, "paper_2608_03473_gb300", "csrc", f), "rb").read())
+    return h.hexdigest()
+
+
 def profiled_traffic(workload_key):
     """DRAM bytes of one step's kernels from the committed ncu summaries, or
     None when the kernel source changed since the counters were taken: the
     entry-row kernels' first, then the warp-tile kernel's."""
-    import hashlib
     import re
-    for source, profile in (("rows.cu", "lex_rows_dram_512mib.md"), ("lexwarp.cu", "lex_warps_dram_512mib.md")):
+    for profile in PROFILED:
         try:
-            src = open(os.path.join(ROOT, "paper_2608_03473_gb300", "csrc", source), "rb").read()
+            h = kernel_hash(profile)
             text = open(os.path.join(ROOT, "profiles", profile)).read()
         except OSError:
             continue
-        h = hashlib.sha256(src).hexdigest()
         for key, val, sha in re.findall(r"<!-- traffic (\S+) (\d+) ([0-9a-f]{64}) -->", text):
             if key == workload_key and sha == h:
                 return int(val)
