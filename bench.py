@@ -162,6 +162,16 @@ def profiled_traffic(workload_key):
     return None
 
 
+# lx_ctx_debug_counts: the kernels of each count
+ROUTES = {"rows": "entry-row kernels", "warps": "warp-tile kernel", "tiles": "tile kernel",
+          "contexts": "entry contexts enumerated, entry-row kernel", "chunks": "chunks scanned from their contexts"}
+
+
+def kernels_run(before, after):
+    """The kernels that calls between two lx_ctx_debug_counts ran, in words."""
+    return ", ".join(ROUTES[k] for k in ROUTES if after[k] != before[k]) or "none"
+
+
 def cpu_cores():
     try:
         return len(os.sched_getaffinity(0))
@@ -729,26 +739,27 @@ def main():
         fmt = lambda m: [f"0x{b:02x}" for b in range(256) if m[b]]
         line["config"]["certified"] = {"exact": fmt(ex_mask), "modulo": fmt(mo_mask)}
         if not full:
-            # the same filtered stream under exact cuts: with no exact-certified
-            # byte, lx_lex cuts at certified two-byte windows (warp-tile kernel)
-            # where the token set has them, else enumerates entry contexts; its
-            # output must equal the modulo-cut output (both are pi_I(tok(w)))
+            # the same filtered stream under exact cuts: certified bytes, certified
+            # two-byte windows where there are none, or enumerated entry contexts;
+            # its output must equal the modulo-cut output (both are pi_I(tok(w)))
             x_k = torch.empty_like(d_k)
             x_l = torch.empty_like(d_l)
             win_ctx = lg.lx_tokenset_walk_table(ts, lg.LX_FILTERED_EXACT)[2].get("n_ctx", 0)
             x_ms = []
+            before = lg.lx_ctx_debug_counts(ctx)
             for i in range(5):
                 rcx, ntx, conx = lg.lx_lex(ctx, ts, d_in, lg.LX_FILTERED_EXACT, x_k, x_l, stream=stream)
                 if i >= 2:
                     x_ms.append(lg.lx_ctx_last_kernel_ms(ctx))
+            route = kernels_run(before, lg.lx_ctx_debug_counts(ctx))
             rc, nt3, con3 = lex_fn(ctx, ts, d_in, mode, d_k, d_l, stream=stream)
             same = (rcx == 0 and ntx == nt3 and conx == con3 and torch.equal(x_k[:ntx], d_k[:nt3])
                     and torch.equal(x_l[:ntx], d_l[:nt3]))
             line["exact_certificate"] = {
                 "mode": "LX_FILTERED_EXACT",
-                "path": "lx_lex (certified cuts)" if ex_mask.any() else
-                        ("lx_lex: no exact-certified byte; cuts at certified two-byte windows (warp-tile kernel)"
-                         if win_ctx else "lx_lex: no exact-certified byte, so the hybrid plan enumerates entry contexts"),
+                "path": "lx_lex (%s): %s" % (
+                    "certified bytes" if ex_mask.any() else "no exact-certified byte; certified two-byte windows"
+                    if win_ctx else "no exact-certified byte or window", route),
                 "window_contexts": win_ctx,
                 "kernel_ms": statistics.median(x_ms), "value": n / (statistics.median(x_ms) / 1e3) / 1e9,
                 "unit": "GB/s", "same_output_as_modulo": bool(same)}

@@ -1,5 +1,6 @@
 """bench.py's DRAM counters belong to all of a kernel's device code: the file
-and the headers that hold parts of it; an edit of any turns them into null."""
+and the headers that hold parts of it; an edit of any turns them into null.
+And the names of the kernels that a call ran."""
 
 import os
 import shutil
@@ -41,3 +42,10 @@ def test_every_header_with_device_code_counts(profile):
             if line.startswith('#include "') and line.split('"')[1].endswith(".cuh"):
                 todo.append(line.split('"')[1])
     assert seen == set(bench.PROFILED[profile])
+
+
+def test_kernels_run():
+    zero = {k: 0 for k in (*bench.ROUTES, "graphs")}
+    assert bench.kernels_run(zero, {**zero, "rows": 5}) == "entry-row kernels"
+    assert bench.kernels_run(zero, {**zero, "rows": 1, "warps": 1}) == "entry-row kernels, warp-tile kernel"
+    assert bench.kernels_run(zero, {**zero, "graphs": 1}) == "none"
