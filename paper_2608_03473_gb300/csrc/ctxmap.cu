@@ -620,6 +620,7 @@ int lex_contexts_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, u
     const size_t o_guess = al(o_nxt + T), o_bmap = al(o_guess + 2 * T);
     const size_t total = al(o_bmap + 4 * ((T + TOP_NT - 1) / TOP_NT));
     rc = grow(&c->e_dev, &c->e_dev_bytes, total);
+    if (rc == LX_E_NOMEM) return LX_ROWS;   // the chunks need a third of it
     if (rc != LX_OK) return rc;
     uint8_t *d = static_cast<uint8_t *>(c->e_dev);
     R.res = reinterpret_cast<RResult *>(d);

@@ -1203,6 +1203,7 @@ int lx::grow(void **p, size_t *have, size_t need)
     *have = 0;
     int rc = cuda_err(cudaMalloc(p, need));   // exactly what is asked: buffers are sized per call
     if (rc == LX_OK) *have = need;
+    else cudaGetLastError();   // (else the next launch's check would find it)
     return rc;
 }
 
@@ -1816,7 +1817,10 @@ int lx::grow_host(void **p, size_t *have, size_t need)
     if (*p) cudaFreeHost(*p);
     *p = nullptr;
     *have = 0;
-    if (cudaMallocHost(p, need) != cudaSuccess) return LX_E_NOMEM;
+    if (cudaMallocHost(p, need) != cudaSuccess) {
+        cudaGetLastError();
+        return LX_E_NOMEM;
+    }
     *have = need;
     return LX_OK;
 }

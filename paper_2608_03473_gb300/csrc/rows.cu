@@ -1030,6 +1030,7 @@ int rows_prepare(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uint64_t
     size_t *have = L.fused ? &c->small_bytes : &c->scratch_bytes;
     if (L.fused && *have < need) c->small_clean = false;
     rc = grow(buf, have, need);
+    if (rc == LX_E_NOMEM) return LX_ROWS;   // (what comes next may need less)
     if (rc != LX_OK) return rc;
     uint8_t *scr = static_cast<uint8_t *>(*buf);
     P.res = reinterpret_cast<RResult *>(scr);
@@ -1267,6 +1268,7 @@ int lex_batch_rows(lx_ctx *c, const std::vector<uint64_t> &sets_key, const lx_do
     void *od = c->b_dev, *oh = c->b_host;
     rc = grow(&c->b_dev, &c->b_dev_bytes, dev_total);
     if (rc == LX_OK) rc = grow_host(&c->b_host, &c->b_host_bytes, host_total);
+    if (rc == LX_E_NOMEM) return LX_ROWS;
     if (rc != LX_OK) return rc;
     const bool moved = od != c->b_dev || oh != c->b_host;
     uint8_t *dv = static_cast<uint8_t *>(c->b_dev), *hs = static_cast<uint8_t *>(c->b_host);

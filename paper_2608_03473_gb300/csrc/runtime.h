@@ -181,8 +181,8 @@ constexpr int LX_SPARSE = -100;   // internal status, never returned by the C AB
 bool warp_path_ok(const lx_tokenset *ts, int mode, const uint8_t *d_in);
 // Lexing from the entry rows of fixed slices (rows.cu; same contract as
 // lx_lex, any input alignment), for token sets with a synchronizing byte.
-// LX_ROWS: the entry rows were not found or do not fit together; the caller
-// lexes the input another way.
+// LX_ROWS: the entry rows were not found or do not fit together, or there is no
+// memory for the scratch; the caller lexes the input another way.
 // LX_FAR: only because synchronizing bytes (or, with rows given, the starts
 // from which they were found) lie too far apart.
 constexpr int LX_ROWS = -102;   // internal statuses, never returned by the C ABI
