@@ -94,9 +94,10 @@ template <int FORM>
 __device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool has)
 {
     uint32_t e = E.pre, w = P.guess;
+    bool hit = true;
     if (P.n_pat && has) {
         w = 0;
-        bool hit = false;
+        hit = false;
         while (!hit && w < GUESS_MAX && w < p) {   // 64 bytes at a time
             uint4 c[4];
 #pragma unroll
@@ -112,7 +113,7 @@ __device__ uint32_t guess_row(const GuessIn &P, const REnv &E, uint64_t p, bool 
             w += back;
         }
     }
-    bool todo = has, lost = false;
+    bool todo = has && (hit || w >= p), lost = false;   // (none in reach: nothing to walk from)
     while (__any_sync(0xffffffffu, todo)) {
         if (todo) {
             uint64_t a = p > w ? p - w : 0;
