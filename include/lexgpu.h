@@ -254,16 +254,20 @@ int lx_ctx_last_kernel_ms(lx_ctx *ctx, float *ms);
  *     table; every 32 to 256 bytes lexed from the row the scanner is in
  *     there) when the token set has an event-code walk table for the mode
  *     (lx_tokenset_walk_table) and a byte after which every run is in one
- *     row; for inputs they refuse, and other sets, the warp-tile kernel (every
- *     warp owns 6144-byte tiles) when there is a walk table and d_in is 16-byte
- *     aligned; the tile kernel (CTAs of 256 threads over 17408-byte tiles,
- *     per-lane token records) otherwise;
+ *     row; for inputs without such a byte for 8 KiB, entry contexts
+ *     (lx_lex_enumerative); for other inputs they refuse (a token backtracks
+ *     to before the slice it failed in), and other sets, the warp-tile kernel
+ *     (every warp owns 6144-byte tiles) when there is a walk table and d_in is
+ *     16-byte aligned; the tile kernel (CTAs of 256 threads over 17408-byte
+ *     tiles, per-lane token records) otherwise.  A set and mode whose inputs
+ *     are refused one after the other goes up to 15 calls without an attempt;
  *   LX_KERNEL_TILE: always the tile kernel;
  *   LX_KERNEL_WARP: always the warp-tile kernel; lx_lex returns LX_E_INVAL
  *     for a call it cannot serve.
  * Both produce the same stream (tests compare them).  Returns LX_E_INVAL
  * for another value.  lx_lex_host follows the same choice; lx_lex_batch
- * takes the one-launch warp-tile batch unless LX_KERNEL_TILE is set.
+ * takes a one-launch batch (of the warp-tile kernel with LX_KERNEL_WARP)
+ * unless LX_KERNEL_TILE is set.
  */
 #define LX_KERNEL_AUTO 0
 #define LX_KERNEL_TILE 1
@@ -392,10 +396,12 @@ int lx_lex_async(lx_ctx *ctx, const lx_tokenset *ts, const uint8_t *d_in, uint64
  * launches run in order on `stream`).  On the entry-row and warp-tile kernels
  * each piece is copied to a 16-byte aligned place and lexed into its own
  * output range, and its tokens are copied out behind the previous pieces';
- * if some piece is refused (entry rows that do not fit, certified bytes too
- * far apart, backtracking past the step budget), the whole input is copied
- * in again and lexed by lx_lex's plan.  Host buffers should be pinned for
- * full copy speed.  Returns after all copies have completed.
+ * pieces whose entry rows do not fit are lexed again by the warp-tile kernel,
+ * and where it refuses one too (certified bytes too far apart, backtracking
+ * past the step budget), or a piece has no synchronizing byte for 8 KiB, the
+ * whole input is copied in again and lexed by the rest of lx_lex's plan.
+ * Host buffers should be pinned for full copy speed.  Returns after all copies
+ * have completed.
  */
 int lx_lex_host(lx_ctx *ctx, const lx_tokenset *ts, const uint8_t *h_in, uint64_t n, int mode,
                 uint16_t *h_kinds, uint32_t *h_lens, uint64_t capacity, uint64_t *n_tokens,
@@ -549,10 +555,13 @@ int lx_model_train_step(lx_model *m, const uint16_t *d_windows, const uint16_t *
  * fix-up rounds that changed an entry, and the round after the judge), chunks
  * scanned again after the first round, judged = 1 when the judge ran.  Where
  * lx_lex_enumerative walks from every candidate context, the rounds run on
- * the chunks' entry-to-exit maps and nothing is scanned again; the stats are
- * the same.  Otherwise each scan also stages the chunk's kept tokens in
- * context scratch (6 bytes of device memory per input byte), so that the
- * settled chunks are copied to the output.
+ * the chunks' entry-to-exit maps and nothing is scanned again; the stats count
+ * as if it were (but for a chunk whose last token, wrongly entered or in a
+ * malformed input, fails beyond its end: a scan sees that, the map does not).
+ * Otherwise (d_in not 16-byte aligned, backtracking across slices, a lexing
+ * error in a later slice than its token began in) each scan also stages the
+ * chunk's kept tokens in context scratch (6 bytes of device memory per input
+ * byte), so that the settled chunks are copied to the output.
  */
 typedef struct {
     uint64_t chunks;
@@ -604,7 +613,7 @@ int lx_lex_speculative(lx_ctx *ctx, const lx_tokenset *ts, lx_model *model, cons
  * for a non-empty document), LX_E_MODE, LX_E_TOOBIG, LX_E_NOMEM, LX_E_CUDA,
  * LX_E_TIMEOUT; LX_E_CAPACITY when *n_total > capacity (results[] are
  * still filled, so the caller can size the buffers and call again).
- * Synchronizes `stream` before returning.
+ * Returns when its work on `stream` is done.
  */
 typedef struct {
     const uint8_t *data;   /* device pointer to the document's bytes       */

@@ -1,6 +1,7 @@
-// devutil.cuh -- device helpers shared by the lexing kernels (lex.cu,
-// lexwarp.cu): shared-memory access through 32-bit shared addresses, the
-// global timer, and the decoupled look-back over per-tile status words.
+// devutil.cuh -- device helpers shared by the lexing kernels (lex.cu, lexwarp.cu
+// and, through rows.cuh, rows.cu and ctxmap.cu): shared-memory access through
+// 32-bit shared addresses, the global timer, the status words of look-backs,
+// and lex.cu's one-level look-back over them (lookback.cuh has the others').
 // Not part of the C ABI.
 #pragma once
 

@@ -1390,10 +1390,12 @@ static int lex_device(lx_ctx *c, const lx_tokenset *ts, const uint8_t *d_in, uin
                       uint16_t *d_kinds, uint32_t *d_lens, uint64_t capacity, uint64_t *n_tokens,
                       uint64_t *consumed, cudaStream_t st, const LaunchCfg *force = nullptr, int refused = LX_OK)
 {
-    // Hybrid plan (Section 9): certified cuts where certified bytes occur;
-    // where the mode certifies no byte, or certified bytes turn out too far
-    // apart, entry contexts are enumerated instead (lx_lex_enumerative), so
-    // no call degenerates to one lane walking the input.
+    // Hybrid plan (Section 9): entry rows first, where the set has a
+    // synchronizing byte; then certified cuts where certified bytes occur;
+    // where the mode certifies no byte, or synchronizing or certified bytes
+    // turn out too far apart, entry contexts are enumerated instead, so that
+    // no call degenerates to one lane walking the input (but for stretches
+    // of more than 64 KiB whose bytes all have more than eight contexts).
     const bool can_enumerate = !force && c->kernel == LX_KERNEL_AUTO && ts->scan.status == LX_OK;
     const lx_tuned *tu = tuned_for(c, ts, mode);
     const bool tuned_tile = c->kernel == LX_KERNEL_AUTO && tu && tu->kernel == LX_KERNEL_TILE;

@@ -1,8 +1,9 @@
 // lexwarp.cu -- GB300 (sm_103a) certified-split lexing with warp-owned tiles,
 // for token sets with an event-code walk table (internal.h) and 16-byte aligned
 // inputs: lx_lex_async, LX_KERNEL_WARP, sets without a synchronizing byte (those
-// cut at two-byte windows) and the inputs that rows.cu hands over (a backtrack
-// to before a slice, no synchronizing byte for 8 KiB).
+// cut at two-byte windows) and what rows.cu hands over: a backtrack to before a
+// slice, and of batches also no synchronizing byte for 8 KiB (single inputs
+// without one go to ctxmap.cu).
 //
 // Every warp claims tiles of WT (6144) input bytes from a global counter and owns
 // them end to end; nothing but the one-time table staging synchronises the

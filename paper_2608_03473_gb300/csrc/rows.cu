@@ -26,7 +26,11 @@
 // Where every slice agrees from START at offset 0 on, the rows are the serial
 // scan's by induction.  A disagreement, an entry row that was not found or a
 // backtrack to before a slice stops the call (ERR_ROWS) and the caller
-// lexes the input another way; what was written is overwritten.
+// lexes the input another way; what was written is overwritten.  That costs up
+// to a pass: C-like text with 40 lines of tokens that backtrack, alone among
+// inputs that are taken, 2 MiB 80 us a call without the attempt, 140 with it, 64
+// MiB 230 and 405 (250 when lexwarp.cu came first); one after the other
+// (Refusals in runtime.h) they cost what they do without.
 //
 // Backtracking inside a slice (SLOW) is replayed by its lane (relex), and the
 // first lexing failure ends the stream (Corollary 1); a token that fails in a
