@@ -37,8 +37,8 @@
 // later slice than its own, with no accepting prefix (WalkTable::noacc: an open
 // string at the input's end), fails at the last event before.  Handing such
 // inputs on took two passes: JSON cut inside a string 107 -> 32 us a call at
-// 1.5 KB, 309 -> 135 at 64 MiB; for it, a register or two of spills more: 512
-// MiB of JSON 519.8 -> 522.2 us, 512 documents 362.7 -> 367.4.
+// 1.5 KB, 309 -> 135 at 64 MiB; what it adds to the others is a few bytes of
+// spills: 512 MiB of JSON 519.3 -> 519.9 us, 512 documents 365.0 -> 367.0.
 //
 // Against the chunks of lexwarp.cu, which start at a certified byte and run
 // on past their lane's bytes to the next one: no lane walks another's bytes
