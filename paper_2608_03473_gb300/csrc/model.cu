@@ -61,7 +61,7 @@ struct lx_model {
     float *act = nullptr;
     size_t act_floats = 0;
     uint16_t *win = nullptr;
-    bool mg_ready = false;          // k_mlp_grad may use its shared memory, k_outer its clusters
+    bool mg_ready = false;          // k_mlp_grad may use its shared memory
     float *h_g = nullptr;           // pinned: the gradient and the loss on their way to the caller
     int device = -1;
 };
@@ -534,11 +534,12 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
 
 // Weight gradients: G[M x N] = A^T D, A [B][M], D [B][N], and the column sums of
 // D (the bias) from the first row of tiles.  64 x 64 tiles, 4 x 4 per thread;
-// blockIdx.z: which of the two layers.  A cluster of CTAs shares a tile, each
-// one slice of the batch; their sums are added in the order of the slices,
-// each CTA its part of the tile from all of them, so that a gradient is the
-// same each time (adding them to G as they came was not).
-constexpr uint32_t OT = 64, OK = 16, OSLICE = 64, OCLUSTER = 16;
+// blockIdx.z: which of the two layers.  One cluster of CTAs shares a tile, or
+// two, each CTA one slice of the batch; a cluster adds its sums in the order of
+// the slices, each CTA its part of the tile from all of them, and the clusters
+// add theirs to the zeros in G, where the order of two does not matter: a
+// gradient is the same each time (adding each slice's as it came was not).
+constexpr uint32_t OT = 64, OK = 16, OSLICE = 64, OCLUSTER = 8;
 
 // The address of this CTA's shared word `a` in the cluster's CTA `rank`.
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank)
@@ -603,9 +604,10 @@ __global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const
         *reinterpret_cast<float4 *>(&part[(4 * ty + i) * OT + 4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
     if (tid < OT) part[OT * OT + tid] = sum;
     cluster_sync();
-    const uint32_t S = gridDim.y, base = (uint32_t)__cvta_generic_to_shared(part);   // the cluster's CTAs: all slices
+    const uint32_t S = gridDim.y > OCLUSTER ? gridDim.y / 2 : gridDim.y, rank = blockIdx.y % S;   // the cluster's CTAs
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(part);
     const uint32_t words = OT * OT + (m0 == 0 ? OT : 0);
-    for (uint32_t i = 4 * (blockIdx.y * 256 + tid); i < words; i += S * 1024) {
+    for (uint32_t i = 4 * (rank * 256 + tid); i < words; i += S * 1024) {
         float4 x[OCLUSTER];   // all loads first
 #pragma unroll
         for (uint32_t q = 0; q < OCLUSTER; q++)
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const
         if (i < OT * OT && m0 + i / OT >= M) continue;
 #pragma unroll
         for (uint32_t j = 0; j < 4; j++)
-            if (n0 + i % OT + j < N) to[n0 + i % OT + j] = v[j];
+            if (n0 + i % OT + j < N) atomicAdd(&to[n0 + i % OT + j], v[j]);
     }
     cluster_sync();   // (until the others have read this CTA's sums)
 }
@@ -948,8 +950,6 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
         if (!m->mg_ready) {   // once per model; the largest sizes', which all models share
             rc = cuda_err(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                4 * MgSmem(MG_MAXH, MG_MAXC).total));
-            if (rc == LX_OK)
-                rc = cuda_err(cudaFuncSetAttribute(k_outer, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             if (rc != LX_OK) return rc;
             m->mg_ready = true;
         }
@@ -959,10 +959,10 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
                                                          w + m->o_w1, w + m->o_b1, w + m->o_w2, w + m->o_b2, h1, dz, dh1,
                                                          g + m->o_emb, g + m->o_wc, g + m->o_bc, g + m->n_params);
         const uint32_t t1 = (MIN_ / OT) * ((H + OT - 1) / OT), t2n = ((H + OT - 1) / OT) * ((C + OT - 1) / OT);
-        // slices of 64 windows, of more where that makes over 16 (8 192 windows: 432 -> 446 us; up to 2 048 as before)
-        uint32_t slices = 1;
-        while (slices < OCLUSTER && slices * OSLICE < B) slices *= 2;
-        const uint32_t slice = ((B + slices - 1) / slices + OK - 1) / OK * OK;
+        // slices of 64 windows, of more where that makes over 16
+        const uint32_t slice = std::max(OSLICE, ((B + 2 * OCLUSTER - 1) / (2 * OCLUSTER) + OK - 1) / OK * OK);
+        const uint32_t ns = (B + slice - 1) / slice, cluster = ns > OCLUSTER ? (ns + 1) / 2 : ns;
+        const uint32_t slices = ns > OCLUSTER ? 2 * cluster : cluster;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(std::max(t1, t2n), slices, 2);
         cfg.blockDim = dim3(256);
@@ -970,7 +970,7 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
         cudaLaunchAttribute at[1] = {};
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = 1;
-        at[0].val.clusterDim.y = slices;
+        at[0].val.clusterDim.y = cluster;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
