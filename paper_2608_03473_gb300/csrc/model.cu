@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
                                                     const __nv_bfloat16 *w1, const __nv_bfloat16 *b1,
                                                     const __nv_bfloat16 *w2, const __nv_bfloat16 *b2, float *h1o,
                                                     float *dzo, float *dho, float *gemb, float *gwc, float *gbc,
-                                                    float *loss)
+                                                    float *lossw)
 {
     extern __shared__ __align__(16) float sm[];
     const MgSmem L(H, C);
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
         for (uint32_t c = lane; c < C; c += 32) se += expf(zr[MG * c] - mx);
         for (int o = 16; o; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
         const float lse = mx + logf(se);
-        if (lane == 0) atomicAdd(loss, (lse - (yb < C ? zr[MG * yb] : 0.0f)) / (float)B);
+        if (lane == 0) lossw[b0 + wid] = lse - (yb < C ? zr[MG * yb] : 0.0f);   // (k_outer takes the mean)
         __syncwarp();
         for (uint32_t c = lane; c < C; c += 32) {
             const float g = (expf(zr[MG * c] - lse) - (c == yb ? 1.0f : 0.0f)) / (float)B;
@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(MG_NT) k_mlp_grad(const uint16_t *win, const u
 // two, each CTA one slice of the batch; a cluster adds its sums in the order of
 // the slices, each CTA its part of the tile from all of them, and the clusters
 // add theirs to the zeros in G, where the order of two does not matter: a
-// gradient is the same each time (adding each slice's as it came was not).
+// gradient is the same each time (adding each slice's as it came was not).  A CTA past the tiles
+// takes the mean of the windows' losses, in 64 bits.
 constexpr uint32_t OT = 64, OK = 16, OSLICE = 64, OCLUSTER = 8;
 
 // The address of this CTA's shared word `a` in the cluster's CTA `rank`.
@@ -559,7 +560,8 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const float *A0, const float *D0, uint32_t M0, uint32_t N0,
+__global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const float *lossw,
+                                               float *loss, const float *A0, const float *D0, uint32_t M0, uint32_t N0,
                                                float *G0, float *s0, const float *A1, const float *D1, uint32_t M1,
                                                uint32_t N1, float *G1, float *s1)
 {
@@ -568,9 +570,22 @@ __global__ void __launch_bounds__(256) k_outer(uint32_t B, uint32_t slice, const
     float *G = one ? G1 : G0, *cs = one ? s1 : s0;
     const uint32_t M = one ? M1 : M0, N = one ? N1 : N0;
     const uint32_t nt = (N + OT - 1) / OT, m0 = (blockIdx.x / nt) * OT, n0 = (blockIdx.x % nt) * OT;
-    if (m0 >= M) return;   // (the whole cluster)
+    const uint32_t tid = threadIdx.x;
+    if (m0 >= M) {   // (the whole cluster)
+        if (blockIdx.x == gridDim.x - 1 && blockIdx.y + blockIdx.z == 0) {
+            __shared__ double red[8];
+            double l = 0.0;
+            for (uint32_t i = tid; i < B; i += 256) l += (double)lossw[i];
+            for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if ((tid & 31u) == 0) red[tid >> 5] = l;
+            __syncthreads();
+            l = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+            if (tid == 0) *loss = (float)(l / (double)B);
+        }
+        return;
+    }
     __shared__ __align__(16) float As[OK][OT], Ds[OK][OT], part[OT * OT + OT];
-    const uint32_t tid = threadIdx.x, tx = tid & 15u, ty = tid >> 4;
+    const uint32_t tx = tid & 15u, ty = tid >> 4;
     const uint32_t k0 = min(B, blockIdx.y * slice), k1 = min(B, k0 + slice);
     float acc[4][4], sum = 0.0f;
 #pragma unroll
@@ -957,14 +972,14 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
         cudaMemsetAsync(g, 0, sizeof(float) * (m->n_params + 1), s);
         k_mlp_grad<<<(B + MG - 1) / MG, MG_NT, smem, s>>>(d_win, d_y, B, H, C, mo, m->arg, w + m->o_emb, w + m->o_wc,
                                                          w + m->o_w1, w + m->o_b1, w + m->o_w2, w + m->o_b2, h1, dz, dh1,
-                                                         g + m->o_emb, g + m->o_wc, g + m->o_bc, g + m->n_params);
+                                                         g + m->o_emb, g + m->o_wc, g + m->o_bc, dm);   // dm: here the windows' losses
         const uint32_t t1 = (MIN_ / OT) * ((H + OT - 1) / OT), t2n = ((H + OT - 1) / OT) * ((C + OT - 1) / OT);
         // slices of 64 windows, of more where that makes over 16
         const uint32_t slice = std::max(OSLICE, ((B + 2 * OCLUSTER - 1) / (2 * OCLUSTER) + OK - 1) / OK * OK);
         const uint32_t ns = (B + slice - 1) / slice, cluster = ns > OCLUSTER ? (ns + 1) / 2 : ns;
         const uint32_t slices = ns > OCLUSTER ? 2 * cluster : cluster;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(std::max(t1, t2n), slices, 2);
+        cfg.gridDim = dim3(std::max(t1, t2n) + 1, slices, 2);   // (the last: the loss)
         cfg.blockDim = dim3(256);
         cfg.stream = s;
         cudaLaunchAttribute at[1] = {};
@@ -974,7 +989,7 @@ int model_pass(lx_model *m, const uint16_t *d_win, const uint16_t *d_y, uint32_t
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        rc = cuda_err(cudaLaunchKernelEx(&cfg, k_outer, B, slice, (const float *)mo, (const float *)dh1, (uint32_t)MIN_, H,
+        rc = cuda_err(cudaLaunchKernelEx(&cfg, k_outer, B, slice, (const float *)dm, g + m->n_params, (const float *)mo, (const float *)dh1, (uint32_t)MIN_, H,
                                          g + m->o_w1, g + m->o_b1, (const float *)h1, (const float *)dz, H, C, g + m->o_w2,
                                          g + m->o_b2));
         if (rc == LX_OK) rc = cuda_err(cudaGetLastError());

@@ -1,7 +1,8 @@
-"""The dense layers' gradients (W1, b1, W2, b2) are the same each time they are
-computed: their sums over the batch have an order of their own, whatever the
-order in which the slices of the batch finish.  (The embedding's and the
-filters' gradients and the loss are summed as they come.)"""
+"""The dense layers' gradients (W1, b1, W2, b2) and the loss are the same each
+time they are computed: their sums over the batch have an order of their own,
+whatever the order in which the slices of the batch finish.  (The embedding's
+and the filters' gradients are summed as they come, and the loss as well past
+256 hidden units.)"""
 
 import numpy as np
 import pytest
@@ -25,7 +26,15 @@ def test_dense_gradients_repeat(lexlib, batch, hidden, contexts):
     dw = torch.from_numpy(win.astype(np.int16)).cuda()
     dy = torch.from_numpy(rng.integers(0, contexts, size=batch).astype(np.int16)).cuda()
     dense = sum(OM.sizes(hidden, contexts)[:3])
-    first = m.gradient(dw, dy)[0][dense:].copy()
+    first, loss = m.gradient(dw, dy)
+    first = first[dense:].copy()
     assert np.all(np.isfinite(first)) and np.any(first != 0)
     for _ in range(30):
-        assert np.array_equal(m.gradient(dw, dy)[0][dense:], first)
+        g, l = m.gradient(dw, dy)
+        assert np.array_equal(g[dense:], first)
+        assert hidden > 256 or l == loss
+    if hidden <= 256:   # a mean in 64 bits of losses that are each within a few units in the last place
+        z, _ = OM.forward(OM.to_bf16(m.get_params().astype(np.float64)), win, hidden, contexts)
+        zmax = z.max(1, keepdims=True)
+        want = np.mean(np.log(np.exp(z - zmax).sum(1)) + zmax[:, 0] - z[np.arange(batch), dy.cpu().numpy()])
+        assert abs(loss - want) <= 4 * np.spacing(np.float32(want))
