@@ -2168,7 +2168,8 @@ extern "C" int lx_autotune(lx_ctx *c, const lx_tokenset *ts, int mode, const uin
         }
     }
     c->warps = saved_warps;
-    // the entry-row kernels, when they apply and do not refuse the sample
+    // the entry-row kernels, when they apply and do not refuse the sample (one
+    // without a synchronizing byte for 8 KiB goes on to the contexts)
     float best_r = 1e30f;
     if (rc == LX_OK && ts->scan.status == LX_OK && rows_path_ok(ts, mode)) {
         uint64_t nt = 0, con = 0;
@@ -2177,6 +2178,9 @@ extern "C" int lx_autotune(lx_ctx *c, const lx_tokenset *ts, int mode, const uin
         for (int rep = 0; rep < 4 && r == LX_OK; rep++) {
             cudaEventRecord(e0, st);
             r = lex_rows_device(c, ts, d_sample, n, mode, d_kinds, d_lens, capacity, &nt, &con, st);
+            if (r == LX_FAR)
+                r = lex_contexts_device(c, ts, d_sample, n, mode, d_kinds, d_lens, capacity, &nt, &con, st, nullptr,
+                                        nullptr);
             cudaEventRecord(e1, st);
             if (r == LX_E_CAPACITY) r = LX_OK;
             if (r != LX_OK) break;

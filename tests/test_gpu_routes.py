@@ -396,3 +396,21 @@ def test_autotune_times_every_kernel(lg, off):
                                      torch.zeros(small.size, dtype=torch.int32))
         assert rc == 0 and (nt, con) == (expected("clike", small, 2)[0].size, expected("clike", small, 2)[2])
         assert ("rows" in ran(lg, ctx, before)) == rows   # the same choice
+
+
+@pytest.mark.parametrize("off", [0, 5])
+def test_autotune_with_a_long_line(lg, off):
+    # the plan that a call on such a sample takes (the entry rows, then the contexts) is what is timed: C-like
+    # text on one line, which the other kernels walk with one lane
+    import torch
+    name, mode = "clike", 2
+    lines = corpus.generate(name, 300_000, seed=92).tobytes().split(b"\n")
+    w = np.frombuffer(b" ".join(x for x in lines if not any(c in x for c in (b'"', b"'", b"//"))), np.uint8)
+    ctx, ts = lg.lx_ctx_create(), tset(lg, name)
+    d = torch.zeros(w.size + 16, dtype=torch.uint8, device="cuda")[off:off + w.size]
+    d.copy_(torch.from_numpy(w.copy()))
+    k = torch.zeros(w.size, dtype=torch.int16, device="cuda")
+    l = torch.zeros(w.size, dtype=torch.int32, device="cuda")
+    assert lg.lx_autotune(ctx, ts, mode, d, k, l) == 0
+    lex = lambda ts, d, k, l: lg.lx_lex(ctx, ts, d, mode, k, l)   # noqa: E731
+    assert call(lg, ctx, name, w, mode, lex, off, ts=ts) == {"rows": 1, "contexts": 1}
